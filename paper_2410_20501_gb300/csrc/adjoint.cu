@@ -27,6 +27,7 @@ __device__ __forceinline__ void tsc_dweights(float d, float w[3]) {
 // acceleration through the kick (x' = x + dt_drift v').
 __global__ void k_adj_accel(const float* __restrict__ xbar_out, const float* __restrict__ vbar_out, int64_t np,
                             float dt_kick, float dt_drift, float* __restrict__ abar) {
+  pdl_entry();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 3 * np;
        i += (int64_t)gridDim.x * blockDim.x)
     abar[i] = dt_kick * fmaf(dt_drift, __ldg(xbar_out + i), __ldg(vbar_out + i));
@@ -46,6 +47,7 @@ template <> struct DStencil<7> {
 // phi_bar = sum_d (1/h) sum_q c_q (g_bar_d(+q) - g_bar_d(-q)).
 template <int ORDER>
 __global__ void k_divergence(const float* __restrict__ gbar, float* __restrict__ phibar, int log2n, float inv_h) {
+  pdl_entry();
   const int64_t N = (int64_t)1 << (3 * log2n);
   const int m = (1 << log2n) - 1;
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < N; c += (int64_t)gridDim.x * blockDim.x) {
@@ -77,6 +79,7 @@ __global__ void __launch_bounds__(256) k_pos_grad(const uint32_t* __restrict__ X
                                                   const float* __restrict__ vbar_out, float dt_drift,
                                                   const uint32_t* __restrict__ perm, float* __restrict__ xbar_in,
                                                   float* __restrict__ vbar_in) {
+  pdl_entry();
   const int m = (1 << log2n) - 1, sh = 32 - log2n;
   const int64_t N = (int64_t)1 << (3 * log2n);
   const float nf = (float)(1 << log2n);

@@ -27,6 +27,7 @@ __global__ void __launch_bounds__(T * T * T) k_deposit(const uint32_t* __restric
                                                        const uint32_t* __restrict__ cellstart, int n,
                                                        int log2n, const float* __restrict__ vals, float scale,
                                                        float* __restrict__ rho, double* __restrict__ partial) {
+  pdl_entry();
   constexpr int E = T + 2, S = E * E * E, NT = T * T * T;
   extern __shared__ float M[];  // [27][S]
   __shared__ double wsum[NT / 32];
@@ -146,6 +147,7 @@ __global__ void __launch_bounds__(DTHREADS, 2) k_deposit_stream(const uint32_t* 
                                                                 float scale, float* __restrict__ rho,
                                                                 double* __restrict__ partial,
                                                                 const float* __restrict__ crowd) {
+  pdl_entry();
   using G = DepositStage<VALS>;
   constexpr int KP = G::KP, NC = G::NC, PL = DPL;
   extern __shared__ float sm[];
@@ -343,6 +345,7 @@ __global__ void __launch_bounds__(256) k_group_moments(const uint32_t* __restric
                                                        const uint32_t* __restrict__ cellstart,
                                                        const uint32_t* __restrict__ list, int log2n,
                                                        const float* __restrict__ vals, float* __restrict__ crowd) {
+  pdl_entry();
   static_assert(G == 8 || G == 16, "group width");
   constexpr int PERW = 32 / G, NOUT = (27 + G - 1) / G;
   const uint32_t ncells = list[0];
@@ -395,6 +398,7 @@ __global__ void __launch_bounds__(256) k_medium_moments(const uint32_t* __restri
                                                         const uint32_t* __restrict__ cellstart,
                                                         const uint32_t* __restrict__ runs, int log2n,
                                                         const float* __restrict__ vals, float* __restrict__ crowd) {
+  pdl_entry();
   const uint32_t ntot = runs[0];
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t warps = gridDim.x * 8;
@@ -434,6 +438,7 @@ __global__ void __launch_bounds__(CT) k_crowded_moments(const uint32_t* __restri
                                                         const uint32_t* __restrict__ cellstart,
                                                         const uint32_t* __restrict__ bigs, int log2n,
                                                         const float* __restrict__ vals, float* __restrict__ crowd) {
+  pdl_entry();
   __shared__ float part[CT / 32][27];
   const uint32_t nruns = bigs[0];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -472,6 +477,7 @@ inline void deposit_stream_plan(int n, int* chunk, int* nitems) {
 // Sum of a float32 array: per-block float64 partials (fixed order).
 __global__ void __launch_bounds__(256) k_sum_partials(const float* __restrict__ f, int64_t count,
                                                       double* __restrict__ partial) {
+  pdl_entry();
   __shared__ double wsum[8];
   float v = 0.0f, c = 0.0f;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count;
@@ -496,6 +502,7 @@ __global__ void __launch_bounds__(256) k_sum_partials(const float* __restrict__ 
 __global__ void __launch_bounds__(1024) k_reduce_partials(const double* __restrict__ partial,
                                                           int64_t count, int64_t stride, int nout,
                                                           double scale, double* __restrict__ out) {
+  pdl_entry();
   __shared__ double red[1024];
   for (int k = blockIdx.x; k < nout; k += gridDim.x) {   // one output per block (fixed order within it)
     double t = 0.0;

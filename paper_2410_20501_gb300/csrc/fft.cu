@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(lines_per_block<M>() * (M / 8)) k_fft_z_r2c(co
                                                                               const double* __restrict__ mean,
                                                                               float2* __restrict__ out,
                                                                               int64_t rows) {
+  pdl_entry();
   constexpr int LB = lines_per_block<M>(), TPL = M / 8, LP = M + 1, H = M + 1, n = 2 * M;
   __shared__ float2 s[LB * LP];
   const int64_t row0 = (int64_t)blockIdx.x * LB;
@@ -194,6 +195,7 @@ template <int M>
 __global__ void __launch_bounds__(lines_per_block<M>() * (M / 8)) k_fft_z_c2r(const float2* __restrict__ in,
                                                                               float* __restrict__ out,
                                                                               int64_t rows) {
+  pdl_entry();
   constexpr int LB = lines_per_block<M>(), TPL = M / 8, LP = M + 1, H = M + 1, n = 2 * M;
   __shared__ float2 s[LB * LP];
   const int64_t row0 = (int64_t)blockIdx.x * LB;
@@ -259,6 +261,7 @@ enum ColMode { FWD = 0, INVT = 1, FWDMUL = 2, MULINV = 3, SOLVE = 4 };
 template <int L, int AXIS, int MODE>
 __global__ void __launch_bounds__(lines_per_block<L>() * (L / 8)) k_fft_cols(const float2* in, float2* out,
                                                                              int ntiles, Mult mu) {
+  pdl_entry();
   constexpr bool MUL = MODE == FWDMUL || MODE == MULINV || MODE == SOLVE;
   constexpr int TW = lines_per_block<L>(), TPL = L / 8, LP = L + 1, n = L, H = n / 2 + 1;
   __shared__ float2 s[TW * LP];
@@ -400,6 +403,7 @@ pm_status launch_fft_poisson(const float* rho, const double* mean, float* phi, f
 // S = phi_xx phi_yy + phi_xx phi_zz + phi_yy phi_zz (H: the three diagonal
 // second derivatives, planes of N), then S -= T^2 for each mixed derivative T.
 __global__ void k_lpt_diag(const float* __restrict__ H, float* __restrict__ S, int64_t N) {
+  pdl_entry();
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < N; c += (int64_t)gridDim.x * blockDim.x) {
     const float a = H[c], b = H[N + c], d = H[2 * N + c];
     S[c] = fmaf(a, b, fmaf(a, d, b * d));
@@ -407,6 +411,7 @@ __global__ void k_lpt_diag(const float* __restrict__ H, float* __restrict__ S, i
 }
 
 __global__ void k_lpt_sub_sq(const float* __restrict__ T, float* __restrict__ S, int64_t N) {
+  pdl_entry();
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < N; c += (int64_t)gridDim.x * blockDim.x)
     S[c] = fmaf(-T[c], T[c], S[c]);
 }
@@ -417,6 +422,7 @@ __global__ void k_lpt_sub_sq(const float* __restrict__ T, float* __restrict__ S,
 // V = v1 Psi1 + v2 Psi2.  V holds Psi1_d on entry; psi2 may be NULL (1LPT).
 __global__ void k_lpt_combine(const float* __restrict__ psi2, float* __restrict__ V, uint32_t* __restrict__ X,
                               int d, int log2n, float d1, float e2, float v1, float v2) {
+  pdl_entry();
   const int64_t N = (int64_t)1 << (3 * log2n);
   const int m = (1 << log2n) - 1;
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x) {

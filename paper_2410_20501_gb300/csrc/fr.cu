@@ -180,6 +180,7 @@ __device__ __forceinline__ float fr_update(float ec, const float nb[6], float bv
 template <int NH>
 __global__ void __launch_bounds__(256) k_fr_sweep(float* __restrict__ e, Src b, int log2n, int colour, float beta,
                                                   float kappa, float q) {
+  pdl_entry();
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (1u << (3 * log2n - 1))) return;
   {   // the box of a batched launch
@@ -217,6 +218,7 @@ __device__ __forceinline__ float fr_flux(float enb, float ec) {
 template <int NH, bool BOXES>
 __global__ void k_fr_restrict(const float* __restrict__ e, Src b, int log2n, float alpha, float kappa,
                               float* __restrict__ eH, float* __restrict__ rH, float* __restrict__ bH) {
+  pdl_entry();
   const int lc = log2n - 1, mc = (1 << lc) - 1;
   const int64_t total = (int64_t)1 << (3 * lc);
   if (BOXES) {   // the box of a batched launch
@@ -271,6 +273,7 @@ __global__ void k_fr_restrict(const float* __restrict__ e, Src b, int log2n, flo
 template <int NH>
 __global__ void k_fr_coarse_op(const float* __restrict__ eH, float* __restrict__ bH, int log2n, float alpha,
                                float kappa) {
+  pdl_entry();
   const uint32_t m = (1u << log2n) - 1;
   const uint32_t quads = 1u << (3 * log2n - 2);
   {   // the box of a batched launch
@@ -312,6 +315,7 @@ __global__ void k_fr_coarse_op(const float* __restrict__ eH, float* __restrict__
 template <int NH>
 __global__ void __launch_bounds__(256) k_fr_norm(const float* __restrict__ e, Src b, int log2n, float alpha,
                                                  float kappa, double* __restrict__ partial) {
+  pdl_entry();
   __shared__ double scratch[32];
   const float mean = load_mean(b);
   const int m = (1 << log2n) - 1;
@@ -337,6 +341,7 @@ template <int NH>
 __global__ void __launch_bounds__(1024) k_fr_coarse(float* __restrict__ e, Src b, int log2n, float alpha,
                                                     float beta, float kappa, float q, int max_sweeps,
                                                     float drop) {
+  pdl_entry();
   __shared__ float se[4096], sbv[4096];
   __shared__ float2 scratch[33];
   const int n = 1 << log2n, m = n - 1, N = n * n * n;

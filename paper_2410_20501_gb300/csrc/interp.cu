@@ -46,6 +46,7 @@ template <> struct Stencil<7> {
 template <int ORDER, bool FR>
 __global__ void k_gradient(const float* __restrict__ phi, const float* __restrict__ eps, float alpha,
                            float* __restrict__ g, int log2n, float inv_h, int nh) {
+  pdl_entry();
   const int m = (1 << log2n) - 1;
   const int64_t total = (int64_t)1 << (3 * log2n);
   phi += (int64_t)blockIdx.z * total;          // the box of a batched launch
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(GNT) k_gradient_stream(const float* __restrict
                                                         const float* __restrict__ eps, float alpha,
                                                         float* __restrict__ g, int log2n, float inv_h,
                                                         int chunk, int nitems, int nh) {
+  pdl_entry();
   constexpr int R = Stencil<ORDER>::R, W = 2 * R + 1, EY = GTY + 2 * R, EZ = GTZ + 2 * R, PL = EY * EZ;
   extern __shared__ float P[];   // [W][EY][EZ]
   const int n = 1 << log2n, m = n - 1;
@@ -148,6 +150,7 @@ __global__ void __launch_bounds__(256) k_interp_kdk(const float* __restrict__ g,
                                                     const float* __restrict__ dtk_box,
                                                     const float* __restrict__ dtd_box,
                                                     float2* __restrict__ blockmax) {
+  pdl_entry();
   const int m = (1 << log2n) - 1, sh = 32 - log2n;
   const int64_t N = (int64_t)1 << (3 * log2n);
   // the box of a batched launch: its grid and its particles p0 .. p0 + np_box
@@ -373,6 +376,7 @@ __global__ void __launch_bounds__(I_THREADS) k_force_interp_stream(
     uint32_t* __restrict__ Xo, float* __restrict__ Vo, uint32_t* __restrict__ ids_out, float dt_kick,
     float drift_scale, int mode, const float* __restrict__ dtk_box, const float* __restrict__ dtd_box,
     float2* __restrict__ blockmax) {
+  pdl_entry();
   constexpr int R = Stencil<ORDER>::R, H = R + 1, PEY = IT_Y + 2 * H, PEZ = IT_Z + 2 * H, PPL = PEY * PEZ,
                 PS = 2 * R + 2, PL_T = (PPL + I_THREADS - 1) / I_THREADS;
   extern __shared__ float fsm[];
@@ -485,6 +489,7 @@ constexpr size_t force_interp_smem() {
 // (float bits of non-negative values order like unsigned integers).
 __global__ void __launch_bounds__(256) k_speed_max(const float* __restrict__ V, int64_t np,
                                                    float2* __restrict__ blockmax) {
+  pdl_entry();
   __shared__ unsigned wv[8];
   unsigned mv = 0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
@@ -504,6 +509,7 @@ __global__ void __launch_bounds__(256) k_speed_max(const float* __restrict__ V, 
 // (float64); one block.
 __global__ void __launch_bounds__(1024) k_max_pairs(const float2* __restrict__ v, int64_t count,
                                                     double* __restrict__ out) {
+  pdl_entry();
   __shared__ unsigned wa[32], wv[32];
   unsigned ma = 0, mv = 0;
   for (int64_t i = threadIdx.x; i < count; i += blockDim.x) {

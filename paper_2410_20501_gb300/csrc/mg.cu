@@ -55,6 +55,7 @@ __device__ __forceinline__ void load_nb(const float* __restrict__ u, int i, int 
 
 // u = -h^2 f / 6 (Eq. multigrid_initial_guess).
 __global__ void k_jacobi_guess(float* __restrict__ u, Src f, int64_t count, float h2) {
+  pdl_entry();
   u += (int64_t)blockIdx.z * count;
   f = box_src(f, count);
   const float mean = load_mean(f);
@@ -65,6 +66,7 @@ __global__ void k_jacobi_guess(float* __restrict__ u, Src f, int64_t count, floa
 
 // u *= a (per box: ab[box] if ab is set).
 __global__ void k_scale(float* __restrict__ u, int64_t count, float a, const float* __restrict__ ab) {
+  pdl_entry();
   u += (int64_t)blockIdx.z * count;
   if (ab) a = __ldg(ab + blockIdx.z);
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < count;
@@ -78,6 +80,7 @@ __global__ void k_scale(float* __restrict__ u, int64_t count, float a, const flo
 // nothing, the black pass ignores its own old value.
 __global__ void k_rb_sweep(float* __restrict__ u, Src f, int log2n, int colour, PoissonUpdate upd,
                            int nb_old, int own_old, int zero) {
+  pdl_entry();
   const int m = (1 << log2n) - 1, half = log2n - 1;
   u += (int64_t)blockIdx.z << (3 * log2n);
   f = box_src(f, (int64_t)1 << (3 * log2n));
@@ -115,6 +118,7 @@ __global__ void k_rb_sweep(float* __restrict__ u, Src f, int log2n, int colour, 
 template <bool COMP>
 __global__ void k_resid_restrict(const float* __restrict__ u, Src f, int log2n, float inv_h2,
                                  float* __restrict__ fc) {
+  pdl_entry();
   const int lc = log2n - 1, mc = (1 << lc) - 1;
   u += (int64_t)blockIdx.z << (3 * log2n);
   f = box_src(f, (int64_t)1 << (3 * log2n));
@@ -183,6 +187,7 @@ __global__ void k_resid_restrict(const float* __restrict__ u, Src f, int log2n, 
 // residual): partial[blockIdx] and partial[gridDim + blockIdx].
 __global__ void __launch_bounds__(256) k_resid_norm(const float* __restrict__ u, Src f, int log2n,
                                                     float inv_h2, double* __restrict__ partial) {
+  pdl_entry();
   __shared__ double scratch[32];
   const float mean = load_mean(f);
   const int m = (1 << log2n) - 1;
@@ -227,6 +232,7 @@ __device__ __forceinline__ void block_sum_f64(double* out, double v, double* scr
 __global__ void __launch_bounds__(256) k_resid_f64(const double* __restrict__ u, const float* __restrict__ f,
                                                    const double* __restrict__ fmean, int log2n, double inv_h2,
                                                    float* __restrict__ r, double* __restrict__ partial) {
+  pdl_entry();
   __shared__ double scratch[32];
   const double mean = *fmean;
   const int m = (1 << log2n) - 1;
@@ -251,6 +257,7 @@ __global__ void __launch_bounds__(256) k_resid_f64(const double* __restrict__ u,
 
 // u += e (float64 iterate, float32 correction).
 __global__ void k_add_correction_f64(double* __restrict__ u, const float* __restrict__ e, int64_t count) {
+  pdl_entry();
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < count; c += (int64_t)gridDim.x * blockDim.x)
     u[c] += (double)__ldg(e + c);
 }
@@ -263,6 +270,7 @@ __global__ void k_add_correction_f64(double* __restrict__ u, const float* __rest
 // x, parent (weight 3/4) before neighbour (1/4), in fused multiply-adds.
 __global__ void k_prolong_correct(float* __restrict__ u, const float* __restrict__ uc,
                                   const float* __restrict__ uc2, int log2n) {
+  pdl_entry();
   const int lc = log2n - 1, mc = (1 << lc) - 1;
   const int64_t total = (int64_t)1 << (3 * lc);
   u += (int64_t)blockIdx.z << (3 * log2n);
@@ -334,6 +342,7 @@ __global__ void k_prolong_correct(float* __restrict__ u, const float* __restrict
 __global__ void __launch_bounds__(1024) k_mg_coarse(float* __restrict__ u, Src f, int log2n, float h2,
                                                     float omega, int max_sweeps, float drop,
                                                     int zero_guess) {
+  pdl_entry();
   __shared__ float su[4096], sf[4096];
   __shared__ float2 scratch[33];
   const int n = 1 << log2n, m = n - 1, N = n * n * n, npair = N >> 1;

@@ -93,6 +93,7 @@ template <class Upd, int MINB>
 __global__ void __launch_bounds__(kQuadThreads, MINB) k_rb_fused4(const float* __restrict__ uin,
                                                                  float* __restrict__ uout, Src f, int log2n,
                                                                  int chunk, int zero, int first, Upd upd) {
+  pdl_entry();
   constexpr int T = kFusedT, EC = kFusedEC, PL = kFusedPL, R = kFusedRing, RO = kFusedRingOld;
   extern __shared__ float4 fsm4[];
   float* Old = reinterpret_cast<float*>(fsm4);   // [RO][ER][EC]

@@ -86,6 +86,7 @@ template <int S, class Upd>
 __global__ void __launch_bounds__(kStreamThreads) k_rb_stream(const float* __restrict__ uin,
                                                              float* __restrict__ uout, Src f, int log2n,
                                                              int chunk, int nitems, int zero_guess, Upd upd) {
+  pdl_entry();
   using G = StreamGeom<S>;
   constexpr int TY = kStreamTY, TZ = kStreamTZ, H = G::H, EY = G::EY, EZ = G::EZ, RW = G::RW;
   constexpr int PL = G::PL, W = G::W, WF = G::WF, NT = kStreamThreads;

@@ -46,6 +46,7 @@ template <bool BOX>
 __global__ void __launch_bounds__(KT) k_cell_count(const uint32_t* __restrict__ X, int64_t np, int log2n,
                                                    int64_t np_box, uint2* __restrict__ kr,
                                                    uint32_t* __restrict__ cnt) {
+  pdl_entry();
   const int64_t i0 = blockIdx.x * (int64_t)(KT * CI) + threadIdx.x;
   const int sh = 32 - log2n;
   const uint32_t lane = threadIdx.x & 31;
@@ -86,6 +87,7 @@ __global__ void __launch_bounds__(KT) k_cell_count(const uint32_t* __restrict__ 
 __global__ void __launch_bounds__(KT) k_cell_scatter(const uint2* __restrict__ kr, int64_t np,
                                                      const uint32_t* __restrict__ cellstart,
                                                      uint32_t* __restrict__ perm) {
+  pdl_entry();
   const int64_t i0 = blockIdx.x * (int64_t)(KT * CI) + threadIdx.x;
   uint2 t[CI];
   uint32_t base[CI];
@@ -118,6 +120,7 @@ __global__ void __launch_bounds__(KT) k_cell_order(const uint32_t* __restrict__ 
                                                    uint32_t* __restrict__ perm, uint32_t* __restrict__ smalls,
                                                    uint32_t* __restrict__ meds, uint32_t* __restrict__ runs,
                                                    uint32_t* __restrict__ bigs) {
+  pdl_entry();
   __shared__ uint32_t wtot[4][KT / 32];
   __shared__ uint32_t lbase[4];
   const int64_t c0 = (blockIdx.x * (int64_t)KT + threadIdx.x) * OC;
@@ -205,6 +208,7 @@ template <int G>
 __global__ void __launch_bounds__(KT) k_cell_order_med(const uint32_t* __restrict__ cellstart,
                                                        const uint32_t* __restrict__ list,
                                                        uint32_t* __restrict__ perm) {
+  pdl_entry();
   constexpr int PERW = 32 / G;
   const uint32_t nlist = list[0];
   const uint32_t lane = threadIdx.x & 31, g = lane & (G - 1);
@@ -256,6 +260,7 @@ __device__ __forceinline__ void warp_rank_sort(const uint32_t* buf, uint32_t m, 
 __global__ void __launch_bounds__(WT) k_cell_order_warp(const uint32_t* __restrict__ cellstart,
                                                         const uint32_t* __restrict__ runs,
                                                         uint32_t* __restrict__ perm) {
+  pdl_entry();
   __shared__ uint32_t sbuf[WT / 32][kWarpRun];
   const uint32_t nruns = runs[0];
   const uint32_t lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -318,6 +323,7 @@ __global__ void __launch_bounds__(LT) k_cell_order_long(const uint32_t* __restri
                                                         const uint32_t* __restrict__ runs,
                                                         uint32_t* __restrict__ perm,
                                                         uint32_t* __restrict__ scratch) {
+  pdl_entry();
   __shared__ uint32_t sv[LCH];
   const uint32_t nruns = runs[0];
   for (uint32_t q = blockIdx.x; q < nruns; q += gridDim.x) {
@@ -406,6 +412,7 @@ __device__ __forceinline__ void scan_load(const uint32_t* __restrict__ a, int64_
 
 __global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const uint32_t* __restrict__ a, int64_t len,
                                                         uint32_t* __restrict__ sums) {
+  pdl_entry();
   __shared__ uint32_t wt[32];
   __shared__ uint32_t tot;
   const int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK + (int64_t)threadIdx.x * SCAN_V;
@@ -418,6 +425,7 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const uint32_t* __restri
 }
 
 __global__ void __launch_bounds__(SCAN_T) k_scan_sums(uint32_t* __restrict__ sums, int64_t nsums) {
+  pdl_entry();
   __shared__ uint32_t wt[32];
   __shared__ uint32_t tot;
   uint32_t carry = 0;
@@ -433,6 +441,7 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_sums(uint32_t* __restrict__ sum
 
 __global__ void __launch_bounds__(SCAN_T) k_scan_apply(uint32_t* __restrict__ a, int64_t len,
                                                        const uint32_t* __restrict__ sums) {
+  pdl_entry();
   __shared__ uint32_t wt[32];
   __shared__ uint32_t tot;
   const int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK + (int64_t)threadIdx.x * SCAN_V;
@@ -468,6 +477,7 @@ __global__ void __launch_bounds__(PT) k_permute(const uint32_t* __restrict__ per
                                                 const uint32_t* __restrict__ X, const float* __restrict__ V,
                                                 const uint32_t* __restrict__ id, uint32_t* __restrict__ Xs,
                                                 float* __restrict__ Vs, uint32_t* __restrict__ ids) {
+  pdl_entry();
   const int64_t j0 = (int64_t)blockIdx.x * (PT * PK) + threadIdx.x;
   uint32_t p[PK];
 #pragma unroll
