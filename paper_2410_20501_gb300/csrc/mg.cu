@@ -329,114 +329,189 @@ __global__ void k_prolong_correct(float* __restrict__ u, const float* __restrict
   }
 }
 
-// Coarsest level (n <= 16) in one CTA of 1024 threads: red-black SOR sweeps
-// (factor omega) until the residual norm dropped by `drop`, its running
-// minimum stalls for 5 sweeps (float32 floor), or `max_sweeps` sweeps.  Thread
-// t owns the cell pairs (2P, 2P+1), P = t and t + 1024 (same i, j; k even and
-// odd), so each colour pass gives every thread one cell per pair.  The
-// residual of a black cell is taken from its own update (its neighbours are
-// red and do not move during the black pass).  The red residuals of a sweep
-// and the next sweep's red values come from the same neighbour sums (the black
-// cells do not move in between): the new red values are held in registers
-// until the sweep's norm has decided whether there is a next sweep.
-__global__ void __launch_bounds__(1024) k_mg_coarse(float* __restrict__ u, Src f, int log2n, float h2,
-                                                    float omega, int max_sweeps, float drop,
-                                                    int zero_guess) {
+// Coarsest level (n = 4, 8 or 16) in one CTA: red-black SOR sweeps (factor
+// omega) until the residual norm dropped by `drop`, its running minimum stalls
+// for 5 sweeps (float32 floor), or `max_sweeps` sweeps.
+//
+// What bounds it is the chain of sweeps on one SM (about 25 of them at 16^3),
+// so the sweep is kept short.  A thread owns a whole row (i, j): its n / 2 red
+// and n / 2 black values stay in registers, the z neighbours with them, and
+// only the four x and y neighbour rows come from shared memory, where the
+// cells of one colour of a row lie together in 16-byte groups: a red cell and
+// its x and y neighbours have the same index kk in their colour's row
+// (z = 2 kk + o, o the parity of row and colour), z + 1 is at kk + o, z - 1
+// at kk + o - 1.  The residual of a black cell comes from its own update (its
+// neighbours do not move in the black pass), that of a red cell from the next
+// sweep's neighbour sums, so a sweep is two passes and two barriers; its norm
+// is summed over the block while the next sweep's red cells are already
+// computed (kept apart until the norm has decided whether there is a next
+// sweep).  16^3: 66 -> 29 us a solve against a thread per two pairs of cells
+// in natural order with four barriers a sweep.
+template <int VW> struct alignas(4 * VW) RowVec { float v[VW]; };
+template <int LOG>
+__global__ void __launch_bounds__(LOG == 2 ? 32 : 1 << (2 * LOG)) k_mg_coarse(float* __restrict__ u, Src f, float h2,
+                                                                              float omega, int max_sweeps, float drop,
+                                                                              int zero_guess) {
   pdl_entry();
-  __shared__ float su[4096], sf[4096];
-  __shared__ float2 scratch[33];
-  const int n = 1 << log2n, m = n - 1, N = n * n * n, npair = N >> 1;
-  u += (int64_t)blockIdx.z * N;   // one CTA per box
-  f = box_src(f, N);
+  constexpr int n = 1 << LOG, m = n - 1, ROWS = n * n, H = n / 2, VW = H < 4 ? H : 4, NV = H / VW;
+  constexpr int NW = ROWS < 32 ? 1 : ROWS / 32;   // warps
+  using Vec = RowVec<VW>;
+  __shared__ Vec S[2][NV][ROWS];   // [colour][group of kk][row]
+  __shared__ float2 part[NW];
+  u += (int64_t)blockIdx.z * ROWS * n;   // one CTA per box
+  f = box_src(f, ROWS * n);
   const float mean = load_mean(f);
   const float inv_h2 = 1.0f / h2;
-  for (int c = threadIdx.x; c < N; c += blockDim.x) {
-    su[c] = zero_guess ? 0.0f : u[c];
-    sf[c] = src_at(f, c, mean);
-  }
-  __syncthreads();
-  auto nbsum = [&](int c) -> float {
-    const int k = c & m, j = (c >> log2n) & m, i = c >> (2 * log2n);
-    return su[(((i + 1) & m) << (2 * log2n)) | (j << log2n) | k] +
-           su[(((i - 1) & m) << (2 * log2n)) | (j << log2n) | k] +
-           su[(i << (2 * log2n)) | (((j + 1) & m) << log2n) | k] +
-           su[(i << (2 * log2n)) | (((j - 1) & m) << log2n) | k] +
-           su[(i << (2 * log2n)) | (j << log2n) | ((k + 1) & m)] +
-           su[(i << (2 * log2n)) | (j << log2n) | ((k - 1) & m)];
-  };
-  // the cell of pair P with colour col: k of 2P is even, so its colour is (i + j) & 1
-  auto cell_of = [&](int P, int col) -> int {
-    const int c0 = P << 1;
-    return c0 + ((col ^ ((c0 >> log2n) + (c0 >> (2 * log2n)))) & 1);
-  };
-  // SOR update of cell c from its neighbour sum
-  auto sor = [&](int c, float nb) -> float {
-    const float ugs = (nb - h2 * sf[c]) * kSixth;
-    return (omega == 1.0f) ? ugs : omega * ugs + (1.0f - omega) * su[c];
-  };
-  const int P0 = threadIdx.x, P1 = threadIdx.x + blockDim.x;   // npair <= 2048 = 2 x 1024
-  float2 r2p;
+  const bool act = threadIdx.x < ROWS;
+  const int row = act ? threadIdx.x : 0, i = row >> LOG, j = row & m, par = (i + j) & 1;
+  const int rxp = (((i + 1) & m) << LOG) | j, rxm = (((i - 1) & m) << LOG) | j;
+  const int ryp = (i << LOG) | ((j + 1) & m), rym = (i << LOG) | ((j - 1) & m);
+  float v[2][H], fv[2][H];   // [colour][kk]
   {
-    float s = 0.0f, cmp = 0.0f;
-    for (int c = threadIdx.x; c < N; c += blockDim.x) {
-      const float d = sf[c] - (nbsum(c) - 6.0f * su[c]) * inv_h2;
-      kahan_add(s, cmp, d * d);
+    float t[n];
+    auto split = [&](float dst[2][H]) {   // natural order -> colours (red first)
+#pragma unroll
+      for (int kk = 0; kk < H; ++kk) {
+        dst[0][kk] = par ? t[2 * kk + 1] : t[2 * kk];
+        dst[1][kk] = par ? t[2 * kk] : t[2 * kk + 1];
+      }
+    };
+#pragma unroll
+    for (int k = 0; k < n; k += 4) {
+      const float4 q = __ldg(reinterpret_cast<const float4*>(f.p + row * n + k));
+      t[k] = f.s * (q.x - mean); t[k + 1] = f.s * (q.y - mean);
+      t[k + 2] = f.s * (q.z - mean); t[k + 3] = f.s * (q.w - mean);
     }
-    r2p = block_pair_sum(s, cmp, scratch);
+    split(fv);
+#pragma unroll
+    for (int k = 0; k < n; k += 4) {
+      const float4 q = zero_guess ? make_float4(0.0f, 0.0f, 0.0f, 0.0f)
+                                  : *reinterpret_cast<const float4*>(u + row * n + k);
+      t[k] = q.x; t[k + 1] = q.y; t[k + 2] = q.z; t[k + 3] = q.w;
+    }
+    split(v);
   }
-  float best = r2p.x + r2p.y;
+  auto put = [&](int c, const float w[H]) {
+    if (!act) return;
+#pragma unroll
+    for (int g = 0; g < NV; ++g) {
+      Vec x;
+#pragma unroll
+      for (int q = 0; q < VW; ++q) x.v[q] = w[g * VW + q];
+      S[c][g][row] = x;
+    }
+  };
+  // neighbour sums of the row's cells of colour c (order x+, x-, y+, y-, z+, z-)
+  auto nbsum = [&](int c, float nb[H]) {
+    const bool o = ((c + par) & 1) != 0;
+    const float* w = v[1 - c];
+#pragma unroll
+    for (int g = 0; g < NV; ++g) {
+      const Vec a = S[1 - c][g][rxp], b = S[1 - c][g][rxm], d = S[1 - c][g][ryp], e = S[1 - c][g][rym];
+#pragma unroll
+      for (int q = 0; q < VW; ++q) {
+        const int kk = g * VW + q;
+        const float zp = o ? w[(kk + 1) % H] : w[kk], zm = o ? w[kk] : w[(kk + H - 1) % H];
+        nb[kk] = a.v[q] + b.v[q] + d.v[q] + e.v[q] + zp + zm;
+      }
+    }
+  };
+  auto sor = [&](float old, float nb, float fc) -> float {
+    const float ugs = (nb - h2 * fc) * kSixth;
+    return (omega == 1.0f) ? ugs : omega * ugs + (1.0f - omega) * old;
+  };
+  float sum[2], cmp[2];   // compensated sums of squared residuals, two chains
+  auto clear = [&]() { sum[0] = sum[1] = cmp[0] = cmp[1] = 0.0f; };
+  auto residuals = [&](int c, const float val[H], const float nb[H]) {
+#pragma unroll
+    for (int kk = 0; kk < H; ++kk) {
+      const float d = fv[c][kk] - (nb[kk] - 6.0f * val[kk]) * inv_h2;
+      kahan_add(sum[kk & 1], cmp[kk & 1], d * d);
+    }
+  };
+  auto pair_add = [](float& s, float& c, float os, float oc) {
+    float t, e;
+    two_sum(s, os, t, e);
+    s = t;
+    c = c + oc + e;
+  };
+  // this warp's sum over its rows into part[] (idle threads add nothing)
+  auto warp_part = [&]() {
+    float s = act ? sum[0] - cmp[0] : 0.0f, c = 0.0f;
+    pair_add(s, c, act ? sum[1] - cmp[1] : 0.0f, 0.0f);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      const float os = __shfl_xor_sync(0xffffffffu, s, d), oc = __shfl_xor_sync(0xffffffffu, c, d);
+      pair_add(s, c, os, oc);
+    }
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_float2(s, c);
+  };
+  // the block's sum from part[], the same in every thread
+  auto block_total = [&]() -> float {
+    float2 t = part[0];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) pair_add(t.x, t.y, part[w].x, part[w].y);
+    return t.x + t.y;
+  };
+
+  put(0, v[0]);
+  put(1, v[1]);
+  __syncthreads();
+  float nb[H];
+  clear();
+  nbsum(1, nb);
+  residuals(1, v[1], nb);
+  nbsum(0, nb);
+  residuals(0, v[0], nb);
+  warp_part();
+  __syncthreads();
+  float best = block_total();
   const float target = drop * drop * best;
   int stale = 0;
-  if (max_sweeps > 0) {   // the first sweep's red cells
-    for (int P = threadIdx.x; P < npair; P += blockDim.x) {
-      const int c = cell_of(P, 0);
-      su[c] = sor(c, nbsum(c));
-    }
-    __syncthreads();
-  }
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    // here the red cells hold this sweep's values
-    float s = 0.0f, cmp = 0.0f;
-    for (int P = threadIdx.x; P < npair; P += blockDim.x) {      // black, with its residual
-      const int c = cell_of(P, 1);
-      const float nb = nbsum(c);
-      const float un = sor(c, nb);
-      su[c] = un;
-      const float d = sf[c] - (nb - 6.0f * un) * inv_h2;
-      kahan_add(s, cmp, d * d);
+    // v, the shared rows: the values after `sweep` sweeps; nb: sums around the
+    // red cells
+    float red[H];
+    if (sweep > 0) {
+      nbsum(0, nb);
+      residuals(0, v[0], nb);
+      warp_part();
     }
+#pragma unroll
+    for (int kk = 0; kk < H; ++kk) red[kk] = sor(v[0][kk], nb[kk], fv[0][kk]);
+    put(0, red);
     __syncthreads();
-    // red residuals, and the next sweep's red values from the same sums
-    float pend0 = 0.0f, pend1 = 0.0f;
-    const int c0 = P0 < npair ? cell_of(P0, 0) : 0, c1 = P1 < npair ? cell_of(P1, 0) : 0;
-    if (P0 < npair) {
-      const float nb = nbsum(c0);
-      const float d = sf[c0] - (nb - 6.0f * su[c0]) * inv_h2;
-      kahan_add(s, cmp, d * d);
-      pend0 = sor(c0, nb);
+    if (sweep > 0) {   // the norm after `sweep` sweeps
+      const float r = block_total();
+      if (r <= target) break;
+      if (r < 0.998f * best) {   // squared norms: a 0.1% improvement of the norm
+        best = r;
+        stale = 0;
+      } else if (++stale >= 5) {
+        break;                  // no progress for 5 sweeps: the float32 floor
+      }
     }
-    if (P1 < npair) {
-      const float nb = nbsum(c1);
-      const float d = sf[c1] - (nb - 6.0f * su[c1]) * inv_h2;
-      kahan_add(s, cmp, d * d);
-      pend1 = sor(c1, nb);
-    }
-    r2p = block_pair_sum(s, cmp, scratch);   // its barriers end every read of this sweep
-    const float r = r2p.x + r2p.y;
-    if (r <= target) break;
-    if (r < 0.998f * best) {   // squared norms: a 0.1% improvement of the norm
-      best = r;
-      stale = 0;
-    } else if (++stale >= 5) {
-      break;                  // no progress for 5 sweeps: the float32 floor
-    }
-    if (sweep + 1 < max_sweeps) {   // the next sweep's red cells
-      if (P0 < npair) su[c0] = pend0;
-      if (P1 < npair) su[c1] = pend1;
-      __syncthreads();
-    }
+#pragma unroll
+    for (int kk = 0; kk < H; ++kk) v[0][kk] = red[kk];
+    nbsum(1, nb);
+    clear();
+#pragma unroll
+    for (int kk = 0; kk < H; ++kk) v[1][kk] = sor(v[1][kk], nb[kk], fv[1][kk]);
+    residuals(1, v[1], nb);
+    put(1, v[1]);
+    __syncthreads();
   }
-  for (int c = threadIdx.x; c < N; c += blockDim.x) u[c] = su[c];
+  if (act) {
+    float t[n];
+#pragma unroll
+    for (int kk = 0; kk < H; ++kk) {
+      t[2 * kk] = par ? v[1][kk] : v[0][kk];
+      t[2 * kk + 1] = par ? v[0][kk] : v[1][kk];
+    }
+#pragma unroll
+    for (int k = 0; k < n; k += 4)
+      *reinterpret_cast<float4*>(u + row * n + k) = make_float4(t[k], t[k + 1], t[k + 2], t[k + 3]);
+  }
 }
 
 // SOR factor of the coarsest level: the caller's, else Young's optimum
@@ -558,8 +633,13 @@ pm_status v_cycle(MG& g, int l, bool zero_guess) {
       const int64_t N = (int64_t)n * n * n;
       PM_LAUNCH(K_MG_GUESS, 8.0 * N * g.B, k_scale, g.grid(grid_for(N, 256)), 256, 0, g.s, u, N, g.gscale, sbox);
     }
-    PM_LAUNCH(K_MG_COARSE, 12.0 * n * n * n * g.B, k_mg_coarse, g.grid(1), 1024, 0, g.s, u, g.f[l], log2n, h2,
-              coarse_omega(p, n), p.coarse_max_sweeps, p.coarse_drop, zero_guess ? 1 : 0);
+#define PM_COARSE(LOG, threads)                                                                                 \
+  PM_LAUNCH(K_MG_COARSE, 12.0 * n * n * n * g.B, k_mg_coarse<LOG>, g.grid(1), threads, 0, g.s, u, g.f[l], h2, \
+            coarse_omega(p, n), p.coarse_max_sweeps, p.coarse_drop, zero_guess ? 1 : 0)
+    if (n == 16) PM_COARSE(4, 256);
+    else if (n == 8) PM_COARSE(3, 64);
+    else PM_COARSE(2, 32);
+#undef PM_COARSE
     return PM_OK;
   }
   float w[64];
