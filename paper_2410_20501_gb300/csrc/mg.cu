@@ -78,34 +78,45 @@ __global__ void k_scale(float* __restrict__ u, int64_t count, float a, const flo
 // shared with the streaming smoother).  zero: the values of this level are
 // taken as 0 (the coarse-level error starts from zero): the red pass reads
 // nothing, the black pass ignores its own old value.
-__global__ void k_rb_sweep(float* __restrict__ u, Src f, int log2n, int colour, PoissonUpdate upd,
-                           int nb_old, int own_old, int zero) {
+//
+// These levels live in L2 and a pass is over in a few microseconds, so what
+// bounds it is the latency of its loads: a thread takes four consecutive z
+// cells (two of the colour) and has its five 16-byte row loads, the z
+// neighbour beyond the run and the sources in flight together.
+constexpr int kSweepThreads = 128;
+__global__ void __launch_bounds__(kSweepThreads) k_rb_sweep(float* __restrict__ u, Src f, int log2n, int colour,
+                                                            PoissonUpdate upd, int nb_old, int own_old, int zero) {
   pdl_entry();
-  const int m = (1 << log2n) - 1, half = log2n - 1;
+  const uint32_t t = blockIdx.x * kSweepThreads + threadIdx.x;
+  if (t >= 1u << (3 * log2n - 2)) return;
   u += (int64_t)blockIdx.z << (3 * log2n);
   f = box_src(f, (int64_t)1 << (3 * log2n));
   upd = upd.box(blockIdx.z);
-  const float mean = load_mean(f);
-  const int64_t total = (int64_t)1 << (3 * log2n - 1);
-  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-    const int kk = (int)(t & ((1 << half) - 1));
-    const int64_t rest = t >> half;
-    const int j = (int)(rest & m), i = (int)(rest >> log2n);
-    const int k = 2 * kk + ((colour + i + j) & 1);
-    const int64_t c = idx3(i, j, k, log2n);
-    float nb[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    float old = 0.0f;
-    if (!(zero && colour == 0)) {
-      nb[0] = u[idx3((i + 1) & m, j, k, log2n)];
-      nb[1] = u[idx3((i - 1) & m, j, k, log2n)];
-      nb[2] = u[idx3(i, (j + 1) & m, k, log2n)];
-      nb[3] = u[idx3(i, (j - 1) & m, k, log2n)];
-      nb[4] = u[idx3(i, j, (k + 1) & m, log2n)];
-      nb[5] = u[idx3(i, j, (k - 1) & m, log2n)];
-    }
-    if (!zero) old = u[c];
-    u[c] = upd(old, nb, src_at(f, c, mean), 0, nb_old != 0, own_old != 0);
+  const int m = (1 << log2n) - 1;
+  const int k0 = (int)(t << 2) & m, j = (int)(t >> (log2n - 2)) & m, i = (int)(t >> (2 * log2n - 2));
+  const bool odd = ((colour + i + j) & 1) != 0;   // cells k0 + odd and k0 + odd + 2
+  const uint32_t c = idx3(i, j, k0, log2n);
+  float4 XP = make_float4(0.0f, 0.0f, 0.0f, 0.0f), XM = XP, YP = XP, YM = XP, C = XP;
+  float ze = 0.0f;
+  auto row4 = [&](int ii, int jj) { return *reinterpret_cast<const float4*>(u + idx3(ii & m, jj & m, k0, log2n)); };
+  if (!(zero && colour == 0)) {
+    XP = row4(i + 1, j);
+    XM = row4(i - 1, j);
+    YP = row4(i, j + 1);
+    YM = row4(i, j - 1);
+    C = row4(i, j);
+    ze = u[idx3(i, j, (odd ? k0 + 4 : k0 - 1) & m, log2n)];
   }
+  const float4 F = __ldg(reinterpret_cast<const float4*>(f.p + c));
+  const float mean = load_mean(f);
+  const float nb0[6] = {odd ? XP.y : XP.x, odd ? XM.y : XM.x, odd ? YP.y : YP.x, odd ? YM.y : YM.x,
+                        odd ? C.z : C.y, odd ? C.x : ze};
+  const float nb1[6] = {odd ? XP.w : XP.z, odd ? XM.w : XM.z, odd ? YP.w : YP.z, odd ? YM.w : YM.z,
+                        odd ? ze : C.w, odd ? C.z : C.y};
+  const float o0 = zero ? 0.0f : odd ? C.y : C.x, o1 = zero ? 0.0f : odd ? C.w : C.z;
+  const float f0 = f.s * ((odd ? F.y : F.x) - mean), f1 = f.s * ((odd ? F.w : F.z) - mean);
+  u[c + odd] = upd(o0, nb0, f0, 0, nb_old != 0, own_old != 0);
+  u[c + odd + 2] = upd(o1, nb1, f1, 0, nb_old != 0, own_old != 0);
 }
 
 // Coarse right-hand side fc = R(f - L u): residual of the 8 children,
@@ -606,14 +617,14 @@ pm_status smooth(MG& g, int l, int count, const float* w, bool zero, float scale
       g.alt[l] = t;
     }
   } else {
-    const unsigned grid = grid_for(N / 2, 256);
+    const unsigned grid = grid_for(N / 4, kSweepThreads);
     for (; done < count; ++done) {
       PoissonUpdate upd{h2, {w[done], 1.0f}, done == 0 ? scale : 1.0f, done == 0 ? sbox : nullptr};
       const int z = (done == 0 && zero) ? 1 : 0;
       const int first = done == 0 ? 1 : 0;
-      PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (z ? 4.0 : 6.0) * N * g.B, k_rb_sweep, g.grid(grid), 256, 0,
+      PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (z ? 4.0 : 6.0) * N * g.B, k_rb_sweep, g.grid(grid), kSweepThreads, 0,
                 g.s, g.u[l], g.f[l], log2n, 0, upd, first, first, z);
-      PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (z ? 4.0 : 6.0) * N * g.B, k_rb_sweep, g.grid(grid), 256, 0,
+      PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (z ? 4.0 : 6.0) * N * g.B, k_rb_sweep, g.grid(grid), kSweepThreads, 0,
                 g.s, g.u[l], g.f[l], log2n, 1, upd, 0, first, z);
     }
   }
