@@ -156,12 +156,11 @@ typedef struct {
                              MG_GUESS_SCALED: guess_scale * phi (the warm start
                              of Eq. rescaming_newtonian_potential)              */
   float guess_scale;
-  int smoother;           /* 2: one fused red-black sweep per pass over memory
-                             on levels with n >= 128 (bitwise equal to the
-                             colour passes), colour passes below;
-                             1: colour passes (one kernel per colour)
-                             everywhere; 0: two sweeps per pass on levels with
-                             n >= 128 (streaming kernel)                       */
+  int smoother;           /* 2 or 0: fused red-black sweeps on levels with
+                             n >= 64, two per pass over memory (mg_*; fr_*: see
+                             fr_params), bitwise equal to the colour passes,
+                             which levels below take; 1: colour passes (one
+                             kernel per colour) everywhere                     */
   float coarse_omega;     /* SOR factor of the coarsest-level sweeps; 0: the
                              optimal one for that grid, 2/(1 + sqrt(1 - mu^2)),
                              mu = (2 + cos(2 pi/n))/3 (1.634 at 16^3)          */
@@ -259,7 +258,9 @@ typedef struct {
   int cycles;        /* cycles to run when tol <= 0                           */
   double tol;        /* > 0: cycle until ||b - N(u)|| <= tol ||b|| (synchronises) */
   int max_cycles;
-  int smoother;      /* as mg_params.smoother                                   */
+  int smoother;      /* 2: one fused sweep per pass on levels with n >= 128,
+                        colour passes below; 1: colour passes everywhere; 0: two
+                        sweeps per pass on levels with n >= 128                 */
   int nhs;           /* Hu-Sawicki exponent n: 1 (cubic per cell) or 2 (quartic,
                         §3.10); 0 is taken as 1                                 */
 } fr_params;
@@ -567,8 +568,8 @@ int pm_timing_collect(const char** names, double* ms, int64_t* launches, double*
 /* ------------------------------------------------------------ autotuning --
  * Batched launches (pm_step_batch) tune how they tile their work, online: for
  * each launch site and shape (n, B) the candidate values of one parameter
- * (the x chunk of the force pass and of the fused multigrid sweep; colour
- * passes or fused sweeps on 64^3 levels) take turns on successive real
+ * (the x chunk of the force pass; colour passes or fused sweeps on 64^3
+ * levels) take turns on successive real
  * launches, timed with CUDA events on the launch stream and read back
  * without synchronising; after two timings each the fastest is kept for the
  * rest of the process.  Every candidate computes bitwise the same result, so
@@ -578,8 +579,8 @@ int pm_timing_collect(const char** names, double* ms, int64_t* launches, double*
 /* mode 0: fixed default tilings; 1 (the default): tune; 2: forget every
  * choice and timing, then tune.  PM_EINVAL for another mode. */
 pm_status pm_autotune(int mode);
-/* Reports the tuned sites, five ints each: site (0 force-pass chunk, 1 fused
- * multigrid sweep chunk, 2 multigrid smoother form: 0 colour passes, 1 fused),
+/* Reports the tuned sites, five ints each: site (0 force-pass chunk, 2
+ * multigrid smoother form: 0 colour passes, 1 fused; 1 is not in use),
  * n, B, the chosen value (-1 while undecided) and the timings read so far.
  * out (host, 5 * cap ints) may be NULL; returns the number of sites. */
 int pm_autotune_report(int* out, int cap);

@@ -12,6 +12,7 @@
 #include "pm_device.cuh"
 #include "pm_internal.cuh"
 #include "rb_fused.cuh"
+#include "rb_march.cuh"
 #include "rb_stream.cuh"
 
 namespace pmgb {
@@ -540,7 +541,7 @@ struct MG {
   const mg_params* p;
   cudaStream_t s;
   float* u[12];     // current iterate of each level
-  float* alt[12];   // ping-pong partner for the streaming smoother (or NULL)
+  float* alt[12];   // ping-pong partner of the fused sweeps (or NULL)
   Src f[12];
   bool first_cycle;
   float gscale;
@@ -549,10 +550,14 @@ struct MG {
   dim3 grid(unsigned gx) const { return dim3(gx, 1, (unsigned)B); }
 };
 
-pm_status stream_attributes() {
-  PM_TRY(smem_attr(k_rb_stream<2, PoissonUpdate>, StreamGeom<2>::smem_bytes));
-  PM_TRY(smem_attr(k_rb_stream<1, PoissonUpdate>, StreamGeom<1>::smem_bytes));
-  PM_TRY(smem_attr(k_rb_fused4<PoissonUpdate, 3>, kFusedSmem));
+pm_status march_attributes() {
+  constexpr size_t one = MarchGeom<1, kMarchTY, kMarchTZ>::smem, two = MarchGeom<2, kMarchTY, kMarchTZ>::smem;
+  PM_TRY(smem_attr(k_rb_march<1, kMarchTY, kMarchTZ, true, true>, one));
+  PM_TRY(smem_attr(k_rb_march<1, kMarchTY, kMarchTZ, false, false>, one));
+  PM_TRY(smem_attr(k_rb_march<2, kMarchTY, kMarchTZ, true, true>, two));
+  PM_TRY(smem_attr(k_rb_march<2, kMarchTY, kMarchTZ, true, false>, two));
+  PM_TRY(smem_attr(k_rb_march<2, kMarchTY, kMarchTZ, false, true>, two));
+  PM_TRY(smem_attr(k_rb_march<2, kMarchTY, kMarchTZ, false, false>, two));
   return PM_OK;
 }
 
@@ -564,57 +569,45 @@ pm_status smooth(MG& g, int l, int count, const float* w, bool zero, float scale
   const float h2 = 1.0f / ((float)n * (float)n);
   const int64_t N = (int64_t)n * n * n;
   int done = 0;
-  if (g.p->smoother == 0 && stream_ok(n) && g.alt[l] && g.B == 1) {
-    int chunk, nitems;
-    stream_plan(n, &chunk, &nitems);
+  // fused sweeps (two per pass over memory) or colour passes (two per sweep),
+  // bitwise the same result.  Two sweeps: 512^3 0.83 -> 0.40 ms, 256^3 130 -> 63
+  // us against one fused sweep a pass, 128^3 28 -> 18 us against the colour
+  // passes; at 64^3 the two forms are even (a V-cycle from there 56 against 55
+  // us), so one launch is taken instead of four.  On 64^3 levels of a batch the
+  // form is tuned.
+  const bool fused_valid = g.p->smoother != 1 && n >= 64 && g.alt[l] && fused_aligned(g.u[l], g.alt[l], g.f[l].p);
+  bool fused = fused_valid;
+  const bool tune_form = fused_valid && g.B > 1 && n < 128;
+  if (tune_form) {
+    static const int forms[2] = {0, 1};
+    fused = tune_begin(TUNE_MG_SMOOTHER, n, g.B, forms, 2, 1, g.s) == 1;
+  }
+  const bool form_timed = tune_form && tune_active();
+  if (fused) {
     while (done < count) {
-      const int S = (count - done) >= 2 ? 2 : 1;
-      PoissonUpdate upd{h2, {w[done], S == 2 ? w[done + 1] : 1.0f}, done == 0 ? scale : 1.0f};
+      const int S = count - done >= 2 ? 2 : 1;
       const int z = (done == 0 && zero) ? 1 : 0;
-      const unsigned grid = (unsigned)(nitems < 152 * 2 ? nitems : 152 * 2);   // 2 CTAs/SM (shared memory)
-      if (S == 2)
-        PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (z ? 20.0 : 24.0) * N, (k_rb_stream<2, PoissonUpdate>), grid, kStreamThreads,
-                  StreamGeom<2>::smem_bytes, g.s, g.u[l], g.alt[l], g.f[l], log2n, chunk, nitems, z, upd);
-      else
-        PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (z ? 8.0 : 12.0) * N, (k_rb_stream<1, PoissonUpdate>), grid, kStreamThreads,
-                  StreamGeom<1>::smem_bytes, g.s, g.u[l], g.alt[l], g.f[l], log2n, chunk, nitems, z, upd);
+      const bool one0 = w[done] == 1.0f, one1 = S == 2 && w[done + 1] == 1.0f;
+      const MarchArgs a{h2, done == 0 ? scale : 1.0f, {w[done], S == 2 ? w[done + 1] : 1.0f},
+                        done == 0 ? sbox : nullptr};
+      const int chunks = march_chunks(n, g.B, S);
+      const dim3 grid = g.grid((unsigned)((n / kMarchTY) * (n / kMarchTZ) * chunks));
+#define PM_MARCH(SW, A, Bn)                                                                                       \
+  PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (z ? 8.0 : 12.0) * N * g.B,                                     \
+            (k_rb_march<SW, kMarchTY, kMarchTZ, A, Bn>), grid, (MarchGeom<SW, kMarchTY, kMarchTZ>::THREADS),     \
+            (MarchGeom<SW, kMarchTY, kMarchTZ>::smem), g.s, g.u[l], g.alt[l], g.f[l], log2n, chunks, z, a)
+      if (S == 1) {
+        if (one0) PM_MARCH(1, true, true); else PM_MARCH(1, false, false);
+      } else if (one0) {
+        if (one1) PM_MARCH(2, true, true); else PM_MARCH(2, true, false);
+      } else {
+        if (one1) PM_MARCH(2, false, true); else PM_MARCH(2, false, false);
+      }
+#undef PM_MARCH
       float* t = g.u[l];
       g.u[l] = g.alt[l];
       g.alt[l] = t;
       done += S;
-    }
-    return PM_OK;
-  }
-  // fused sweeps (one pass per sweep) or colour passes (two per sweep), bitwise
-  // the same result; on 64^3 levels of a batch the form is tuned, and the
-  // fused sweep's x chunk is tuned on every batched level
-  const bool fused_valid = g.p->smoother == 2 && n >= 64 && g.alt[l] && fused_aligned(g.u[l], g.alt[l], g.f[l].p);
-  bool fused = fused_valid && fused_ok(n, g.B);
-  const bool tune_form = fused_valid && g.B > 1 && n < 128;
-  if (tune_form) {
-    static const int forms[2] = {0, 1};
-    fused = tune_begin(TUNE_MG_SMOOTHER, n, g.B, forms, 2, fused ? 1 : 0, g.s) == 1;
-  }
-  const bool form_timed = tune_form && tune_active();
-  if (fused) {
-    for (; done < count; ++done) {
-      int chunk = fused_chunk(n);
-      const bool tune_chunk = g.B > 1 && !form_timed;   // one timing at a time
-      if (tune_chunk) {
-        int cand[3], nc = 0;
-        for (int c = 16; c <= 64 && c <= n; c *= 2) cand[nc++] = c;
-        chunk = tune_begin(TUNE_MG_FUSED_CHUNK, n, g.B, cand, nc, chunk, g.s);
-      }
-      const unsigned grid = (unsigned)((n / kFusedT) * (n / kFusedT) * (n / chunk));
-      PoissonUpdate upd{h2, {w[done], 1.0f}, done == 0 ? scale : 1.0f, done == 0 ? sbox : nullptr};
-      const int z = (done == 0 && zero) ? 1 : 0;
-      PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (z ? 8.0 : 12.0) * N * g.B, (k_rb_fused4<PoissonUpdate, 3>),
-                g.grid(grid), kQuadThreads, kFusedSmem, g.s, g.u[l], g.alt[l], g.f[l], log2n, chunk, z,
-                done == 0 ? 1 : 0, upd);
-      if (tune_chunk) tune_end(g.s);
-      float* t = g.u[l];
-      g.u[l] = g.alt[l];
-      g.alt[l] = t;
     }
   } else {
     const unsigned grid = grid_for(N / 4, kSweepThreads);
@@ -717,7 +710,7 @@ pm_status mg_solve_batch_src(Src f, float* phi, int n, int B, const mg_params& p
     }
     g.alt[l] = w.mg_alt[l];
   }
-  PM_TRY(stream_attributes());
+  PM_TRY(march_attributes());
   g.first_cycle = true;
   g.gscale = 1.0f;
   g.gbox = prm.first_guess == MG_GUESS_SCALED ? gbox : nullptr;
@@ -752,7 +745,7 @@ pm_status mg_solve_src(Src f, float* phi, int n, const mg_params& prm, mg_stats*
     }
     g.alt[l] = w.mg_alt[l];
   }
-  PM_TRY(stream_attributes());
+  PM_TRY(march_attributes());
   g.first_cycle = true;
   g.gscale = prm.first_guess == MG_GUESS_SCALED ? prm.guess_scale : 1.0f;
   const int64_t N = (int64_t)n * n * n;

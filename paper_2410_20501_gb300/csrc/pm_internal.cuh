@@ -24,7 +24,7 @@ extern const char* const kKernelClassNames[K_NCLASS];
 // tune_begin before its launch(es) with candidate values that compute bitwise
 // the same result, uses the value returned, and calls tune_end after them on
 // the same stream; tune_active() says whether this call is being timed.
-enum TuneSite { TUNE_FORCE_CHUNK, TUNE_MG_FUSED_CHUNK, TUNE_MG_SMOOTHER };
+enum TuneSite { TUNE_FORCE_CHUNK = 0, TUNE_MG_SMOOTHER = 2 };
 int tune_begin(int site, int n, int B, const int* cand, int ncand, int dflt, cudaStream_t s);
 void tune_end(cudaStream_t s);
 bool tune_active();

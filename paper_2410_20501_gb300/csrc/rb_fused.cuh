@@ -57,9 +57,8 @@ inline int fused_chunk(int n) {
   return c;
 }
 
-// Levels the fused kernel takes: n >= 128, or n = 64 in a batch of at least 8
-// boxes (enough CTAs to fill the GPU).
-inline bool fused_ok(int n, int B = 1) { return n >= 128 || (n >= 64 && B >= 8); }
+// Levels the fused kernel takes.
+inline bool fused_ok(int n) { return n >= 128; }
 
 // float4 plane, source and run loads and stores need 16-byte aligned level
 // arrays (workspace levels always are; caller arrays are checked on entry).
@@ -81,7 +80,10 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_group2() { asm volatile("cp.async.wait_group 2;\n" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void cp_async_wait_group() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(PENDING) : "memory");
+}
 
 // Update functor interface: upd(old, nb[6] (x+, x-, y+, y-, z+, z-), source,
 // sweep index (0 here), neighbours-never-updated, own-never-updated).  first:
@@ -249,7 +251,7 @@ __global__ void __launch_bounds__(kQuadThreads, MINB) k_rb_fused4(const float* _
     if (!zero) {
       if (t + 3 <= x1 + 1) issue(t + 3);
       cp_async_commit_group();
-      cp_async_wait_group2();
+      cp_async_wait_group<2>();
     }
     const float4 F_t = Fa;
     if (t + 2 <= x1) Fa = fetch_f(t + 2);

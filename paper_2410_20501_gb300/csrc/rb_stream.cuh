@@ -19,7 +19,8 @@
 // split index in the other colour's row, the two z neighbours at index kk + o
 // and kk + o - 1 where o is the row's parity.  The next plane is fetched into
 // registers while the current plane's stages run.  The update rule is a
-// functor: linear SOR (Poisson) or the f(R) cubic.
+// functor (the f(R) cell equation; the linear smoother has its own kernel in
+// rb_march.cuh, its colour passes share the functor below).
 #pragma once
 
 #include "pm_internal.cuh"
@@ -64,8 +65,8 @@ struct PoissonUpdate {
     if (gbox) u.gscale = __ldg(gbox + b);
     return u;
   }
-  // Explicit rounding intrinsics (no contraction) so that the fused and the
-  // colour-by-colour kernels produce bitwise identical updates.
+  // Explicit rounding intrinsics (no other contraction) so that the fused and
+  // the colour-by-colour kernels produce bitwise identical updates.
   __device__ __forceinline__ float operator()(float old, const float nb[6], float fv, int sweep,
                                               bool nb_old, bool own_old) const {
     float s = __fadd_rn(nb[0], nb[1]);
@@ -78,7 +79,7 @@ struct PoissonUpdate {
     const float w = omega[sweep];
     if (w == 1.0f) return ugs;
     const float o = own_old ? __fmul_rn(gscale, old) : old;
-    return __fadd_rn(__fmul_rn(w, ugs), __fmul_rn(1.0f - w, o));
+    return __fmaf_rn(w, ugs, __fmul_rn(1.0f - w, o));
   }
 };
 

@@ -1,0 +1,56 @@
+"""The linear smoother's fused sweeps (one or two sweeps per pass over memory,
+levels with n >= 64) against the colour passes, bitwise, over sweep counts,
+factors, guesses and batches; the coarsest-level solve at each size it takes
+against the oracle."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import poisson
+from paper_2410_20501_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pm():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import os
+    from paper_2410_20501_gb300 import build, pm as _pm
+    if not os.path.exists(_pm.LIB_PATH):
+        build.build()
+    _pm.lib()
+    return _pm
+
+
+@pytest.mark.parametrize("n,npre,npost,omega,scale", [(64, 1, 0, 1.25, 1.0), (64, 2, 1, 1.25, 0.9), (128, 3, 2, 1.1, 1.3),
+                                                      (64, 4, 4, 1.0, 1.1), (256, 2, 3, 1.25, 0.7)])
+def test_fused_sweeps_are_bitwise_the_colour_passes(pm, n, npre, npost, omega, scale):
+    f = torch.from_numpy(inputs.random_field(n, 11).astype(np.float32)).cuda()
+    phi0 = torch.from_numpy(inputs.random_field(n, 12).astype(np.float32)).cuda()
+    outs = []
+    for smoother in (2, 0, 1):
+        phi, _ = pm.mg_solve(f, phi=phi0.clone(), fixed_cycles=2, first_guess=pm.MG_GUESS_SCALED, guess_scale=scale,
+                             npre=npre, npost=npost, omega=omega, smoother=smoother)
+        outs.append(phi.cpu().numpy())
+    assert np.array_equal(outs[0], outs[2]) and np.array_equal(outs[1], outs[2])
+
+
+@pytest.mark.parametrize("n,B", [(64, 1), (64, 5), (128, 3)])
+def test_fused_sweeps_of_a_batch(pm, n, B):
+    f = torch.from_numpy(np.stack([inputs.random_field(n, 20 + b) for b in range(B)]).astype(np.float32)).cuda()
+    phi = [pm.mg_solve_batch(f, fixed_cycles=2, smoother=s).cpu().numpy() for s in (2, 1)]
+    assert np.array_equal(phi[0], phi[1])
+
+
+@pytest.mark.parametrize("coarsest,sweeps", [(4, 200), (8, 200), (16, 200), (16, 0), (16, 3)])
+def test_coarsest_sizes_match_the_oracle(pm, coarsest, sweeps):
+    n = 32
+    f = inputs.random_field(n, 5).astype(np.float32).astype(np.float64)
+    phi, _ = pm.mg_solve(torch.from_numpy(f.astype(np.float32)).cuda(), fixed_cycles=2, coarsest=coarsest,
+                         coarse_max_sweeps=sweeps, first_guess=pm.MG_GUESS_JACOBI)
+    ref, _ = poisson.mg_solve(f, 1.0 / n, prm=poisson.MGParams(coarsest=coarsest, coarse_max_sweeps=sweeps), cycles=2)
+    # the bar of the 16^3 case: float32 against float64 after the same steps
+    assert np.linalg.norm(phi.cpu().numpy() - ref) < 1e-5 * np.linalg.norm(ref)
