@@ -110,7 +110,7 @@ size_t layout_workspace(Workspace* w, void* base, int n, int64_t np, uint32_t fl
     w->Vs = (float*)take((size_t)np * 12);
     if (flags & PM_WS_IDS) w->ids = (uint32_t*)take((size_t)np * 4);
     w->rho = (float*)take((size_t)N * 4);
-    w->g = (float*)take((size_t)N * 16);   // three planes, or float4 per cell
+    w->g = (float*)take((size_t)N * 12);
   }
   if (flags & PM_WS_ADJ) {
     w->adj_abar = (float*)take((size_t)np * 12);
@@ -406,13 +406,24 @@ pm_status pm_lpt2(const float* noise, const float* amp, int n, double d1, double
 
 pm_status pm_gradient(const float* phi, float* g, int n, int order, void* stream) {
   if (!valid_n(n) || !phi || !g || (order != 3 && order != 5 && order != 7) || !all_a16(phi, g)) return PM_EINVAL;
-  return gradient_launch(phi, nullptr, 0.0f, g, n, order, false, as_stream(stream));
+  return gradient_launch(phi, nullptr, 0.0f, g, n, order, as_stream(stream));
 }
 
 pm_status pm_interp(const float* g, const uint32_t* X, int64_t np, int n, float* acc, void* stream) {
   if (!valid_n(n) || !valid_np(np) || !g || (np > 0 && (!X || !acc)) || !all_a16(g, X, acc)) return PM_EINVAL;
-  return interp_launch(g, X, nullptr, nullptr, np, n, acc, nullptr, nullptr, nullptr, 0.0f, 0.0f, 0, false,
+  return interp_launch(g, X, nullptr, nullptr, np, n, acc, nullptr, nullptr, nullptr, 0.0f, 0.0f, 0,
                        as_stream(stream));
+}
+
+pm_status pm_interp_packed(const float* g, const uint32_t* X, int64_t np, int n, float* acc, void* ws, size_t ws_bytes,
+                           void* stream) {
+  if (!valid_n(n) || !valid_np(np) || !g || (np > 0 && (!X || !acc)) || !all_a16(g, X, acc)) return PM_EINVAL;
+  if (!ws || !aligned(ws)) return PM_EINVAL;
+  if (ws_bytes < (size_t)n * n * n * sizeof(float4) + 256) return PM_ENOMEM;
+  // from 2^17 particles and a fortieth of the cells on, random order pays for the extra launches and the packing
+  if (np < 1 << 17 || 40 * np < (int64_t)n * n * n) return pm_interp(g, X, np, n, acc, stream);
+  return interp_packed_launch(g, X, np, n, acc, static_cast<int*>(ws),
+                              reinterpret_cast<float4*>(static_cast<char*>(ws) + 256), as_stream(stream));
 }
 
 // The step; with V_host, the velocities are copied from that host array on
@@ -528,9 +539,9 @@ pm_status step_impl(pm_state* st_, const pm_step_params* prm, pm_stats* stats, v
                                S.acc, S.X, S.V, S.id, (float)prm->dt_kick, (float)prm->dt_drift, 1, s, Batch{},
                                blockmax, max_out));
   } else {
-    PM_TRY(gradient_launch(S.phi, eps_force, alpha, w.g, n, prm->grad_order, false, s, 1, nh));
+    PM_TRY(gradient_launch(S.phi, eps_force, alpha, w.g, n, prm->grad_order, s, 1, nh));
     PM_TRY(interp_launch(w.g, w.Xs, w.Vs, w.ids, np, n, S.acc, S.X, S.V, S.id, (float)prm->dt_kick,
-                         (float)prm->dt_drift, 1, false, s, Batch{}, blockmax, max_out));
+                         (float)prm->dt_drift, 1, s, Batch{}, blockmax, max_out));
   }
   if (max_out) {
     double h[2] = {0.0, 0.0};
@@ -735,7 +746,7 @@ pm_status pm_step_adj(pm_state* st_, const pm_step_params* prm, const float* phi
     if (r != PM_OK && r != PM_ENOCONV) return r;
     phi = w.adj_phi;
   }
-  PM_TRY(gradient_launch(phi, nullptr, 0.0f, w.g, n, prm->grad_order, false, s));
+  PM_TRY(gradient_launch(phi, nullptr, 0.0f, w.g, n, prm->grad_order, s));
   // reverse sweep
   PM_TRY(adj_accel_launch(X_bar_out, V_bar_out, np, (float)prm->dt_kick, (float)prm->dt_drift, w.adj_abar, s));
   const int64_t N = (int64_t)n * n * n;
@@ -867,7 +878,7 @@ pm_status fr_solve_batch(const float* rho, float* eps, int n, int B, const fr_pa
 pm_status pm_gradient_batch(const float* phi, float* g, int n, int B, int order, void* stream) {
   if (!valid_n(n) || B < 1 || !phi || !g || (order != 3 && order != 5 && order != 7) || !all_a16(phi, g))
     return PM_EINVAL;
-  return gradient_launch(phi, nullptr, 0.0f, g, n, order, false, as_stream(stream), B);
+  return gradient_launch(phi, nullptr, 0.0f, g, n, order, as_stream(stream), B);
 }
 
 pm_status pm_interp_batch(const float* g, const uint32_t* X, int64_t np_box, int n, int B, float* acc,
@@ -879,7 +890,7 @@ pm_status pm_interp_batch(const float* g, const uint32_t* X, int64_t np_box, int
   Batch bt;
   bt.B = B;
   bt.np_box = np_box;
-  return interp_launch(g, X, nullptr, nullptr, np, n, acc, nullptr, nullptr, nullptr, 0.0f, 0.0f, 0, false,
+  return interp_launch(g, X, nullptr, nullptr, np, n, acc, nullptr, nullptr, nullptr, 0.0f, 0.0f, 0,
                        as_stream(stream), bt);
 }
 

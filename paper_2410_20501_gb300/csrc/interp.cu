@@ -17,19 +17,6 @@ __device__ __forceinline__ int64_t idx3(int i, int j, int k, int log2n) {
   return ((int64_t)i << (2 * log2n)) | ((int64_t)j << log2n) | k;
 }
 
-// phi + alpha (u^(n+1) - 1), u = 1 + eps: the combined potential up to a
-// constant (alpha = -(c~^2/2) fbar; n = nh, 1 or 2).
-template <bool FR>
-__device__ __forceinline__ float pot(const float* __restrict__ phi, const float* __restrict__ eps, float alpha,
-                                     int64_t c, int nh) {
-  float v = __ldg(phi + c);
-  if (FR) {
-    const float e = __ldg(eps + c);
-    v = fmaf(alpha, nh == 2 ? e * fmaf(e, 3.0f + e, 3.0f) : e * (2.0f + e), v);
-  }
-  return v;
-}
-
 // Table 1 coefficients c_1..c_3 of the antisymmetric central derivative
 // (1/h) sum_k c_k (u_{i+k} - u_{i-k}).
 template <int ORDER> struct Stencil;
@@ -43,104 +30,82 @@ template <> struct Stencil<7> {
   __device__ static float c(int k) { return k == 1 ? 0.75f : (k == 2 ? -0.15f : 1.0f / 60.0f); }
 };
 
+// A thread owns four consecutive z cells of a row and marches over a chunk of
+// x planes with the 2R + 1 potential runs around its plane in registers, so a
+// plane step loads one new run, the 2R rows beside it and the runs on either
+// side in z (16 bytes each, all in flight together; the CTA's rows share them
+// through L1) and writes three runs.  Bound by HBM and L2: 16 bytes a cell.
+// 256^3, order 7: 166 -> 65 us, 512^3 order 5: 0.92 -> 0.35 ms against planes staged in shared
+// memory with two barriers each.
+constexpr int GNT = 256;
+
 template <int ORDER, bool FR>
-__global__ void k_gradient(const float* __restrict__ phi, const float* __restrict__ eps, float alpha,
-                           float* __restrict__ g, int log2n, float inv_h, int nh) {
+__global__ void __launch_bounds__(GNT) k_gradient(const float* __restrict__ phi, const float* __restrict__ eps,
+                                                  float alpha, float* __restrict__ g, int log2n, float inv_h, int chunk,
+                                                  int nh) {
   pdl_entry();
-  const int m = (1 << log2n) - 1;
-  const int64_t total = (int64_t)1 << (3 * log2n);
-  phi += (int64_t)blockIdx.z * total;          // the box of a batched launch
-  if (FR) eps += (int64_t)blockIdx.z * total;
-  g += (int64_t)blockIdx.z * 3 * total;
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < total;
-       c += (int64_t)gridDim.x * blockDim.x) {
-    const int k = (int)(c & m), j = (int)((c >> log2n) & m), i = (int)(c >> (2 * log2n));
-    float gx = 0.0f, gy = 0.0f, gz = 0.0f;
-#pragma unroll
-    for (int q = Stencil<ORDER>::R; q >= 1; --q) {
-      const float w = Stencil<ORDER>::c(q);
-      gx = fmaf(w, pot<FR>(phi, eps, alpha, idx3((i + q) & m, j, k, log2n), nh) -
-                       pot<FR>(phi, eps, alpha, idx3((i - q) & m, j, k, log2n), nh), gx);
-      gy = fmaf(w, pot<FR>(phi, eps, alpha, idx3(i, (j + q) & m, k, log2n), nh) -
-                       pot<FR>(phi, eps, alpha, idx3(i, (j - q) & m, k, log2n), nh), gy);
-      gz = fmaf(w, pot<FR>(phi, eps, alpha, idx3(i, j, (k + q) & m, log2n), nh) -
-                       pot<FR>(phi, eps, alpha, idx3(i, j, (k - q) & m, log2n), nh), gz);
-    }
-    const int64_t N = total;
-    g[c] = -gx * inv_h;
-    g[N + c] = -gy * inv_h;
-    g[2 * N + c] = -gz * inv_h;
-  }
-}
-
-// Streaming gradient for n >= 64: a CTA owns a 16 x 64 (y, z) column and a
-// chunk of x planes, keeps the 2R + 1 planes of Phi (with a halo of R in y and
-// z) that the stencil needs in shared memory, so every Phi value is read from
-// HBM once (plus halos).  Same arithmetic order as k_gradient.  VEC4 writes
-// g interleaved as float4 (gx, gy, gz, 0) for the interpolation.
-constexpr int GTY = 16, GTZ = 64, GNT = 256;
-
-template <int ORDER, bool FR, bool VEC4>
-__global__ void __launch_bounds__(GNT) k_gradient_stream(const float* __restrict__ phi,
-                                                        const float* __restrict__ eps, float alpha,
-                                                        float* __restrict__ g, int log2n, float inv_h,
-                                                        int chunk, int nitems, int nh) {
-  pdl_entry();
-  constexpr int R = Stencil<ORDER>::R, W = 2 * R + 1, EY = GTY + 2 * R, EZ = GTZ + 2 * R, PL = EY * EZ;
-  extern __shared__ float P[];   // [W][EY][EZ]
-  const int n = 1 << log2n, m = n - 1;
-  const int tiles_z = n / GTZ, tiles = (n / GTY) * tiles_z;
+  constexpr int R = Stencil<ORDER>::R, W = 2 * R + 1;
+  const int m = (1 << log2n) - 1, lq = log2n - 2;
   const int64_t N = (int64_t)1 << (3 * log2n);
-  const int tid = threadIdx.x;
+  const uint32_t t = blockIdx.x * GNT + threadIdx.x;          // run of the plane
+  if (t >= 1u << (2 * log2n - 2)) return;
   phi += (int64_t)blockIdx.z * N;              // the box of a batched launch
   if (FR) eps += (int64_t)blockIdx.z * N;
-  g += (int64_t)blockIdx.z * (VEC4 ? 4 : 3) * N;
-  for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
-    const int tile = item % tiles, xc = item / tiles;
-    const int y0 = (tile / tiles_z) * GTY, z0 = (tile % tiles_z) * GTZ;
-    const int x0 = xc * chunk, x1 = x0 + chunk;
-    for (int t = x0 - R; t < x1 + R; ++t) {
-      float* Pt = P + (((t % W) + W) % W) * PL;
-      const int64_t pb = (int64_t)(t & m) << (2 * log2n);
-      for (int e = tid; e < PL; e += GNT) {
-        const int ly = e / EZ, lz = e - ly * EZ;
-        Pt[e] = pot<FR>(phi, eps, alpha, pb | ((int64_t)((y0 - R + ly) & m) << log2n) | ((z0 - R + lz) & m), nh);
-      }
-      __syncthreads();
-      const int xo = t - R;
-      if (xo >= x0) {
-        const float* Pc = P + (((xo % W) + W) % W) * PL;
-        for (int e = tid; e < GTY * GTZ; e += GNT) {
-          const int ly = e / GTZ, lz = e - ly * GTZ;
-          const int c = (ly + R) * EZ + lz + R;
-          float gx = 0.0f, gy = 0.0f, gz = 0.0f;
-#pragma unroll
-          for (int q = R; q >= 1; --q) {
-            const float w = Stencil<ORDER>::c(q);
-            const float* Pp = P + ((((xo + q) % W) + W) % W) * PL;
-            const float* Pm = P + ((((xo - q) % W) + W) % W) * PL;
-            gx = fmaf(w, Pp[c] - Pm[c], gx);
-            gy = fmaf(w, Pc[c + q * EZ] - Pc[c - q * EZ], gy);
-            gz = fmaf(w, Pc[c + q] - Pc[c - q], gz);
-          }
-          const int64_t cell = ((int64_t)xo << (2 * log2n)) | ((int64_t)(y0 + ly) << log2n) | (z0 + lz);
-          if (VEC4) {
-            reinterpret_cast<float4*>(g)[cell] = make_float4(-gx * inv_h, -gy * inv_h, -gz * inv_h, 0.0f);
-          } else {
-            g[cell] = -gx * inv_h;
-            g[N + cell] = -gy * inv_h;
-            g[2 * N + cell] = -gz * inv_h;
-          }
-        }
-      }
-      __syncthreads();
+  g += (int64_t)blockIdx.z * 3 * N;
+  const int j = (int)(t >> lq), k = (int)(t & ((1 << lq) - 1)) << 2, x0 = blockIdx.y * chunk;
+  auto run = [&](int x, int y, int z) -> float4 {
+    const int64_t c = idx3(x & m, y & m, z & m, log2n);
+    float4 v = __ldg(reinterpret_cast<const float4*>(phi + c));
+    if (FR) {
+      const float4 e = __ldg(reinterpret_cast<const float4*>(eps + c));
+      auto both = [&](float p, float q) {
+        return fmaf(alpha, nh == 2 ? q * fmaf(q, 3.0f + q, 3.0f) : q * (2.0f + q), p);
+      };
+      v = make_float4(both(v.x, e.x), both(v.y, e.y), both(v.z, e.z), both(v.w, e.w));
     }
+    return v;
+  };
+  float4 P[W];   // planes x - R .. x + R
+#pragma unroll
+  for (int q = 0; q < W - 1; ++q) P[q + 1] = run(x0 - R + q, j, k);
+  for (int x = x0; x < x0 + chunk; ++x) {
+#pragma unroll
+    for (int q = 0; q < W - 1; ++q) P[q] = P[q + 1];
+    P[W - 1] = run(x + R, j, k);
+    const float4 left = run(x, j, k - 4), right = run(x, j, k + 4);
+    float4 yp[R], ym[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      yp[q] = run(x, j + q + 1, k);
+      ym[q] = run(x, j - q - 1, k);
+    }
+    const float zr[12] = {left.x, left.y, left.z, left.w, P[R].x, P[R].y, P[R].z, P[R].w,
+                          right.x, right.y, right.z, right.w};
+    auto at = [](const float4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; };
+    float o[3][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float gx = 0.0f, gy = 0.0f, gz = 0.0f;
+#pragma unroll
+      for (int q = R; q >= 1; --q) {
+        const float w = Stencil<ORDER>::c(q);
+        gx = fmaf(w, at(P[R + q], i) - at(P[R - q], i), gx);
+        gy = fmaf(w, at(yp[q - 1], i) - at(ym[q - 1], i), gy);
+        gz = fmaf(w, zr[4 + i + q] - zr[4 + i - q], gz);
+      }
+      o[0][i] = -gx * inv_h;
+      o[1][i] = -gy * inv_h;
+      o[2][i] = -gz * inv_h;
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      *reinterpret_cast<float4*>(g + d * N + idx3(x, j, k, log2n)) = make_float4(o[d][0], o[d][1], o[d][2], o[d][3]);
   }
 }
 
 // Inverse TSC; mode 1 also kicks and drifts.  Particles are read in cell
 // order (Xs, Vs) and written in the same order (Xo, Vo).
-template <bool VEC4, bool MAXES>
+template <bool MAXES>
 __global__ void __launch_bounds__(256) k_interp_kdk(const float* __restrict__ g, const uint32_t* __restrict__ Xs,
                                                     const float* __restrict__ Vs,
                                                     const uint32_t* __restrict__ ids_in, int64_t np, int log2n,
@@ -156,7 +121,7 @@ __global__ void __launch_bounds__(256) k_interp_kdk(const float* __restrict__ g,
   // the box of a batched launch: its grid and its particles p0 .. p0 + np_box
   // (np stays the plane stride of the particle arrays)
   const int64_t p0 = (int64_t)blockIdx.z * np_box, p1 = p0 + np_box;
-  g += (int64_t)blockIdx.z * (VEC4 ? 4 : 3) * N;
+  g += (int64_t)blockIdx.z * 3 * N;
   if (dtk_box) dt_kick = __ldg(dtk_box + blockIdx.z);
   if (dtd_box) drift_scale = __ldg(dtd_box + blockIdx.z) * 4294967296.0f;
   float amax = 0.0f, vmax = 0.0f;   // largest |a| and |v after the kick| of this thread
@@ -180,16 +145,9 @@ __global__ void __launch_bounds__(256) k_interp_kdk(const float* __restrict__ g,
         for (int oz = 0; oz < 3; ++oz) {
           const int64_t c = idx3(ci, cj, (iz + oz - 1) & m, log2n);
           const float w = wxy * wz[oz];
-          if (VEC4) {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(g) + c);
-            ax = fmaf(w, v.x, ax);
-            ay = fmaf(w, v.y, ay);
-            az = fmaf(w, v.z, az);
-          } else {
-            ax = fmaf(w, __ldg(g + c), ax);
-            ay = fmaf(w, __ldg(g + N + c), ay);
-            az = fmaf(w, __ldg(g + 2 * N + c), az);
-          }
+          ax = fmaf(w, __ldg(g + c), ax);
+          ay = fmaf(w, __ldg(g + N + c), ay);
+          az = fmaf(w, __ldg(g + 2 * N + c), az);
         }
       }
     }
@@ -231,6 +189,130 @@ __global__ void __launch_bounds__(256) k_interp_kdk(const float* __restrict__ g,
       blockmax[(int64_t)blockIdx.z * gridDim.x + blockIdx.x] = make_float2(__uint_as_float(ma), __uint_as_float(mv));
     }
   }
+}
+
+// Whether the gather is worth packing the field for, from a sample of the
+// particles' order (one block): *flag = 1 if `gain` lookups saved per row of
+// cells that 32 neighbouring particles touch exceed `cost`.
+__global__ void __launch_bounds__(1024) k_interp_order(const uint32_t* __restrict__ Xs, int64_t np, int log2n,
+                                                       float gain, float cost, int* __restrict__ flag) {
+  pdl_entry();
+  __shared__ int total;
+  constexpr int PER_WARP = 8, GROUPS = 32 * PER_WARP;
+  const int sh = 32 - log2n, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) total = 0;
+  __syncthreads();
+  uint32_t x[PER_WARP], y[PER_WARP];
+#pragma unroll
+  for (int k = 0; k < PER_WARP; ++k) {   // groups spread evenly over the particles (np >= 32)
+    const int64_t p = (np - 32) * ((threadIdx.x >> 5) * PER_WARP + k) / (GROUPS - 1) + lane;
+    x[k] = __ldg(Xs + p) >> sh;
+    y[k] = __ldg(Xs + np + p) >> sh;
+  }
+  int rows = 0;
+#pragma unroll
+  for (int k = 0; k < PER_WARP; ++k) {
+    const uint32_t row = (x[k] << log2n) | y[k], prev = __shfl_up_sync(0xffffffffu, row, 1);
+    rows += __popc(__ballot_sync(0xffffffffu, lane == 0 || row != prev));
+  }
+  if (lane == 0) atomicAdd(&total, rows);   // integers: any order
+  __syncthreads();
+  if (threadIdx.x == 0) *flag = gain * ((float)total / GROUPS) > cost;
+}
+
+// Cells of the force field as float4 (g_x, g_y, g_z, 0), if *flag; a thread
+// packs four at a time.
+__global__ void __launch_bounds__(256) k_pack_force(const float* __restrict__ g, float4* __restrict__ out, int64_t N,
+                                                    const int* __restrict__ flag) {
+  pdl_entry();
+  if (!*flag) return;
+  for (int64_t c = 4 * (blockIdx.x * (int64_t)256 + threadIdx.x); c < N; c += 4 * (int64_t)gridDim.x * 256) {
+    const float4 x = __ldg(reinterpret_cast<const float4*>(g + c));
+    const float4 y = __ldg(reinterpret_cast<const float4*>(g + N + c));
+    const float4 z = __ldg(reinterpret_cast<const float4*>(g + 2 * N + c));
+    out[c] = make_float4(x.x, y.x, z.x, 0.0f);
+    out[c + 1] = make_float4(x.y, y.y, z.y, 0.0f);
+    out[c + 2] = make_float4(x.z, y.z, z.z, 0.0f);
+    out[c + 3] = make_float4(x.w, y.w, z.w, 0.0f);
+  }
+}
+
+// Two neighbouring packed cells (32 bytes, aligned) in one load.
+struct CellPair {
+  float4 a, b;
+};
+__device__ __forceinline__ CellPair load_pair(const float4* p) {
+  CellPair v;
+  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(v.a.x), "=f"(v.a.y), "=f"(v.a.z), "=f"(v.a.w), "=f"(v.b.x), "=f"(v.b.y), "=f"(v.b.z), "=f"(v.b.w)
+      : "l"(p));
+  return v;
+}
+
+// Inverse TSC at particles in any order, from the packed field if *flag, else
+// from the three planes: the sums of k_interp_kdk in the same order (bitwise the
+// same).  What bounds the gather at scattered positions is the line lookups of
+// L1, one per load and lane, so the three z cells of a row come in two aligned
+// 32-byte loads instead of nine 4-byte ones.  10^7 random positions on 256^3:
+// 3.3 -> 1.6 ms with the packing.
+__global__ void __launch_bounds__(256) k_interp_packed(const float4* __restrict__ gp, const float* __restrict__ g,
+                                                       const uint32_t* __restrict__ Xs, int64_t np, int log2n,
+                                                       float* __restrict__ acc, const int* __restrict__ flag) {
+  pdl_entry();
+  const int m = (1 << log2n) - 1, sh = 32 - log2n;
+  const int64_t N = (int64_t)1 << (3 * log2n);
+  const int64_t p = blockIdx.x * (int64_t)256 + threadIdx.x;
+  if (p >= np) return;
+  const bool packed = *flag != 0;
+  const uint32_t x = __ldg(Xs + p), y = __ldg(Xs + np + p), z = __ldg(Xs + 2 * np + p);
+  float wx[3], wy[3], wz[3];
+  tsc_weights(cell_offset(x, log2n), wx);
+  tsc_weights(cell_offset(y, log2n), wy);
+  tsc_weights(cell_offset(z, log2n), wz);
+  const int ix = (int)(x >> sh), iy = (int)(y >> sh), iz = (int)(z >> sh);
+  float ax = 0.0f, ay = 0.0f, az = 0.0f;
+  if (packed) {
+    const int z0 = (iz - 1) & m, k0 = z0 & ~1, k1 = (k0 + 2) & m;
+    const bool odd = z0 & 1;                     // the row's cells are b, a, b of two pairs, else a, b, a
+#pragma unroll
+    for (int ox = 0; ox < 3; ++ox) {
+#pragma unroll
+      for (int oy = 0; oy < 3; ++oy) {
+        const float4* row = gp + idx3((ix + ox - 1) & m, (iy + oy - 1) & m, 0, log2n);
+        const CellPair u = load_pair(row + k0), v = load_pair(row + k1);
+        const float wxy = wx[ox] * wy[oy];
+        const float w0 = wxy * wz[0], w1 = wxy * wz[1], w2 = wxy * wz[2];
+        ax = fmaf(w0, odd ? u.b.x : u.a.x, ax);
+        ay = fmaf(w0, odd ? u.b.y : u.a.y, ay);
+        az = fmaf(w0, odd ? u.b.z : u.a.z, az);
+        ax = fmaf(w1, odd ? v.a.x : u.b.x, ax);
+        ay = fmaf(w1, odd ? v.a.y : u.b.y, ay);
+        az = fmaf(w1, odd ? v.a.z : u.b.z, az);
+        ax = fmaf(w2, odd ? v.b.x : v.a.x, ax);
+        ay = fmaf(w2, odd ? v.b.y : v.a.y, ay);
+        az = fmaf(w2, odd ? v.b.z : v.a.z, az);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int ox = 0; ox < 3; ++ox) {
+#pragma unroll
+      for (int oy = 0; oy < 3; ++oy) {
+        const float wxy = wx[ox] * wy[oy];
+#pragma unroll
+        for (int oz = 0; oz < 3; ++oz) {
+          const int64_t c = idx3((ix + ox - 1) & m, (iy + oy - 1) & m, (iz + oz - 1) & m, log2n);
+          const float w = wxy * wz[oz];
+          ax = fmaf(w, __ldg(g + c), ax);
+          ay = fmaf(w, __ldg(g + N + c), ay);
+          az = fmaf(w, __ldg(g + 2 * N + c), az);
+        }
+      }
+    }
+  }
+  acc[p] = ax;
+  acc[np + p] = ay;
+  acc[2 * np + p] = az;
 }
 
 // Force and inverse TSC + kick-drift-kick in one pass for cell-sorted
@@ -535,50 +617,50 @@ __global__ void __launch_bounds__(1024) k_max_pairs(const float2* __restrict__ v
 }
 
 template <int ORDER>
-pm_status launch_grad(const float* phi, const float* eps, float alpha, float* g, int n, bool vec4, cudaStream_t s,
-                      int B, int nh) {
+pm_status launch_grad(const float* phi, const float* eps, float alpha, float* g, int n, cudaStream_t s, int B, int nh) {
   const int64_t N = (int64_t)n * n * n;
-  const double bytes = ((eps ? 8.0 : 4.0) * N + (vec4 ? 16.0 : 12.0) * N) * B;
-  if (n >= 64) {
-    constexpr int R = Stencil<ORDER>::R;
-    constexpr size_t smem = sizeof(float) * (2 * R + 1) * (GTY + 2 * R) * (GTZ + 2 * R);
-    const int tiles = (n / GTY) * (n / GTZ);
-    int chunk = n;
-    while (chunk > 16 && (int64_t)tiles * (n / chunk) < 8 * 152) chunk >>= 1;
-    const int nitems = tiles * (n / chunk);
-    unsigned gx = (unsigned)(nitems < 152 * 4 ? nitems : 152 * 4);
-    if (B > 1) gx = (unsigned)nitems;   // the boxes fill the GPU: one item per CTA
-    const dim3 grid(gx, 1, (unsigned)B);
-#define PM_GRAD_STREAM(FRB, V4)                                                                                    \
-  PM_LAUNCH(K_GRADIENT, bytes, (k_gradient_stream<ORDER, FRB, V4>), grid, GNT, smem, s, phi, eps, alpha, g, ilog2(n), \
-            (float)n, chunk, nitems, nh)
-    if (eps) {
-      if (vec4) PM_GRAD_STREAM(true, true); else PM_GRAD_STREAM(true, false);
-    } else {
-      if (vec4) PM_GRAD_STREAM(false, true); else PM_GRAD_STREAM(false, false);
-    }
-#undef PM_GRAD_STREAM
-    return launch_status();
-  }
-  if (vec4) return PM_EINVAL;
-  const dim3 grid(grid_for(N, 256), 1, (unsigned)B);
+  const double bytes = ((eps ? 8.0 : 4.0) * N + 12.0 * N) * B;
+  const unsigned gx = grid_for((int64_t)n * n / 4, GNT);
+  int chunk = n < 16 ? n : 16;   // planes a thread marches over, as many as leave four CTAs per SM
+  while (chunk > 1 && (int64_t)gx * (n / chunk) * B < 4 * 152) chunk >>= 1;
+  const dim3 grid(gx, (unsigned)(n / chunk), (unsigned)B);
   if (eps)
-    PM_LAUNCH(K_GRADIENT, bytes, (k_gradient<ORDER, true>), grid, 256, 0, s, phi, eps, alpha, g, ilog2(n), (float)n,
-              nh);
+    PM_LAUNCH(K_GRADIENT, bytes, (k_gradient<ORDER, true>), grid, GNT, 0, s, phi, eps, alpha, g, ilog2(n), (float)n,
+              chunk, nh);
   else
-    PM_LAUNCH(K_GRADIENT, bytes, (k_gradient<ORDER, false>), grid, 256, 0, s, phi, eps, alpha, g, ilog2(n), (float)n,
-              nh);
+    PM_LAUNCH(K_GRADIENT, bytes, (k_gradient<ORDER, false>), grid, GNT, 0, s, phi, eps, alpha, g, ilog2(n), (float)n,
+              chunk, nh);
   return launch_status();
 }
 
 }  // namespace
 
-pm_status gradient_launch(const float* phi, const float* eps, float alpha, float* g, int n, int order, bool vec4,
-                          cudaStream_t s, int batch, int nh) {
-  if (order == 3) return launch_grad<3>(phi, eps, alpha, g, n, vec4, s, batch, nh);
-  if (order == 5) return launch_grad<5>(phi, eps, alpha, g, n, vec4, s, batch, nh);
-  if (order == 7) return launch_grad<7>(phi, eps, alpha, g, n, vec4, s, batch, nh);
+pm_status gradient_launch(const float* phi, const float* eps, float alpha, float* g, int n, int order, cudaStream_t s,
+                          int batch, int nh) {
+  if (order == 3) return launch_grad<3>(phi, eps, alpha, g, n, s, batch, nh);
+  if (order == 5) return launch_grad<5>(phi, eps, alpha, g, n, s, batch, nh);
+  if (order == 7) return launch_grad<7>(phi, eps, alpha, g, n, s, batch, nh);
   return PM_EINVAL;
+}
+
+// The field is packed where that pays.  Per warp of particles the gather costs
+// 81 lookups for each row of cells the warp touches from the planes and 18 (and
+// some more for the wider cells) from the packed field; packing a cell costs
+// about as much as 43 lookups a warp at one particle per cell (all measured at
+// 256^3: cell-ordered particles planes 0.36, packed 0.40 ms at one particle per
+// cell and 0.13, 0.23 ms at a quarter; in random order 5.7 against 2.6 and 1.4
+// against 0.73 ms).
+pm_status interp_packed_launch(const float* g, const uint32_t* X, int64_t np, int n, float* acc, int* flag,
+                               float4* packed, cudaStream_t s) {
+  if (np < 32) return PM_EINVAL;
+  const int64_t N = (int64_t)n * n * n;
+  const float gain = 81.0f - 18.0f, cost = 108.0f + 43.0f * (float)N / (float)np;
+  PM_LAUNCH(K_INTERP, 0.0, k_interp_order, 1, 1024, 0, s, X, np, ilog2(n), gain, cost, flag);
+  // counted as small, so that its launch overlaps the sample (most of it exits at once where the flag is 0)
+  PM_LAUNCH(K_INTERP, 0.0, k_pack_force, grid_for(N / 4, 256, 152 * 8), 256, 0, s, g, packed, N, flag);
+  PM_LAUNCH(K_INTERP, 12.0 * N + 24.0 * np, k_interp_packed, grid_for(np, 256), 256, 0, s, packed, g, X, np, ilog2(n),
+            acc, flag);
+  return launch_status();
 }
 
 template <int ORDER>
@@ -654,23 +736,19 @@ pm_status force_interp_launch(const float* phi, const float* eps, float alpha, i
 
 pm_status interp_launch(const float* g, const uint32_t* Xs, const float* Vs, const uint32_t* ids_in, int64_t np,
                         int n, float* acc, uint32_t* Xo, float* Vo, uint32_t* ids_out, float dt_kick,
-                        float dt_drift, int mode, bool vec4, cudaStream_t s, const Batch& bt,
+                        float dt_drift, int mode, cudaStream_t s, const Batch& bt,
                         float2* blockmax, double* max_out) {
   if (np == 0) return PM_OK;
   const float drift_scale = (float)((double)dt_drift * 4294967296.0);
-  const double bytes = (vec4 ? 16.0 : 12.0) * n * n * (double)n * bt.B +
+  const double bytes = 12.0 * n * n * (double)n * bt.B +
                        np * (12.0 + (mode ? 36.0 : 0.0) + (acc ? 12.0 : 0.0) + (ids_out ? 8.0 : 0.0));
   const int64_t np_box = bt.B > 1 ? bt.np_box : np;
   const dim3 grid(grid_for(np_box, 256), 1, (unsigned)bt.B);
   if (!max_out) blockmax = nullptr;
-#define PM_INTERP(V4, MX)                                                                                       \
-  PM_LAUNCH(K_INTERP, bytes, (k_interp_kdk<V4, MX>), grid, 256, 0, s, g, Xs, Vs, ids_in, np, ilog2(n), acc, Xo, Vo, \
-            ids_out, dt_kick, drift_scale, mode, np_box, bt.dt_kick, bt.dt_drift, blockmax)
-  if (vec4) {
-    if (blockmax) PM_INTERP(true, true); else PM_INTERP(true, false);
-  } else {
-    if (blockmax) PM_INTERP(false, true); else PM_INTERP(false, false);
-  }
+#define PM_INTERP(MX)                                                                                               \
+  PM_LAUNCH(K_INTERP, bytes, k_interp_kdk<MX>, grid, 256, 0, s, g, Xs, Vs, ids_in, np, ilog2(n), acc, Xo, Vo, ids_out, \
+            dt_kick, drift_scale, mode, np_box, bt.dt_kick, bt.dt_drift, blockmax)
+  if (blockmax) PM_INTERP(true); else PM_INTERP(false);
 #undef PM_INTERP
   if (blockmax) {
     const int64_t nb = (int64_t)grid.x * grid.z;

@@ -224,17 +224,21 @@ pm_status prolong_correct_launch(float* u, const float* uc, const float* uc2, in
 // Background constants of the f(R) equation (host, float64).
 void fr_background(const fr_params& p, double* fbar, double* kappa, double* c2);
 
-// g = -grad(phi [+ alpha ((1 + eps)^(nh+1) - 1)]); vec4: g interleaved as float4
-// (gx, gy, gz, 0) per cell (n >= 64 only), else three planes.
-pm_status gradient_launch(const float* phi, const float* eps, float alpha, float* g, int n,
-                          int order, bool vec4, cudaStream_t s, int batch = 1, int nh = 1);
-// mode 0: acc only; mode 1: kick + drift into Xo/Vo (and acc if non-NULL);
-// vec4: g interleaved as float4.  With max_out (2 doubles, device) also the
-// largest |a| and |v after the kick| (blockmax: one float2 per block).
+// g = -grad(phi [+ alpha ((1 + eps)^(nh+1) - 1)]), three planes.
+pm_status gradient_launch(const float* phi, const float* eps, float alpha, float* g, int n, int order, cudaStream_t s,
+                          int batch = 1, int nh = 1);
+// mode 0: acc only; mode 1: kick + drift into Xo/Vo (and acc if non-NULL).
+// With max_out (2 doubles, device) also the largest |a| and |v after the kick|
+// (blockmax: one float2 per block).
 pm_status interp_launch(const float* g, const uint32_t* Xs, const float* Vs, const uint32_t* ids_in,
                         int64_t np, int n, float* acc, uint32_t* Xo, float* Vo, uint32_t* ids_out,
-                        float dt_kick, float dt_drift, int mode, bool vec4, cudaStream_t s,
+                        float dt_kick, float dt_drift, int mode, cudaStream_t s,
                         const Batch& bt = Batch{}, float2* blockmax = nullptr, double* max_out = nullptr);
+// acc = the force at X (np >= 32), by way of the field packed as float4 cells
+// (packed: n^3, 32-byte aligned) where the particles' order makes that the
+// faster one; bitwise interp_launch.
+pm_status interp_packed_launch(const float* g, const uint32_t* X, int64_t np, int n, float* acc, int* flag,
+                               float4* packed, cudaStream_t s);
 
 // The force g = -grad(phi [+ alpha ((1 + eps)^(nh+1) - 1)]) (order 3, 5 or
 // 7) computed in shared memory and interpolated at the cell-sorted particles
@@ -280,9 +284,14 @@ pm_status fetch_scalars(const double* dev, double* host, int count, cudaStream_t
 namespace pmgb {
 // First statement of every kernel: waits until the kernels before it in the
 // stream have finished and their writes are visible, then lets the next
-// kernel's blocks be placed as soon as this kernel's last ones are.
+// kernel's blocks be placed as soon as this kernel's last ones are.  Loads
+// through __ldg count as invariant and may be moved across a memory clobber,
+// but not out of the block behind a branch on a value the compiler cannot see
+// (always 0): they stay behind the wait.
 __device__ __forceinline__ void pdl_entry() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  unsigned never;
+  asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(never)::"memory");
+  if (never) asm volatile("exit;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 

@@ -119,6 +119,8 @@ _SIGS = {
     "pm_gradient": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_void_p]),
     "pm_interp": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, ctypes.c_void_p,
                                  ctypes.c_void_p]),
+    "pm_interp_packed": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64, ctypes.c_int,
+                                        ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p]),
     "pm_step": (ctypes.c_int, [ctypes.POINTER(pm_state), ctypes.POINTER(pm_step_params), ctypes.POINTER(pm_stats),
                                ctypes.c_void_p]),
     "pm_step_host": (ctypes.c_int, [ctypes.POINTER(pm_state), ctypes.POINTER(pm_step_params),
@@ -344,6 +346,15 @@ def interp(g, X):
     n = g.shape[1]
     np_ = X.shape[1]
     acc = torch.empty((3, np_), dtype=torch.float32, device=X.device)
+    if np_ >= 2 ** 17 and 40 * np_ >= n ** 3:   # below, pm_interp_packed takes pm_interp's way
+        try:
+            ws = torch.empty(16 * n ** 3 + 256, dtype=torch.uint8, device=X.device)
+        except torch.cuda.OutOfMemoryError:
+            ws = None
+        if ws is not None:
+            _check(lib().pm_interp_packed(_p(g, torch.float32), _p(X, torch.int32), np_, n, _p(acc), _p(ws),
+                                          ws.numel(), _stream()), "pm_interp_packed")
+            return acc
     _check(lib().pm_interp(_p(g, torch.float32), _p(X, torch.int32), np_, n, _p(acc), _stream()), "pm_interp")
     return acc
 

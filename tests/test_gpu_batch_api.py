@@ -69,3 +69,24 @@ def test_gradient_and_interp_batch_equal_single_boxes(pm):
         assert torch.equal(g[b], gb), b
         Xb = pm.positions_to_device(np.ascontiguousarray(X[:, b * np_box:(b + 1) * np_box]))
         assert np.array_equal(acc[:, b * np_box:(b + 1) * np_box], pm.interp(gb, Xb).cpu().numpy()), b
+
+
+@pytest.mark.parametrize("n,N,order", [(64, 1 << 17, "random"), (64, (1 << 17) + 1, "cells"), (128, 300007, "random"),
+                                       (4, 1 << 17, "random")])
+def test_interp_of_many_particles_is_bitwise_the_plain_gather(pm, n, N, order):
+    """Many particles take the packed field where their order is scattered
+    (and the planes where it is not): bitwise pm_interp either way."""
+    import ctypes
+    g = torch.from_numpy(np.stack([inputs.random_field(n, 40 + d) for d in range(3)]).astype(np.float32)).cuda()
+    X = inputs.uniform_particles(N, 6)
+    if order == "cells":
+        c = X >> np.uint32(32 - int(np.log2(n)))
+        X = X[:, np.lexsort((c[2], c[1], c[0]))]
+    Xd = pm.positions_to_device(X)
+    plain = torch.empty((3, N), dtype=torch.float32, device="cuda")
+    code = pm.lib().pm_interp(pm._p(g), pm._p(Xd), N, n, pm._p(plain), pm._stream())
+    assert code == 0
+    assert torch.equal(pm.interp(g, Xd), plain)
+    small = torch.empty(16 * n ** 3, dtype=torch.uint8, device="cuda")
+    assert pm.lib().pm_interp_packed(pm._p(g), pm._p(Xd), N, n, pm._p(plain), pm._p(small),
+                                     ctypes.c_size_t(small.numel()), pm._stream()) == 2
