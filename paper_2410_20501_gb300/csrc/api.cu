@@ -118,10 +118,10 @@ size_t layout_workspace(Workspace* w, void* base, int n, int64_t np, uint32_t fl
     w->adj_psi = (float*)take((size_t)N * 4);
     w->adj_gbar = (float*)take((size_t)N * 12);
   }
-  if (flags & PM_WS_FFT) w->spec = (float2*)take((size_t)n * n * (n / 2 + 1) * 8 * batch);
+  if (flags & PM_WS_FFT) w->spec = (float2*)take((size_t)n * n * (n / 2 + 8) * 8 * batch);   // rows of pitch n/2 + 8
   if (flags & PM_WS_LPT) {
-    w->lpt_a = (float2*)take((size_t)n * n * (n / 2 + 1) * 8);
-    w->lpt_b = (float2*)take((size_t)n * n * (n / 2 + 1) * 8);
+    w->lpt_a = (float2*)take((size_t)n * n * (n / 2 + 8) * 8);
+    w->lpt_b = (float2*)take((size_t)n * n * (n / 2 + 8) * 8);
     w->lpt_r = (float*)take((size_t)N * 4 * 5);
   }
   if (flags & PM_WS_REFINE) {

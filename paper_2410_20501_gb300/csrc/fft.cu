@@ -3,10 +3,11 @@
 // compensation) and FFT (-1 / (k^2 W_TSC(k)^2), W_TSC = prod_d sinc(pi m_d / n)^3).
 //
 // phi = scale * IFFT[ G(k) FFT[rho] ] with G(0) = 0 (which also removes the
-// mean of rho).  The transforms are hand-written: a shared-memory Stockham
-// FFT (radix 8, then 4 or 2; a thread holds 8 points per stage), twiddles from
-// a float2 table built in float64 on the host.  Passes over HBM, with the
-// half-spectrum C[x][y][kz], kz = 0 .. n/2, stored as float2 rows of n/2 + 1:
+// mean of rho).  The transforms are hand-written: a Stockham FFT (radix 8, then
+// 4 or 2) whose points stay in registers, eight to a thread, and pass through
+// shared memory only between stages; twiddles from a float2 table built in
+// float64 on the host.  Passes over HBM, with the half-spectrum C[x][y][kz],
+// kz = 0 .. n/2, stored as float2 rows of pitch n/2 + 8 (64-byte aligned):
 //   z: real rows -> n/2-point complex FFT of the even/odd pairs -> n/2 + 1
 //      outputs (R2C);
 //   y: forward FFT of the columns;
@@ -99,59 +100,103 @@ template <int R, bool INV> __device__ __forceinline__ void dft_r(float2* v) {
   else dft2<INV>(v[0], v[1]);
 }
 
-// One Stockham stage of radix R on a line of L points at a (stride-1), done
-// by the L/8 threads of the line (thread t): 8/R butterflies per thread.
-template <int L, int R, bool INV>
-__device__ __forceinline__ void stockham_stage(float2* a, int t, int Ns) {
-  constexpr int PER = 8 / R, Q = L / R;
-  float2 v[8];
-  int base[PER];
+// Place of point i in a line's shared memory, without bank conflicts for the
+// accesses of 16 lanes in a line's first stages: points 1, 8 and 8 + a jump of
+// 64 apart.  Where a line's lanes follow each other (z passes) the place is the
+// point with its low bits exchanged by its high ones; where the lanes run over
+// the lines first (column passes, COLS) one float2 of padding follows every
+// eight.
+template <bool COLS>
+__device__ __forceinline__ constexpr int place(int i) {
+  return COLS ? i + (i >> 3) : i ^ ((i >> 4) & 7) ^ ((i >> 3) & 8);
+}
+
+// One Stockham stage of radix R after Ns points were combined: 8/R butterflies
+// on v, thread t of the line's L/8; v[q + (8/R) r] is point
+// t + (q + (8/R) r) L/8 of the line on entry.
+template <int L, int R, int NS, bool INV>
+__device__ __forceinline__ void butterflies(float2 v[8], int t) {
+  constexpr int PER = 8 / R;
 #pragma unroll
   for (int q = 0; q < PER; ++q) {
-    const int j = t + q * (L / 8);
-    const int k = j & (Ns - 1);                  // Ns is a power of two
-    base[q] = (j - k) * R + k;
+    float2 w[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[q * R + r] = a[j + r * Q];
-    if (Ns > 1) {
-      const int step = L / (Ns * R);
+    for (int r = 0; r < R; ++r) w[r] = v[q + PER * r];
+    if (NS > 1) {
+      constexpr int step = L / (NS * R);
+      const int k = (t + q * (L / 8)) & (NS - 1);
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        float2 w = g_tw[L + r * k * step];
-        if (INV) w = cconj(w);
-        v[q * R + r] = cmul(v[q * R + r], w);
+        float2 tw = g_tw[L + r * k * step];
+        if (INV) tw = cconj(tw);
+        w[r] = cmul(w[r], tw);
       }
     }
-    dft_r<R, INV>(v + q * R);
+    dft_r<R, INV>(w);
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[q + PER * r] = w[r];
+  }
+}
+
+// Moves the results of a stage of radix R (after NS combined points) to where
+// the next stage reads them: v[i] is point t + i L/8 again.
+template <int L, int R, int NS, bool COLS>
+__device__ __forceinline__ void exchange(float2 v[8], float2* line, int t) {
+  constexpr int PER = 8 / R;
+  __syncthreads();   // the line is free
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const int j = t + q * (L / 8), k = j & (NS - 1), base = (j - k) * R + k;
+#pragma unroll
+    for (int r = 0; r < R; ++r) line[place<COLS>(base + r * NS)] = v[q + PER * r];
   }
   __syncthreads();
 #pragma unroll
-  for (int q = 0; q < PER; ++q)
-#pragma unroll
-    for (int r = 0; r < R; ++r) a[base[q] + r * Ns] = v[q * R + r];
-  __syncthreads();
+  for (int i = 0; i < 8; ++i) v[i] = line[place<COLS>(t + i * (L / 8))];
 }
 
-// In-place FFT of the line at a (L points, unnormalised), by its L/8
-// threads; all threads of the block must call it (it synchronises).
-template <int L, bool INV>
-__device__ __forceinline__ void fft_line(float2* a, int t) {
+// FFT of a line of L points, unnormalised: v[i] is point t + i L/8 before and
+// after, for the line's L/8 threads t.  All threads of the block must call it
+// (it synchronises); line: this line's shared memory (line_places).
+template <int L, bool INV, bool COLS>
+__device__ __forceinline__ void fft_line(float2 v[8], float2* line, int t) {
   constexpr int LOG = (L >= 1024) ? 10 : (L >= 512) ? 9 : (L >= 256) ? 8 : (L >= 128) ? 7 : (L >= 64) ? 6 :
                       (L >= 32) ? 5 : (L >= 16) ? 4 : 3;
-  constexpr int S8 = LOG / 3, REM = LOG % 3;
-  int Ns = 1;
-#pragma unroll
-  for (int s = 0; s < S8; ++s) {
-    stockham_stage<L, 8, INV>(a, t, Ns);
-    Ns *= 8;
+  constexpr int S8 = LOG / 3, LAST = 1 << (LOG % 3);   // radix-8 stages, then one of radix LAST (if above 1)
+  butterflies<L, 8, 1, INV>(v, t);
+  if constexpr (S8 >= 2) {
+    exchange<L, 8, 1, COLS>(v, line, t);
+    butterflies<L, 8, 8, INV>(v, t);
   }
-  if constexpr (REM == 2) stockham_stage<L, 4, INV>(a, t, Ns);
-  if constexpr (REM == 1) stockham_stage<L, 2, INV>(a, t, Ns);
+  if constexpr (S8 >= 3) {
+    exchange<L, 8, 8, COLS>(v, line, t);
+    butterflies<L, 8, 64, INV>(v, t);
+  }
+  if constexpr (LAST > 1) {
+    constexpr int NS = L / LAST;
+    exchange<L, 8, NS / 8, COLS>(v, line, t);
+    butterflies<L, LAST, NS, INV>(v, t);
+  }
 }
 
-// Lines per block: 4096 points per block (32 KB of shared memory), capped
-// by the number of lines available.
-template <int L> __host__ __device__ constexpr int lines_per_block() { return 4096 / L < 1 ? 1 : 4096 / L; }
+// Lines per block: 4096 points a block, at least 8 lines (64-byte runs of a
+// column pass) and at most 32.
+template <int L> __host__ __device__ constexpr int lines_per_block() {
+  return 4096 / L < 8 ? 8 : 4096 / L > 32 ? 32 : 4096 / L;
+}
+// Shared places of a line: a column pass, whose lanes take eight lines times two
+// points or sixteen lines at a time, staggers its lines over the banks.
+template <int L, bool COLS> __host__ __device__ constexpr int line_places() {
+  return COLS ? (L + L / 8 + 15) / 16 * 16 + (lines_per_block<L>() == 8 ? 2 : 1) : L < 16 ? 16 : L;
+}
+template <int L, bool COLS> constexpr size_t lines_smem() {
+  return sizeof(float2) * lines_per_block<L>() * line_places<L, COLS>();
+}
+// Pitch of the half spectrum's rows (float2).
+__host__ __device__ constexpr int spec_pitch(int n) { return n / 2 + 8; }
+
+// 512^3: a whole solve 2.90 -> 1.45 ms, 256^3 0.39 -> 0.20 ms against stages
+// that each read and write shared memory.
 
 // ---- z pass: real rows of n = 2M values <-> n/2 + 1 complex ----
 // Forward: Z_m = x_2m + i x_2m+1, Z = FFT_M(Z), X[k] = E + w_n^k O with
@@ -165,27 +210,32 @@ __global__ void __launch_bounds__(lines_per_block<M>() * (M / 8)) k_fft_z_r2c(co
                                                                               float2* __restrict__ out,
                                                                               int64_t rows) {
   pdl_entry();
-  constexpr int LB = lines_per_block<M>(), TPL = M / 8, LP = M + 1, H = M + 1, n = 2 * M;
-  __shared__ float2 s[LB * LP];
+  constexpr int LB = lines_per_block<M>(), TPL = M / 8, LP = line_places<M, false>(), H = M + 1, n = 2 * M;
+  extern __shared__ float2 fft_sm[];
   const int64_t row0 = (int64_t)blockIdx.x * LB;
   const int nl = (int)((rows - row0) < LB ? (rows - row0) : LB);
   const float mu = mean ? (float)*mean : 0.0f;
-  for (int e = threadIdx.x; e < nl * M; e += blockDim.x) {
-    const int l = e / M, m = e - l * M;
-    const float2 v = __ldg(reinterpret_cast<const float2*>(in + (row0 + l) * n) + m);
-    s[l * LP + m] = make_float2(v.x - mu, v.y - mu);
-  }
-  __syncthreads();
   const int line = threadIdx.x / TPL, t = threadIdx.x - line * TPL;
-  fft_line<M, false>(s + line * LP, t);
+  float2 v[8];
+  const float2* src = reinterpret_cast<const float2*>(in + (row0 + (line < nl ? line : 0)) * n) + t;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __ldg(src + i * TPL);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = make_float2(v[i].x - mu, v[i].y - mu);
+  float2* s = fft_sm + line * LP;
+  fft_line<M, false, false>(v, s, t);
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) s[place<false>(t + i * TPL)] = v[i];
+  __syncthreads();
   for (int e = threadIdx.x; e < nl * H; e += blockDim.x) {
     const int l = e / H, k = e - l * H;
-    const float2 zk = s[l * LP + (k == M ? 0 : k)];
-    const float2 zc = cconj(s[l * LP + (k == 0 ? 0 : M - k)]);
+    const float2 zk = fft_sm[l * LP + place<false>(k == M ? 0 : k)];
+    const float2 zc = cconj(fft_sm[l * LP + place<false>(k == 0 ? 0 : M - k)]);
     const float2 E = make_float2(0.5f * (zk.x + zc.x), 0.5f * (zk.y + zc.y));
     const float2 D = csub(zk, zc);
     const float2 O = make_float2(0.5f * D.y, -0.5f * D.x);        // -i D / 2
-    out[(row0 + l) * H + k] = cadd(E, cmul(g_tw[n + k], O));      // k <= M < n
+    out[(row0 + l) * spec_pitch(n) + k] = cadd(E, cmul(g_tw[n + k], O));      // k <= M < n
   }
 }
 
@@ -196,37 +246,31 @@ __global__ void __launch_bounds__(lines_per_block<M>() * (M / 8)) k_fft_z_c2r(co
                                                                               float* __restrict__ out,
                                                                               int64_t rows) {
   pdl_entry();
-  constexpr int LB = lines_per_block<M>(), TPL = M / 8, LP = M + 1, H = M + 1, n = 2 * M;
-  __shared__ float2 s[LB * LP];
+  constexpr int LB = lines_per_block<M>(), TPL = M / 8, LP = line_places<M, false>(), n = 2 * M;
+  extern __shared__ float2 fft_sm[];
   const int64_t row0 = (int64_t)blockIdx.x * LB;
   const int nl = (int)((rows - row0) < LB ? (rows - row0) : LB);
-  for (int e = threadIdx.x; e < nl * H; e += blockDim.x) {
-    const int l = e / H, k = e - l * H;
-    s[l * LP + k] = __ldg(in + (row0 + l) * H + k);
+  const int line = threadIdx.x / TPL, t = threadIdx.x - line * TPL;
+  const float2* src = in + (row0 + (line < nl ? line : 0)) * spec_pitch(n);
+  float2 v[8], c[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    v[i] = __ldg(src + t + i * TPL);
+    c[i] = __ldg(src + M - t - i * TPL);
   }
-  __syncthreads();
-  float2 z[(LB * M + lines_per_block<M>() * (M / 8) - 1) / (lines_per_block<M>() * (M / 8))];
-  int cnt = 0;
-  for (int e = threadIdx.x; e < nl * M; e += blockDim.x, ++cnt) {
-    const int l = e / M, k = e - l * M;
-    const float2 xk = s[l * LP + k], xc = cconj(s[l * LP + M - k]);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float2 xk = v[i], xc = cconj(c[i]);
     const float2 E = make_float2(0.5f * (xk.x + xc.x), 0.5f * (xk.y + xc.y));
     const float2 D = make_float2(0.5f * (xk.x - xc.x), 0.5f * (xk.y - xc.y));
-    const float2 O = cmul(D, cconj(g_tw[n + k]));
-    z[cnt] = make_float2(E.x - O.y, E.y + O.x);                   // E + i O
+    const float2 O = cmul(D, cconj(g_tw[n + t + i * TPL]));
+    v[i] = make_float2(E.x - O.y, E.y + O.x);                   // E + i O
   }
-  __syncthreads();
-  cnt = 0;
-  for (int e = threadIdx.x; e < nl * M; e += blockDim.x, ++cnt) {
-    const int l = e / M, k = e - l * M;
-    s[l * LP + k] = z[cnt];
-  }
-  __syncthreads();
-  const int line = threadIdx.x / TPL, t = threadIdx.x - line * TPL;
-  fft_line<M, true>(s + line * LP, t);
-  for (int e = threadIdx.x; e < nl * M; e += blockDim.x) {
-    const int l = e / M, m = e - l * M;
-    reinterpret_cast<float2*>(out + (row0 + l) * n)[m] = s[l * LP + m];
+  fft_line<M, true, false>(v, fft_sm + line * LP, t);
+  if (line < nl) {
+    float2* dst = reinterpret_cast<float2*>(out + (row0 + line) * n) + t;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) dst[i * TPL] = v[i];
   }
 }
 
@@ -258,31 +302,41 @@ struct Mult {
 // inverse, write `out` (x pass); SOLVE: forward, multiply, inverse (x pass).
 enum ColMode { FWD = 0, INVT = 1, FWDMUL = 2, MULINV = 3, SOLVE = 4 };
 
+// A block's lanes run over its columns first (64-byte runs of every row), so a
+// point of a line is read from memory into the register the first butterfly
+// takes it from and written from the one the last leaves it in; the spectral
+// multiplier meets its points in registers too.  16 bytes a point: at 512^3 a y
+// pass takes 0.19 ms (5.7 TB/s, bound by HBM), the x pass with both transforms
+// 0.41 ms (bound by its exchanges: shared memory and issue), against 0.56 ms
+// each with every stage through shared memory.  Registers are sized for four
+// resident CTAs of 512 threads per SM, for three in the x pass (0.42 ms with
+// four, 0.58 with two); 1024-point lines keep the compiler's choice.
 template <int L, int AXIS, int MODE>
-__global__ void __launch_bounds__(lines_per_block<L>() * (L / 8)) k_fft_cols(const float2* in, float2* out,
+__global__ void __launch_bounds__(lines_per_block<L>() * (L / 8), L <= 512 ? (MODE == SOLVE ? 3 : 4) : 0) k_fft_cols(const float2* in, float2* out,
                                                                              int ntiles, Mult mu) {
   pdl_entry();
   constexpr bool MUL = MODE == FWDMUL || MODE == MULINV || MODE == SOLVE;
-  constexpr int TW = lines_per_block<L>(), TPL = L / 8, LP = L + 1, n = L, H = n / 2 + 1;
-  __shared__ float2 s[TW * LP];
+  constexpr int TW = lines_per_block<L>(), TPL = L / 8, LP = line_places<L, true>(), n = L, H = n / 2 + 1, P = spec_pitch(n);
+  extern __shared__ float2 fft_sm[];
   __shared__ float ta[MUL ? n : 1], tb[MUL ? n : 1];
   const int tile = blockIdx.x % ntiles, other = blockIdx.x / ntiles;   // other: x (AXIS 1) or y (AXIS 0)
-  const int kz0 = tile * TW;
-  const int tw = (H - kz0) < TW ? (H - kz0) : TW;
-  const int64_t stride = AXIS == 1 ? H : (int64_t)n * H;
-  const int64_t base = (AXIS == 1 ? (int64_t)other * n * H : (int64_t)other * H) + kz0;
-  for (int e = threadIdx.x; e < tw * L; e += blockDim.x) {
-    const int i = e / tw, l = e - i * tw;
-    s[l * LP + i] = in[base + i * stride + l];
-  }
+  const int l = threadIdx.x % TW, t = threadIdx.x / TW;
+  const int kz = tile * TW + l;
+  const bool live = kz < H;
+  constexpr int64_t stride = AXIS == 1 ? P : (int64_t)n * P;
+  const int64_t base = (AXIS == 1 ? (int64_t)other * n * P : (int64_t)other * P) + (live ? kz : 0) + t * stride;
+  float2 v[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = in[base + i * (TPL * stride)];
   if (MUL) {
-    // per-axis tables: GREEN7: sin^2(pi m/n); GREENTSC: k^2 and sinc^6;
-    // LPT kinds: k (0 on the Nyquist index, which also flags it in tb)
+    // per-axis tables: GREEN7: 4 n^2 sin^2(pi m/n) and 1; GREENTSC: k^2 and
+    // sinc^6; LPT kinds: k (0 on the Nyquist index, which also flags it in tb)
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
       const int m = i < n / 2 ? i : i - n;
       const float sp = sinpif((float)m / (float)n);
       if (mu.kind == GREEN7) {
-        ta[i] = sp * sp;
+        ta[i] = 4.0f * (float)n * (float)n * (sp * sp);
+        tb[i] = 1.0f;
       } else if (mu.kind == GREENTSC) {
         ta[i] = 39.47841760435743f * (float)m * (float)m;
         const float sc = m == 0 ? 1.0f : sp / (3.14159265358979f * (float)m / (float)n);
@@ -295,50 +349,50 @@ __global__ void __launch_bounds__(lines_per_block<L>() * (L / 8)) k_fft_cols(con
       }
     }
   }
-  __syncthreads();
-  const int line = threadIdx.x / TPL, t = threadIdx.x - line * TPL;
-  if (MODE == FWD || MODE == FWDMUL || MODE == SOLVE) fft_line<L, false>(s + line * LP, t);
-  if (MODE == INVT) fft_line<L, true>(s + line * LP, t);
+  float2* line = fft_sm + l * LP;
+  if (MODE == FWD || MODE == FWDMUL || MODE == SOLVE) fft_line<L, false, true>(v, line, t);
+  if (MODE == INVT) fft_line<L, true, true>(v, line, t);
   if (MUL) {
-    for (int e = threadIdx.x; e < tw * L; e += blockDim.x) {
-      const int l = e / L, i = e - l * L;          // kx index i, kz = kz0 + l
-      const int kz = kz0 + l;
-      float2& v = s[l * LP + i];
-      const int ix[3] = {i, other, kz};
-      if (mu.kind == GREEN7) {
-        const float lam = ta[i] + ta[other] + ta[kz];
-        const float g = lam > 0.0f ? -mu.scale / (4.0f * (float)n * (float)n * lam) : 0.0f;
-        v = make_float2(v.x * g, v.y * g);
-      } else if (mu.kind == GREENTSC) {
-        const float k2 = ta[i] + ta[other] + ta[kz];
-        const float g = k2 > 0.0f ? -mu.scale / (k2 * tb[i] * tb[other] * tb[kz]) : 0.0f;
-        v = make_float2(v.x * g, v.y * g);
-      } else {
-        const bool zero = tb[i] + tb[other] + tb[kz] > 0.0f || (i == 0 && other == 0 && kz == 0);
+    __syncthreads();   // the tables are complete
+    const int kzc = live ? kz : 0;
+    if constexpr (MODE == SOLVE) {
+      const float ao = ta[other], ak = ta[kzc], bo = tb[other], bk = tb[kzc];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int i = t + q * TPL;                   // kx index
+        const float k2 = ta[i] + ao + ak;
+        const float g = k2 > 0.0f ? -mu.scale / (k2 * tb[i] * bo * bk) : 0.0f;
+        v[q] = make_float2(v[q].x * g, v[q].y * g);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int i = t + q * TPL;                   // kx index
+        const int ix[3] = {i, other, kzc};
+        const bool zero = tb[i] + tb[other] + tb[kzc] > 0.0f || (i == 0 && other == 0 && kzc == 0);
         if (zero) {
-          v = make_float2(0.0f, 0.0f);
+          v[q] = make_float2(0.0f, 0.0f);
         } else if (mu.kind == DERIV) {
           const float k = mu.scale * ta[ix[mu.d1]];
-          v = make_float2(-k * v.y, k * v.x);                 // i k v
+          v[q] = make_float2(-k * v[q].y, k * v[q].x);                 // i k v
         } else {
           float g;
           if (mu.kind == HESS) {
             g = -mu.scale * ta[ix[mu.d1]] * ta[ix[mu.d2]];
           } else {
-            const float k2 = ta[i] * ta[i] + ta[other] * ta[other] + ta[kz] * ta[kz];
+            const float k2 = ta[i] * ta[i] + ta[other] * ta[other] + ta[kzc] * ta[kzc];
             g = -mu.scale / k2;
-            if (mu.kind == AMPLAP) g *= __ldg(mu.amp + ((int64_t)i * n + other) * H + kz);
+            if (mu.kind == AMPLAP) g *= __ldg(mu.amp + ((int64_t)i * n + other) * H + kzc);
           }
-          v = make_float2(v.x * g, v.y * g);
+          v[q] = make_float2(v[q].x * g, v[q].y * g);
         }
       }
     }
-    __syncthreads();
-    if (MODE == MULINV || MODE == SOLVE) fft_line<L, true>(s + line * LP, t);
+    if (MODE == MULINV || MODE == SOLVE) fft_line<L, true, true>(v, line, t);
   }
-  for (int e = threadIdx.x; e < tw * L; e += blockDim.x) {
-    const int i = e / tw, l = e - i * tw;
-    out[base + i * stride + l] = s[l * LP + i];
+  if (live) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) out[base + i * (TPL * stride)] = v[i];
   }
 }
 
@@ -346,6 +400,7 @@ __global__ void __launch_bounds__(lines_per_block<L>() * (L / 8)) k_fft_cols(con
 template <int N>
 struct FftPlan {
   static constexpr int M = N / 2, H = M + 1, LBz = lines_per_block<M>(), LBc = lines_per_block<N>();
+  static constexpr size_t smz = lines_smem<M, false>(), smc = lines_smem<N, true>();
   static constexpr int64_t rows = (int64_t)N * N;
   static constexpr double cells = (double)N * N * N, spec = (double)N * N * H * 8.0;
   static unsigned zblocks() { return (unsigned)((rows + LBz - 1) / LBz); }
@@ -353,15 +408,28 @@ struct FftPlan {
   static unsigned cblocks() { return (unsigned)(ntiles() * N); }
 };
 
+// Shared-memory limits of the column passes of an n^3 grid (above the default at
+// n = 1024 only).
+template <int N>
+pm_status fft_attributes() {
+  constexpr size_t b = FftPlan<N>::smc;
+  if (b <= 40 * 1024) return PM_OK;
+  PM_TRY(smem_attr(k_fft_cols<N, 1, FWD>, b));
+  PM_TRY(smem_attr(k_fft_cols<N, 1, INVT>, b));
+  PM_TRY(smem_attr(k_fft_cols<N, 0, SOLVE>, b));
+  PM_TRY(smem_attr(k_fft_cols<N, 0, FWDMUL>, b));
+  return smem_attr(k_fft_cols<N, 0, MULINV>, b);
+}
+
 // spec = M(k) FFT[real]  (unnormalised forward transform, then the multiplier)
 template <int N>
 pm_status fft_forward_mul(const float* real, const double* mean, float2* spec, const Mult& mu, cudaStream_t s) {
   using P = FftPlan<N>;
-  PM_LAUNCH(K_FFT, 4.0 * P::cells + P::spec, k_fft_z_r2c<P::M>, P::zblocks(), P::LBz * (P::M / 8), 0, s, real, mean,
+  PM_LAUNCH(K_FFT, 4.0 * P::cells + P::spec, k_fft_z_r2c<P::M>, P::zblocks(), P::LBz * (P::M / 8), P::smz, s, real, mean,
             spec, P::rows);
-  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 1, FWD>), P::cblocks(), P::LBc * (N / 8), 0, s, spec, spec,
+  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 1, FWD>), P::cblocks(), P::LBc * (N / 8), P::smc, s, spec, spec,
             P::ntiles(), mu);
-  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 0, FWDMUL>), P::cblocks(), P::LBc * (N / 8), 0, s, spec, spec,
+  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 0, FWDMUL>), P::cblocks(), P::LBc * (N / 8), P::smc, s, spec, spec,
             P::ntiles(), mu);
   return launch_status();
 }
@@ -371,11 +439,11 @@ pm_status fft_forward_mul(const float* real, const double* mean, float2* spec, c
 template <int N>
 pm_status fft_mul_inverse(const float2* spec, float2* tmp, float* real, const Mult& mu, cudaStream_t s) {
   using P = FftPlan<N>;
-  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 0, MULINV>), P::cblocks(), P::LBc * (N / 8), 0, s, spec, tmp,
+  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 0, MULINV>), P::cblocks(), P::LBc * (N / 8), P::smc, s, spec, tmp,
             P::ntiles(), mu);
-  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 1, INVT>), P::cblocks(), P::LBc * (N / 8), 0, s, tmp, tmp,
+  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 1, INVT>), P::cblocks(), P::LBc * (N / 8), P::smc, s, tmp, tmp,
             P::ntiles(), mu);
-  PM_LAUNCH(K_FFT, P::spec + 4.0 * P::cells, k_fft_z_c2r<P::M>, P::zblocks(), P::LBz * (P::M / 8), 0, s, tmp, real,
+  PM_LAUNCH(K_FFT, P::spec + 4.0 * P::cells, k_fft_z_c2r<P::M>, P::zblocks(), P::LBz * (P::M / 8), P::smz, s, tmp, real,
             P::rows);
   return launch_status();
 }
@@ -384,18 +452,19 @@ template <int N>
 pm_status launch_fft_poisson(const float* rho, const double* mean, float* phi, float2* C, int kind, double scale,
                              cudaStream_t s) {
   using P = FftPlan<N>;
+  PM_TRY(fft_attributes<N>());
   // the y and x transform pairs scale by n each, the z pair by n/2 (the
   // inverse runs an n/2-point transform of the packed pairs): divide by n^3/2
   const Mult mu{kind == 1 ? GREEN7 : GREENTSC, 0, 0, (float)(2.0 * scale / P::cells), nullptr};
-  PM_LAUNCH(K_FFT, 4.0 * P::cells + P::spec, k_fft_z_r2c<P::M>, P::zblocks(), P::LBz * (P::M / 8), 0, s, rho, mean,
+  PM_LAUNCH(K_FFT, 4.0 * P::cells + P::spec, k_fft_z_r2c<P::M>, P::zblocks(), P::LBz * (P::M / 8), P::smz, s, rho, mean,
             C, P::rows);
-  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 1, FWD>), P::cblocks(), P::LBc * (N / 8), 0, s, C, C, P::ntiles(),
+  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 1, FWD>), P::cblocks(), P::LBc * (N / 8), P::smc, s, C, C, P::ntiles(),
             mu);
-  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 0, SOLVE>), P::cblocks(), P::LBc * (N / 8), 0, s, C, C,
+  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 0, SOLVE>), P::cblocks(), P::LBc * (N / 8), P::smc, s, C, C,
             P::ntiles(), mu);
-  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 1, INVT>), P::cblocks(), P::LBc * (N / 8), 0, s, C, C,
+  PM_LAUNCH(K_FFT, 2.0 * P::spec, (k_fft_cols<N, 1, INVT>), P::cblocks(), P::LBc * (N / 8), P::smc, s, C, C,
             P::ntiles(), mu);
-  PM_LAUNCH(K_FFT, P::spec + 4.0 * P::cells, k_fft_z_c2r<P::M>, P::zblocks(), P::LBz * (P::M / 8), 0, s, C, phi,
+  PM_LAUNCH(K_FFT, P::spec + 4.0 * P::cells, k_fft_z_c2r<P::M>, P::zblocks(), P::LBz * (P::M / 8), P::smz, s, C, phi,
             P::rows);
   return launch_status();
 }
@@ -439,6 +508,7 @@ template <int N>
 pm_status launch_lpt2(const float* noise, const float* amp, float d1, float e2, float v1, float v2, uint32_t* X,
                       float* V, float2* A, float2* B, float* R, cudaStream_t s) {
   using P = FftPlan<N>;
+  PM_TRY(fft_attributes<N>());
   const int64_t NC = (int64_t)N * N * N;
   const float inv = (float)(2.0 / P::cells);
   float *H = R, *S = R + 3 * NC, *T = R + 4 * NC;

@@ -137,7 +137,7 @@ struct Workspace {
   // adjoint buffers
   float* adj_abar; float* adj_phi; float* adj_psi; float* adj_gbar;
   double* box_mean;   // per-box mean density of a batch
-  float2* spec;       // half spectrum n^2 (n/2 + 1) of the FFT Poisson path
+  float2* spec;       // half spectrum n^2 (n/2 + 8) of the FFT Poisson path
   float2* lpt_a; float2* lpt_b; float* lpt_r;   // LPT: two half spectra, five real grids
   float* ref_r; float* ref_e;                   // refinement: float32 residual and correction
   int64_t np; int n; int batch;
@@ -252,7 +252,7 @@ pm_status force_interp_launch(const float* phi, const float* eps, float alpha, i
 
 // phi = scale * IFFT[G FFT[rho - mean]], G(0) = 0; kind 1: FFT_7pt, 2: FFT
 // with the exact kernel and TSC deconvolution (§3.7); mean (device float64)
-// may be NULL.  C: n^2 (n/2 + 1) float2.
+// may be NULL.  C: n^2 (n/2 + 8) float2.
 pm_status fft_poisson_launch(const float* rho, const double* mean, float* phi, float2* C, int n, int kind,
                              double scale, cudaStream_t s);
 

@@ -102,3 +102,17 @@ def test_step_accelerations_with_fft_solvers(pm, kind):
     phi = poisson.solve_fft7(f, 1.0 / n) if kind == 1 else poisson.solve_fft_tsc(f, 1.0 / n)
     ref = mesh.interp_tsc(mesh.force_from_potential(phi, 1.0 / n), pos)
     assert rel_l2(acc.T, ref) < 1e-5
+
+
+@pytest.mark.parametrize("n", [16, 32, 1024])
+def test_fft7_of_a_plane_wave_at_the_smallest_and_largest_sizes(pm, n):
+    """phi of f = cos(2 pi (3 x + y) / L) along a few rows against the 7-point
+    symbol; the mode is exact, so the error is the transforms' rounding."""
+    k = torch.arange(n, device="cuda", dtype=torch.float32)
+    phase = 2.0 * np.pi * ((3.0 * k[:, None, None] + k[None, :, None]) % n) / n
+    rho = (1.0 + torch.cos(phase) * torch.ones(n, device="cuda")).contiguous()
+    phi = pm.poisson_fft(rho, kind=pm.PM_POISSON_FFT7)
+    lam = 4.0 * n * n * (np.sin(3.0 * np.pi / n) ** 2 + np.sin(np.pi / n) ** 2)
+    ref = -torch.cos(phase) / lam
+    # a transform of n^3 points rounds to about log2(n) ulp of the largest mode
+    assert float((phi - ref).abs().max()) < 3.0 * np.log2(n) * 6e-8 / lam * 4.0
