@@ -23,8 +23,7 @@
 
 #include "pm_device.cuh"
 #include "pm_internal.cuh"
-#include "rb_fused.cuh"
-#include "rb_stream.cuh"
+#include "rb_march.cuh"
 
 namespace pmgb {
 
@@ -40,16 +39,15 @@ __device__ __forceinline__ uint32_t idx3(int i, int j, int k, int log2n) {
 }
 
 // Root eps > -1 of g(e) = e^3 + 3e^2 + c1 e + c0 (g(-1) = q < 0, g convex on
-// e > -1, so the root is unique).  One Halley step from the current value
-// reaches float32 resolution in a warm sweep (the value moved little since
-// the last one); otherwise up to two plain Newton steps from the Halley
-// point, then Newton inside a shrinking bracket [lo, hi]; when a step leaves
-// the bracket (or g' <= 0) the upper end is set from the bound
-// u* <= sqrt(max(-p, 0)) + (-q)^(1/3), p = c1 - 3, and the step falls back to
-// bisection.  Stops when g is at its float32 rounding level or the step is
-// below 2e-7 relative.
+// e > -1, so the root is unique).  One step of root_step from the current value
+// reaches float32 resolution in a warm sweep (the value moved little since the
+// last one); what is left goes to Newton inside a shrinking bracket [lo, hi]
+// (fr_root): when a step leaves the bracket (or g' <= 0) the upper end is set
+// from the bound u* <= sqrt(max(-p, 0)) + (-q)^(1/3), p = c1 - 3, and the step
+// falls back to bisection.  It stops when g is at its float32 rounding level or
+// the step is below 2e-7 relative.
 // g(e) of the cell equation in eps = u - 1 (NH = 1: cubic, NH = 2: quartic),
-// its derivative, half its second and a sixth of its third derivative, the
+// its derivative, the
 // float32 rounding level of its evaluation, and an upper bound of the root
 // (from u* <= sqrt(max(-p, 0)) + (-q)^(1/3) for the cubic,
 // u* <= max(1, (|p| + |q|)^(1/3)) for the quartic).
@@ -57,8 +55,6 @@ template <int NH> struct CellPoly;
 template <> struct CellPoly<1> {
   __device__ static float g(float e, float c1, float c0) { return ((e + 3.0f) * e + c1) * e + c0; }
   __device__ static float gp(float e, float c1) { return (3.0f * e + 6.0f) * e + c1; }
-  __device__ static float half_gpp(float e) { return 3.0f * e + 3.0f; }
-  __device__ static float sixth_gppp(float) { return 1.0f; }
   __device__ static float noise(float e, float c1, float c0) {
     const float e2 = e * e;
     return 1.5e-7f * (fabsf(c0) + fabsf(c1 * e) + 3.0f * e2 + fabsf(e2 * e));
@@ -70,8 +66,6 @@ template <> struct CellPoly<1> {
 template <> struct CellPoly<2> {
   __device__ static float g(float e, float c1, float c0) { return (((e + 4.0f) * e + 6.0f) * e + c1) * e + c0; }
   __device__ static float gp(float e, float c1) { return ((4.0f * e + 12.0f) * e + 12.0f) * e + c1; }
-  __device__ static float half_gpp(float e) { const float u = e + 1.0f; return 6.0f * u * u; }
-  __device__ static float sixth_gppp(float e) { return 4.0f * (e + 1.0f); }
   __device__ static float noise(float e, float c1, float c0) {
     const float e2 = e * e;
     return 1.5e-7f * (fabsf(c0) + fabsf(c1 * e) + 6.0f * e2 + 4.0f * fabsf(e2 * e) + e2 * e2);
@@ -86,39 +80,6 @@ __device__ __forceinline__ float fr_root(float e, float c1, float c0, float q) {
   using P = CellPoly<NH>;
   float lo = -1.0f, hi = __int_as_float(0x7f800000);  // +inf until needed
   if (!(e > lo)) e = 0.0f;
-  {
-    // Halley: e1 = e - g g' / (g'^2 - g g''/2); its remaining error is about
-    // C d^3 for a step d, C = (g''/2g')^2 - g'''/(6 g') (Halley's cubic error
-    // constant), tested without a division
-    const float g0 = P::g(e, c1, c0), gp0 = P::gp(e, c1), hg = P::half_gpp(e);
-    const float den = gp0 * gp0 - g0 * hg;
-    const float e1 = e - __fdividef(g0 * gp0, den);
-    if (gp0 > 0.0f && den > 0.0f && e1 > lo) {
-      const float d = e1 - e;
-      if (fabsf(hg * hg - P::sixth_gppp(e) * gp0) * fabsf(d * d * d) <= (1e-7f * fabsf(e1) + 1e-20f) * (gp0 * gp0))
-        return e1;
-      e = e1;   // not yet at resolution: the Newton steps start from here
-    }
-  }
-  {
-    // one or two plain Newton steps;
-    // accepted when the remaining error is at float32 resolution and the root
-    // is admissible.  Newton's error after a step of length d is about K d^2,
-    // K = g''/(2 g')
-    const float g0 = P::g(e, c1, c0), gp0 = P::gp(e, c1);
-    const float e1 = e - __fdividef(g0, gp0);
-    {
-      const float d0 = e1 - e;
-      if (gp0 > 0.0f && e1 > lo && d0 * d0 * P::half_gpp(e) <= (1e-7f * fabsf(e1) + 1e-20f) * gp0) return e1;
-    }
-    const float g1 = P::g(e1, c1, c0), gp1 = P::gp(e1, c1);
-    const float e2 = e1 - __fdividef(g1, gp1);
-    // the same test for the second step, d = e2 - e1
-    const float d = e2 - e1;
-    if (gp0 > 0.0f && gp1 > 0.0f && e2 > lo && d * d * P::half_gpp(e1) <= (1e-7f * fabsf(e2) + 1e-20f) * gp1)
-      return e2;
-    if (gp1 > 0.0f && e2 > lo) e = e2;   // continue from the better point
-  }
   for (int it = 0; it < 30; ++it) {
     const float g = P::g(e, c1, c0);
     const float gp = P::gp(e, c1);
@@ -164,42 +125,171 @@ __device__ __forceinline__ float fr_op(float ec, const float nb[6], float alpha,
   return alpha * L + kappa * ec / (1.0f + ec);
 }
 
-template <int NH>
-__device__ __forceinline__ float fr_update(float ec, const float nb[6], float bv, float beta, float kappa,
-                                           float q) {
-  float S = 0.0f;
-#pragma unroll
-  for (int t = 0; t < 6; ++t)
-    S = NH == 1 ? fmaf(nb[t], 2.0f + nb[t], S) : fmaf(nb[t], fmaf(nb[t], 3.0f + nb[t], 3.0f), S);
-  const float S6 = S * (1.0f / 6.0f);
-  const float c1 = (NH == 1 ? 2.0f : 3.0f) + beta * (bv - kappa) - S6;
-  const float c0 = beta * bv - S6;
-  return fr_root<NH>(ec, c1, c0, q);
+// Approximate reciprocal (one instruction; a denormal argument gives infinity).
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
+// Cells in pairs (the paired float instructions halve the arithmetic of the
+// root, which is most of a sweep).  Accumulates a neighbour's term of S:
+// nb (2 + nb), for NH = 2 nb (3 + 3 nb + nb^2).
 template <int NH>
-__global__ void __launch_bounds__(256) k_fr_sweep(float* __restrict__ e, Src b, int log2n, int colour, float beta,
-                                                  float kappa, float q) {
+__device__ __forceinline__ float2 add_term(float2 s, float2 nb) {
+  return NH == 1 ? fma2(nb, add2(nb, both(2.0f)), s) : fma2(nb, fma2(nb, add2(nb, both(3.0f)), both(3.0f)), s);
+}
+
+// One step of a pair: Halley's, and from its point a Newton step with the slope
+// g' + g'' d/2 that Halley's denominator holds; the value of g there is its
+// (finite) Taylor sum.  With x = g g'' / (2 g'^2) (about g'' d / (2 g')) and
+// s = d^2 times a sixth of the third derivative over g' the remaining error is about (x^3 + x s) d, so the step
+// counts as done (ok) for |x| <= 0.006 and s < 1e-5, when that is below 3e-7 d.
+// Written with few constants and signs (a pair instruction takes neither
+// immediates nor, cheaply, a negated operand) and a test of five instructions a
+// cell: the arithmetic is what a sweep takes.
+template <int NH>
+__device__ __forceinline__ float2 root_step(float2 e, float2 c1, float2 c0, bool& okx, bool& oky) {
+  float2 g, gp, hg, sixth;   // g, its derivative, half its second and (NH = 2) a sixth of its third
+  if (NH == 1) {
+    const float2 t = mul2(e, add2(e, both(2.0f)));   // e^2 + 2 e
+    g = fma2(add2(add2(t, e), c1), e, c0);
+    gp = fma2(t, both(3.0f), c1);
+    hg = fma2(e, both(3.0f), both(3.0f));
+  } else {
+    const float2 u = add2(e, both(1.0f));
+    g = fma2(fma2(fma2(add2(e, both(4.0f)), e, both(6.0f)), e, c1), e, c0);
+    gp = fma2(fma2(fma2(e, both(4.0f), both(12.0f)), e, both(12.0f)), e, c1);
+    hg = mul2(mul2(u, u), both(6.0f));
+    sixth = mul2(u, both(4.0f));
+  }
+  const float2 n = mul2(g, hg), gp2 = mul2(gp, gp);
+  const float2 slope = make_float2(-gp.x * rcp_approx(gp2.x - n.x), -gp.y * rcp_approx(gp2.y - n.y));
+  const float2 d = mul2(g, slope), e1 = add2(e, d);
+  const float2 g1 = NH == 1 ? fma2(fma2(add2(hg, d), d, gp), d, g)
+                            : fma2(fma2(fma2(add2(sixth, d), d, hg), d, gp), d, g);
+  const float2 e2 = fma2(g1, slope, e1);
+  const float2 s = NH == 1 ? mul2(d, d) : mul2(mul2(d, d), sixth);
+  okx = fmaf(0.006f, gp2.x, -fabsf(n.x)) >= 0.0f && fmaf(1e-5f, gp.x, -s.x) > 0.0f && e2.x > -1.0f;
+  oky = fmaf(0.006f, gp2.y, -fabsf(n.y)) >= 0.0f && fmaf(1e-5f, gp.y, -s.y) > 0.0f && e2.y > -1.0f;
+  return e2;
+}
+
+// Roots of NP pairs of cell equations from the current values e: one step for
+// all, which settles nearly every warm cell, and for those of the cells `need`
+// (two bits a pair) that it does not a second one and then fr_root, one by one
+// (selected, not indexed or called: the pairs stay in registers).
+template <int NH, int NP>
+__device__ __forceinline__ void fr_roots(float2 (&e)[NP], const float2 (&c1)[NP], const float2 (&c0)[NP], float q,
+                                         unsigned need) {
+  static_assert(NP == 1 || NP == 2, "one or two pairs");
+  unsigned fail = 0;
+  float2 n[NP];
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    bool okx, oky;
+    n[i] = root_step<NH>(e[i], c1[i], c0[i], okx, oky);
+    if (!okx) fail |= 1u << (2 * i);
+    if (!oky) fail |= 2u << (2 * i);
+  }
+  fail &= need;
+  if (fail) {
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      // from the step's point, or where it left the admissible range from its start
+      const float2 f = make_float2(n[i].x > -1.0f && n[i].x < 1e3f ? n[i].x : e[i].x,
+                                   n[i].y > -1.0f && n[i].y < 1e3f ? n[i].y : e[i].y);
+      bool okx, oky;
+      const float2 r = root_step<NH>(f, c1[i], c0[i], okx, oky);
+      if (fail & (1u << (2 * i))) n[i].x = okx ? r.x : f.x;
+      if (fail & (2u << (2 * i))) n[i].y = oky ? r.y : f.y;
+      if (okx) fail &= ~(1u << (2 * i));
+      if (oky) fail &= ~(2u << (2 * i));
+    }
+    for (; fail; fail &= fail - 1u) {
+      const bool hi = NP == 2 && (fail & 3u) == 0u, y = ((hi ? fail >> 2 : fail) & 1u) == 0u;
+      const float2 pe = hi ? n[NP - 1] : n[0], p1 = hi ? c1[NP - 1] : c1[0], p0 = hi ? c0[NP - 1] : c0[0];
+      const float r = fr_root<NH>(y ? pe.y : pe.x, y ? p1.y : p1.x, y ? p0.y : p0.x, q);
+      if (!hi && !y) n[0].x = r;
+      if (!hi && y) n[0].y = r;
+      if (hi && !y) n[NP - 1].x = r;
+      if (hi && y) n[NP - 1].y = r;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NP; ++i) e[i] = n[i];
+}
+
+// The cell equations of NP pairs with neighbour terms S and sources b (as
+// beta b): c0 = beta b - S/6, c1 = c0 + k1, k1 = 2 - beta kappa (3 for NH = 2).
+template <int NH, int NP>
+__device__ __forceinline__ void fr_updates(float2 (&e)[NP], const float2 (&S)[NP], const float2 (&bb)[NP], float k1,
+                                           float q, unsigned need = ~0u) {
+  float2 c0[NP], c1[NP];
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    c0[i] = fma2(S[i], both(-1.0f / 6.0f), bb[i]);
+    c1[i] = add2(c0[i], both(k1));
+  }
+  fr_roots<NH, NP>(e, c1, c0, q, need);
+}
+
+// The sweeps of a level as the policy of k_rb_march; sources enter as beta b.
+template <int NH>
+struct CellSweeps {
+  float beta, k1, q;
+  __device__ __forceinline__ void box(int) {}
+  __device__ __forceinline__ float2 source(float2 b) const { return mul2(both(beta), b); }
+  __device__ __forceinline__ static float2 first(float2 a, float2 b) {
+    return add_term<NH>(add_term<NH>(both(0.0f), a), b);
+  }
+  __device__ __forceinline__ static float2 add(float2 s, float2 nb) { return add_term<NH>(s, nb); }
+  __device__ __forceinline__ static float2 add(float2 s, float x, float y) {
+    return add_term<NH>(s, make_float2(x, y));
+  }
+  template <int ST>
+  __device__ __forceinline__ void update(float2 (&v)[2], const float2 (&s)[2], const float2 (&bb)[2],
+                                         unsigned need) const {
+    fr_updates<NH, 2>(v, s, bb, k1, q, need);
+  }
+};
+
+// One colour of a sweep, four z cells (one pair of the colour) a thread with
+// 16-byte row loads, as the linear k_rb_sweep: these levels live in L2, and the
+// latency of the loads and of the root is what a pass takes.
+constexpr int kSweepThreads = 128;
+template <int NH>
+__global__ void __launch_bounds__(kSweepThreads) k_fr_sweep(float* __restrict__ e, Src b, int log2n, int colour,
+                                                            float beta, float k1, float q) {
   pdl_entry();
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (1u << (3 * log2n - 1))) return;
+  const uint32_t t = blockIdx.x * kSweepThreads + threadIdx.x;
+  if (t >= 1u << (3 * log2n - 2)) return;
   {   // the box of a batched launch
     const int64_t N = (int64_t)1 << (3 * log2n);
     e += (int64_t)blockIdx.z * N;
     b = box_src(b, N);
   }
-  const uint32_t m = (1u << log2n) - 1;
-  const uint32_t kk = t & ((1u << (log2n - 1)) - 1), row = t >> (log2n - 1);
-  const uint32_t j = row & m, i = row >> log2n;
-  const uint32_t k = 2 * kk + ((colour + i + j) & 1);
-  const uint32_t c = (row << log2n) | k;
-  uint32_t qi[6];
-  nb_index(c, i, j, k, log2n, qi);
-  float nb[6];
-#pragma unroll
-  for (int r = 0; r < 6; ++r) nb[r] = e[qi[r]];
-  const float bv = b.s * (__ldg(b.p + c) - load_mean(b));
-  e[c] = fr_update<NH>(e[c], nb, bv, beta, kappa, q);
+  const int m = (1 << log2n) - 1;
+  const int k0 = (int)(t << 2) & m, j = (int)(t >> (log2n - 2)) & m, i = (int)(t >> (2 * log2n - 2));
+  const bool odd = ((colour + i + j) & 1) != 0;   // cells k0 + odd and k0 + odd + 2
+  const uint32_t c = idx3(i, j, k0, log2n);
+  auto row4 = [&](int ii, int jj) { return *reinterpret_cast<const float4*>(e + idx3(ii & m, jj & m, k0, log2n)); };
+  const float4 XP = row4(i + 1, j), XM = row4(i - 1, j), YP = row4(i, j + 1), YM = row4(i, j - 1), C = row4(i, j);
+  const float ze = e[idx3(i, j, (odd ? k0 + 4 : k0 - 1) & m, log2n)];
+  const float4 F = __ldg(reinterpret_cast<const float4*>(b.p + c));
+  const float mean = load_mean(b);
+  auto mine = [&](const float4& v) { return odd ? make_float2(v.y, v.w) : make_float2(v.x, v.z); };
+  float2 S[1] = {add_term<NH>(both(0.0f), mine(XP))};
+  S[0] = add_term<NH>(S[0], mine(XM));
+  S[0] = add_term<NH>(S[0], mine(YP));
+  S[0] = add_term<NH>(S[0], mine(YM));
+  S[0] = add_term<NH>(S[0], odd ? make_float2(C.z, ze) : make_float2(C.y, C.w));
+  S[0] = add_term<NH>(S[0], odd ? make_float2(C.x, C.z) : make_float2(ze, C.y));
+  const float2 bb[1] = {mul2(both(beta), mul2(both(b.s), add2(mine(F), both(-mean))))};
+  float2 v[1] = {mine(C)};
+  fr_updates<NH, 1>(v, S, bb, k1, q);
+  e[c + odd] = v[0].x;
+  e[c + odd + 2] = v[0].y;
 }
 
 // The non-linear flux of N_h through one face, (u_nb^(n+1) - u^(n+1)) in
@@ -334,95 +424,210 @@ __global__ void __launch_bounds__(256) k_fr_norm(const float* __restrict__ e, Sr
   block_sum_to(partial + gridDim.x + blockIdx.x, sb, cb, scratch);
 }
 
-// Coarsest level (n <= 16) in one CTA: non-linear sweeps until the residual
-// dropped by `drop`, its running minimum stalls for 5 sweeps (float32 floor), or
-// `max_sweeps` sweeps.
-template <int NH>
-__global__ void __launch_bounds__(1024) k_fr_coarse(float* __restrict__ e, Src b, int log2n, float alpha,
-                                                    float beta, float kappa, float q, int max_sweeps,
-                                                    float drop) {
+// Coarsest level (n = 4, 8 or 16) in one CTA: non-linear sweeps until the
+// residual dropped by `drop`, its running minimum stalls for 5 sweeps (float32
+// floor), or `max_sweeps` sweeps.
+//
+// One SM's arithmetic bounds it (a root for each of 4096 cells a sweep), and the
+// barriers.  A thread owns up to eight z cells of a row, two pairs of either
+// colour, in registers; shared memory holds the colours of a row apart (as in
+// k_mg_coarse), so its x and y neighbours come in 16-byte loads.  The residual
+// of a black pair is taken when it has been updated, that of a red pair when the
+// next sweep updates it, from the neighbours that are at hand; the block's norm
+// is summed by one warp beside the black pass, and a sweep too many is undone
+// from the values kept: two barriers a sweep.  16^3: 46 -> 25 us a
+// solve against separate passes for the norm and a cell at a time.
+template <int NH, int LOG>
+struct FrCoarse {
+  static constexpr int n = 1 << LOG, H = n / 2, NP = H >= 4 ? 2 : 1, PARTS = H / (2 * NP);   // threads per row
+  static constexpr int RUNS = n * n * PARTS, THREADS = RUNS < 32 ? 32 : RUNS;
+};
+template <int NH, int LOG>
+__global__ void __launch_bounds__(FrCoarse<NH, LOG>::THREADS) k_fr_coarse(float* __restrict__ e, Src b, float alpha,
+                                                                          float beta, float kappa, float k1, float q,
+                                                                          int max_sweeps, float drop) {
   pdl_entry();
-  __shared__ float se[4096], sbv[4096];
-  __shared__ float2 scratch[33];
-  const int n = 1 << log2n, m = n - 1, N = n * n * n;
+  using C = FrCoarse<NH, LOG>;
+  constexpr int n = C::n, m = n - 1, H = C::H, NP = C::NP, HK = 2 * NP, N = n * n * n, NW = C::THREADS / 32;
+  __shared__ alignas(16) float S[2][N / 2];   // [colour][row][kk]: cell z = 2 kk + parity of (row, colour)
+  __shared__ float2 part[NW];
+  __shared__ float total;
   e += (int64_t)blockIdx.z * N;   // one CTA per box of a batched launch
   b = box_src(b, N);
   const float mean = load_mean(b);
-  for (int c = threadIdx.x; c < N; c += blockDim.x) {
-    se[c] = e[c];
-    sbv[c] = src_at(b, c, mean);
+  const bool act = threadIdx.x < C::RUNS;
+  const int t = act ? threadIdx.x : 0, row = t / C::PARTS, kk0 = (t - row * C::PARTS) * HK;
+  const int i = row >> LOG, j = row & m, par = (i + j) & 1;
+  const int own = row * H + kk0;
+  const int xp = ((((i + 1) & m) << LOG) | j) * H + kk0, xm = ((((i - 1) & m) << LOG) | j) * H + kk0;
+  const int yp = ((i << LOG) | ((j + 1) & m)) * H + kk0, ym = ((i << LOG) | ((j - 1) & m)) * H + kk0;
+  float2 v[2][NP], src[2][NP];   // [colour]: values and sources
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {   // natural order -> colours (red: z = 2 kk + par)
+    const int z = row * n + 2 * kk0 + 4 * p;
+    const float4 u = *reinterpret_cast<const float4*>(e + z), f = __ldg(reinterpret_cast<const float4*>(b.p + z));
+    const float fs[4] = {b.s * (f.x - mean), b.s * (f.y - mean), b.s * (f.z - mean), b.s * (f.w - mean)};
+    v[0][p] = par ? make_float2(u.y, u.w) : make_float2(u.x, u.z);
+    v[1][p] = par ? make_float2(u.x, u.z) : make_float2(u.y, u.w);
+    src[0][p] = par ? make_float2(fs[1], fs[3]) : make_float2(fs[0], fs[2]);
+    src[1][p] = par ? make_float2(fs[0], fs[2]) : make_float2(fs[1], fs[3]);
   }
-  __syncthreads();
-  auto nbs = [&](int c, float nb[6]) {
-    const int k = c & m, j = (c >> log2n) & m, i = c >> (2 * log2n);
-    nb[0] = se[(((i + 1) & m) << (2 * log2n)) | (j << log2n) | k];
-    nb[1] = se[(((i - 1) & m) << (2 * log2n)) | (j << log2n) | k];
-    nb[2] = se[(i << (2 * log2n)) | (((j + 1) & m) << log2n) | k];
-    nb[3] = se[(i << (2 * log2n)) | (((j - 1) & m) << log2n) | k];
-    nb[4] = se[(i << (2 * log2n)) | (j << log2n) | ((k + 1) & m)];
-    nb[5] = se[(i << (2 * log2n)) | (j << log2n) | ((k - 1) & m)];
+  auto put = [&](int c, const float2 (&w)[NP]) {
+    if (!act) return;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) *reinterpret_cast<float2*>(&S[c][own + 2 * p]) = w[p];
   };
-  // squared residual norm: per-thread compensated sums, then a compensated
-  // float pair over the block, the same in every thread
-  auto norm2 = [&]() -> float {
-    float s = 0.0f, cmp = 0.0f;
-    for (int c = threadIdx.x; c < N; c += blockDim.x) {
-      float nb[6];
-      nbs(c, nb);
-      const float d = sbv[c] - fr_op<NH>(se[c], nb, alpha, kappa);
-      kahan_add(s, cmp, d * d);
+  // the six neighbours of the thread's pairs of colour c, x+ .. z-
+  auto neighbours = [&](int c, float2 (&nb)[6][NP]) {
+    const float* w = S[1 - c];
+    const int at[4] = {xp, xm, yp, ym};
+#pragma unroll
+    for (int d = 0; d < 4; ++d)
+#pragma unroll
+      for (int p = 0; p < NP; ++p) nb[d][p] = *reinterpret_cast<const float2*>(w + at[d] + 2 * p);
+    const bool o = ((c + par) & 1) != 0;
+    const float ze = w[row * H + (o ? (kk0 + HK) & (H - 1) : (kk0 + H - 1) & (H - 1))];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const float2 x = v[1 - c][p];
+      const float before = p > 0 ? v[1 - c][p > 0 ? p - 1 : 0].y : ze, after = p < NP - 1 ? v[1 - c][p < NP - 1 ? p + 1 : p].x : ze;
+      nb[4][p] = o ? make_float2(x.y, after) : x;
+      nb[5][p] = o ? x : make_float2(before, x.x);
     }
-    const float2 r = block_pair_sum(s, cmp, scratch);
-    return r.x + r.y;
   };
-  float best = norm2();
+  float sum = 0.0f, cmp = 0.0f;   // compensated sum of squared residuals
+  auto residuals = [&](int c, const float2 (&nb)[6][NP]) {
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const float2 x = v[c][p], nx = mul2(x, both(-1.0f));
+      float2 L = both(0.0f);
+#pragma unroll
+      for (int d = 0; d < 6; ++d) {
+        const float2 s = add2(nb[d][p], x), df = add2(nb[d][p], nx);
+        const float2 w = NH == 1 ? add2(s, both(2.0f)) : add2(fma2(s, both(3.0f), both(3.0f)), fma2(nb[d][p], s, mul2(x, x)));
+        L = fma2(df, w, L);
+      }
+      const float d0 = src[c][p].x - fmaf(alpha, L.x, kappa * x.x / (1.0f + x.x));
+      const float d1 = src[c][p].y - fmaf(alpha, L.y, kappa * x.y / (1.0f + x.y));
+      kahan_add(sum, cmp, d0 * d0);
+      kahan_add(sum, cmp, d1 * d1);
+    }
+  };
+  auto update = [&](int c, const float2 (&nb)[6][NP], float2 (&out)[NP]) {
+    float2 T[NP], bb[NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      T[p] = both(0.0f);
+#pragma unroll
+      for (int d = 0; d < 6; ++d) T[p] = add_term<NH>(T[p], nb[d][p]);
+      bb[p] = mul2(both(beta), src[c][p]);
+      out[p] = v[c][p];
+    }
+    fr_updates<NH, NP>(out, T, bb, k1, q);
+  };
+  auto pair_add = [](float& s, float& c, float os, float oc) {
+    float r, err;
+    two_sum(s, os, r, err);
+    s = r;
+    c = c + oc + err;
+  };
+  auto lanes_sum = [&](float& s, float& c) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      const float os = __shfl_xor_sync(0xffffffffu, s, d), oc = __shfl_xor_sync(0xffffffffu, c, d);
+      pair_add(s, c, os, oc);
+    }
+  };
+  auto warp_part = [&]() {   // this warp's sum into part[] (idle threads add nothing)
+    float s = act ? sum - cmp : 0.0f, c = 0.0f;
+    lanes_sum(s, c);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_float2(s, c);
+    sum = cmp = 0.0f;
+  };
+  auto block_total = [&]() {   // warp 0: the block's sum into total
+    if (threadIdx.x >= 32) return;
+    float2 x = threadIdx.x < NW ? part[threadIdx.x < NW ? threadIdx.x : 0] : make_float2(0.0f, 0.0f);
+    lanes_sum(x.x, x.y);
+    if (threadIdx.x == 0) total = x.x + x.y;
+  };
+
+  put(0, v[0]);
+  put(1, v[1]);
+  __syncthreads();
+  float2 nb[6][NP];
+  neighbours(1, nb);
+  residuals(1, nb);
+  neighbours(0, nb);
+  residuals(0, nb);
+  warp_part();
+  __syncthreads();
+  block_total();
+  __syncthreads();
+  float best = total;
   const float target = drop * drop * best;
   int stale = 0;
-  // the cell of pair P (cells 2P, 2P + 1: same i, j) with colour col: k of
-  // 2P is even, so its colour is (i + j) & 1; every thread gets one cell of a
-  // pair per colour pass (the cells of one colour are independent)
-  auto cell_of = [&](int P, int col) -> int {
-    const int c0 = P << 1;
-    return c0 + ((col ^ ((c0 >> log2n) + (c0 >> (2 * log2n)))) & 1);
-  };
+  float2 before[2][NP];   // the values one sweep earlier
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    for (int colour = 0; colour < 2; ++colour) {
-      for (int P = threadIdx.x; P < (N >> 1); P += blockDim.x) {
-        const int c = cell_of(P, colour);
-        float nb[6];
-        nbs(c, nb);
-        se[c] = fr_update<NH>(se[c], nb, sbv[c], beta, kappa, q);
+    // v, the shared rows: the values after `sweep` sweeps
+    neighbours(0, nb);
+    if (sweep > 0) {
+      residuals(0, nb);
+      warp_part();
+    }
+    float2 next[NP];
+    update(0, nb, next);
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      before[0][p] = v[0][p];
+      before[1][p] = v[1][p];
+      v[0][p] = next[p];
+    }
+    put(0, v[0]);
+    __syncthreads();
+    if (sweep > 0) block_total();   // the norm after `sweep` sweeps
+    neighbours(1, nb);
+    update(1, nb, next);
+#pragma unroll
+    for (int p = 0; p < NP; ++p) v[1][p] = next[p];
+    residuals(1, nb);
+    put(1, v[1]);
+    __syncthreads();
+    if (sweep > 0) {
+      const float r = total;
+      bool stop = r <= target;
+      if (!stop) {
+        if (r < 0.998f * best) {   // squared norms: a 0.1% improvement of the norm
+          best = r;
+          stale = 0;
+        } else {
+          stop = ++stale >= 5;     // no progress for 5 sweeps: the float32 floor
+        }
       }
-      __syncthreads();
-    }
-    const float r = norm2();
-    if (r <= target) break;
-    if (r < 0.998f * best) {   // squared norms: a 0.1% improvement of the norm
-      best = r;
-      stale = 0;
-    } else if (++stale >= 5) {
-      break;                  // no progress for 5 sweeps: the float32 floor
+      if (stop) {                  // it was the sweep before this one
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          v[0][p] = before[0][p];
+          v[1][p] = before[1][p];
+        }
+        break;
+      }
     }
   }
-  for (int c = threadIdx.x; c < N; c += blockDim.x) e[c] = se[c];
+  if (act) {
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const float2 ev = par ? v[1][p] : v[0][p], od = par ? v[0][p] : v[1][p];
+      *reinterpret_cast<float4*>(e + row * n + 2 * kk0 + 4 * p) = make_float4(ev.x, od.x, ev.y, od.y);
+    }
+  }
 }
-
-// The non-linear Gauss-Seidel update as a functor for the streaming smoother.
-template <int NH>
-struct FRUpdate {
-  float beta, kappa, q;
-  __device__ __forceinline__ FRUpdate box(int) const { return *this; }
-  __device__ __forceinline__ float operator()(float old, const float nb[6], float bv, int, bool, bool) const {
-    return fr_update<NH>(old, nb, bv, beta, kappa, q);
-  }
-};
 
 struct FR {
   int n0;
   const fr_params* p;
   cudaStream_t s;
   float* e[12];
-  float* alt[12];   // ping-pong partner for the streaming smoother (or NULL)
+  float* alt[12];   // ping-pong partner of the fused sweeps (or NULL)
   float* r[12];
   Src b[12];
   double fbar, kappa;
@@ -446,6 +651,7 @@ struct FR {
 struct LevelConst {
   int n, log2n;
   float alpha, beta, kappa, q;
+  float k1;   // 2 - beta kappa (3 - beta kappa for n = 2)
 };
 
 LevelConst level_const(const FR& f, int l) {
@@ -457,68 +663,45 @@ LevelConst level_const(const FR& f, int l) {
   c.beta = (float)(h2 / (6.0 * f.fbar));
   c.kappa = (float)f.kappa;
   c.q = (float)(h2 * f.kappa / (6.0 * f.fbar));
+  c.k1 = (float)((f.nh == 2 ? 3.0 : 2.0) - h2 * f.kappa / (6.0 * f.fbar));
   return c;
 }
 
-// Resident CTAs per SM that the four-cell fused f(R) sweep's registers are
-// sized for.
-constexpr int kFrRunsMinBlocks = 3;
-
-template <int NH>
-pm_status stream_attributes_nh() {
-  PM_TRY(smem_attr(k_rb_stream<2, FRUpdate<NH>>, StreamGeom<2>::smem_bytes));
-  PM_TRY(smem_attr(k_rb_stream<1, FRUpdate<NH>>, StreamGeom<1>::smem_bytes));
-  PM_TRY(smem_attr(k_rb_fused4<FRUpdate<NH>, kFrRunsMinBlocks>, kFusedSmem));
-  return PM_OK;
-}
-
-pm_status stream_attributes(int nh) { return nh == 2 ? stream_attributes_nh<2>() : stream_attributes_nh<1>(); }
+// The fused sweeps' column tile.  Two rows of 64 x 32 cells a thread need 160
+// registers, so a CTA of 352 threads has an SM to itself; 64 x 64 (96 registers,
+// spilling) is slower: 0.49 against 0.47 ms at 512^3.  Against one cell at a time
+// in shared memory (three CTAs per SM) a warm sweep went 0.57 -> 0.47 ms, 256^3
+// 86 -> 73 us, 128^3 25 -> 17 us, a cold one at 512^3 0.73 -> 0.50 ms.  The colour
+// passes take 2 x 0.27 ms there; below 128^3 they are the faster form (an F-cycle
+// from 128^3 0.417 against 0.433 ms with fused sweeps at 64^3 too).
+constexpr int kFrTY = 32, kFrTZ = 64;
 
 template <int NH>
 pm_status fr_smooth_nh(FR& f, int l, int count) {
-  using FRUpdate = ::pmgb::FRUpdate<NH>;
   const LevelConst c = level_const(f, l);
   const double N = (double)c.n * c.n * c.n * f.B;
-  if (f.p->smoother == 0 && stream_ok(c.n) && f.alt[l] && f.B == 1) {
-    int chunk, nitems;
-    stream_plan(c.n, &chunk, &nitems);
-    const unsigned grid = (unsigned)(nitems < 152 * 2 ? nitems : 152 * 2);   // 2 CTAs/SM (shared memory)
-    const FRUpdate upd{c.beta, c.kappa, c.q};
-    for (int done = 0; done < count;) {
-      const int S = (count - done) >= 2 ? 2 : 1;
-      if (S == 2)
-        PM_LAUNCH(l == 0 ? K_FR_SMOOTH0 : K_FR_SMOOTH, 24.0 * N, (k_rb_stream<2, FRUpdate>), grid, kStreamThreads, StreamGeom<2>::smem_bytes,
-                  f.s, f.e[l], f.alt[l], f.b[l], c.log2n, chunk, nitems, 0, upd);
-      else
-        PM_LAUNCH(l == 0 ? K_FR_SMOOTH0 : K_FR_SMOOTH, 12.0 * N, (k_rb_stream<1, FRUpdate>), grid, kStreamThreads, StreamGeom<1>::smem_bytes,
-                  f.s, f.e[l], f.alt[l], f.b[l], c.log2n, chunk, nitems, 0, upd);
-      float* t = f.e[l];
-      f.e[l] = f.alt[l];
-      f.alt[l] = t;
-      done += S;
-    }
-    return PM_OK;
-  }
-  // a box of a batch takes the kernels it would take alone (fused_ok of one
-  // box), so every box evolves bitwise as in a batch of one
-  if (f.p->smoother == 2 && fused_ok(c.n) && f.alt[l] && fused_aligned(f.e[l], f.alt[l], f.b[l].p)) {
-    const int chunk = fused_chunk(c.n);
-    const dim3 grid = f.grid((unsigned)((c.n / kFusedT) * (c.n / kFusedT) * (c.n / chunk)));
-    const FRUpdate upd{c.beta, c.kappa, c.q};
+  // a box of a batch takes the kernels it would take alone, so every box
+  // evolves bitwise as in a batch of one
+  if (f.p->smoother != 1 && c.n >= 128 && f.alt[l] && march_aligned(f.e[l], f.alt[l], f.b[l].p)) {
+    using G = MarchGeom<1, kFrTY, kFrTZ>;
+    PM_TRY((march_attribute<CellSweeps<NH>, 1, kFrTY, kFrTZ>()));
+    const int chunks = march_chunks<1, kFrTY, kFrTZ>(c.n, 1);
+    const dim3 grid = f.grid((unsigned)((c.n / kFrTY) * (c.n / kFrTZ) * chunks));
+    const CellSweeps<NH> sweeps{c.beta, c.k1, c.q};
     for (int it = 0; it < count; ++it) {
-      PM_LAUNCH(l == 0 ? K_FR_SMOOTH0 : K_FR_SMOOTH, 12.0 * N, (k_rb_fused4<FRUpdate, kFrRunsMinBlocks>), grid,
-                kQuadThreads, kFusedSmem, f.s, f.e[l], f.alt[l], f.b[l], c.log2n, chunk, 0, 0, upd);
+      PM_LAUNCH(l == 0 ? K_FR_SMOOTH0 : K_FR_SMOOTH, 12.0 * N, (k_rb_march<CellSweeps<NH>, 1, kFrTY, kFrTZ>), grid,
+                G::THREADS, G::smem, f.s, f.e[l], f.alt[l], f.b[l], c.log2n, chunks, 0, sweeps);
       float* t = f.e[l];
       f.e[l] = f.alt[l];
       f.alt[l] = t;
     }
     return PM_OK;
   }
-  const dim3 grid = f.grid(grid_for(((int64_t)c.n * c.n * c.n) / 2, 256));
+  const dim3 grid = f.grid(grid_for(((int64_t)c.n * c.n * c.n) / 4, kSweepThreads));
   for (int it = 0; it < count; ++it)
     for (int colour = 0; colour < 2; ++colour)
-      PM_LAUNCH(l == 0 ? K_FR_SMOOTH0 : K_FR_SMOOTH, 6.0 * N, k_fr_sweep<NH>, grid, 256, 0, f.s, f.e[l], f.b[l],
-                c.log2n, colour, c.beta, c.kappa, c.q);
+      PM_LAUNCH(l == 0 ? K_FR_SMOOTH0 : K_FR_SMOOTH, 6.0 * N, k_fr_sweep<NH>, grid, kSweepThreads, 0, f.s, f.e[l],
+                f.b[l], c.log2n, colour, c.beta, c.k1, c.q);
   return PM_OK;
 }
 
@@ -533,9 +716,14 @@ bool is_coarsest(const FR& f, int l) {
 
 pm_status fr_coarse(FR& f, int l) {
   const LevelConst c = level_const(f, l);
-  FR_NH(f, PM_LAUNCH(K_FR_COARSE, 12.0 * c.n * c.n * (double)c.n * f.B, k_fr_coarse<NH>, f.grid(1), 1024, 0, f.s,
-                     f.e[l], f.b[l],
-                     c.log2n, c.alpha, c.beta, c.kappa, c.q, f.p->coarse_max_sweeps, f.p->coarse_drop));
+#define PM_FR_COARSE(LOG)                                                                                             \
+  FR_NH(f, PM_LAUNCH(K_FR_COARSE, 12.0 * c.n * c.n * (double)c.n * f.B, (k_fr_coarse<NH, LOG>), f.grid(1),           \
+                     (FrCoarse<NH, LOG>::THREADS), 0, f.s, f.e[l], f.b[l], c.alpha, c.beta, c.kappa, c.k1, c.q,       \
+                     f.p->coarse_max_sweeps, f.p->coarse_drop))
+  if (c.n == 16) PM_FR_COARSE(4);
+  else if (c.n == 8) PM_FR_COARSE(3);
+  else PM_FR_COARSE(2);
+#undef PM_FR_COARSE
   return PM_OK;
 }
 
@@ -604,7 +792,6 @@ pm_status fr_solve_src(Src b, float* eps, int n, const fr_params& prm, mg_stats*
     f.alt[l] = w.fr_alt[l];
   }
   f.nh = prm.nhs == 2 ? 2 : 1;
-  PM_TRY(stream_attributes(f.nh));
   double c2;
   fr_background(prm, &f.fbar, &f.kappa, &c2);
   mg_stats local{PM_OK, 0, -1.0, -1.0, -1.0};

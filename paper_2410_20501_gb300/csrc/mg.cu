@@ -11,9 +11,7 @@
 
 #include "pm_device.cuh"
 #include "pm_internal.cuh"
-#include "rb_fused.cuh"
 #include "rb_march.cuh"
-#include "rb_stream.cuh"
 
 namespace pmgb {
 
@@ -75,8 +73,34 @@ __global__ void k_scale(float* __restrict__ u, int64_t count, float a, const flo
     u[c] *= a;
 }
 
-// One colour of a red-black SOR sweep (the update rule is PoissonUpdate,
-// shared with the streaming smoother).  zero: the values of this level are
+// The linear update rule: (old value, 6 neighbours in the order x+, x-, y+, y-,
+// z+, z-, source value, neighbours-never-updated, own-never-updated) -> new value.
+struct PoissonUpdate {
+  float h2, omega;
+  float gscale;        // warm-start rescale applied to never-updated values
+  const float* gbox;   // per-box gscale of a batched launch (replaces gscale), or NULL
+  __device__ __forceinline__ PoissonUpdate box(int b) const {
+    PoissonUpdate u = *this;
+    if (gbox) u.gscale = __ldg(gbox + b);
+    return u;
+  }
+  // Explicit rounding intrinsics (no other contraction) so that the fused and
+  // the colour-by-colour kernels produce bitwise identical updates.
+  __device__ __forceinline__ float operator()(float old, const float nb[6], float fv, bool nb_old, bool own_old) const {
+    float s = __fadd_rn(nb[0], nb[1]);
+    s = __fadd_rn(s, nb[2]);
+    s = __fadd_rn(s, nb[3]);
+    s = __fadd_rn(s, nb[4]);
+    s = __fadd_rn(s, nb[5]);
+    if (nb_old) s = __fmul_rn(gscale, s);
+    const float ugs = __fmul_rn(__fsub_rn(s, __fmul_rn(h2, fv)), 1.0f / 6.0f);
+    if (omega == 1.0f) return ugs;
+    const float o = own_old ? __fmul_rn(gscale, old) : old;
+    return __fmaf_rn(omega, ugs, __fmul_rn(1.0f - omega, o));
+  }
+};
+
+// One colour of a red-black SOR sweep.  zero: the values of this level are
 // taken as 0 (the coarse-level error starts from zero): the red pass reads
 // nothing, the black pass ignores its own old value.
 //
@@ -116,8 +140,8 @@ __global__ void __launch_bounds__(kSweepThreads) k_rb_sweep(float* __restrict__ 
                         odd ? ze : C.w, odd ? C.z : C.y};
   const float o0 = zero ? 0.0f : odd ? C.y : C.x, o1 = zero ? 0.0f : odd ? C.w : C.z;
   const float f0 = f.s * ((odd ? F.y : F.x) - mean), f1 = f.s * ((odd ? F.w : F.z) - mean);
-  u[c + odd] = upd(o0, nb0, f0, 0, nb_old != 0, own_old != 0);
-  u[c + odd + 2] = upd(o1, nb1, f1, 0, nb_old != 0, own_old != 0);
+  u[c + odd] = upd(o0, nb0, f0, nb_old != 0, own_old != 0);
+  u[c + odd + 2] = upd(o1, nb1, f1, nb_old != 0, own_old != 0);
 }
 
 // Coarse right-hand side fc = R(f - L u): residual of the 8 children,
@@ -551,13 +575,12 @@ struct MG {
 };
 
 pm_status march_attributes() {
-  constexpr size_t one = MarchGeom<1, kMarchTY, kMarchTZ>::smem, two = MarchGeom<2, kMarchTY, kMarchTZ>::smem;
-  PM_TRY(smem_attr(k_rb_march<1, kMarchTY, kMarchTZ, true, true>, one));
-  PM_TRY(smem_attr(k_rb_march<1, kMarchTY, kMarchTZ, false, false>, one));
-  PM_TRY(smem_attr(k_rb_march<2, kMarchTY, kMarchTZ, true, true>, two));
-  PM_TRY(smem_attr(k_rb_march<2, kMarchTY, kMarchTZ, true, false>, two));
-  PM_TRY(smem_attr(k_rb_march<2, kMarchTY, kMarchTZ, false, true>, two));
-  PM_TRY(smem_attr(k_rb_march<2, kMarchTY, kMarchTZ, false, false>, two));
+  PM_TRY((march_attribute<LinearSweeps<true, true>, 1, kMarchTY, kMarchTZ>()));
+  PM_TRY((march_attribute<LinearSweeps<false, false>, 1, kMarchTY, kMarchTZ>()));
+  PM_TRY((march_attribute<LinearSweeps<true, true>, 2, kMarchTY, kMarchTZ>()));
+  PM_TRY((march_attribute<LinearSweeps<true, false>, 2, kMarchTY, kMarchTZ>()));
+  PM_TRY((march_attribute<LinearSweeps<false, true>, 2, kMarchTY, kMarchTZ>()));
+  PM_TRY((march_attribute<LinearSweeps<false, false>, 2, kMarchTY, kMarchTZ>()));
   return PM_OK;
 }
 
@@ -575,7 +598,7 @@ pm_status smooth(MG& g, int l, int count, const float* w, bool zero, float scale
   // passes; at 64^3 the two forms are even (a V-cycle from there 56 against 55
   // us), so one launch is taken instead of four.  On 64^3 levels of a batch the
   // form is tuned.
-  const bool fused_valid = g.p->smoother != 1 && n >= 64 && g.alt[l] && fused_aligned(g.u[l], g.alt[l], g.f[l].p);
+  const bool fused_valid = g.p->smoother != 1 && n >= 64 && g.alt[l] && march_aligned(g.u[l], g.alt[l], g.f[l].p);
   bool fused = fused_valid;
   const bool tune_form = fused_valid && g.B > 1 && n < 128;
   if (tune_form) {
@@ -588,14 +611,17 @@ pm_status smooth(MG& g, int l, int count, const float* w, bool zero, float scale
       const int S = count - done >= 2 ? 2 : 1;
       const int z = (done == 0 && zero) ? 1 : 0;
       const bool one0 = w[done] == 1.0f, one1 = S == 2 && w[done + 1] == 1.0f;
-      const MarchArgs a{h2, done == 0 ? scale : 1.0f, {w[done], S == 2 ? w[done + 1] : 1.0f},
-                        done == 0 ? sbox : nullptr};
-      const int chunks = march_chunks(n, g.B, S);
+      const int chunks = S == 2 ? march_chunks<2, kMarchTY, kMarchTZ>(n, g.B) : march_chunks<1, kMarchTY, kMarchTZ>(n, g.B);
       const dim3 grid = g.grid((unsigned)((n / kMarchTY) * (n / kMarchTZ) * chunks));
-#define PM_MARCH(SW, A, Bn)                                                                                       \
-  PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (z ? 8.0 : 12.0) * N * g.B,                                     \
-            (k_rb_march<SW, kMarchTY, kMarchTZ, A, Bn>), grid, (MarchGeom<SW, kMarchTY, kMarchTZ>::THREADS),     \
-            (MarchGeom<SW, kMarchTY, kMarchTZ>::smem), g.s, g.u[l], g.alt[l], g.f[l], log2n, chunks, z, a)
+#define PM_MARCH(SW, ONE0, ONE1)                                                                                   \
+  do {                                                                                                             \
+    const LinearSweeps<ONE0, ONE1> sweeps{h2, done == 0 ? scale : 1.0f, w[done], SW == 2 ? w[done + 1] : 1.0f,      \
+                                          done == 0 ? sbox : nullptr};                                             \
+    PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (z ? 8.0 : 12.0) * N * g.B,                                     \
+              (k_rb_march<LinearSweeps<ONE0, ONE1>, SW, kMarchTY, kMarchTZ>), grid,                                \
+              (MarchGeom<SW, kMarchTY, kMarchTZ>::THREADS), (MarchGeom<SW, kMarchTY, kMarchTZ>::smem), g.s, g.u[l], \
+              g.alt[l], g.f[l], log2n, chunks, z, sweeps);                                                         \
+  } while (0)
       if (S == 1) {
         if (one0) PM_MARCH(1, true, true); else PM_MARCH(1, false, false);
       } else if (one0) {
@@ -612,7 +638,7 @@ pm_status smooth(MG& g, int l, int count, const float* w, bool zero, float scale
   } else {
     const unsigned grid = grid_for(N / 4, kSweepThreads);
     for (; done < count; ++done) {
-      PoissonUpdate upd{h2, {w[done], 1.0f}, done == 0 ? scale : 1.0f, done == 0 ? sbox : nullptr};
+      const PoissonUpdate upd{h2, w[done], done == 0 ? scale : 1.0f, done == 0 ? sbox : nullptr};
       const int z = (done == 0 && zero) ? 1 : 0;
       const int first = done == 0 ? 1 : 0;
       PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (z ? 4.0 : 6.0) * N * g.B, k_rb_sweep, g.grid(grid), kSweepThreads, 0,

@@ -1,5 +1,5 @@
-// S full red-black sweeps (S = 1 or 2) of the linear SOR smoother in one pass
-// over memory, for the levels of the Poisson multigrid.
+// S full red-black sweeps (S = 1 or 2) of a level in one pass over memory; the
+// update is a policy: linear SOR (LinearSweeps, below) or the f(R) cell equation.
 //
 // A CTA owns a TY x TZ column of (y, z) cells and a chunk of x planes and
 // marches along x.  Every thread keeps two rows (the even one first) of four z
@@ -13,9 +13,9 @@
 // other colour in the step before.  Each stage is valid on one ring less of
 // the halo than the one before, so the last is valid on the column; plane
 // t - 2S + 1 is then final and written.  Every update sees the neighbour
-// values of the plain colour passes in the order x+, x-, y+, y-, z+, z- and
-// rounds as PoissonUpdate does: the result is bitwise theirs.  Old values come
-// from `uin`, the result goes to `uout`.
+// values of the plain colour passes in the order x+, x-, y+, y-, z+, z-; the
+// linear one rounds as PoissonUpdate does, so its result is bitwise theirs.  Old
+// values come from `uin`, the result goes to `uout`.
 //
 // What bounds it: the shared-memory and load wavefronts and the instructions
 // per update, as memory moves 12 bytes a cell for S sweeps.  Therefore two
@@ -27,16 +27,31 @@
 // every access is conflict-free.  Two buffers per stage make one barrier a
 // step enough; old values and sources arrive by asynchronous copies four planes
 // ahead.  Measured at 512^3: 0.40 ms for two sweeps (4.0 TB/s of the 12 bytes a
-// cell), against 0.83 ms with one sweep a pass (k_rb_fused4); ncu at 256^3: 47
+// cell), against 0.83 ms with one sweep a pass in shared memory; ncu at 256^3: 47
 // us of 63 at the shared-memory pipe's half rate, 0.37 instructions a cycle and
 // scheduler, the 12 warps waiting for it and each other.  One row a thread (23
 // warps) takes 0.42 ms: more instructions, as many wavefronts.
 #pragma once
 
 #include "pm_internal.cuh"
-#include "rb_fused.cuh"
 
 namespace pmgb {
+
+__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void cp_async_wait_group() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(PENDING) : "memory");
+}
+
+// Runs of four cells move in 16-byte accesses (workspace levels are aligned;
+// caller arrays are checked on entry).
+inline bool march_aligned(const float* u, const float* alt, const float* f) {
+  return (((uintptr_t)u | (uintptr_t)alt | (uintptr_t)f) & 15) == 0;
+}
 
 template <int S, int TY, int TZ>
 struct MarchGeom {
@@ -59,30 +74,59 @@ struct MarchGeom {
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
 
-struct MarchArgs {
-  float h2, gscale;
-  float omega[2];
-  const float* gbox;   // per-box gscale of a batched launch (replaces gscale)
+// Linear SOR sweeps with factors om0, om1 (ONE0, ONE1: the factor is 1), as
+// PoissonUpdate rounds them; gscale multiplies the values present before the
+// first sweep (gbox: per box of a batched launch).  Sources enter as -h^2 f.
+template <bool ONE0, bool ONE1>
+struct LinearSweeps {
+  float h2, gscale, om0, om1;
+  const float* gbox;
+  __device__ __forceinline__ void box(int b) { if (gbox) gscale = __ldg(gbox + b); }
+  __device__ __forceinline__ float2 source(float2 f) const { return mul2(both(-h2), f); }
+  __device__ __forceinline__ static float2 first(float2 a, float2 b) { return add2(a, b); }
+  __device__ __forceinline__ static float2 add(float2 s, float2 nb) { return add2(s, nb); }
+  __device__ __forceinline__ static float2 add(float2 s, float x, float y) {   // a pair from two places
+    return make_float2(__fadd_rn(s.x, x), __fadd_rn(s.y, y));
+  }
+  // the rows' values v after stage ST (1 .. 2S) from their neighbour sums s (need:
+  // the cells, two bits a row, that have to be right)
+  template <int ST>
+  __device__ __forceinline__ void update(float2 (&v)[2], float2 (&s)[2], const float2 (&nhf)[2], unsigned) const {
+    constexpr bool ONE = ST <= 2 ? ONE0 : ONE1;
+    const float om = ST <= 2 ? om0 : om1;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      if (ST == 1) s[j] = make_float2(__fmul_rn(gscale, s[j].x), __fmul_rn(gscale, s[j].y));   // rounded before the next sum
+      const float2 g = mul2(add2(s[j], nhf[j]), both(1.0f / 6.0f));
+      if (ONE) {
+        v[j] = g;
+      } else {
+        if (ST <= 2) v[j] = mul2(both(gscale), v[j]);
+        v[j] = fma2(both(om), g, mul2(both(1.0f - om), v[j]));
+      }
+    }
+  }
 };
 
-// The registers of one thread's runs and its part of a step.  ONE0 / ONE1: the
-// factor of the first / second sweep is 1.
-template <int S, int TY, int TZ, bool ONE0, bool ONE1>
+// The registers of one thread's runs and its part of a step.
+template <class P, int S, int TY, int TZ>
 struct MarchRun {
   using G = MarchGeom<S, TY, TZ>;
   static constexpr int W = G::W;                // plane t in slot K of step<K>
-  float2 R[W][2], B[W][2], FR[W][2], FB[W][2];  // [slot][row]: red and black pairs and -h^2 f of the planes held
+  float2 R[W][2], B[W][2], FR[W][2], FB[W][2];  // [slot][row]: red and black pairs and sources of the planes held
   float4* in;                                   // this run's place in the planes in flight
   const float *uin, *fp;
   float* uout;
   float* buf;
-  float h2, gscale, om0, om1, fs, mean;
+  P pol;
+  float fs, mean;
   uint32_t base, m;
   int log2n, up, dn, x0, x1;
+  unsigned need[2];   // S = 1: the red cells (two bits a row) with all neighbours at hand, by the step's parity
   bool useful, zero;
 
-  __device__ __forceinline__ static float2 both(float v) { return make_float2(v, v); }
   __device__ __forceinline__ uint32_t plane(int p) const { return ((uint32_t)p & m) << (2 * log2n); }
   // puts plane p in flight into slot K (read back by this thread only)
   template <int K>
@@ -99,8 +143,8 @@ struct MarchRun {
     }
     cp_async_commit_group();
   }
-  __device__ __forceinline__ float2 hsrc(float a, float b) const {
-    return mul2(both(-h2), mul2(both(fs), add2(make_float2(a, b), both(-mean))));
+  __device__ __forceinline__ float2 source(float a, float b) const {
+    return pol.source(mul2(both(fs), add2(make_float2(a, b), both(-mean))));
   }
   __device__ __forceinline__ float* buffer(int stage, int p) const { return buf + (2 * stage + (p & 1)) * G::BUF; }
   __device__ __forceinline__ void put(int stage, int p, const float2 (&v)[2]) const {
@@ -109,22 +153,6 @@ struct MarchRun {
     b[G::PL] = v[0].y;
     b[2 * G::PL] = v[1].x;
     b[3 * G::PL] = v[1].y;
-  }
-  // what stage ST takes from other threads on plane p: row 1 of the row pair
-  // below, row 0 of the one above, either row's z neighbour outside the run
-  struct Others {
-    float2 below, above;
-    float ze[2];
-  };
-  template <int ST, int ODD>
-  __device__ __forceinline__ Others others(int p) const {
-    const float* b = buffer(ST - 1, p);
-    Others o;
-    o.below = make_float2(b[2 * G::PL + dn], b[3 * G::PL + dn]);
-    o.above = make_float2(b[up], b[G::PL + up]);
-    o.ze[0] = ODD ? b[1] : b[G::PL - 1];
-    o.ze[1] = ODD ? b[3 * G::PL - 1] : b[2 * G::PL + 1];
-    return o;
   }
   // The plane that has arrived for slot K enters the registers; ODD: its parity
   // (x chunks start at even planes): row j's red cells are z + 1, z + 3 if
@@ -138,50 +166,44 @@ struct MarchRun {
       if ((ODD + j) & 1) {
         R[K][j] = make_float2(u.y, u.w);
         B[K][j] = make_float2(u.x, u.z);
-        FR[K][j] = hsrc(s.y, s.w);
-        FB[K][j] = hsrc(s.x, s.z);
+        FR[K][j] = source(s.y, s.w);
+        FB[K][j] = source(s.x, s.z);
       } else {
         R[K][j] = make_float2(u.x, u.z);
         B[K][j] = make_float2(u.y, u.w);
-        FR[K][j] = hsrc(s.x, s.z);
-        FB[K][j] = hsrc(s.y, s.w);
+        FR[K][j] = source(s.x, s.z);
+        FB[K][j] = source(s.y, s.w);
       }
     }
   }
   // Stage ST of a step on plane p in slot K: the pairs v[K] of one colour from
-  // those of the other, w[.]; ODD: the step's parity (row j's cells of the
-  // stage's colour are z + 1, z + 3 if ODD + j is odd, in every stage of a step).
+  // those of the other, w[.], and the sources fv; ODD: the step's parity (row
+  // j's cells of the stage's colour are z + 1, z + 3 if ODD + j is odd, in every
+  // stage of a step).  From other threads come row 1 of the row pair below, row
+  // 0 of the one above and either row's z neighbour outside the run.
   template <int K, int ST, int ODD>
   __device__ __forceinline__ void stage(int p, float2 (&v)[W][2], const float2 (&w)[W][2],
-                                        const float2 (&nhf)[W][2]) const {
-    constexpr int KP = (K + 1) % W, KM = (K + W - 1) % W;
-    constexpr bool ONE = ST <= 2 ? ONE0 : ONE1;
-    const Others x = others<ST, ODD>(p);
+                                        const float2 (&fv)[W][2]) const {
+    constexpr int KP = (K + 1) % W, KM = (K + W - 1) % W, PL = G::PL;
+    const float* b = buffer(ST - 1, p);
+    const float2 below = make_float2(b[2 * PL + dn], b[3 * PL + dn]), above = make_float2(b[up], b[PL + up]);
+    const float ze[2] = {ODD ? b[1] : b[PL - 1], ODD ? b[3 * PL - 1] : b[2 * PL + 1]};
+    float2 s[2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      float2 s = add2(w[KP][j], w[KM][j]);
-      s = add2(s, j == 0 ? w[K][1] : x.above);
-      s = add2(s, j == 0 ? x.below : w[K][0]);
+      s[j] = P::first(w[KP][j], w[KM][j]);
+      s[j] = P::add(s[j], j == 0 ? w[K][1] : above);
+      s[j] = P::add(s[j], j == 0 ? below : w[K][0]);
       if ((ODD + j) & 1) {
-        s.x = __fadd_rn(s.x, w[K][j].y);
-        s.y = __fadd_rn(s.y, x.ze[j]);
-        s = add2(s, w[K][j]);
+        s[j] = P::add(s[j], w[K][j].y, ze[j]);
+        s[j] = P::add(s[j], w[K][j]);
       } else {
-        s = add2(s, w[K][j]);
-        s.x = __fadd_rn(s.x, x.ze[j]);
-        s.y = __fadd_rn(s.y, w[K][j].x);
-      }
-      if (ST == 1) s = make_float2(__fmul_rn(gscale, s.x), __fmul_rn(gscale, s.y));   // rounded before the next sum
-      const float2 g = mul2(add2(s, nhf[K][j]), both(1.0f / 6.0f));
-      if (ONE) {
-        v[K][j] = g;
-      } else {
-        const float om = ST <= 2 ? om0 : om1;
-        float2 o = v[K][j];
-        if (ST <= 2) o = mul2(both(gscale), o);
-        v[K][j] = fma2(both(om), g, mul2(both(1.0f - om), o));
+        s[j] = P::add(s[j], w[K][j]);
+        s[j] = P::add(s[j], ze[j], w[K][j].x);
       }
     }
+    // cells whose value is used or has all its neighbours (S = 1; of S = 2 the policy does not ask)
+    pol.template update<ST>(v[K], s, fv[K], ST == 1 ? need[ODD] : useful ? 15u : 0u);
     if (ST < 2 * S) put(ST, p, v[K]);
   }
   // One step with plane t, of parity ODD, in slot K: plane t + 1 enters, every
@@ -213,29 +235,25 @@ struct MarchRun {
   }
 };
 
-// zero: the level's values are taken as 0.  gscale multiplies the values
-// present before the first sweep.  chunks: at most n / 2.
-template <int S, int TY, int TZ, bool ONE0, bool ONE1>
+// zero: the level's values are taken as 0.  chunks: at most n / 2.
+template <class P, int S, int TY, int TZ>
 __global__ void __launch_bounds__(MarchGeom<S, TY, TZ>::THREADS, 1)
-    k_rb_march(const float* __restrict__ uin, float* __restrict__ uout, Src f, int log2n, int chunks, int zero,
-               MarchArgs a) {
+    k_rb_march(const float* __restrict__ uin, float* __restrict__ uout, Src f, int log2n, int chunks, int zero, P pol) {
   pdl_entry();
   using G = MarchGeom<S, TY, TZ>;
   constexpr int W = G::W;
   extern __shared__ float4 march_sm4[];
-  MarchRun<S, TY, TZ, ONE0, ONE1> r;
+  MarchRun<P, S, TY, TZ> r;
   const uint32_t n = 1u << log2n;
   const int64_t off = (int64_t)blockIdx.z << (3 * log2n);   // the box of a batched launch
   f = box_src(f, (int64_t)1 << (3 * log2n));
+  r.pol = pol;
+  r.pol.box(blockIdx.z);
   r.uin = uin + off;
   r.uout = uout + off;
   r.fp = f.p;
   r.fs = f.s;
   r.mean = f.mean ? (float)*f.mean : 0.0f;
-  r.gscale = a.gbox ? __ldg(a.gbox + blockIdx.z) : a.gscale;
-  r.h2 = a.h2;
-  r.om0 = a.omega[0];
-  r.om1 = a.omega[1];
   r.m = n - 1;
   r.log2n = log2n;
   r.zero = zero != 0;
@@ -253,6 +271,13 @@ __global__ void __launch_bounds__(MarchGeom<S, TY, TZ>::THREADS, 1)
   r.buf = reinterpret_cast<float*>(march_sm4 + W * G::STAGED) + 1 + run;   // this run's place in every buffer
   r.up = pair < G::EP - 1 ? G::ER : 0;
   r.dn = pair > 0 ? -G::ER : 0;
+#pragma unroll
+  for (int odd = 0; odd < 2; ++odd) {   // not the outermost rows, nor a halo run's outermost cell
+    unsigned k = (pair > 0 ? 3u : 0u) | (pair < G::EP - 1 ? 12u : 0u);
+    if (q == 0) k &= odd ? ~4u : ~1u;                // z is red in the row of even parity
+    if (q == G::ER - 1) k &= odd ? ~2u : ~8u;        // z + 3 in the other
+    r.need[odd] = k;
+  }
 #pragma unroll
   for (int k = 0; k < W; ++k)
 #pragma unroll
@@ -282,12 +307,12 @@ __global__ void __launch_bounds__(MarchGeom<S, TY, TZ>::THREADS, 1)
   }
 }
 
-// The sweeps' column tile, and into how many x chunks (of nearly equal, even
-// length) a level is cut: the count with the fewest plane steps in sequence, waves of
-// one CTA per SM times the longest chunk and its 2S steps of run-up.
-constexpr int kMarchTY = 32, kMarchTZ = 64;
-inline int march_chunks(int n, int B, int S) {
-  const int64_t columns = (int64_t)(n / kMarchTY) * (n / kMarchTZ) * B;
+// Into how many x chunks (of nearly equal, even length) a level is cut: the
+// count with the fewest plane steps in sequence, waves of one CTA per SM times
+// the longest chunk and its 2S steps of run-up.
+template <int S, int TY, int TZ>
+inline int march_chunks(int n, int B) {
+  const int64_t columns = (int64_t)(n / TY) * (n / TZ) * B;
   int best = 1;
   int64_t least = INT64_MAX;
   for (int c = 1; c <= n / 2; ++c) {
@@ -299,5 +324,13 @@ inline int march_chunks(int n, int B, int S) {
   }
   return best;
 }
+
+template <class P, int S, int TY, int TZ>
+inline pm_status march_attribute() {
+  return smem_attr(k_rb_march<P, S, TY, TZ>, MarchGeom<S, TY, TZ>::smem);
+}
+
+// The linear sweeps' column tile.
+constexpr int kMarchTY = 32, kMarchTZ = 64;
 
 }  // namespace pmgb

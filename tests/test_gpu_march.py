@@ -54,3 +54,30 @@ def test_coarsest_sizes_match_the_oracle(pm, coarsest, sweeps):
     ref, _ = poisson.mg_solve(f, 1.0 / n, prm=poisson.MGParams(coarsest=coarsest, coarse_max_sweeps=sweeps), cycles=2)
     # the bar of the 16^3 case: float32 against float64 after the same steps
     assert np.linalg.norm(phi.cpu().numpy() - ref) < 1e-5 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("nhs,a,n", [(1, 0.05, 128), (1, 1.0, 128), (2, 0.5, 128), (2, 1.0, 256)])
+def test_fused_fr_sweeps_match_the_colour_passes(pm, nhs, a, n):
+    """From the unscreened to the screened regime (eps towards -1), from a cold
+    start: the pair root's second step and its fallback are taken."""
+    rho = np.exp(1.2 * inputs.random_field(n, 31))
+    rho = torch.from_numpy((rho / rho.mean()).astype(np.float32)).cuda()
+    outs = [pm.fr_solve(rho, a=a, Om=0.3, OL=0.7, fR0=-1e-5, boxsize=float(n), cycles=1, nhs=nhs,
+                        smoother=s)[0].cpu().numpy().astype(np.float64) for s in (2, 1)]
+    assert np.all(np.isfinite(outs[0])) and outs[0].min() > -1.0
+    # the same cell equations on the same neighbours, each root to float32 resolution
+    assert np.linalg.norm(outs[0] - outs[1]) < 1e-6 * np.linalg.norm(outs[1])
+
+
+@pytest.mark.parametrize("coarsest", [4, 8, 16])
+def test_fr_coarsest_sizes_match_the_oracle(pm, coarsest):
+    from oracle import fr as ofr
+    n = 32
+    rho = np.exp(0.8 * inputs.random_field(n, 8))
+    rho = (rho / rho.mean()).astype(np.float32).astype(np.float64)
+    model = ofr.FRModel(Om=0.3, OL=0.7, fR0=-1e-5, boxsize=float(n))
+    eps, _ = pm.fr_solve(torch.from_numpy(rho.astype(np.float32)).cuda(), a=0.6, Om=0.3, OL=0.7, fR0=-1e-5,
+                         boxsize=float(n), coarsest=coarsest, cycles=1)
+    u, _ = ofr.fr_solve(rho, 0.6, model, prm=ofr.FASParams(coarsest=coarsest), cycles=1)
+    # the bar of the 16^3 case
+    assert np.linalg.norm(eps.cpu().numpy() - (u - 1.0)) < 1e-4 * np.linalg.norm(u - 1.0)
