@@ -4,9 +4,9 @@
 // correction, a single-CTA coarsest-level solve, V-cycles.
 //
 // Precision: smoothing and transfers in float32.  The finest-level residual is
-// formed as sum_nb (u_nb - u) with every difference and partial sum kept
-// exactly (TwoSum), so the float32-stored iterate is tested against f with
-// float64-class accuracy; norms are accumulated in float64.
+// formed from sums that carry their rounding (TwoSum), so the float32-stored
+// iterate is tested against f with float64-class accuracy; norms are accumulated
+// in float64.
 #include <math.h>
 
 #include "pm_device.cuh"
@@ -29,38 +29,17 @@ __device__ __forceinline__ uint32_t idx3(int i, int j, int k, int log2n) {
   return ((uint32_t)i << (2 * log2n)) | ((uint32_t)j << log2n) | (uint32_t)k;
 }
 
-// sum_nb (u_nb - u) with TwoSum on every difference and partial sum: S + E.
-__device__ __forceinline__ void lap_diff_comp(float uc, const float nb[6], float& S, float& E) {
-  float s, e, t;
-  two_sum(nb[0], -uc, S, E);
-#pragma unroll
-  for (int q = 1; q < 6; ++q) {
-    two_sum(nb[q], -uc, s, e);
-    two_sum(S, s, S, t);
-    E += t + e;
-  }
-}
-
-__device__ __forceinline__ void load_nb(const float* __restrict__ u, int i, int j, int k, int log2n,
-                                        float nb[6]) {
-  const int m = (1 << log2n) - 1;
-  nb[0] = __ldg(u + idx3((i + 1) & m, j, k, log2n));
-  nb[1] = __ldg(u + idx3((i - 1) & m, j, k, log2n));
-  nb[2] = __ldg(u + idx3(i, (j + 1) & m, k, log2n));
-  nb[3] = __ldg(u + idx3(i, (j - 1) & m, k, log2n));
-  nb[4] = __ldg(u + idx3(i, j, (k + 1) & m, log2n));
-  nb[5] = __ldg(u + idx3(i, j, (k - 1) & m, log2n));
-}
-
-// u = -h^2 f / 6 (Eq. multigrid_initial_guess).
+// u = -h^2 f / 6 (Eq. multigrid_initial_guess), four cells a thread.
 __global__ void k_jacobi_guess(float* __restrict__ u, Src f, int64_t count, float h2) {
   pdl_entry();
+  const int64_t c = 4 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
+  if (c >= count) return;
   u += (int64_t)blockIdx.z * count;
   f = box_src(f, count);
   const float mean = load_mean(f);
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < count;
-       c += (int64_t)gridDim.x * blockDim.x)
-    u[c] = -h2 * src_at(f, c, mean) * kSixth;
+  const float4 v = __ldg(reinterpret_cast<const float4*>(f.p + c));
+  auto guess = [&](float x) { return -h2 * (f.s * (x - mean)) * kSixth; };
+  *reinterpret_cast<float4*>(u + c) = make_float4(guess(v.x), guess(v.y), guess(v.z), guess(v.w));
 }
 
 // u *= a (per box: ab[box] if ab is set).
@@ -144,104 +123,150 @@ __global__ void __launch_bounds__(kSweepThreads) k_rb_sweep(float* __restrict__ 
   u[c + odd + 2] = upd(o1, nb1, f1, nb_old != 0, own_old != 0);
 }
 
+// A pair of floats with what rounding took from it: s + e is exact after every
+// add (TwoSum per component; e itself is a float sum).
+struct PairSum {
+  float2 s, e;
+  __device__ __forceinline__ explicit PairSum(float2 v) : s(v), e(both(0.0f)) {}
+  __device__ __forceinline__ void add(float2 v) {
+    const float2 m = both(-1.0f);
+    const float2 t = add2(s, v), vp = fma2(s, m, t);               // t - s
+    const float2 se = fma2(fma2(vp, m, t), m, s), ve = fma2(vp, m, v);   // s - (t - vp), v - vp
+    e = add2(e, add2(se, ve));
+    s = t;
+  }
+  // subtracts k times another sum (k v split exactly by a fused multiply-add)
+  __device__ __forceinline__ void sub_times(float k, const PairSum& v) {
+    const float2 p = mul2(v.s, both(-k)), pe = fma2(v.s, both(-k), mul2(p, both(-1.0f)));
+    add(p);
+    e = add2(e, fma2(v.e, both(-k), pe));
+  }
+};
+
 // Coarse right-hand side fc = R(f - L u): residual of the 8 children,
 // averaged.  Summed over the 2x2x2 block the Laplacian fluxes through the 12
-// inner faces cancel pairwise, so  h^2 sum_c L u_c  is the sum of
-// (u_nb - u_c) over the 24 outer faces only.  With COMP the differences are
-// exact (TwoSum) and summed with compensation, as is the sum of the sources,
-// and the one cancelling subtraction is a single rounding (fused
-// multiply-add).
+// inner faces cancel pairwise, so  h^2 sum_c L u_c  is the sum of the 24 outer
+// neighbours minus three times that of the 8 children.  With COMP both sums
+// carry their rounding (PairSum), as does the sum of the sources, and the one
+// cancelling subtraction is a single rounding (fused multiply-add).
+//
+// The compensated sums' arithmetic and the number of loads in flight bound it:
+// a thread takes two coarse cells along z, so its fine rows come in 16-byte
+// loads and the two cells go through the paired float instructions.  512^3:
+// 0.314 -> 0.231 ms against one cell a thread with the 24 differences
+// summed one by one; 256^3 42 -> 32 us.
 template <bool COMP>
-__global__ void k_resid_restrict(const float* __restrict__ u, Src f, int log2n, float inv_h2,
-                                 float* __restrict__ fc) {
+__global__ void __launch_bounds__(128) k_resid_restrict(const float* __restrict__ u, Src f, int log2n, float inv_h2,
+                                                        float* __restrict__ fc) {
   pdl_entry();
-  const int lc = log2n - 1, mc = (1 << lc) - 1;
+  const int lc = log2n - 1, mc = (1 << lc) - 1, m = (1 << log2n) - 1, lg = lc - 1;
   u += (int64_t)blockIdx.z << (3 * log2n);
   f = box_src(f, (int64_t)1 << (3 * log2n));
   fc += (int64_t)blockIdx.z << (3 * lc);
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;   // two coarse cells, K = 2 G and 2 G + 1
+  if (t >= 1u << (3 * lc - 1)) return;
+  const int G = (int)(t & ((1u << lg) - 1u)), J = (int)(t >> lg) & mc, I = (int)(t >> (lg + lc));
+  const int z0 = 4 * G;
+  auto row = [&](const float* p, int x, int y) {
+    return __ldg(reinterpret_cast<const float4*>(p + idx3(x & m, y & m, z0, log2n)));
+  };
+  float4 core[2][2], xf[2][2], yf[2][2], fr[2][2];   // [x][y], [side][y], [x][side]
+  float zl[2][2], zr[2][2];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      core[a][b] = row(u, 2 * I + a, 2 * J + b);
+      zl[a][b] = __ldg(u + idx3(2 * I + a, 2 * J + b, (z0 - 1) & m, log2n));
+      zr[a][b] = __ldg(u + idx3(2 * I + a, 2 * J + b, (z0 + 4) & m, log2n));
+      xf[a][b] = row(u, a ? 2 * I + 2 : 2 * I - 1, 2 * J + b);
+      yf[a][b] = row(u, 2 * I + a, b ? 2 * J + 2 : 2 * J - 1);
+      fr[a][b] = row(f.p, 2 * I + a, 2 * J + b);
+    }
   const float mean = load_mean(f);
-  const int64_t total = (int64_t)1 << (3 * lc);
-  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-    const int K = (int)(t & mc), J = (int)((t >> lc) & mc), I = (int)(t >> (2 * lc));
-    float core[2][2][4], xf[2][2][2], yf[2][2][2];
-    load_children_block(u, I, J, K, log2n, core, xf, yf);
-    float fz[8];
+  // (first coarse cell, second coarse cell): even fine cells, odd fine cells
+  auto ev = [](const float4& v) { return make_float2(v.x, v.z); };
+  auto od = [](const float4& v) { return make_float2(v.y, v.w); };
+  auto source = [&](float2 v) { return mul2(both(f.s), add2(v, both(-mean))); };
+  float2 d;
+  if (COMP) {
+    PairSum S(ev(xf[0][0])), C(ev(core[0][0])), F(source(ev(fr[0][0])));
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
-        const float2 fr = __ldg(reinterpret_cast<const float2*>(f.p + idx3(2 * I + a, 2 * J + b, 2 * K, log2n)));
-        fz[(a * 2 + b) * 2] = f.s * (fr.x - mean);
-        fz[(a * 2 + b) * 2 + 1] = f.s * (fr.y - mean);
-      }
-    // outer faces (neighbour, child): x-, x+ for each (b, c); y-, y+ for each
-    // (a, c); z-, z+ for each (a, b)
-    float nbv[24], chv[24];
-#pragma unroll
-    for (int b = 0; b < 2; ++b)
-#pragma unroll
-      for (int c = 0; c < 2; ++c)
-#pragma unroll
-        for (int side = 0; side < 2; ++side) {
-          const int q = (b * 2 + c) * 2 + side;
-          nbv[q] = xf[side][b][c];
-          chv[q] = core[side][b][c + 1];
-          nbv[8 + q] = yf[b][side][c];          // here b plays a (x offset)
-          chv[8 + q] = core[b][side][c + 1];
-          nbv[16 + q] = core[b][c][side ? 3 : 0];   // here (b, c) play (a, b)
-          chv[16 + q] = core[b][c][side ? 2 : 1];
+        if (a + b) {
+          S.add(ev(xf[a][b]));
+          C.add(ev(core[a][b]));
+          F.add(source(ev(fr[a][b])));
         }
-    float d;
-    if (COMP) {
-      float S, E, sq, eq, tq;
-      two_sum(nbv[0], -chv[0], S, E);
-#pragma unroll
-      for (int q = 1; q < 24; ++q) {
-        two_sum(nbv[q], -chv[q], sq, eq);
-        two_sum(S, sq, S, tq);
-        E += tq + eq;
+        S.add(od(xf[a][b]));
+        S.add(ev(yf[a][b]));
+        S.add(od(yf[a][b]));
+        S.add(make_float2(zl[a][b], core[a][b].y));
+        S.add(make_float2(core[a][b].z, zr[a][b]));
+        C.add(od(core[a][b]));
+        F.add(source(od(fr[a][b])));
       }
-      float F = fz[0], Fe = 0.0f;
+    S.sub_times(3.0f, C);
+    d = add2(fma2(both(-inv_h2), S.s, F.s), fma2(both(-inv_h2), S.e, F.e));
+  } else {
+    // per row, so that what cancels is subtracted early: neighbours minus three times the children
+    float2 L = both(0.0f), F = both(0.0f);
 #pragma unroll
-      for (int q = 1; q < 8; ++q) {
-        two_sum(F, fz[q], F, tq);
-        Fe += tq;
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const float2 ce = mul2(ev(core[a][b]), both(-1.0f)), co = mul2(od(core[a][b]), both(-1.0f));
+        const float2 fe = add2(ev(xf[a][b]), ce), fo = add2(od(xf[a][b]), co);
+        const float2 ge = add2(ev(yf[a][b]), ce), go = add2(od(yf[a][b]), co);
+        const float2 lo = add2(make_float2(zl[a][b], core[a][b].y), ce), hi = add2(make_float2(core[a][b].z, zr[a][b]), co);
+        L = add2(L, add2(add2(add2(fe, fo), add2(ge, go)), add2(lo, hi)));
+        F = add2(F, add2(source(ev(fr[a][b])), source(od(fr[a][b]))));
       }
-      d = fmaf(-inv_h2, S, F) + (Fe - inv_h2 * E);
-    } else {
-      float L[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-      for (int q = 0; q < 24; ++q) L[q & 3] += nbv[q] - chv[q];
-      const float F = ((fz[0] + fz[1]) + (fz[2] + fz[3])) + ((fz[4] + fz[5]) + (fz[6] + fz[7]));
-      d = fmaf(-inv_h2, (L[0] + L[1]) + (L[2] + L[3]), F);
-    }
-    fc[t] = 0.125f * d;
+    d = fma2(both(-inv_h2), L, F);
   }
+  *reinterpret_cast<float2*>(fc + 2 * t) = mul2(d, both(0.125f));
 }
 
 // Residual norm^2 and source norm^2 partials (finest level, compensated
-// residual): partial[blockIdx] and partial[gridDim + blockIdx].
+// residual): partial[blockIdx] and partial[gridDim + blockIdx].  A thread takes
+// four z cells at a time: 16-byte loads, and the neighbour sum minus 6 u with its
+// rounding (PairSum) in the paired float instructions, which is what it spends
+// its time on.  256^3: 100 -> 45 us against one cell a time with the six
+// differences summed one by one.
 __global__ void __launch_bounds__(256) k_resid_norm(const float* __restrict__ u, Src f, int log2n,
                                                     float inv_h2, double* __restrict__ partial) {
   pdl_entry();
   __shared__ double scratch[32];
   const float mean = load_mean(f);
   const int m = (1 << log2n) - 1;
-  const int64_t total = (int64_t)1 << (3 * log2n);
-  float sd = 0.0f, cd = 0.0f, sf = 0.0f, cf = 0.0f;
-  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < total; c += gridDim.x * blockDim.x) {
-    const int k = (int)(c & m), j = (int)((c >> log2n) & m), i = (int)(c >> (2 * log2n));
-    float nb[6];
-    load_nb(u, i, j, k, log2n, nb);
-    const float uc = __ldg(u + c), fv = src_at(f, c, mean);
-    float S, E;
-    lap_diff_comp(uc, nb, S, E);
-    const float d = fmaf(-inv_h2, S, fv) - inv_h2 * E;
-    kahan_add(sd, cd, d * d);
-    kahan_add(sf, cf, fv * fv);
+  const uint32_t runs = 1u << (3 * log2n - 2);
+  PairSum D(both(0.0f)), F(both(0.0f));
+  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < runs; t += gridDim.x * blockDim.x) {
+    const int k = (int)(t << 2) & m, j = (int)(t >> (log2n - 2)) & m, i = (int)(t >> (2 * log2n - 2));
+    auto row = [&](int x, int y) { return __ldg(reinterpret_cast<const float4*>(u + idx3(x & m, y & m, k, log2n))); };
+    const float4 c = row(i, j), xp = row(i + 1, j), xm = row(i - 1, j), yp = row(i, j + 1), ym = row(i, j - 1);
+    const float zl = __ldg(u + idx3(i, j, (k - 1) & m, log2n)), zr = __ldg(u + idx3(i, j, (k + 4) & m, log2n));
+    const float4 fr = __ldg(reinterpret_cast<const float4*>(f.p + 4 * (int64_t)t));
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {   // cells 0, 1, then 2, 3
+      auto two = [&](const float4& v) { return h ? make_float2(v.z, v.w) : make_float2(v.x, v.y); };
+      PairSum S(two(xp));
+      S.add(two(xm));
+      S.add(two(yp));
+      S.add(two(ym));
+      S.add(h ? make_float2(c.w, zr) : make_float2(c.y, c.z));
+      S.add(h ? make_float2(c.y, c.z) : make_float2(zl, c.x));
+      S.sub_times(6.0f, PairSum(two(c)));
+      const float2 fv = mul2(both(f.s), add2(two(fr), both(-mean)));
+      const float2 d = add2(fma2(both(-inv_h2), S.s, fv), mul2(both(-inv_h2), S.e));
+      D.add(mul2(d, d));
+      F.add(mul2(fv, fv));
+    }
   }
-  block_sum_to(partial + blockIdx.x, sd, cd, scratch);
-  block_sum_to(partial + gridDim.x + blockIdx.x, sf, cf, scratch);
+  block_sum_to(partial + blockIdx.x, D.s.x + D.s.y, -(D.e.x + D.e.y), scratch);
+  block_sum_to(partial + gridDim.x + blockIdx.x, F.s.x + F.s.y, -(F.e.x + F.e.y), scratch);
 }
 
 // Block sum of per-thread float64 values, written by thread 0 to *out (a
@@ -683,12 +708,12 @@ pm_status v_cycle(MG& g, int l, bool zero_guess) {
     PM_TRY(smooth(g, l, p.npre, w, zero_guess, scaled ? g.gscale : 1.0f, sbox));
   }
   const int64_t nc = ((int64_t)n * n * n) / 8;
-  const unsigned grid = grid_for(nc, 256);
+  const unsigned grid = grid_for(nc / 2, 128);
   if (l == 0)
-    PM_LAUNCH(K_MG_RESTRICT, 68.0 * nc * g.B, k_resid_restrict<true>, g.grid(grid), 256, 0, g.s, g.u[l], g.f[l],
+    PM_LAUNCH(K_MG_RESTRICT, 68.0 * nc * g.B, k_resid_restrict<true>, g.grid(grid), 128, 0, g.s, g.u[l], g.f[l],
               log2n, (float)n * (float)n, const_cast<float*>(g.f[l + 1].p));
   else
-    PM_LAUNCH(K_MG_RESTRICT, 68.0 * nc * g.B, k_resid_restrict<false>, g.grid(grid), 256, 0, g.s, g.u[l], g.f[l],
+    PM_LAUNCH(K_MG_RESTRICT, 68.0 * nc * g.B, k_resid_restrict<false>, g.grid(grid), 128, 0, g.s, g.u[l], g.f[l],
               log2n, (float)n * (float)n, const_cast<float*>(g.f[l + 1].p));
   PM_TRY(v_cycle(g, l + 1, true));
   PM_LAUNCH(K_MG_PROLONG, 68.0 * nc * g.B, k_prolong_correct, g.grid(grid_for(nc / 2, 256)), 256, 0, g.s, g.u[l],
@@ -743,7 +768,7 @@ pm_status mg_solve_batch_src(Src f, float* phi, int n, int B, const mg_params& p
   const int64_t N = (int64_t)n * n * n;
   const float h2 = 1.0f / ((float)n * (float)n);
   if (prm.first_guess == MG_GUESS_JACOBI)
-    PM_LAUNCH(K_MG_GUESS, 8.0 * N * B, k_jacobi_guess, g.grid(grid_for(N, 256)), 256, 0, s, phi, f, N, h2);
+    PM_LAUNCH(K_MG_GUESS, 8.0 * N * B, k_jacobi_guess, g.grid(grid_for(N / 4, 256)), 256, 0, s, phi, f, N, h2);
   for (int c = 0; c < prm.fixed_cycles; ++c) {
     PM_TRY(v_cycle(g, 0, false));
     g.first_cycle = false;
@@ -777,7 +802,7 @@ pm_status mg_solve_src(Src f, float* phi, int n, const mg_params& prm, mg_stats*
   const int64_t N = (int64_t)n * n * n;
   const float h2 = 1.0f / ((float)n * (float)n);
   if (prm.first_guess == MG_GUESS_JACOBI)
-    PM_LAUNCH(K_MG_GUESS, 8.0 * N, k_jacobi_guess, grid_for(N, 256), 256, 0, s, phi, f, N, h2);
+    PM_LAUNCH(K_MG_GUESS, 8.0 * N, k_jacobi_guess, grid_for(N / 4, 256), 256, 0, s, phi, f, N, h2);
   mg_stats local{PM_OK, 0, -1.0, -1.0, -1.0};
   auto cycle = [&]() -> pm_status {
     PM_TRY(v_cycle(g, 0, false));

@@ -81,3 +81,19 @@ def test_fr_coarsest_sizes_match_the_oracle(pm, coarsest):
     u, _ = ofr.fr_solve(rho, 0.6, model, prm=ofr.FASParams(coarsest=coarsest), cycles=1)
     # the bar of the 16^3 case
     assert np.linalg.norm(eps.cpu().numpy() - (u - 1.0)) < 1e-4 * np.linalg.norm(u - 1.0)
+
+
+@pytest.mark.parametrize("n,coarsest", [(8, 4), (16, 4), (64, 16), (128, 16)])
+def test_residual_norm_in_wide_loads(pm, n, coarsest):
+    """The residual norm that ends a solve, from the smallest grid above the
+    coarsest on, against float64 on the same iterate."""
+    f = inputs.random_field(n, 12)
+    f = (f - f.mean()).astype(np.float32)
+    phi, st = pm.mg_solve(torch.from_numpy(f).cuda(), tol=0.9, coarsest=coarsest)
+    u = phi.cpu().numpy().astype(np.float64)
+    lap = sum(np.roll(u, s, d) for s in (1, -1) for d in range(3)) - 6.0 * u
+    f = f.astype(np.float64)
+    r = np.linalg.norm(f - lap * n * n)
+    assert st["cycles"] == 1 and st["norm_f"] == pytest.approx(np.linalg.norm(f), rel=1e-6)
+    # the residual is exact to a rounding of each cell's (and of the source less its float32 mean)
+    assert st["res"] == pytest.approx(r, abs=2e-7 * st["norm_f"])
