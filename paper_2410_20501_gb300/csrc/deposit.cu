@@ -466,10 +466,16 @@ __global__ void __launch_bounds__(CT) k_crowded_moments(const uint32_t* __restri
   }
 }
 
-inline void deposit_stream_plan(int n, int* chunk, int* nitems) {
+// x planes per CTA and CTAs a box.  A chunk repeats the planes on its two sides:
+// 16 or more while the grid fills the SMs several times over (256^3 297 us at 32,
+// 316 at 16, 363 at 8), fewer only where SMs would have no CTA at all (32^3 with
+// its other launches 45 us at 16, 35 at 2; 64^3 47 at 16, 39 at 4; 128^3 77 at 16,
+// 79 at 8).
+inline void deposit_stream_plan(int n, int B, int* chunk, int* nitems) {
   const int tiles = (n / DTY) * (n / DTZ);
   int c = n;
-  while (c > 16 && (int64_t)tiles * (n / c) < 8 * 152) c >>= 1;
+  while (c > 16 && (int64_t)tiles * (n / c) * B < 8 * 152) c >>= 1;
+  while (c > 2 && (int64_t)tiles * (n / c) * B < 152) c >>= 1;
   *chunk = c;
   *nitems = tiles * (n / c);
 }
@@ -535,12 +541,6 @@ pm_status launch_deposit(const uint32_t* Xs, int64_t np, const uint32_t* cellsta
 
 }  // namespace
 
-int deposit_items(int n) {
-  int chunk, nitems;
-  deposit_stream_plan(n, &chunk, &nitems);
-  return nitems;
-}
-
 int64_t reduce_partials_capacity(int n, int64_t np) {
   int64_t t = (int64_t)n / 4;
   int64_t c = t * t * t;               // deposit blocks with 4^3 tiles (upper bound)
@@ -592,7 +592,7 @@ pm_status deposit_sorted_values(const uint32_t* Xs, int64_t np, const uint32_t* 
     PM_TRY(crowded_moments(Xs, np, cellstart, n, vals, cr, s));
     const float* crowd = cr.runs && np > 0 ? cr.moments : nullptr;
     int chunk, nitems;
-    deposit_stream_plan(n, &chunk, &nitems);
+    deposit_stream_plan(n, 1, &chunk, &nitems);
     const unsigned grid = (unsigned)nitems;   // one item per CTA, two 512-thread CTAs per SM
     const double bytes = (vals ? 16.0 : 12.0) * np + 8.0 * n * n * (double)n + 4.0;
     if (vals) {
@@ -618,7 +618,7 @@ pm_status deposit_sorted_batch(const uint32_t* Xs, int64_t np_box, int B, const 
   PM_TRY(crowded_moments(Xs, np_box * B, cellstart, n, nullptr, cr, s));
   PM_TRY(smem_attr(k_deposit_stream<false>, DepositStage<false>::smem));
   int chunk, nitems;
-  deposit_stream_plan(n, &chunk, &nitems);
+  deposit_stream_plan(n, B, &chunk, &nitems);
   const float scale = np_box > 0 ? (float)((double)n * n * n / (double)np_box) : 0.0f;
   // one item per CTA: B x nitems CTAs balance over the SMs (two resident each)
   const int gx = nitems;

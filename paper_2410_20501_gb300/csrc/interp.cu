@@ -675,8 +675,14 @@ pm_status launch_force_interp(const float* phi, const float* eps, float alpha, i
   PM_TRY(smem_attr(k_force_interp_stream<ORDER, true, false>, smem));
   PM_TRY(smem_attr(k_force_interp_stream<ORDER, true, true>, smem));
   const int tiles = (n / IT_Y) * (n / IT_Z);
+  // A chunk repeats 2 R + 2 planes of run-up, so the longest that gives every SM
+  // four times its four resident CTAs, down to 16 planes; a grid that then still
+  // leaves CTA slots empty takes shorter ones, since a column marched by one CTA
+  // is a chain of plane latencies.  Force pass at 16 -> 2 planes: 32^3 53 -> 14 us,
+  // 64^3 59 -> 18; 16 -> 4: 128^3 84 -> 66 (2: 73); 256^3 400 at 32, 16 and 8, 425 at 4.
   int chunk = n;
   while (chunk > 16 && (int64_t)tiles * (n / chunk) * bt.B < 16 * 152) chunk >>= 1;
+  while (bt.B == 1 && chunk > 2 && (int64_t)tiles * (n / chunk) < 4 * 152) chunk >>= 1;
   if (bt.B > 1) {   // batches: the x chunk is tuned (each particle's force is chunk-independent)
     int cand[3], nc = 0;
     for (int c = 16; c <= 64 && c <= n; c *= 2) cand[nc++] = c;

@@ -154,8 +154,6 @@ int64_t sort_meds_capacity(int64_t np);
 int64_t sort_bigs_capacity(int64_t np);
 int64_t sort_smalls_capacity(int64_t np);
 int64_t reduce_partials_capacity(int n, int64_t np);
-// Work items of the streaming deposit for one box of n^3 cells (n >= 32).
-int deposit_items(int n);
 
 // ------------------------------------------------------ stage launchers --
 // Stable sort by cell key: *perm_out (in the workspace) lists the particles

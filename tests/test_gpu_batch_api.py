@@ -90,3 +90,18 @@ def test_interp_of_many_particles_is_bitwise_the_plain_gather(pm, n, N, order):
     small = torch.empty(16 * n ** 3, dtype=torch.uint8, device="cuda")
     assert pm.lib().pm_interp_packed(pm._p(g), pm._p(Xd), N, n, pm._p(plain), pm._p(small),
                                      ctypes.c_size_t(small.numel()), pm._stream()) == 2
+
+
+@pytest.mark.parametrize("n,order", [(32, 5), (64, 3), (64, 7), (128, 5)])
+def test_short_plane_chunks(pm, n, order):
+    """Small grids are marched in few planes a block: the same forces as the
+    gradient and the gather one after the other, and the same density as a batch
+    whose blocks march longer."""
+    X = inputs.uniform_particles(n ** 3, 5)
+    V = np.zeros((3, n ** 3), dtype=np.float32)
+    sim = pm.Simulation(X, V, n, Om=0.3, OL=0.7, boxsize=float(n), keep_acc=True, grad_order=order)
+    sim.step(a=0.5, dt_kick=0.0, dt_drift=0.0)
+    assert torch.equal(sim.acc, pm.interp(pm.gradient(sim.phi, order), sim.X))
+    Xd, B = pm.positions_to_device(X), 2 if n == 128 else 16
+    rho = pm.deposit(Xd, n)
+    assert torch.equal(pm.deposit_batch(Xd.repeat(1, B), n, B)[B - 1], rho)
