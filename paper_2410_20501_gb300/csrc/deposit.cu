@@ -10,8 +10,7 @@
 //
 // n >= 32: the streaming kernel k_deposit_stream walks the x planes of a
 // column of cells (cells of up to kWalkRun particles weighed there, larger
-// ones summed beforehand by k_group_moments, k_medium_moments and
-// k_crowded_moments into the moment buffer).  n < 32: k_deposit<T>, one CTA
+// ones summed beforehand by k_list_moments into the moment buffer).  n < 32: k_deposit<T>, one CTA
 // per T^3 tile: one thread per source cell of the tile plus a one-cell halo
 // walks the cell's particles into moments in shared memory, then every
 // destination cell sums its 27.
@@ -118,7 +117,7 @@ __global__ void __launch_bounds__(T * T * T) k_deposit(const uint32_t* __restric
 //
 // Cells of more than kWalkRun particles are not walked here: eight or sixteen
 // lanes, a warp or a block per cell summed their moments beforehand
-// (k_group_moments, k_medium_moments, k_crowded_moments), and the cell's
+// (k_list_moments), and the cell's
 // thread adds the 27 sums, so a source thread weighs at most kWalkRun
 // particles per plane.
 constexpr int DTY = 16, DTZ = 16, DEY = DTY + 2, DEZ = DTZ + 2, DNT = DTY * DTZ;
@@ -341,14 +340,12 @@ __device__ __forceinline__ void add_moments(const uint32_t* __restrict__ Xs, int
 // adds the lanes' sums in a fixed shuffle tree.  The moments go to
 // crowd[kMomStride a .. + 26] (a = the cell's first rank).
 template <bool VALS, int G>
-__global__ void __launch_bounds__(256) k_group_moments(const uint32_t* __restrict__ Xs, int64_t np,
-                                                       const uint32_t* __restrict__ cellstart,
-                                                       const uint32_t* __restrict__ list, int log2n,
-                                                       const float* __restrict__ vals, float* __restrict__ crowd) {
-  pdl_entry();
+__device__ __forceinline__ void group_moments(const uint32_t* __restrict__ Xs, int64_t np,
+                                              const uint32_t* __restrict__ cellstart,
+                                              const uint32_t* __restrict__ list, uint32_t ncells, int log2n,
+                                              const float* __restrict__ vals, float* __restrict__ crowd) {
   static_assert(G == 8 || G == 16, "group width");
   constexpr int PERW = 32 / G, NOUT = (27 + G - 1) / G;
-  const uint32_t ncells = list[0];
   const uint32_t lane = threadIdx.x & 31, g = lane & (G - 1);
   const uint32_t groups = gridDim.x * 8 * PERW;
   // the groups of a warp take consecutive list entries; a warp with no entry
@@ -394,12 +391,10 @@ __global__ void __launch_bounds__(256) k_group_moments(const uint32_t* __restric
 // the lanes' sums in a fixed shuffle tree.  The moments go to
 // crowd[kMomStride a .. + 26] (a = the cell's first rank).
 template <bool VALS>
-__global__ void __launch_bounds__(256) k_medium_moments(const uint32_t* __restrict__ Xs, int64_t np,
-                                                        const uint32_t* __restrict__ cellstart,
-                                                        const uint32_t* __restrict__ runs, int log2n,
-                                                        const float* __restrict__ vals, float* __restrict__ crowd) {
-  pdl_entry();
-  const uint32_t ntot = runs[0];
+__device__ __forceinline__ void medium_moments(const uint32_t* __restrict__ Xs, int64_t np,
+                                               const uint32_t* __restrict__ cellstart,
+                                               const uint32_t* __restrict__ runs, uint32_t ntot, int log2n,
+                                               const float* __restrict__ vals, float* __restrict__ crowd) {
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t warps = gridDim.x * 8;
   for (uint32_t q = blockIdx.x * 8 + (threadIdx.x >> 5); q < ntot; q += warps) {
@@ -434,13 +429,11 @@ __global__ void __launch_bounds__(256) k_medium_moments(const uint32_t* __restri
 // crowd[kMomStride a .. + 26], as for medium cells.
 constexpr int CT = 256;
 template <bool VALS>
-__global__ void __launch_bounds__(CT) k_crowded_moments(const uint32_t* __restrict__ Xs, int64_t np,
-                                                        const uint32_t* __restrict__ cellstart,
-                                                        const uint32_t* __restrict__ bigs, int log2n,
-                                                        const float* __restrict__ vals, float* __restrict__ crowd) {
-  pdl_entry();
+__device__ __forceinline__ void crowded_moments_block(const uint32_t* __restrict__ Xs, int64_t np,
+                                                      const uint32_t* __restrict__ cellstart,
+                                                      const uint32_t* __restrict__ bigs, uint32_t nruns, int log2n,
+                                                      const float* __restrict__ vals, float* __restrict__ crowd) {
   __shared__ float part[CT / 32][27];
-  const uint32_t nruns = bigs[0];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (uint32_t q = blockIdx.x; q < nruns; q += gridDim.x) {
     const uint32_t c = bigs[1 + q];
@@ -464,6 +457,22 @@ __global__ void __launch_bounds__(CT) k_crowded_moments(const uint32_t* __restri
     }
     __syncthreads();
   }
+}
+
+// The moments of all listed cells, the largest first.  One launch for the four
+// lists: most are empty or short, and a launch of its own costs more than its
+// work (32^3, alone: four launches 12.3 us, one 3.4; 10^7 on 256^3 42 -> 28; 256^3
+// late 88 -> 87).
+template <bool VALS>
+__global__ void __launch_bounds__(CT, 4) k_list_moments(const uint32_t* __restrict__ Xs, int64_t np,
+                                                     const uint32_t* __restrict__ cellstart, Crowded cr, int log2n,
+                                                     const float* __restrict__ vals) {
+  pdl_entry();
+  const uint32_t nb = cr.bigs[0], nr = cr.runs[0], nm = cr.meds[0], ns = cr.smalls[0];
+  crowded_moments_block<VALS>(Xs, np, cellstart, cr.bigs, nb, log2n, vals, cr.moments);
+  medium_moments<VALS>(Xs, np, cellstart, cr.runs, nr, log2n, vals, cr.moments);
+  group_moments<VALS, 16>(Xs, np, cellstart, cr.meds, nm, log2n, vals, cr.moments);
+  group_moments<VALS, 8>(Xs, np, cellstart, cr.smalls, ns, log2n, vals, cr.moments);
 }
 
 // x planes per CTA and CTAs a box.  A chunk repeats the planes on its two sides:
@@ -504,22 +513,27 @@ __global__ void __launch_bounds__(256) k_sum_partials(const float* __restrict__ 
 }
 
 // out[k] = scale * sum_i partial[k * stride + i], i < count, for k < nout
-// (one block, fixed order: strided per-thread sums then a tree).
+// (one block, fixed order: strided per-thread sums, then the lanes and the warps
+// in shuffle trees).  Latency is all it costs: two barriers instead of ten.
 __global__ void __launch_bounds__(1024) k_reduce_partials(const double* __restrict__ partial,
                                                           int64_t count, int64_t stride, int nout,
                                                           double scale, double* __restrict__ out) {
   pdl_entry();
-  __shared__ double red[1024];
+  __shared__ double red[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int k = blockIdx.x; k < nout; k += gridDim.x) {   // one output per block (fixed order within it)
     double t = 0.0;
     for (int64_t i = threadIdx.x; i < count; i += blockDim.x) t += partial[k * stride + i];
-    red[threadIdx.x] = t;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) red[warp] = t;
     __syncthreads();
-    for (int o = 512; o > 0; o >>= 1) {
-      if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-      __syncthreads();
+    if (warp == 0) {
+      t = red[lane];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+      if (lane == 0) out[k] = t * scale;
     }
-    if (threadIdx.x == 0) out[k] = red[0] * scale;
     __syncthreads();
   }
 }
@@ -561,26 +575,10 @@ namespace {
 pm_status crowded_moments(const uint32_t* Xs, int64_t np, const uint32_t* cellstart, int n, const float* vals,
                           const Crowded& cr, cudaStream_t s) {
   if (!cr.runs || np == 0) return PM_OK;
-  const int l2 = ilog2(n);
-  if (vals) {
-    PM_LAUNCH(K_DEPOSIT, 0.0, (k_group_moments<true, 8>), 8 * 152, 256, 0, s, Xs, np, cellstart, cr.smalls, l2, vals,
-              cr.moments);
-    PM_LAUNCH(K_DEPOSIT, 0.0, (k_group_moments<true, 16>), 8 * 152, 256, 0, s, Xs, np, cellstart, cr.meds, l2, vals,
-              cr.moments);
-    PM_LAUNCH(K_DEPOSIT, 0.0, k_medium_moments<true>, 8 * 152, 256, 0, s, Xs, np, cellstart, cr.runs, l2, vals,
-              cr.moments);
-    PM_LAUNCH(K_DEPOSIT, 0.0, k_crowded_moments<true>, 4 * 152, CT, 0, s, Xs, np, cellstart, cr.bigs, l2, vals,
-              cr.moments);
-  } else {
-    PM_LAUNCH(K_DEPOSIT, 0.0, (k_group_moments<false, 8>), 8 * 152, 256, 0, s, Xs, np, cellstart, cr.smalls, l2,
-              vals, cr.moments);
-    PM_LAUNCH(K_DEPOSIT, 0.0, (k_group_moments<false, 16>), 8 * 152, 256, 0, s, Xs, np, cellstart, cr.meds, l2, vals,
-              cr.moments);
-    PM_LAUNCH(K_DEPOSIT, 0.0, k_medium_moments<false>, 8 * 152, 256, 0, s, Xs, np, cellstart, cr.runs, l2, vals,
-              cr.moments);
-    PM_LAUNCH(K_DEPOSIT, 0.0, k_crowded_moments<false>, 4 * 152, CT, 0, s, Xs, np, cellstart, cr.bigs, l2, vals,
-              cr.moments);
-  }
+  if (vals)
+    PM_LAUNCH(K_DEPOSIT, 0.0, k_list_moments<true>, 8 * 152, CT, 0, s, Xs, np, cellstart, cr, ilog2(n), vals);
+  else
+    PM_LAUNCH(K_DEPOSIT, 0.0, k_list_moments<false>, 8 * 152, CT, 0, s, Xs, np, cellstart, cr, ilog2(n), vals);
   return PM_OK;
 }
 }  // namespace

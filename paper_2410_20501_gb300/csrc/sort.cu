@@ -30,11 +30,15 @@ constexpr int SCAN_CHUNK = SCAN_V * SCAN_T;
 constexpr int KT = 256;             // threads of the key, scatter and order kernels
 constexpr int CI = 4;               // particles per thread of the counting kernel
 constexpr uint32_t SHORT_RUN = kLongRun;  // runs up to this length are ordered by one thread or warp
-constexpr int WT = 256;             // threads of the warp-per-run kernel
-constexpr int LT = 256;             // threads of a long-run block
+constexpr int LT = 256;             // threads of the kernel that orders the listed runs
 constexpr int LCH = 4096;           // elements sorted in shared memory at once
-constexpr int LONG_BLOCKS = 8 * 152;
+constexpr int LIST_BLOCKS = 8 * 152;
 
+
+// The counters of the crowded-cell lists (their entries follow).
+struct ListHeads {
+  uint32_t *smalls, *meds, *runs, *bigs;
+};
 
 // key = (i n + j) n + k of the cell holding each particle; with np_box > 0
 // (a batch of boxes) prefixed by the box, i / np_box.  Counts the particles of
@@ -86,8 +90,9 @@ __global__ void __launch_bounds__(KT) k_cell_count(const uint32_t* __restrict__ 
 // their loads in flight together.
 __global__ void __launch_bounds__(KT) k_cell_scatter(const uint2* __restrict__ kr, int64_t np,
                                                      const uint32_t* __restrict__ cellstart,
-                                                     uint32_t* __restrict__ perm) {
+                                                     uint32_t* __restrict__ perm, ListHeads lists) {
   pdl_entry();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *lists.smalls = *lists.meds = *lists.runs = *lists.bigs = 0;   // for k_cell_order
   const int64_t i0 = blockIdx.x * (int64_t)(KT * CI) + threadIdx.x;
   uint2 t[CI];
   uint32_t base[CI];
@@ -104,10 +109,10 @@ __global__ void __launch_bounds__(KT) k_cell_scatter(const uint2* __restrict__ k
 // cellstart[c+1]-1, in ascending particle index.  A thread takes OC
 // consecutive cells (16-byte loads of their starts).  Runs of at most
 // kWalkRun are insertion-sorted here; runs of at most kMedRun are listed in
-// smalls[1 ..] (for k_cell_order_med<16> and the deposit), runs of at most
-// SHORT_RUN in meds[1 ..] for k_cell_order_med<32>, longer ones in runs[1 ..] for
-// k_cell_order_warp and, if longer than kWarpRun, in bigs[1 ..] for
-// k_cell_order_long as well (list[0] counts the entries, zeroed).  A block
+// smalls[1 ..] (for order_groups<16> and the deposit), runs of at most
+// SHORT_RUN in meds[1 ..] for order_groups<32>, longer ones in runs[1 ..] for
+// order_warps and, if longer than kWarpRun, in bigs[1 ..] for
+// order_long as well (list[0] counts the entries, zeroed).  A block
 // reserves the room for its entries of each list with one atomic (the lists'
 // counters are shared by the whole grid), its warps and lanes in order after
 // it; a block without entries skips the reservation and its second barrier.
@@ -171,7 +176,7 @@ __global__ void __launch_bounds__(KT) k_cell_order(const uint32_t* __restrict__ 
 #pragma unroll
   for (int k = 0; k < OC; ++k) {
     const uint32_t a = st[k], b = st[k + 1];
-    if (b - a < 2 || b - a > kWalkRun) continue;   // larger runs: k_cell_order_med
+    if (b - a < 2 || b - a > kWalkRun) continue;   // larger runs: k_cell_order_lists
     for (uint32_t p = a + 1; p < b; ++p) {
       const uint32_t v = perm[p];
       uint32_t q = p;
@@ -205,17 +210,14 @@ __global__ void __launch_bounds__(KT) k_cell_order(const uint32_t* __restrict__ 
 // over the group by shuffles.  G = 16 for the small runs (kWalkRun + 1 ..
 // kMedRun particles), G = 32 for the medium ones (kMedRun + 1 .. SHORT_RUN).
 template <int G>
-__global__ void __launch_bounds__(KT) k_cell_order_med(const uint32_t* __restrict__ cellstart,
-                                                       const uint32_t* __restrict__ list,
-                                                       uint32_t* __restrict__ perm) {
-  pdl_entry();
+__device__ __forceinline__ void order_groups(const uint32_t* __restrict__ cellstart, const uint32_t* __restrict__ list,
+                                             uint32_t nlist, uint32_t* __restrict__ perm) {
   constexpr int PERW = 32 / G;
-  const uint32_t nlist = list[0];
   const uint32_t lane = threadIdx.x & 31, g = lane & (G - 1);
-  const uint32_t groups = gridDim.x * (KT / 32) * PERW;
+  const uint32_t groups = gridDim.x * (LT / 32) * PERW;
   // the groups of a warp take consecutive list entries; a warp with no entry
   // left stops as a whole (the shuffles need every lane)
-  for (uint32_t q0 = (blockIdx.x * (KT / 32) + (threadIdx.x >> 5)) * PERW; q0 < nlist; q0 += groups) {
+  for (uint32_t q0 = (blockIdx.x * (LT / 32) + (threadIdx.x >> 5)) * PERW; q0 < nlist; q0 += groups) {
     const uint32_t q = q0 + lane / G;
     uint32_t a = 0, m = 0;
     if (q < nlist) {
@@ -256,17 +258,13 @@ __device__ __forceinline__ void warp_rank_sort(const uint32_t* buf, uint32_t m, 
 // The crowded runs listed by k_cell_order of at most kWarpRun particles, one
 // warp each (many runs in flight per SM): the run is copied to the warp's
 // shared-memory buffer and every element moved to its rank.  Longer runs are
-// skipped here (k_cell_order_long orders them).
-__global__ void __launch_bounds__(WT) k_cell_order_warp(const uint32_t* __restrict__ cellstart,
-                                                        const uint32_t* __restrict__ runs,
-                                                        uint32_t* __restrict__ perm) {
-  pdl_entry();
-  __shared__ uint32_t sbuf[WT / 32][kWarpRun];
-  const uint32_t nruns = runs[0];
+// skipped here (order_long orders them).
+__device__ __forceinline__ void order_warps(const uint32_t* __restrict__ cellstart, const uint32_t* __restrict__ runs,
+                                            uint32_t nruns, uint32_t* __restrict__ perm, uint32_t* sbuf) {
   const uint32_t lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  uint32_t* buf = sbuf[wib];
-  const uint32_t warps = gridDim.x * (WT / 32);
-  for (uint32_t q = blockIdx.x * (WT / 32) + wib; q < nruns; q += warps) {
+  uint32_t* buf = sbuf + wib * kWarpRun;
+  const uint32_t warps = gridDim.x * (LT / 32);
+  for (uint32_t q = blockIdx.x * (LT / 32) + wib; q < nruns; q += warps) {
     const uint32_t c = runs[1 + q];
     const uint32_t a = cellstart[c], m = cellstart[c + 1] - a;
     if (m > kWarpRun) continue;   // the same for the whole warp
@@ -319,13 +317,9 @@ __device__ void block_merge(const uint32_t* A, int64_t la, const uint32_t* B, in
 // LCH-element chunks sorted in shared memory, then pairwise merges between
 // the run and the same ranks of `scratch`.  Runs already in order are left as
 // they are.
-__global__ void __launch_bounds__(LT) k_cell_order_long(const uint32_t* __restrict__ cellstart,
-                                                        const uint32_t* __restrict__ runs,
-                                                        uint32_t* __restrict__ perm,
-                                                        uint32_t* __restrict__ scratch) {
-  pdl_entry();
-  __shared__ uint32_t sv[LCH];
-  const uint32_t nruns = runs[0];
+__device__ __forceinline__ void order_long(const uint32_t* __restrict__ cellstart, const uint32_t* __restrict__ runs,
+                                           uint32_t nruns, uint32_t* __restrict__ perm, uint32_t* __restrict__ scratch,
+                                           uint32_t* sv) {
   for (uint32_t q = blockIdx.x; q < nruns; q += gridDim.x) {
     const uint32_t c = runs[1 + q];
     const uint32_t a = cellstart[c];
@@ -362,6 +356,27 @@ __global__ void __launch_bounds__(LT) k_cell_order_long(const uint32_t* __restri
     }
     __syncthreads();
   }
+}
+
+// Orders the listed runs: the longest first, then warps and groups of lanes over
+// the lists in equal shares.  One launch for the four lists: each is empty or
+// short in most calls, and a launch of its own costs more than its work (32^3,
+// alone: four launches 12.6 us, one 3.8; 10^7 on 256^3 38 -> 28).  Eight blocks an
+// SM: the short lists wait on loads, and at five 256^3 late took 72 us instead of 51.
+__global__ void __launch_bounds__(LT, 8) k_cell_order_lists(const uint32_t* __restrict__ cellstart,
+                                                         const uint32_t* __restrict__ smalls,
+                                                         const uint32_t* __restrict__ meds,
+                                                         const uint32_t* __restrict__ runs,
+                                                         const uint32_t* __restrict__ bigs, uint32_t* __restrict__ perm,
+                                                         uint32_t* __restrict__ scratch) {
+  pdl_entry();
+  __shared__ uint32_t sv[LCH];
+  static_assert(LT / 32 * kWarpRun <= LCH, "the warps' buffers share the block's");
+  const uint32_t nb = bigs[0], nr = runs[0], nm = meds[0], ns = smalls[0];
+  order_long(cellstart, bigs, nb, perm, scratch, sv);   // ends at a barrier, if it ran
+  order_warps(cellstart, runs, nr, perm, sv);
+  order_groups<32>(cellstart, meds, nm, perm);
+  order_groups<16>(cellstart, smalls, ns, perm);
 }
 
 // ---- exclusive scan of a uint32 array (three kernels) ----
@@ -439,6 +454,9 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_sums(uint32_t* __restrict__ sum
   }
 }
 
+// SUMS: sums holds the chunks' totals and not their prefix, and each block adds up
+// those before its own (a launch less: see scan_u32).
+template <bool SUMS>
 __global__ void __launch_bounds__(SCAN_T) k_scan_apply(uint32_t* __restrict__ a, int64_t len,
                                                        const uint32_t* __restrict__ sums) {
   pdl_entry();
@@ -449,7 +467,15 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_apply(uint32_t* __restrict__ a,
   scan_load(a, len, base, v);
 #pragma unroll
   for (int k = 0; k < SCAN_V; ++k) t += v[k];
-  uint32_t e = block_exclusive_scan(t, wt, &tot) + sums[blockIdx.x];
+  uint32_t before = 0;
+  if (SUMS) {
+    for (uint32_t i = threadIdx.x; i < blockIdx.x; i += SCAN_T) before += sums[i];
+    block_exclusive_scan(before, wt, &tot);
+    before = tot;   // (the scan ends at a barrier, and the next one begins before it writes tot)
+  } else {
+    before = sums[blockIdx.x];
+  }
+  uint32_t e = block_exclusive_scan(t, wt, &tot) + before;
   if (base + SCAN_V <= len && ((uintptr_t)a & 15) == 0) {
 #pragma unroll
     for (int q = 0; q < SCAN_V / 4; ++q) {
@@ -519,8 +545,14 @@ pm_status scan_u32(uint32_t* a, int64_t len, uint32_t* sums, cudaStream_t s) {
   int64_t nb = (len + SCAN_CHUNK - 1) / SCAN_CHUNK;
   if (nb == 0) return PM_OK;
   PM_LAUNCH(K_SORT_SCAN, 4.0 * len, k_scan_reduce, (unsigned)nb, SCAN_T, 0, s, a, len, sums);
+  // up to two totals a thread, every block adds the ones before it itself (2048
+  // blocks read 8 MB from L2 in all); 512^3 has 8193, where a scan of its own is cheaper
+  if (nb <= 2 * SCAN_T) {
+    PM_LAUNCH(K_SORT_SCAN, 8.0 * len, k_scan_apply<true>, (unsigned)nb, SCAN_T, 0, s, a, len, sums);
+    return PM_OK;
+  }
   PM_LAUNCH(K_SORT_SCAN, 8.0 * nb, k_scan_sums, 1, SCAN_T, 0, s, sums, nb);
-  PM_LAUNCH(K_SORT_SCAN, 8.0 * len, k_scan_apply, (unsigned)nb, SCAN_T, 0, s, a, len, sums);
+  PM_LAUNCH(K_SORT_SCAN, 8.0 * len, k_scan_apply<false>, (unsigned)nb, SCAN_T, 0, s, a, len, sums);
   return PM_OK;
 }
 
@@ -540,11 +572,10 @@ pm_status sort_cells(const uint32_t* X, int64_t np, int n, Workspace& w, cudaStr
   const int64_t ncells = (int64_t)n * n * n * bt.B;
   *perm_out = w.perm;
   PM_TRY(cuda_status(cudaMemsetAsync(cellstart, 0, (size_t)(ncells + 1) * 4, s)));
-  PM_TRY(cuda_status(cudaMemsetAsync(w.runs, 0, 4, s)));   // no crowded or medium cells yet
-  PM_TRY(cuda_status(cudaMemsetAsync(w.meds, 0, 4, s)));
-  PM_TRY(cuda_status(cudaMemsetAsync(w.bigs, 0, 4, s)));
-  PM_TRY(cuda_status(cudaMemsetAsync(w.smalls, 0, 4, s)));
-  if (np == 0) return PM_OK;
+  if (np == 0) {   // no cell is crowded
+    for (uint32_t* c : {w.smalls, w.meds, w.runs, w.bigs}) PM_TRY(cuda_status(cudaMemsetAsync(c, 0, 4, s)));
+    return PM_OK;
+  }
   const int64_t np_box = bt.B > 1 ? bt.np_box : 0;
   const unsigned gc = grid_for(np, KT * CI);
   if (np_box > 0)
@@ -552,14 +583,12 @@ pm_status sort_cells(const uint32_t* X, int64_t np, int n, Workspace& w, cudaStr
   else
     PM_LAUNCH(K_KEYS, 28.0 * np, k_cell_count<false>, gc, KT, 0, s, X, np, log2n, np_box, w.keyrank, cellstart);
   PM_TRY(scan_u32(cellstart, ncells + 1, w.scan_blocks, s));
-  PM_LAUNCH(K_SCATTER, 16.0 * np, k_cell_scatter, gc, KT, 0, s, w.keyrank, np, cellstart, w.perm);
+  PM_LAUNCH(K_SCATTER, 16.0 * np, k_cell_scatter, gc, KT, 0, s, w.keyrank, np, cellstart, w.perm,
+            ListHeads{w.smalls, w.meds, w.runs, w.bigs});
   PM_LAUNCH(K_ORDER, 4.0 * ncells + 8.0 * np, k_cell_order, grid_for(ncells / OC, KT), KT, 0, s, cellstart, ncells,
             w.perm, w.smalls, w.meds, w.runs, w.bigs);
-  PM_LAUNCH(K_ORDER, 0.0, k_cell_order_med<16>, 8 * 152, KT, 0, s, cellstart, w.smalls, w.perm);
-  PM_LAUNCH(K_ORDER, 0.0, k_cell_order_med<32>, 8 * 152, KT, 0, s, cellstart, w.meds, w.perm);
-  PM_LAUNCH(K_ORDER, 0.0, k_cell_order_warp, 8 * 152, WT, 0, s, cellstart, w.runs, w.perm);
-  PM_LAUNCH(K_ORDER, 0.0, k_cell_order_long, LONG_BLOCKS, LT, 0, s, cellstart, w.bigs, w.perm,
-            reinterpret_cast<uint32_t*>(w.keyrank));
+  PM_LAUNCH(K_ORDER, 0.0, k_cell_order_lists, LIST_BLOCKS, LT, 0, s, cellstart, w.smalls, w.meds, w.runs, w.bigs,
+            w.perm, reinterpret_cast<uint32_t*>(w.keyrank));
   return launch_status();
 }
 

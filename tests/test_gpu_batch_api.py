@@ -105,3 +105,15 @@ def test_short_plane_chunks(pm, n, order):
     Xd, B = pm.positions_to_device(X), 2 if n == 128 else 16
     rho = pm.deposit(Xd, n)
     assert torch.equal(pm.deposit_batch(Xd.repeat(1, B), n, B)[B - 1], rho)
+
+
+@pytest.mark.parametrize("B", [127, 128])
+def test_cell_starts_on_both_sides_of_the_scan_rule(pm, B):
+    """2033 chunks of cell counts (each block adds the totals before its own) and
+    2049 (a scan of the totals): every box's density as if it were alone."""
+    n, np_box = 64, 1537
+    X = inputs.uniform_particles(B * np_box, 9)
+    rho = pm.deposit_batch(pm.positions_to_device(X), n, B)
+    for b in (0, 63, B - 1):
+        one = pm.positions_to_device(np.ascontiguousarray(X[:, b * np_box:(b + 1) * np_box]))
+        assert torch.equal(rho[b], pm.deposit(one, n)), b
