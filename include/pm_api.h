@@ -157,10 +157,11 @@ typedef struct {
                              of Eq. rescaming_newtonian_potential)              */
   float guess_scale;
   int smoother;           /* 2 or 0: fused red-black sweeps on levels with
-                             n >= 64, two per pass over memory (mg_*; fr_*: see
-                             fr_params), bitwise equal to the colour passes,
-                             which levels below take; 1: colour passes (one
-                             kernel per colour) everywhere                     */
+                             n >= 64, two per pass over memory, and on smaller
+                             ones up to two with the transfer next to them
+                             (mg_*; fr_*: see fr_params), bitwise equal to the
+                             colour passes; 1: colour passes (one kernel per
+                             colour) everywhere                                */
   float coarse_omega;     /* SOR factor of the coarsest-level sweeps; 0: the
                              optimal one for that grid, 2/(1 + sqrt(1 - mu^2)),
                              mu = (2 + cos(2 pi/n))/3 (1.634 at 16^3)          */

@@ -135,13 +135,13 @@ size_t layout_workspace(Workspace* w, void* base, int n, int64_t np, uint32_t fl
     const int nl = n >> l;
     if (nl < 4) break;
     const size_t bytes = (size_t)nl * nl * nl * 4 * batch;
-    const bool streamed = nl >= 64;   // levels smoothed out of place (fused or streaming sweeps) need a ping-pong partner
+    const bool streamed = nl >= 64;   // f(R) levels smoothed out of place need a ping-pong partner
     if (mg) {
       if (l > 0) {
         w->mg_u[l] = (float*)take(bytes);
         w->mg_f[l] = (float*)take(bytes);
       }
-      if (streamed) w->mg_alt[l] = (float*)take(bytes);
+      if (nl >= 8) w->mg_alt[l] = (float*)take(bytes);   // every level but the smallest possible is smoothed out of place
     }
     if (fr) {
       if (l > 0) {

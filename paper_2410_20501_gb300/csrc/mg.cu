@@ -143,6 +143,60 @@ struct PairSum {
   }
 };
 
+// The right-hand sides of two coarse cells next to each other in z from their
+// children's rows (core [x][y], four cells along z), the rows beyond them in x
+// (xf [side][y]) and y (yf [x][side]), the cells before (zl) and after (zr) the
+// rows and the sources' rows (fr [x][y]; source fs (fr - mean)).
+template <bool COMP>
+__device__ __forceinline__ float2 restrict_pair(const float4 (&core)[2][2], const float4 (&xf)[2][2],
+                                                const float4 (&yf)[2][2], const float4 (&fr)[2][2],
+                                                const float (&zl)[2][2], const float (&zr)[2][2], float fs, float mean,
+                                                float inv_h2) {
+  // (first coarse cell, second coarse cell): even fine cells, odd fine cells
+  auto ev = [](const float4& v) { return make_float2(v.x, v.z); };
+  auto od = [](const float4& v) { return make_float2(v.y, v.w); };
+  auto source = [&](float2 v) { return mul2(both(fs), add2(v, both(-mean))); };
+  float2 d;
+  if (COMP) {
+    PairSum S(ev(xf[0][0])), C(ev(core[0][0])), F(source(ev(fr[0][0])));
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        if (a + b) {
+          S.add(ev(xf[a][b]));
+          C.add(ev(core[a][b]));
+          F.add(source(ev(fr[a][b])));
+        }
+        S.add(od(xf[a][b]));
+        S.add(ev(yf[a][b]));
+        S.add(od(yf[a][b]));
+        S.add(make_float2(zl[a][b], core[a][b].y));
+        S.add(make_float2(core[a][b].z, zr[a][b]));
+        C.add(od(core[a][b]));
+        F.add(source(od(fr[a][b])));
+      }
+    S.sub_times(3.0f, C);
+    d = add2(fma2(both(-inv_h2), S.s, F.s), fma2(both(-inv_h2), S.e, F.e));
+  } else {
+    // per row, so that what cancels is subtracted early: neighbours minus three times the children
+    float2 L = both(0.0f), F = both(0.0f);
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const float2 ce = mul2(ev(core[a][b]), both(-1.0f)), co = mul2(od(core[a][b]), both(-1.0f));
+        const float2 fe = add2(ev(xf[a][b]), ce), fo = add2(od(xf[a][b]), co);
+        const float2 ge = add2(ev(yf[a][b]), ce), go = add2(od(yf[a][b]), co);
+        const float2 lo = add2(make_float2(zl[a][b], core[a][b].y), ce), hi = add2(make_float2(core[a][b].z, zr[a][b]), co);
+        L = add2(L, add2(add2(add2(fe, fo), add2(ge, go)), add2(lo, hi)));
+        F = add2(F, add2(source(ev(fr[a][b])), source(od(fr[a][b]))));
+      }
+    d = fma2(both(-inv_h2), L, F);
+  }
+  return mul2(d, both(0.125f));
+}
+
 // Coarse right-hand side fc = R(f - L u): residual of the 8 children,
 // averaged.  Summed over the 2x2x2 block the Laplacian fluxes through the 12
 // inner faces cancel pairwise, so  h^2 sum_c L u_c  is the sum of the 24 outer
@@ -183,50 +237,8 @@ __global__ void __launch_bounds__(128) k_resid_restrict(const float* __restrict_
       yf[a][b] = row(u, 2 * I + a, b ? 2 * J + 2 : 2 * J - 1);
       fr[a][b] = row(f.p, 2 * I + a, 2 * J + b);
     }
-  const float mean = load_mean(f);
-  // (first coarse cell, second coarse cell): even fine cells, odd fine cells
-  auto ev = [](const float4& v) { return make_float2(v.x, v.z); };
-  auto od = [](const float4& v) { return make_float2(v.y, v.w); };
-  auto source = [&](float2 v) { return mul2(both(f.s), add2(v, both(-mean))); };
-  float2 d;
-  if (COMP) {
-    PairSum S(ev(xf[0][0])), C(ev(core[0][0])), F(source(ev(fr[0][0])));
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        if (a + b) {
-          S.add(ev(xf[a][b]));
-          C.add(ev(core[a][b]));
-          F.add(source(ev(fr[a][b])));
-        }
-        S.add(od(xf[a][b]));
-        S.add(ev(yf[a][b]));
-        S.add(od(yf[a][b]));
-        S.add(make_float2(zl[a][b], core[a][b].y));
-        S.add(make_float2(core[a][b].z, zr[a][b]));
-        C.add(od(core[a][b]));
-        F.add(source(od(fr[a][b])));
-      }
-    S.sub_times(3.0f, C);
-    d = add2(fma2(both(-inv_h2), S.s, F.s), fma2(both(-inv_h2), S.e, F.e));
-  } else {
-    // per row, so that what cancels is subtracted early: neighbours minus three times the children
-    float2 L = both(0.0f), F = both(0.0f);
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        const float2 ce = mul2(ev(core[a][b]), both(-1.0f)), co = mul2(od(core[a][b]), both(-1.0f));
-        const float2 fe = add2(ev(xf[a][b]), ce), fo = add2(od(xf[a][b]), co);
-        const float2 ge = add2(ev(yf[a][b]), ce), go = add2(od(yf[a][b]), co);
-        const float2 lo = add2(make_float2(zl[a][b], core[a][b].y), ce), hi = add2(make_float2(core[a][b].z, zr[a][b]), co);
-        L = add2(L, add2(add2(add2(fe, fo), add2(ge, go)), add2(lo, hi)));
-        F = add2(F, add2(source(ev(fr[a][b])), source(od(fr[a][b]))));
-      }
-    d = fma2(both(-inv_h2), L, F);
-  }
-  *reinterpret_cast<float2*>(fc + 2 * t) = mul2(d, both(0.125f));
+  *reinterpret_cast<float2*>(fc + 2 * t) =
+      restrict_pair<COMP>(core, xf, yf, fr, zl, zr, f.s, load_mean(f), inv_h2);
 }
 
 // Residual norm^2 and source norm^2 partials (finest level, compensated
@@ -323,6 +335,56 @@ __global__ void k_add_correction_f64(double* __restrict__ u, const float* __rest
     u[c] += (double)__ldg(e + c);
 }
 
+// P(uc - uc2) at the 16 children of the coarse cells (I, J, K) and (I, J, K + 1), K
+// even: put(x, y, the four along z).  Interpolated along z, then y, then x.
+template <class Put>
+__device__ __forceinline__ void prolong_pair(const float* __restrict__ uc, const float* __restrict__ uc2, int I, int J,
+                                             int K, int lc, const Put& put) {
+  const int mc = (1 << lc) - 1;
+  float c[3][3][4];   // [x][y][z]: x, y = I-1 .. I+1, J-1 .. J+1; z = K-1 .. K+2
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int64_t base = idx3((I + a - 1) & mc, (J + b - 1) & mc, 0, lc);
+      const float2 mid = __ldg(reinterpret_cast<const float2*>(uc + base + K));
+      float v[4] = {__ldg(uc + base + ((K - 1) & mc)), mid.x, mid.y, __ldg(uc + base + ((K + 2) & mc))};
+      if (uc2) {
+        const float2 m2 = __ldg(reinterpret_cast<const float2*>(uc2 + base + K));
+        v[0] -= __ldg(uc2 + base + ((K - 1) & mc));
+        v[1] -= m2.x;
+        v[2] -= m2.y;
+        v[3] -= __ldg(uc2 + base + ((K + 2) & mc));
+      }
+#pragma unroll
+      for (int z = 0; z < 4; ++z) c[a][b][z] = v[z];
+    }
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    const int jn = b ? 2 : 0;
+    // z then y contractions: vy[x][q] for the fine z offsets q = 0..3 (coarse
+    // cell q / 2 at column q / 2 + 1, child q & 1)
+    float vy[3][4];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int kc = (q >> 1) + 1, kn = (q & 1) ? kc + 1 : kc - 1;
+        const float vz0 = fmaf(0.25f, c[a][1][kn], fmaf(0.75f, c[a][1][kc], 0.0f));
+        const float vz1 = fmaf(0.25f, c[a][jn][kn], fmaf(0.75f, c[a][jn][kc], 0.0f));
+        vy[a][q] = fmaf(0.25f, vz1, fmaf(0.75f, vz0, 0.0f));
+      }
+#pragma unroll
+    for (int ax = 0; ax < 2; ++ax) {
+      const int in = ax ? 2 : 0;
+      put(ax, b, make_float4(fmaf(0.25f, vy[in][0], fmaf(0.75f, vy[1][0], 0.0f)),
+                             fmaf(0.25f, vy[in][1], fmaf(0.75f, vy[1][1], 0.0f)),
+                             fmaf(0.25f, vy[in][2], fmaf(0.75f, vy[1][2], 0.0f)),
+                             fmaf(0.25f, vy[in][3], fmaf(0.75f, vy[1][3], 0.0f))));
+    }
+  }
+}
+
 // u += P(uc - uc2): cell-centred trilinear prolongation, weights 27/9/3/1 over
 // 64 (§3.6.1); uc2 may be NULL.  One thread per two coarse cells along z
 // (K = 2G, 2G + 1): it reads their 3x3x4 coarse neighbourhood once (a float2
@@ -342,50 +404,134 @@ __global__ void k_prolong_correct(float* __restrict__ u, const float* __restrict
     const int K = 2 * (int)(t & ((1 << hz) - 1));
     const int64_t row = t >> hz;
     const int J = (int)(row & mc), I = (int)(row >> lc);
-    float c[3][3][4];   // [x][y][z]: x, y = I-1 .. I+1, J-1 .. J+1; z = K-1 .. K+2
+    prolong_pair(uc, uc2, I, J, K, lc, [&](int ax, int b, float4 e) {
+      float4* dst = reinterpret_cast<float4*>(u + idx3(2 * I + ax, 2 * J + b, 2 * K, log2n));
+      float4 w = *dst;
+      *dst = make_float4(w.x + e.x, w.y + e.y, w.z + e.z, w.w + e.w);
+    });
+  }
+}
+
+// One side of a V-cycle on a level of up to 32^3 in one launch: the red-black
+// sweeps before the coarse correction and the restriction after them (PRE), or
+// the prolongation and the sweeps after it.  Such a level is a megabyte at most
+// and a colour pass over it is all latency (2.3 us a launch, ten launches a
+// cycle), so the sweeps are repeated instead of synchronised: a CTA takes TX x TY
+// rows of full length with a halo of as many rows as the passes (and the
+// residual) reach, every pass updates a row less on each side, and CTAs never
+// exchange anything.  Rows are kept by colour (a thread's two cells of one colour
+// are one 8-byte word, as are the neighbours' that it reads), so a pass reads one
+// colour and writes the other.  The updates, the restriction and the
+// prolongation are those of the kernels above, cell by cell: bitwise the same.
+//
+// Rows of 4 x 4 while one CTA an SM takes them all, of 8 x 8, which repeat less,
+// beyond (16 boxes 52 us a V-cycle against 46; 4 boxes 31 against 34).  V-cycle from
+// 32^3 against colour passes and the transfers' own launches, coarsest solve
+// included: one box 33 -> 26 us, 16 boxes 70 -> 46, 64 boxes 111 -> 105.
+//
+// uin: the iterate (NULL: zeros), uout: not uin.  n >= 8.
+constexpr int kTileN = 32;
+template <int TX, int TY, bool PRE> struct TileGeom {
+  static constexpr int H = PRE ? 5 : 4, EX = TX + 2 * H, EY = TY + 2 * H, ROWS = EX * EY;
+  static constexpr int ITEMS = 4, THREADS = (ROWS * (kTileN / 4) / ITEMS + 31) / 32 * 32;   // items: four cells of a row
+  static constexpr size_t smem = 2 * sizeof(float2) * ROWS * (kTileN / 4);
+};
+template <int TX, int TY, bool PRE, bool COMP>
+__global__ void __launch_bounds__(TileGeom<TX, TY, PRE>::THREADS)
+    k_rb_tile(const float* __restrict__ uin, float* __restrict__ uout, Src f, const float* __restrict__ uc,
+              float* __restrict__ fc, int log2n, int sweeps, PoissonUpdate u0, PoissonUpdate u1) {
+  pdl_entry();
+  using T = TileGeom<TX, TY, PRE>;
+  constexpr int H = T::H, EX = T::EX, EY = T::EY;
+  extern __shared__ float4 tile_sm[];
+  const int n = 1 << log2n, m = n - 1, lq = log2n - 2, Q = 1 << lq, items = T::ROWS << lq;
+  float2* U = reinterpret_cast<float2*>(tile_sm);   // [colour][item]
+  const int64_t box = (int64_t)blockIdx.z << (3 * log2n);
+  f = box_src(f, (int64_t)1 << (3 * log2n));
+  u0 = u0.box(blockIdx.z);
+  const int x0 = (int)(blockIdx.x / (unsigned)(n / TY)) * TX - H, y0 = (int)(blockIdx.x % (unsigned)(n / TY)) * TY - H;
+  const int tid = threadIdx.x;
+  auto cell = [&](int x, int y, int q) { return idx3((x0 + x) & m, (y0 + y) & m, 4 * q, log2n); };
+  auto put = [&](int x, int y, int q, const float4& v) {
+    const int o = (x0 + x + y0 + y) & 1, i = ((x * EY + y) << lq) + q;
+    U[o * items + i] = make_float2(v.x, v.z);
+    U[(o ^ 1) * items + i] = make_float2(v.y, v.w);
+  };
+  auto get = [&](int x, int y, int q) {
+    const int o = (x0 + x + y0 + y) & 1, i = ((x * EY + y) << lq) + q;
+    const float2 e = U[o * items + i], d = U[(o ^ 1) * items + i];
+    return make_float4(e.x, d.x, e.y, d.y);
+  };
+  const float mean = load_mean(f);
+  float4 F[T::ITEMS];
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+  for (int k = 0; k < T::ITEMS; ++k) {
+    const int i = tid + k * T::THREADS;
+    if (i >= items) break;
+    const int q = i & (Q - 1), row = i >> lq, x = row / EY, y = row - x * EY;
+    const float4 v = __ldg(reinterpret_cast<const float4*>(f.p + cell(x, y, q)));
+    F[k] = make_float4(f.s * (v.x - mean), f.s * (v.y - mean), f.s * (v.z - mean), f.s * (v.w - mean));
+    if (PRE)
+      put(x, y, q, uin ? *reinterpret_cast<const float4*>(uin + box + cell(x, y, q)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f));
+  }
+  if (!PRE) {
+    const int lc = log2n - 1, mc = (1 << lc) - 1;
+    const float* ucb = uc + ((int64_t)blockIdx.z << (3 * lc));
+    for (int i = tid; i < (EX / 2) * (EY / 2) << lq; i += T::THREADS) {
+      const int q = i & (Q - 1), blk = i >> lq, bx = blk / (EY / 2), by = blk - bx * (EY / 2);
+      prolong_pair(ucb, nullptr, ((x0 >> 1) + bx) & mc, ((y0 >> 1) + by) & mc, 2 * q, lc, [&](int ax, int ay, float4 e) {
+        const int x = 2 * bx + ax, y = 2 * by + ay;
+        const float4 w = *reinterpret_cast<const float4*>(uin + box + cell(x, y, q));
+        put(x, y, q, make_float4(w.x + e.x, w.y + e.y, w.z + e.z, w.w + e.w));
+      });
+    }
+  }
+  for (int p = 0; p < 2 * sweeps; ++p) {
+    __syncthreads();
+    const int colour = p & 1;
+    const PoissonUpdate upd = p < 2 ? u0 : u1;
+    float2* own = U + colour * items;
+    const float2* opp = U + (colour ^ 1) * items;
 #pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const int64_t base = idx3((I + a - 1) & mc, (J + b - 1) & mc, 0, lc);
-        const float2 mid = __ldg(reinterpret_cast<const float2*>(uc + base + K));
-        float v[4] = {__ldg(uc + base + ((K - 1) & mc)), mid.x, mid.y, __ldg(uc + base + ((K + 2) & mc))};
-        if (uc2) {
-          const float2 m2 = __ldg(reinterpret_cast<const float2*>(uc2 + base + K));
-          v[0] -= __ldg(uc2 + base + ((K - 1) & mc));
-          v[1] -= m2.x;
-          v[2] -= m2.y;
-          v[3] -= __ldg(uc2 + base + ((K + 2) & mc));
+    for (int k = 0; k < T::ITEMS; ++k) {
+      const int i = tid + k * T::THREADS;
+      if (i >= items) break;
+      const int q = i & (Q - 1), row = i >> lq, x = row / EY, y = row - x * EY;
+      if (x <= p || x >= EX - 1 - p || y <= p || y >= EY - 1 - p) continue;
+      const bool odd = ((colour + x0 + x + y0 + y) & 1) != 0;   // cells 4 q + odd and 4 q + odd + 2
+      const float2 xp = opp[i + (EY << lq)], xm = opp[i - (EY << lq)], yp = opp[i + Q], ym = opp[i - Q], c = opp[i];
+      const float2 side = opp[i - q + ((odd ? q + 1 : q - 1) & (Q - 1))], o = own[i];
+      const float nb0[6] = {xp.x, xm.x, yp.x, ym.x, odd ? c.y : c.x, odd ? c.x : side.y};
+      const float nb1[6] = {xp.y, xm.y, yp.y, ym.y, odd ? side.x : c.y, odd ? c.y : c.x};
+      own[i] = make_float2(upd(o.x, nb0, odd ? F[k].y : F[k].x, p == 0, p < 2),
+                           upd(o.y, nb1, odd ? F[k].w : F[k].z, p == 0, p < 2));
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < TX * TY << lq; i += T::THREADS) {
+    const int q = i & (Q - 1), row = i >> lq, x = H + row / TY, y = H + row % TY;
+    *reinterpret_cast<float4*>(uout + box + cell(x, y, q)) = get(x, y, q);
+  }
+  if (PRE) {
+    const float inv_h2 = (float)n * (float)n;
+    for (int i = tid; i < (TX / 2) * (TY / 2) << lq; i += T::THREADS) {
+      const int q = i & (Q - 1), row = i >> lq, x = H + 2 * (row / (TY / 2)), y = H + 2 * (row % (TY / 2));
+      float4 core[2][2], xf[2][2], yf[2][2], fr[2][2];
+      float zl[2][2], zr[2][2];
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          core[a][b] = get(x + a, y + b, q);
+          zl[a][b] = get(x + a, y + b, (q - 1) & (Q - 1)).w;
+          zr[a][b] = get(x + a, y + b, (q + 1) & (Q - 1)).x;
+          xf[a][b] = get(a ? x + 2 : x - 1, y + b, q);
+          yf[a][b] = get(x + a, b ? y + 2 : y - 1, q);
+          fr[a][b] = __ldg(reinterpret_cast<const float4*>(f.p + cell(x + a, y + b, q)));
         }
-#pragma unroll
-        for (int z = 0; z < 4; ++z) c[a][b][z] = v[z];
-      }
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-      const int jn = b ? 2 : 0;
-      // z then y contractions: vy[x][q] for the fine z offsets q = 0..3 (coarse
-      // cell q / 2 at column q / 2 + 1, child q & 1)
-      float vy[3][4];
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int kc = (q >> 1) + 1, kn = (q & 1) ? kc + 1 : kc - 1;
-          const float vz0 = fmaf(0.25f, c[a][1][kn], fmaf(0.75f, c[a][1][kc], 0.0f));
-          const float vz1 = fmaf(0.25f, c[a][jn][kn], fmaf(0.75f, c[a][jn][kc], 0.0f));
-          vy[a][q] = fmaf(0.25f, vz1, fmaf(0.75f, vz0, 0.0f));
-        }
-#pragma unroll
-      for (int ax = 0; ax < 2; ++ax) {
-        const int in = ax ? 2 : 0;
-        float4* dst = reinterpret_cast<float4*>(u + idx3(2 * I + ax, 2 * J + b, 2 * K, log2n));
-        float4 w = *dst;
-        w.x += fmaf(0.25f, vy[in][0], fmaf(0.75f, vy[1][0], 0.0f));
-        w.y += fmaf(0.25f, vy[in][1], fmaf(0.75f, vy[1][1], 0.0f));
-        w.z += fmaf(0.25f, vy[in][2], fmaf(0.75f, vy[1][2], 0.0f));
-        w.w += fmaf(0.25f, vy[in][3], fmaf(0.75f, vy[1][3], 0.0f));
-        *dst = w;
-      }
+      const int lc = log2n - 1;
+      const int64_t at = ((int64_t)blockIdx.z << (3 * lc)) + idx3(((x0 + x) & m) >> 1, ((y0 + y) & m) >> 1, 2 * q, lc);
+      *reinterpret_cast<float2*>(fc + at) = restrict_pair<COMP>(core, xf, yf, fr, zl, zr, f.s, mean, inv_h2);
     }
   }
 }
@@ -676,6 +822,35 @@ pm_status smooth(MG& g, int l, int count, const float* w, bool zero, float scale
   return PM_OK;
 }
 
+// One side of the V-cycle on a small level (k_rb_tile); zero: from zeros.
+template <bool PRE>
+pm_status tile_side(MG& g, int l, int count, const float* w, bool zero, float scale, const float* sbox) {
+  const int n = g.n0 >> l, log2n = ilog2(n);
+  const float h2 = 1.0f / ((float)n * (float)n);
+  const double N = (double)n * n * n;
+  const PoissonUpdate u0{h2, w[0], scale, sbox}, u1{h2, count > 1 ? w[1] : 1.0f, 1.0f, nullptr};
+  float* out = zero ? g.u[l] : g.alt[l];
+  const float* in = zero ? nullptr : g.u[l];
+  const float* uc = PRE ? nullptr : g.u[l + 1];
+  float* fc = PRE ? const_cast<float*>(g.f[l + 1].p) : nullptr;
+  const bool large = (n / 4) * (n / 4) * (int64_t)g.B > 152;
+#define PM_TILE(TX, TY, COMP)                                                                                     \
+  PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (zero ? 8.0 : 12.0) * N * g.B, (k_rb_tile<TX, TY, PRE, PRE && COMP>), \
+            g.grid((unsigned)((n / TX) * (n / TY))), (TileGeom<TX, TY, PRE>::THREADS), (TileGeom<TX, TY, PRE>::smem), \
+            g.s, in, out, g.f[l], uc, fc, log2n, count, u0, u1)
+  if (l == 0 && PRE) {
+    if (large) PM_TILE(8, 8, true); else PM_TILE(4, 4, true);
+  } else {
+    if (large) PM_TILE(8, 8, false); else PM_TILE(4, 4, false);
+  }
+#undef PM_TILE
+  if (!zero) {
+    g.alt[l] = g.u[l];
+    g.u[l] = out;
+  }
+  return PM_OK;
+}
+
 pm_status v_cycle(MG& g, int l, bool zero_guess) {
   const int n = g.n0 >> l, log2n = ilog2(n);
   const mg_params& p = *g.p;
@@ -698,6 +873,14 @@ pm_status v_cycle(MG& g, int l, bool zero_guess) {
     return PM_OK;
   }
   float w[64];
+  if (p.smoother != 1 && n <= kTileN && p.npre >= 1 && p.npre <= 2 && p.npost >= 1 && p.npost <= 2 && g.alt[l] &&
+      march_aligned(g.u[l], g.alt[l], g.f[l].p)) {
+    for (int si = 0; si < p.npre; ++si) w[si] = si == 0 ? 1.0f : p.omega;
+    PM_TRY(tile_side<true>(g, l, p.npre, w, zero_guess, scaled ? g.gscale : 1.0f, sbox));
+    PM_TRY(v_cycle(g, l + 1, true));
+    for (int si = 0; si < p.npost; ++si) w[si] = si == p.npost - 1 ? 1.0f : p.omega;
+    return tile_side<false>(g, l, p.npost, w, false, 1.0f, nullptr);
+  }
   if (p.npre == 0) {
     const int64_t N = (int64_t)n * n * n;
     if (zero_guess) PM_TRY(cuda_status(cudaMemsetAsync(g.u[l], 0, N * g.B * sizeof(float), g.s)));

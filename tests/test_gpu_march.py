@@ -97,3 +97,16 @@ def test_residual_norm_in_wide_loads(pm, n, coarsest):
     assert st["cycles"] == 1 and st["norm_f"] == pytest.approx(np.linalg.norm(f), rel=1e-6)
     # the residual is exact to a rounding of each cell's (and of the source less its float32 mean)
     assert st["res"] == pytest.approx(r, abs=2e-7 * st["norm_f"])
+
+
+@pytest.mark.parametrize("n,B,npre,npost,coarsest", [(8, 1, 2, 2, 4), (16, 1, 1, 2, 4), (32, 1, 2, 2, 16),
+                                                     (32, 2, 2, 1, 16), (32, 3, 2, 2, 8), (64, 5, 1, 1, 4)])
+def test_small_levels_in_tiles_bitwise_equal_the_colour_passes(pm, n, B, npre, npost, coarsest):
+    """Levels of up to 32^3 (tiles of 4 x 4 rows, of 8 x 8 in larger batches)
+    against colour passes and transfers of their own."""
+    f = np.stack([inputs.random_field(n, 60 + b) for b in range(B)]).astype(np.float32)
+    f = torch.from_numpy(f).cuda()
+    kw = dict(fixed_cycles=2, npre=npre, npost=npost, coarsest=coarsest, first_guess=pm.MG_GUESS_JACOBI)
+    solve = (lambda s: pm.mg_solve(f[0], smoother=s, **kw)[0]) if B == 1 else (
+        lambda s: pm.mg_solve_batch(f, smoother=s, **kw))
+    assert torch.equal(solve(2), solve(1))
