@@ -391,8 +391,8 @@ __device__ __forceinline__ void prolong_pair(const float* __restrict__ uc, const
 // and two scalars per coarse row) and corrects their 16 children (runs of
 // four along z as float4).  Per child the interpolation runs z, then y, then
 // x, parent (weight 3/4) before neighbour (1/4), in fused multiply-adds.
-__global__ void k_prolong_correct(float* __restrict__ u, const float* __restrict__ uc,
-                                  const float* __restrict__ uc2, int log2n) {
+__global__ void __launch_bounds__(256, 5) k_prolong_correct(float* __restrict__ u, const float* __restrict__ uc,
+                                                            const float* __restrict__ uc2, int log2n) {
   pdl_entry();
   const int lc = log2n - 1, mc = (1 << lc) - 1;
   const int64_t total = (int64_t)1 << (3 * lc);

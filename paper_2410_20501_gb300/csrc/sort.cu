@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_sums(uint32_t* __restrict__ sum
 // SUMS: sums holds the chunks' totals and not their prefix, and each block adds up
 // those before its own (a launch less: see scan_u32).
 template <bool SUMS>
-__global__ void __launch_bounds__(SCAN_T) k_scan_apply(uint32_t* __restrict__ a, int64_t len,
+__global__ void __launch_bounds__(SCAN_T, 2) k_scan_apply(uint32_t* __restrict__ a, int64_t len,
                                                        const uint32_t* __restrict__ sums) {
   pdl_entry();
   __shared__ uint32_t wt[32];
