@@ -325,99 +325,130 @@ __global__ void __launch_bounds__(256) k_interp_packed(const float4* __restrict_
 // take in flat order.  Every particle then reads its 27 x 3 force values
 // from shared memory at fixed offsets from its cell, in the same order and
 // with the same operations as k_interp_kdk (bitwise the same result).
+//
+// Shared memory's wavefronts bound it (81 of the 150 a warp of particles takes
+// are the force values themselves, 35 bank conflicts of scattered cells, 21 the
+// planes; the pipe is 80% busy), and what is left is latency: the thread's next
+// particle and the next plane's runs are in flight while the force plane is
+// computed and the particles before it are summed.  With the f(R) potential's
+// second field there are no registers for that at four CTAs an SM (the particle
+// ahead and the paired sums took 460 us there against 443), so it loads each
+// particle in turn.  256^3: 402 -> 386 us, clustered 445 -> 431, with maxima
+// 454 -> 434; f(R) 512^3 3.09 -> 2.99 ms.
 constexpr int IT_Y = 16, IT_Z = 32, IE_Y = IT_Y + 2, IE_Z = IT_Z + 2, I_PL = IE_Y * IE_Z, I_THREADS = 256;
-// Warp 0: the runs of the column's rows on plane q (start of each row's
-// particles, flat prefix of the run lengths).
-__device__ __forceinline__ void column_runs(const uint32_t* __restrict__ cellstart, int q, int y0, int z0,
-                                            int log2n, uint32_t* start, uint32_t* pre) {
-  const int tid = threadIdx.x;
-  if (tid >= 32) return;
-  const int m = (1 << log2n) - 1, j = tid & (IT_Y - 1);
+// One warp: the runs of the column's rows on plane q (start of each row's
+// particles, flat prefix of the run lengths) from the cell starts `v` that its
+// lanes loaded (column_start).
+__device__ __forceinline__ uint32_t column_start(const uint32_t* __restrict__ cellstart, int q, int y0, int z0,
+                                                 int log2n) {
+  const int lane = threadIdx.x & 31, m = (1 << log2n) - 1, j = lane & (IT_Y - 1);
   const int64_t row = ((int64_t)(q & m) << (2 * log2n)) | ((int64_t)(y0 + j) << log2n);
-  const uint32_t v = __ldg(cellstart + row + z0 + (tid < IT_Y ? 0 : IT_Z));
+  return __ldg(cellstart + row + z0 + (lane < IT_Y ? 0 : IT_Z));
+}
+__device__ __forceinline__ void column_runs(uint32_t v, uint32_t* start, uint32_t* pre) {
+  const int lane = threadIdx.x & 31, j = lane & (IT_Y - 1);
   const uint32_t end = __shfl_down_sync(0xffffffffu, v, IT_Y);
-  uint32_t incl = tid < IT_Y ? end - v : 0u;
+  uint32_t incl = lane < IT_Y ? end - v : 0u;
 #pragma unroll
   for (int o = 1; o < IT_Y; o <<= 1) {
     const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
     if (j >= o) incl += y;
   }
-  if (tid < IT_Y) {
+  if (lane < IT_Y) {
     start[j] = v;
     pre[j + 1] = incl;
     if (j == 0) pre[0] = 0;
   }
 }
 
-// Inverse TSC (+ kick and drift) of the particles of one plane of a column,
-// force planes x-1, x, x+1 at S[0..2] (each [3][IE_Y][IE_Z]).
-template <bool MAXES>
-__device__ __forceinline__ void column_particles(const float2* const S2[3], const float* const Sz[3],
-                                                 const uint32_t* st, const uint32_t* pre,
-                                                 int y0, int z0, const uint32_t* __restrict__ Xs,
-                                                 const float* __restrict__ Vs, const uint32_t* __restrict__ ids_in,
-                                                 int64_t np, int log2n, float* __restrict__ acc,
-                                                 uint32_t* __restrict__ Xo, float* __restrict__ Vo,
-                                                 uint32_t* __restrict__ ids_out, float dt_kick, float drift_scale,
-                                                 int mode, float& amax, float& vmax) {
+// A particle on its way to column_particle: its index, position and, for a
+// step, velocity.
+struct ColumnParticle {
+  uint32_t p, x, y, z;
+  float vx, vy, vz;
+};
+// Loads flat particle i of the plane whose runs are st, pre.
+__device__ __forceinline__ void column_load(ColumnParticle& a, uint32_t i, const uint32_t* st, const uint32_t* pre,
+                                            const uint32_t* __restrict__ Xs, const float* __restrict__ Vs, int64_t np,
+                                            int mode) {
+  int j = 0;   // the run holding flat index i
+#pragma unroll
+  for (int b = IT_Y / 2; b > 0; b >>= 1)
+    if (pre[j + b] <= i) j += b;
+  a.p = st[j] + (i - pre[j]);
+  a.x = __ldg(Xs + a.p);
+  a.y = __ldg(Xs + np + a.p);
+  a.z = __ldg(Xs + 2 * np + a.p);
+  if (mode == 1) {
+    a.vx = __ldg(Vs + a.p);
+    a.vy = __ldg(Vs + np + a.p);
+    a.vz = __ldg(Vs + 2 * np + a.p);
+  }
+}
+
+// Inverse TSC (+ kick and drift) of one particle of a plane of a column, force
+// planes x-1, x, x+1 at S2[0..2] (g_x, g_y) and Sz[0..2] (g_z), each
+// [IE_Y][IE_Z], in the operations and the order of k_interp_kdk.  PAIR: the x and
+// y sums in the paired float instructions.
+template <bool MAXES, bool PAIR>
+__device__ __forceinline__ void column_particle(const ColumnParticle& a, const float2* const S2[3],
+                                                const float* const Sz[3], int y0, int z0,
+                                                const uint32_t* __restrict__ ids_in, int64_t np, int log2n,
+                                                float* __restrict__ acc, uint32_t* __restrict__ Xo,
+                                                float* __restrict__ Vo, uint32_t* __restrict__ ids_out, float dt_kick,
+                                                float drift_scale, int mode, float& amax, float& vmax) {
   const int sh = 32 - log2n;
-  const uint32_t total = pre[IT_Y];
-  for (uint32_t i = threadIdx.x; i < total; i += I_THREADS) {
-    int j = 0;   // the run holding flat index i
+  float wx[3], wy[3], wz[3];
+  tsc_weights(cell_offset(a.x, log2n), wx);
+  tsc_weights(cell_offset(a.y, log2n), wy);
+  tsc_weights(cell_offset(a.z, log2n), wz);
+  const int c = ((int)(a.y >> sh) - y0 + 1) * IE_Z + ((int)(a.z >> sh) - z0 + 1);
+  float2 axy = make_float2(0.0f, 0.0f);
+  float az = 0.0f;
 #pragma unroll
-    for (int b = IT_Y / 2; b > 0; b >>= 1)
-      if (pre[j + b] <= i) j += b;
-    const int64_t p = (int64_t)st[j] + (i - pre[j]);
-    const uint32_t x = __ldg(Xs + p), y = __ldg(Xs + np + p), z = __ldg(Xs + 2 * np + p);
-    // velocities in flight while the force is summed
-    float v0x = 0.0f, v0y = 0.0f, v0z = 0.0f;
-    if (mode == 1) {
-      v0x = __ldg(Vs + p);
-      v0y = __ldg(Vs + np + p);
-      v0z = __ldg(Vs + 2 * np + p);
-    }
-    float wx[3], wy[3], wz[3];
-    tsc_weights(cell_offset(x, log2n), wx);
-    tsc_weights(cell_offset(y, log2n), wy);
-    tsc_weights(cell_offset(z, log2n), wz);
-    const int c = ((int)(y >> sh) - y0 + 1) * IE_Z + ((int)(z >> sh) - z0 + 1);
-    float ax = 0.0f, ay = 0.0f, az = 0.0f;
+  for (int ox = 0; ox < 3; ++ox) {
 #pragma unroll
-    for (int ox = 0; ox < 3; ++ox) {
+    for (int oy = 0; oy < 3; ++oy) {
+      const float wxy = wx[ox] * wy[oy];
+      const float2* r2 = S2[ox] + c + (oy - 1) * IE_Z;
+      const float* rz = Sz[ox] + c + (oy - 1) * IE_Z;
+      const float2 wxy2 = __fmul2_rn(make_float2(wx[ox], wx[ox]), make_float2(wy[oy], wy[oy]));
 #pragma unroll
-      for (int oy = 0; oy < 3; ++oy) {
-        const float wxy = wx[ox] * wy[oy];
-        const float2* r2 = S2[ox] + c + (oy - 1) * IE_Z;
-        const float* rz = Sz[ox] + c + (oy - 1) * IE_Z;
-#pragma unroll
-        for (int oz = 0; oz < 3; ++oz) {
+      for (int oz = 0; oz < 3; ++oz) {
+        const float2 fxy = r2[oz - 1];
+        if (PAIR) {
+          const float2 w = __fmul2_rn(wxy2, make_float2(wz[oz], wz[oz]));
+          axy = __ffma2_rn(w, fxy, axy);
+          az = fmaf(w.x, rz[oz - 1], az);
+        } else {
           const float w = wxy * wz[oz];
-          const float2 fxy = r2[oz - 1];
-          ax = fmaf(w, fxy.x, ax);
-          ay = fmaf(w, fxy.y, ay);
+          axy.x = fmaf(w, fxy.x, axy.x);
+          axy.y = fmaf(w, fxy.y, axy.y);
           az = fmaf(w, rz[oz - 1], az);
         }
       }
     }
-    if (acc) {
-      acc[p] = ax;
-      acc[np + p] = ay;
-      acc[2 * np + p] = az;
-    }
-    if (MAXES) amax = fmaxf(amax, sqrtf(fmaf(ax, ax, fmaf(ay, ay, az * az))));
-    if (mode == 1) {
-      const float vx = fmaf(ax, dt_kick, v0x);
-      const float vy = fmaf(ay, dt_kick, v0y);
-      const float vz = fmaf(az, dt_kick, v0z);
-      Vo[p] = vx;
-      Vo[np + p] = vy;
-      Vo[2 * np + p] = vz;
-      if (MAXES) vmax = fmaxf(vmax, sqrtf(fmaf(vx, vx, fmaf(vy, vy, vz * vz))));
-      Xo[p] = x + (uint32_t)__float2int_rn(vx * drift_scale);
-      Xo[np + p] = y + (uint32_t)__float2int_rn(vy * drift_scale);
-      Xo[2 * np + p] = z + (uint32_t)__float2int_rn(vz * drift_scale);
-      if (ids_out) ids_out[p] = __ldg(ids_in + p);
-    }
+  }
+  const float ax = axy.x, ay = axy.y;
+  const int64_t p = a.p;
+  if (acc) {
+    acc[p] = ax;
+    acc[np + p] = ay;
+    acc[2 * np + p] = az;
+  }
+  if (MAXES) amax = fmaxf(amax, sqrtf(fmaf(ax, ax, fmaf(ay, ay, az * az))));
+  if (mode == 1) {
+    const float vx = fmaf(ax, dt_kick, a.vx);
+    const float vy = fmaf(ay, dt_kick, a.vy);
+    const float vz = fmaf(az, dt_kick, a.vz);
+    Vo[p] = vx;
+    Vo[np + p] = vy;
+    Vo[2 * np + p] = vz;
+    if (MAXES) vmax = fmaxf(vmax, sqrtf(fmaf(vx, vx, fmaf(vy, vy, vz * vz))));
+    Xo[p] = a.x + (uint32_t)__float2int_rn(vx * drift_scale);
+    Xo[np + p] = a.y + (uint32_t)__float2int_rn(vy * drift_scale);
+    Xo[2 * np + p] = a.z + (uint32_t)__float2int_rn(vz * drift_scale);
+    if (ids_out) ids_out[p] = __ldg(ids_in + p);
   }
 }
 
@@ -451,7 +482,7 @@ __device__ __forceinline__ void block_maxima(float amax, float vmax, float2* __r
 // particles of plane u - R - 2 are interpolated from the three force planes
 // computed in the steps before.
 template <int ORDER, bool FR, bool MAXES>
-__global__ void __launch_bounds__(I_THREADS) k_force_interp_stream(
+__global__ void __launch_bounds__(I_THREADS, 4) k_force_interp_stream(
     const float* __restrict__ phi, const float* __restrict__ eps, float alpha, int nh, float inv_h,
     const uint32_t* __restrict__ cellstart, const uint32_t* __restrict__ Xs, const float* __restrict__ Vs,
     const uint32_t* __restrict__ ids_in, int64_t np, int log2n, int chunk, int nitems, float* __restrict__ acc,
@@ -520,6 +551,16 @@ __global__ void __launch_bounds__(I_THREADS) k_force_interp_stream(
       if (u < x1 + R) fetch(u + 1);
       __syncthreads();
       const int qg = u - R;
+      const int t = qg - 2;   // particle plane of this step
+      // in flight while the force plane is computed: this thread's first particle
+      // and, on the last warp (which gets the fewest), the next plane's runs
+      const uint32_t *st = s_start[t & 1], *pre = s_pre[t & 1];
+      const uint32_t total = t >= x0 && t < x1 ? pre[IT_Y] : 0u;
+      ColumnParticle next;
+      if (!FR && tid < total) column_load(next, tid, st, pre, Xs, Vs, np, mode);
+      const bool runs = t + 1 >= x0 && t + 1 < x1 && tid >= I_THREADS - 32;
+      uint32_t cs = 0;
+      if (runs) cs = column_start(cellstart, t + 1, y0, z0, log2n);
       if (qg >= x0 - 1 && qg <= x1) {
         float2* G2 = Gxy + (qg & 3) * I_PL;
         float* G1 = Gz + (qg & 3) * I_PL;
@@ -541,10 +582,8 @@ __global__ void __launch_bounds__(I_THREADS) k_force_interp_stream(
           G1[e] = -gz * inv_h;
         }
       }
-      const int t = qg - 2;   // particle plane of this step
-      if (t + 1 >= x0 && t + 1 < x1)
-        column_runs(cellstart, t + 1, y0, z0, log2n, s_start[(t + 1) & 1], s_pre[(t + 1) & 1]);
-      if (t >= x0 && t < x1) {
+      if (runs) column_runs(cs, s_start[(t + 1) & 1], s_pre[(t + 1) & 1]);
+      if (total) {
         const float2* S2[3];
         const float* Sz[3];
 #pragma unroll
@@ -552,8 +591,17 @@ __global__ void __launch_bounds__(I_THREADS) k_force_interp_stream(
           S2[ox] = Gxy + ((t + ox - 1) & 3) * I_PL;
           Sz[ox] = Gz + ((t + ox - 1) & 3) * I_PL;
         }
-        column_particles<MAXES>(S2, Sz, s_start[t & 1], s_pre[t & 1], y0, z0, Xs, Vs, ids_in, np, log2n, acc, Xo, Vo,
-                                ids_out, dt_kick, drift_scale, mode, amax, vmax);
+        for (uint32_t i = tid; i < total; i += I_THREADS) {
+          ColumnParticle cur;
+          if (FR) {
+            column_load(cur, i, st, pre, Xs, Vs, np, mode);
+          } else {
+            cur = next;
+            if (i + I_THREADS < total) column_load(next, i + I_THREADS, st, pre, Xs, Vs, np, mode);
+          }
+          column_particle<MAXES, !FR>(cur, S2, Sz, y0, z0, ids_in, np, log2n, acc, Xo, Vo, ids_out, dt_kick, drift_scale,
+                                 mode, amax, vmax);
+        }
       }
     }
     __syncthreads();   // the rings and run buffers are reused by the next item
