@@ -101,9 +101,19 @@ __global__ void __launch_bounds__(T * T * T) k_deposit(const uint32_t* __restric
 // planes x - 1, x and x + 1, after which plane x - 1 has everything from this
 // column and its 9 sums go to shared memory.  Destination warps (two cells
 // per thread, rows ty and ty + DTY / 2) add, in a fixed order, the 9 column
-// sums that point at each of their cells and write the density.  The sums
-// are double-buffered: sources emit plane x - 1 while the destinations add
-// plane x - 2 (one barrier per plane), on different warps.
+// sums that point at each of their cells and write the density.
+//
+// Its instructions bound it: a source warp weighs as many particles a plane as the
+// fullest of its 32 cells holds (3.6 on average at one a cell), and no plane's
+// fullest cell should hold up the other warps as well.  So there is no barrier
+// over the CTA: source and destination warps meet on two barriers per buffer of
+// column sums (full: every source warp has written; empty: the destinations have
+// read), where filling one and freeing one do not wait, and a source warp runs up
+// to kColBufs planes ahead of the slowest.  One barrier a plane -> four buffers:
+// 256^3 alone 269 -> 266 us, clustered 501 -> 469, 10^7 on 256^3 437 -> 413, with
+// values on 128^3 75 -> 68.  (Two columns a thread in
+// the paired float instructions halve the walks, but 128 registers leave 16 warps
+// an SM: 278 us against 277, clustered 668 against 570 with the moments' launch.)
 //
 // Particle loads: a source thread copies the first KP particles of its cell
 // on the next plane into its own shared-memory slots with asynchronous copies
@@ -126,11 +136,24 @@ constexpr int DSRC_T = (DPL + 31) / 32 * 32;       // source warps
 constexpr int DDST_T = DNT / 2;                    // destination threads (two cells each)
 constexpr int DTHREADS = DSRC_T + DDST_T;
 static_assert(DDST_T % 32 == 0 && DTY % 2 == 0, "whole destination warps, two rows per thread");
+constexpr int kSumPlanes = 16;                    // planes of a partial sum of the density in a batch
+constexpr int kColBufs = 4;                        // column-sum buffers (a power of two)
 // Staged particles per cell and words per particle (x, y, z [, value]).
 template <bool VALS> struct DepositStage {
   static constexpr int KP = kWalkRun, NC = VALS ? 4 : 3;
-  static constexpr size_t smem = sizeof(float) * (2 * 9 * DPL + 2 * KP * NC * DPL);
+  static constexpr size_t smem = sizeof(float) * (kColBufs * 9 * DPL + 2 * KP * NC * DPL);
 };
+
+// Named barriers between the source warps and the destination warps of a CTA
+// (DTHREADS threads on each): `arrive` does not wait.
+__device__ __forceinline__ void barrier_sync(int id) {
+  __syncwarp();
+  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "n"(DTHREADS) : "memory");
+}
+__device__ __forceinline__ void barrier_arrive(int id) {
+  __syncwarp();
+  asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "n"(DTHREADS) : "memory");
+}
 
 __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
@@ -139,26 +162,29 @@ __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
+// Partial sums of the density: one per destination warp and chunk, or with
+// sum_planes < chunk one per warp and run of sum_planes planes (then they do not
+// depend on the chunk, which a batch's size may change).
 template <bool VALS>
 __global__ void __launch_bounds__(DTHREADS, 2) k_deposit_stream(const uint32_t* __restrict__ Xs, int64_t np,
                                                                 const uint32_t* __restrict__ cellstart, int log2n,
                                                                 int chunk, int nitems, const float* __restrict__ vals,
                                                                 float scale, float* __restrict__ rho,
-                                                                double* __restrict__ partial,
+                                                                double* __restrict__ partial, int sum_planes,
                                                                 const float* __restrict__ crowd) {
   pdl_entry();
   using G = DepositStage<VALS>;
-  constexpr int KP = G::KP, NC = G::NC, PL = DPL;
+  constexpr int KP = G::KP, NC = G::NC, PL = DPL, DW = DDST_T / 32;
   extern __shared__ float sm[];
   {   // the box of a batched launch: its cell starts (global particle indices), density, partials
     const int64_t off = (int64_t)blockIdx.z << (3 * log2n);
     cellstart += off;
     rho += off;
-    partial += (int64_t)blockIdx.z * nitems;
+    partial += (int64_t)blockIdx.z * nitems * (chunk / sum_planes) * DW;
   }
-  float* Col = sm;                                                 // [2][9][PL] column sums
-  uint32_t* Slot = reinterpret_cast<uint32_t*>(sm + 2 * 9 * PL);   // [2][KP][NC][PL]
-  __shared__ double wsum[DTHREADS / 32];
+  float* Col = sm;                                                        // [kColBufs][9][PL] column sums
+  uint32_t* Slot = reinterpret_cast<uint32_t*>(sm + kColBufs * 9 * PL);   // [2][KP][NC][PL]
+  constexpr int FULL = 1, EMPTY = 1 + kColBufs;                           // barriers of a buffer
   const int n = 1 << log2n, mask = n - 1;
   const int tiles_z = n / DTZ, tiles = (n / DTY) * tiles_z;
   const int tid = threadIdx.x;
@@ -196,15 +222,12 @@ __global__ void __launch_bounds__(DTHREADS, 2) k_deposit_stream(const uint32_t* 
       stage((x0 - 1) & 1, b0, e0);
       cp_async_commit();
     }
-    // one plane step: source plane xs adds to the column sums of destination
-    // planes xs - 1 (A), xs (B) and xs + 1 (C, started here), emits A; the
-    // destinations add the column sums of plane xs - 2 emitted in the step
-    // before.  The caller rotates the roles of the three register arrays.
+    // one plane step of a source warp: source plane xs adds to the column sums of
+    // destination planes xs - 1 (A), xs (B) and xs + 1 (C, started here) and emits
+    // A.  The caller rotates the roles of the three register arrays.
     auto step = [&](int xs, float (&A)[9], float (&B)[9], float (&C)[9]) {
-      float* ColW = Col + (xs & 1) * 9 * PL;
-      const float* ColR = Col + ((xs - 1) & 1) * 9 * PL;
       uint32_t b2 = 0, e2 = 0;
-      if (src && xs <= x1) {
+      if (src) {
         if (xs + 1 <= x1) stage((xs + 1) & 1, b1, e1);   // the next plane's particles, in flight
         cp_async_commit();
         if (xs + 2 <= x1) {
@@ -237,11 +260,19 @@ __global__ void __launch_bounds__(DTHREADS, 2) k_deposit_stream(const uint32_t* 
         const uint32_t cnt = e0 - b0;
         if (crowd && cnt > kWalkRun) {   // its moments were summed already
           const float* mo = crowd + kMomStride * (int64_t)b0;
+          float s[28];
+#pragma unroll
+          for (int o = 0; o < 26; o += 2) {
+            const float2 v = __ldg(reinterpret_cast<const float2*>(mo + o));
+            s[o] = v.x;
+            s[o + 1] = v.y;
+          }
+          s[26] = __ldg(mo + 26);
 #pragma unroll
           for (int o = 0; o < 9; ++o) {
-            A[o] += __ldg(mo + o);
-            B[o] += __ldg(mo + 9 + o);
-            C[o] += __ldg(mo + 18 + o);
+            A[o] += s[o];
+            B[o] += s[9 + o];
+            C[o] += s[18 + o];
           }
         } else {
 #pragma unroll
@@ -263,12 +294,38 @@ __global__ void __launch_bounds__(DTHREADS, 2) k_deposit_stream(const uint32_t* 
             }
           }
         }
-        // destination plane xs - 1 has all of this column's contributions
-#pragma unroll
-        for (int o = 0; o < 9; ++o) ColW[o * PL + tid] = A[o];
       }
-      const int done = xs - 2;   // the destination plane whose column sums were emitted in the step before
-      if (dst && done >= x0 && done < x1) {
+      // destination plane xs - 1 has all of this column's contributions
+      const int done = xs - 1, buf = done & (kColBufs - 1);
+      if (done >= x0) {
+        if (done >= x0 + kColBufs) barrier_sync(EMPTY + buf);
+        if (src) {
+#pragma unroll
+          for (int o = 0; o < 9; ++o) Col[(buf * 9 + o) * PL + tid] = A[o];
+        }
+        barrier_arrive(FULL + buf);
+      }
+      b0 = b1; e0 = e1; b1 = b2; e1 = e2;
+    };
+    if (!dst) {
+      // column sums of destination planes xs - 1 and xs (the first source plane
+      // reaches planes x0 - 2 .. x0; the first two are outside the chunk)
+      float R0[9], R1[9], R2[9];
+#pragma unroll
+      for (int o = 0; o < 9; ++o) {
+        R0[o] = 0.0f;
+        R1[o] = 0.0f;
+      }
+      for (int xs = x0 - 1; xs <= x1; xs += 3) {
+        step(xs, R0, R1, R2);
+        if (xs + 1 <= x1) step(xs + 1, R1, R2, R0);
+        if (xs + 2 <= x1) step(xs + 2, R2, R0, R1);
+      }
+    } else {
+      for (int d = x0; d < x1; ++d) {
+        const int buf = d & (kColBufs - 1);
+        const float* ColR = Col + buf * 9 * PL;
+        barrier_sync(FULL + buf);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int ry = ty + h * (DTY / 2);
@@ -278,35 +335,17 @@ __global__ void __launch_bounds__(DTHREADS, 2) k_deposit_stream(const uint32_t* 
 #pragma unroll
             for (int oz = 0; oz < 3; ++oz) a += ColR[(oy * 3 + oz) * PL + (ry + 2 - oy) * DEZ + (tz + 2 - oz)];
           const float r = a * scale;
-          rho[((((int64_t)done << log2n) | (y0 + ry)) << log2n) | (z0 + tz)] = r;
+          rho[((((int64_t)d << log2n) | (y0 + ry)) << log2n) | (z0 + tz)] = r;
           kahan_add(wsum_s, wsum_c, r);
         }
+        if (d + kColBufs < x1) barrier_arrive(EMPTY + buf);
+        if (((d + 1 - x0) & (sum_planes - 1)) == 0) {
+          const double ws = warp_sum_comp(wsum_s - wsum_c);
+          if ((dt & 31) == 0) partial[((int64_t)(d / sum_planes) * tiles + tile) * DW + (dt >> 5)] = ws;
+          wsum_s = wsum_c = 0.0f;
+        }
       }
-      __syncthreads();
-      b0 = b1; e0 = e1; b1 = b2; e1 = e2;
-    };
-    // column sums of destination planes xs - 1 and xs (the first source plane
-    // reaches planes x0 - 2 .. x0; the first two are outside the chunk)
-    float R0[9], R1[9], R2[9];
-#pragma unroll
-    for (int o = 0; o < 9; ++o) {
-      R0[o] = 0.0f;
-      R1[o] = 0.0f;
     }
-    for (int xs = x0 - 1; xs <= x1 + 1; xs += 3) {
-      step(xs, R0, R1, R2);
-      if (xs + 1 <= x1 + 1) step(xs + 1, R1, R2, R0);
-      if (xs + 2 <= x1 + 1) step(xs + 2, R2, R0, R1);
-    }
-    const double ws = warp_sum_comp(wsum_s - wsum_c);
-    if ((tid & 31) == 0) wsum[tid >> 5] = ws;
-    __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      for (int w = 0; w < DTHREADS / 32; ++w) t += wsum[w];
-      partial[item] = t;
-    }
-    __syncthreads();
   }
 }
 
@@ -480,11 +519,11 @@ __global__ void __launch_bounds__(CT, 4) k_list_moments(const uint32_t* __restri
 // 316 at 16, 363 at 8), fewer only where SMs would have no CTA at all (32^3 with
 // its other launches 45 us at 16, 35 at 2; 64^3 47 at 16, 39 at 4; 128^3 77 at 16,
 // 79 at 8).
-inline void deposit_stream_plan(int n, int B, int* chunk, int* nitems) {
+inline void deposit_stream_plan(int n, int B, int* chunk, int* nitems) {   // B = 0: not a batch
   const int tiles = (n / DTY) * (n / DTZ);
   int c = n;
-  while (c > 16 && (int64_t)tiles * (n / c) * B < 8 * 152) c >>= 1;
-  while (c > 2 && (int64_t)tiles * (n / c) * B < 152) c >>= 1;
+  while (c > kSumPlanes && (int64_t)tiles * (n / c) * (B ? B : 1) < 8 * 152) c >>= 1;
+  while (!B && c > 2 && (int64_t)tiles * (n / c) < 152) c >>= 1;
   *chunk = c;
   *nitems = tiles * (n / c);
 }
@@ -590,19 +629,20 @@ pm_status deposit_sorted_values(const uint32_t* Xs, int64_t np, const uint32_t* 
     PM_TRY(crowded_moments(Xs, np, cellstart, n, vals, cr, s));
     const float* crowd = cr.runs && np > 0 ? cr.moments : nullptr;
     int chunk, nitems;
-    deposit_stream_plan(n, 1, &chunk, &nitems);
+    deposit_stream_plan(n, 0, &chunk, &nitems);
     const unsigned grid = (unsigned)nitems;   // one item per CTA, two 512-thread CTAs per SM
     const double bytes = (vals ? 16.0 : 12.0) * np + 8.0 * n * n * (double)n + 4.0;
     if (vals) {
       PM_TRY(smem_attr(k_deposit_stream<true>, DepositStage<true>::smem));
       PM_LAUNCH(K_DEPOSIT, bytes, k_deposit_stream<true>, grid, DTHREADS, DepositStage<true>::smem, s, Xs, np,
-                cellstart, ilog2(n), chunk, nitems, vals, scale, rho, partials, crowd);
+                cellstart, ilog2(n), chunk, nitems, vals, scale, rho, partials, chunk, crowd);
     } else {
       PM_TRY(smem_attr(k_deposit_stream<false>, DepositStage<false>::smem));
       PM_LAUNCH(K_DEPOSIT, bytes, k_deposit_stream<false>, grid, DTHREADS, DepositStage<false>::smem, s, Xs, np,
-                cellstart, ilog2(n), chunk, nitems, vals, scale, rho, partials, crowd);
+                cellstart, ilog2(n), chunk, nitems, vals, scale, rho, partials, chunk, crowd);
     }
-    PM_LAUNCH(K_REDUCE, 8.0 * nitems, k_reduce_partials, 1, 1024, 0, s, partials, (int64_t)nitems, (int64_t)0, 1,
+    const int64_t nsums = (int64_t)nitems * (DDST_T / 32);
+    PM_LAUNCH(K_REDUCE, 8.0 * nsums, k_reduce_partials, 1, 1024, 0, s, partials, nsums, (int64_t)0, 1,
               1.0 / ((double)n * n * n), mean_out);
     return launch_status();
   }
@@ -617,15 +657,18 @@ pm_status deposit_sorted_batch(const uint32_t* Xs, int64_t np_box, int B, const 
   PM_TRY(smem_attr(k_deposit_stream<false>, DepositStage<false>::smem));
   int chunk, nitems;
   deposit_stream_plan(n, B, &chunk, &nitems);
+  // the mean of a box must not depend on the boxes it is batched with: partial
+  // sums over a fixed number of planes, of which every chunk here is a multiple
+  const int64_t nsums = (int64_t)nitems * (chunk / kSumPlanes) * (DDST_T / 32);
   const float scale = np_box > 0 ? (float)((double)n * n * n / (double)np_box) : 0.0f;
   // one item per CTA: B x nitems CTAs balance over the SMs (two resident each)
   const int gx = nitems;
   const int64_t np = np_box * B;
   PM_LAUNCH(K_DEPOSIT, 12.0 * np + 8.0 * n * n * (double)n * B + 4.0, k_deposit_stream<false>, dim3(gx, 1, B),
             DTHREADS, DepositStage<false>::smem, s, Xs, np, cellstart, ilog2(n), chunk, nitems, (const float*)nullptr, scale, rho,
-            partials, cr.runs && np > 0 ? (const float*)cr.moments : nullptr);
-  PM_LAUNCH(K_REDUCE, 8.0 * nitems * B, k_reduce_partials, B, 1024, 0, s, partials, (int64_t)nitems,
-            (int64_t)nitems, B, 1.0 / ((double)n * n * n), mean_out);
+            partials, kSumPlanes, cr.runs && np > 0 ? (const float*)cr.moments : nullptr);
+  PM_LAUNCH(K_REDUCE, 8.0 * nsums * B, k_reduce_partials, B, 1024, 0, s, partials, nsums, nsums, B,
+            1.0 / ((double)n * n * n), mean_out);
   return launch_status();
 }
 

@@ -117,3 +117,19 @@ def test_cell_starts_on_both_sides_of_the_scan_rule(pm, B):
     for b in (0, 63, B - 1):
         one = pm.positions_to_device(np.ascontiguousarray(X[:, b * np_box:(b + 1) * np_box]))
         assert torch.equal(rho[b], pm.deposit(one, n)), b
+
+
+def test_large_batch_is_bitwise_a_batch_of_one(pm):
+    """40 boxes of 64^3 march more planes a block than one box does: neither the
+    density nor its mean depends on that."""
+    w = inputs.ensemble_workload(n=64, B=1, boxsize=128.0, steps=2)
+    out = []
+    for B in (1, 40):
+        X, V = np.repeat(w["X"], B, axis=0), np.repeat(w["V"], B, axis=0)
+        ens = pm.Ensemble(X, V, 64, np.repeat(w["Om"], B), w["boxsize"], cold_cycles=4)
+        coef = ens.coefficients(w["a_steps"][:3])
+        for i in range(2):
+            ens.step(coef[i])
+        out.append((ens.positions(), ens.velocities()))
+    for b in (0, 17, 39):
+        assert np.array_equal(out[1][0][b], out[0][0][0]) and np.array_equal(out[1][1][b], out[0][1][0]), b
