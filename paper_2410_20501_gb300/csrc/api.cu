@@ -345,8 +345,10 @@ pm_status pm_deposit(const uint32_t* X, int64_t np, int n, float* rho, void* ws,
   PM_TRY(check_ws(w, ws, ws_bytes, n, np, PM_WS_SORT));
   cudaStream_t s = as_stream(stream);
   uint32_t* p;
-  PM_TRY(sort_cells(X, np, n, w, s, w.cellstart, &p));
-  PM_TRY(permute_particles(p, np, X, nullptr, nullptr, w.Xs, nullptr, nullptr, s));
+  Packed pk;
+  PM_TRY(pack_scattered(X, np, n, w, &pk, s));
+  PM_TRY(sort_cells(X, np, n, w, s, w.cellstart, &p, Batch{}, pk));
+  PM_TRY(permute_particles(p, np, X, nullptr, nullptr, w.Xs, nullptr, nullptr, s, pk));
   PM_TRY(deposit_sorted(w.Xs, np, w.cellstart, n, rho, w.partials, w.scalars, s, crowded(w)));
   return launch_status();
 }
@@ -694,9 +696,11 @@ pm_status pm_interp_adj(const float* g, const uint32_t* X, int64_t np, int n, co
   cudaStream_t s = as_stream(stream);
   const int64_t N = (int64_t)n * n * n;
   uint32_t* perm;
-  PM_TRY(sort_cells(X, np, n, w, s, w.cellstart, &perm));
+  Packed pk;
+  PM_TRY(pack_scattered(X, np, n, w, &pk, s));
+  PM_TRY(sort_cells(X, np, n, w, s, w.cellstart, &perm, Batch{}, pk));
   // sorted positions and sorted acc_bar (the three planes permuted like X)
-  PM_TRY(permute_particles(perm, np, X, acc_bar, nullptr, w.Xs, w.adj_abar, nullptr, s));
+  PM_TRY(permute_particles(perm, np, X, acc_bar, nullptr, w.Xs, w.adj_abar, nullptr, s, pk));
   for (int d = 0; d < 3; ++d)
     PM_TRY(deposit_sorted_values(w.Xs, np, w.cellstart, n, w.adj_abar + d * np, 1.0f, g_bar + d * N, w.partials,
                                  w.scalars + 12, s, crowded(w)));

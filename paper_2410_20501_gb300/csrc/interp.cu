@@ -191,10 +191,10 @@ __global__ void __launch_bounds__(256) k_interp_kdk(const float* __restrict__ g,
   }
 }
 
-// Whether the gather is worth packing the field for, from a sample of the
-// particles' order (one block): *flag = 1 if `gain` lookups saved per row of
-// cells that 32 neighbouring particles touch exceed `cost`.
-__global__ void __launch_bounds__(1024) k_interp_order(const uint32_t* __restrict__ Xs, int64_t np, int log2n,
+// Whether packing what scattered particles look up is worth it, from a sample of
+// their order (one block): *flag = 1 if `gain` lookups saved per row of cells that
+// 32 neighbouring particles touch exceed `cost`.
+__global__ void __launch_bounds__(1024) k_order_sample(const uint32_t* __restrict__ Xs, int64_t np, int log2n,
                                                        float gain, float cost, int* __restrict__ flag) {
   pdl_entry();
   __shared__ int total;
@@ -691,6 +691,12 @@ pm_status gradient_launch(const float* phi, const float* eps, float alpha, float
   return PM_EINVAL;
 }
 
+pm_status order_sample(const uint32_t* X, int64_t np, int n, float gain, float cost, int* flag, cudaStream_t s) {
+  if (np < 32) return PM_EINVAL;
+  PM_LAUNCH(K_INTERP, 0.0, k_order_sample, 1, 1024, 0, s, X, np, ilog2(n), gain, cost, flag);
+  return launch_status();
+}
+
 // The field is packed where that pays.  Per warp of particles the gather costs
 // 81 lookups for each row of cells the warp touches from the planes and 18 (and
 // some more for the wider cells) from the packed field; packing a cell costs
@@ -703,7 +709,7 @@ pm_status interp_packed_launch(const float* g, const uint32_t* X, int64_t np, in
   if (np < 32) return PM_EINVAL;
   const int64_t N = (int64_t)n * n * n;
   const float gain = 81.0f - 18.0f, cost = 108.0f + 43.0f * (float)N / (float)np;
-  PM_LAUNCH(K_INTERP, 0.0, k_interp_order, 1, 1024, 0, s, X, np, ilog2(n), gain, cost, flag);
+  PM_TRY(order_sample(X, np, n, gain, cost, flag, s));
   // counted as small, so that its launch overlaps the sample (most of it exits at once where the flag is 0)
   PM_LAUNCH(K_INTERP, 0.0, k_pack_force, grid_for(N / 4, 256, 152 * 8), 256, 0, s, g, packed, N, flag);
   PM_LAUNCH(K_INTERP, 12.0 * N + 24.0 * np, k_interp_packed, grid_for(np, 256), 256, 0, s, packed, g, X, np, ilog2(n),

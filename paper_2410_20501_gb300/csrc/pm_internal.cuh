@@ -155,6 +155,18 @@ int64_t sort_bigs_capacity(int64_t np);
 int64_t sort_smalls_capacity(int64_t np);
 int64_t reduce_partials_capacity(int n, int64_t np);
 
+// Positions as (x, y, z, 0) beside their planes, written by the sort's count if
+// *scattered; x = NULL: planes only.
+struct Packed {
+  uint4* x = nullptr;
+  int* scattered = nullptr;
+};
+// *flag = 1 if `gain` times the rows of cells that 32 neighbouring particles touch
+// (a sample's mean) exceeds `cost`; np >= 32.
+pm_status order_sample(const uint32_t* X, int64_t np, int n, float gain, float cost, int* flag, cudaStream_t s);
+// Where to pack the positions of particles in an unknown order (*pk unchanged: not at all).
+pm_status pack_scattered(const uint32_t* X, int64_t np, int n, const Workspace& w, Packed* pk, cudaStream_t s);
+
 // ------------------------------------------------------ stage launchers --
 // Stable sort by cell key: *perm_out (in the workspace) lists the particles
 // in cell order, ties in input order, and cellstart[c] .. cellstart[c+1]-1 are
@@ -162,10 +174,10 @@ int64_t reduce_partials_capacity(int n, int64_t np);
 // a batch the key is prefixed by the box (particle index / np_box), so the
 // order is by box, then cell, and ncells = B n^3.
 pm_status sort_cells(const uint32_t* X, int64_t np, int n, Workspace& w, cudaStream_t s, uint32_t* cellstart,
-                     uint32_t** perm_out, const Batch& bt = Batch{});
+                     uint32_t** perm_out, const Batch& bt = Batch{}, const Packed& pk = Packed{});
 pm_status permute_particles(const uint32_t* perm, int64_t np, const uint32_t* X, const float* V,
                             const uint32_t* id, uint32_t* Xs, float* Vs, uint32_t* ids,
-                            cudaStream_t s);
+                            cudaStream_t s, const Packed& pk = Packed{});
 // The cell lists of the last cell sort (smalls, meds, runs, bigs) and the
 // moment buffer (kMomStride floats per particle): the deposit sums the 27
 // moments of every cell of more than kWalkRun particles into it, at

@@ -46,25 +46,33 @@ struct ListHeads {
 // its cell's particles).  A thread takes CI particles, KT apart (coalesced),
 // with their loads and atomics all in flight together; a run of equal keys
 // in adjacent lanes takes one atomic (its head's) and ranks in lane order.
-template <bool BOX>
+//
+// PACK and *scattered: the positions also go to packed[i] (x, y, z, 0), for the
+// gather in cell order (k_permute).  The atomics on scattered cells bound this
+// kernel then, so the 16 bytes more a particle are nearly free, as long as what
+// streams through does not push the counters out of L2 (evict-first accesses: 155
+// us against 209 for 10^7 on 256^3, 144 without packing).
+template <bool BOX, bool PACK>
 __global__ void __launch_bounds__(KT) k_cell_count(const uint32_t* __restrict__ X, int64_t np, int log2n,
                                                    int64_t np_box, uint2* __restrict__ kr,
-                                                   uint32_t* __restrict__ cnt) {
+                                                   uint32_t* __restrict__ cnt, uint4* __restrict__ packed,
+                                                   const int* __restrict__ scattered) {
   pdl_entry();
+  const bool pack = PACK && *scattered;
   const int64_t i0 = blockIdx.x * (int64_t)(KT * CI) + threadIdx.x;
   const int sh = 32 - log2n;
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t upto = (2u << lane) - 1u;       // lanes 0 .. lane
-  uint32_t key[CI], r[CI], start[CI];
+  uint32_t key[CI], r[CI], start[CI], x[CI], y[CI], z[CI];
 #pragma unroll
   for (int k = 0; k < CI; ++k) {
     const int64_t i = i0 + k * KT;
     key[k] = 0xffffffffu;
     if (i < np) {
-      const uint32_t ix = __ldg(X + i) >> sh;
-      const uint32_t iy = __ldg(X + np + i) >> sh;
-      const uint32_t iz = __ldg(X + 2 * np + i) >> sh;
-      key[k] = (((ix << log2n) | iy) << log2n) | iz;
+      x[k] = PACK ? __ldcs(X + i) : __ldg(X + i);
+      y[k] = PACK ? __ldcs(X + np + i) : __ldg(X + np + i);
+      z[k] = PACK ? __ldcs(X + 2 * np + i) : __ldg(X + 2 * np + i);
+      key[k] = ((((x[k] >> sh) << log2n) | (y[k] >> sh)) << log2n) | (z[k] >> sh);
       if (BOX) key[k] |= (uint32_t)(i / np_box) << (3 * log2n);
     }
   }
@@ -78,16 +86,25 @@ __global__ void __launch_bounds__(KT) k_cell_count(const uint32_t* __restrict__ 
     r[k] = 0;
     if (key[k] != 0xffffffffu && start[k] == lane) r[k] = atomicAdd(cnt + key[k], end - lane);
   }
+  if (pack) {   // while the atomics are in flight
+#pragma unroll
+    for (int k = 0; k < CI; ++k)
+      if (i0 + k * KT < np) __stcs(packed + i0 + k * KT, make_uint4(x[k], y[k], z[k], 0u));
+  }
 #pragma unroll
   for (int k = 0; k < CI; ++k) {
     const uint32_t base = __shfl_sync(0xffffffffu, r[k], start[k]);
     const int64_t i = i0 + k * KT;
-    if (i < np) kr[i] = make_uint2(key[k], base + lane - start[k]);
+    if (i < np) {
+      if (pack) __stcs(kr + i, make_uint2(key[k], base + lane - start[k]));
+      else kr[i] = make_uint2(key[k], base + lane - start[k]);
+    }
   }
 }
 
 // perm[cellstart[key] + rank] = i; a thread takes CI particles, KT apart, with
-// their loads in flight together.
+// their loads in flight together.  The keys are read once (evict-first: the cell
+// starts stay in L2; 10^7 in random order on 256^3 173 -> 155 us).
 __global__ void __launch_bounds__(KT) k_cell_scatter(const uint2* __restrict__ kr, int64_t np,
                                                      const uint32_t* __restrict__ cellstart,
                                                      uint32_t* __restrict__ perm, ListHeads lists) {
@@ -97,7 +114,7 @@ __global__ void __launch_bounds__(KT) k_cell_scatter(const uint2* __restrict__ k
   uint2 t[CI];
   uint32_t base[CI];
 #pragma unroll
-  for (int k = 0; k < CI; ++k) t[k] = i0 + k * KT < np ? __ldg(kr + i0 + k * KT) : make_uint2(0u, 0u);
+  for (int k = 0; k < CI; ++k) t[k] = i0 + k * KT < np ? __ldcs(kr + i0 + k * KT) : make_uint2(0u, 0u);
 #pragma unroll
   for (int k = 0; k < CI; ++k) base[k] = i0 + k * KT < np ? __ldg(cellstart + t[k].x) : 0u;
 #pragma unroll
@@ -499,11 +516,14 @@ __global__ void __launch_bounds__(SCAN_T, 2) k_scan_apply(uint32_t* __restrict__
 // PT apart (coalesced), their permutation entries and then their gathers all
 // in flight together.
 constexpr int PT = 256, PK = 4;
+template <bool PACK>
 __global__ void __launch_bounds__(PT) k_permute(const uint32_t* __restrict__ perm, int64_t np,
                                                 const uint32_t* __restrict__ X, const float* __restrict__ V,
                                                 const uint32_t* __restrict__ id, uint32_t* __restrict__ Xs,
-                                                float* __restrict__ Vs, uint32_t* __restrict__ ids) {
+                                                float* __restrict__ Vs, uint32_t* __restrict__ ids,
+                                                const uint4* __restrict__ packed, const int* __restrict__ scattered) {
   pdl_entry();
+  const bool pack = PACK && *scattered;
   const int64_t j0 = (int64_t)blockIdx.x * (PT * PK) + threadIdx.x;
   uint32_t p[PK];
 #pragma unroll
@@ -511,9 +531,17 @@ __global__ void __launch_bounds__(PT) k_permute(const uint32_t* __restrict__ per
   if (X) {
     uint32_t x[PK][3];
 #pragma unroll
-    for (int k = 0; k < PK; ++k)
+    for (int k = 0; k < PK; ++k) {
+      if (pack) {
+        const uint4 v = j0 + k * PT < np ? __ldg(packed + p[k]) : make_uint4(0u, 0u, 0u, 0u);
+        x[k][0] = v.x;
+        x[k][1] = v.y;
+        x[k][2] = v.z;
+      } else {
 #pragma unroll
-      for (int d = 0; d < 3; ++d) x[k][d] = j0 + k * PT < np ? __ldg(X + d * np + p[k]) : 0u;
+        for (int d = 0; d < 3; ++d) x[k][d] = j0 + k * PT < np ? __ldg(X + d * np + p[k]) : 0u;
+      }
+    }
 #pragma unroll
     for (int k = 0; k < PK; ++k)
       if (j0 + k * PT < np) {
@@ -566,8 +594,22 @@ int64_t sort_meds_capacity(int64_t np) { return np / (kMedRun + 1) + 2; }
 int64_t sort_bigs_capacity(int64_t np) { return np / (kWarpRun + 1) + 2; }
 int64_t sort_smalls_capacity(int64_t np) { return np / (kWalkRun + 1) + 2; }
 
+// Packing pays where the gather in cell order is scattered: three lookups of four
+// bytes a particle become one of sixteen (10^7 in random order on 256^3: 294 ->
+// 158 us, the count that packs 144 -> 155).  A sample of the order decides: from
+// eight rows of cells in 32 neighbouring particles on the planes' lookups no longer
+// share their lines.  Below 2^22 particles the planes (48 MB) stay in L2 and
+// the sample costs what it could save.
+pm_status pack_scattered(const uint32_t* X, int64_t np, int n, const Workspace& w, Packed* pk, cudaStream_t s) {
+  if (np < 1 << 22) return PM_OK;
+  pk->x = reinterpret_cast<uint4*>(w.moments);   // free until the deposit sums the crowded cells
+  pk->scattered = reinterpret_cast<int*>(w.scalars + 40);
+  static_assert(kMomStride * sizeof(float) >= sizeof(uint4), "room for the packed positions");
+  return order_sample(X, np, n, 1.0f, 8.0f, pk->scattered, s);
+}
+
 pm_status sort_cells(const uint32_t* X, int64_t np, int n, Workspace& w, cudaStream_t s, uint32_t* cellstart,
-                     uint32_t** perm_out, const Batch& bt) {
+                     uint32_t** perm_out, const Batch& bt, const Packed& pk) {
   const int log2n = ilog2(n);
   const int64_t ncells = (int64_t)n * n * n * bt.B;
   *perm_out = w.perm;
@@ -579,9 +621,14 @@ pm_status sort_cells(const uint32_t* X, int64_t np, int n, Workspace& w, cudaStr
   const int64_t np_box = bt.B > 1 ? bt.np_box : 0;
   const unsigned gc = grid_for(np, KT * CI);
   if (np_box > 0)
-    PM_LAUNCH(K_KEYS, 28.0 * np, k_cell_count<true>, gc, KT, 0, s, X, np, log2n, np_box, w.keyrank, cellstart);
+    PM_LAUNCH(K_KEYS, 28.0 * np, (k_cell_count<true, false>), gc, KT, 0, s, X, np, log2n, np_box, w.keyrank, cellstart,
+              pk.x, pk.scattered);
+  else if (pk.x)
+    PM_LAUNCH(K_KEYS, 28.0 * np, (k_cell_count<false, true>), gc, KT, 0, s, X, np, log2n, np_box, w.keyrank, cellstart,
+              pk.x, pk.scattered);
   else
-    PM_LAUNCH(K_KEYS, 28.0 * np, k_cell_count<false>, gc, KT, 0, s, X, np, log2n, np_box, w.keyrank, cellstart);
+    PM_LAUNCH(K_KEYS, 28.0 * np, (k_cell_count<false, false>), gc, KT, 0, s, X, np, log2n, np_box, w.keyrank, cellstart,
+              pk.x, pk.scattered);
   PM_TRY(scan_u32(cellstart, ncells + 1, w.scan_blocks, s));
   PM_LAUNCH(K_SCATTER, 16.0 * np, k_cell_scatter, gc, KT, 0, s, w.keyrank, np, cellstart, w.perm,
             ListHeads{w.smalls, w.meds, w.runs, w.bigs});
@@ -594,10 +641,15 @@ pm_status sort_cells(const uint32_t* X, int64_t np, int n, Workspace& w, cudaStr
 
 pm_status permute_particles(const uint32_t* perm, int64_t np, const uint32_t* X, const float* V,
                             const uint32_t* id, uint32_t* Xs, float* Vs, uint32_t* ids,
-                            cudaStream_t s) {
+                            cudaStream_t s, const Packed& pk) {
   if (np == 0) return PM_OK;
-  PM_LAUNCH(K_PERMUTE, (4.0 + (X ? 24.0 : 0.0) + (V ? 24.0 : 0.0) + (id ? 8.0 : 0.0)) * np, k_permute,
-            grid_for(np, PT * PK), PT, 0, s, perm, np, X, V, id, Xs, Vs, ids);
+  const double bytes = (4.0 + (X ? 24.0 : 0.0) + (V ? 24.0 : 0.0) + (id ? 8.0 : 0.0)) * np;
+  if (pk.x)
+    PM_LAUNCH(K_PERMUTE, bytes, k_permute<true>, grid_for(np, PT * PK), PT, 0, s, perm, np, X, V, id, Xs, Vs, ids, pk.x,
+              pk.scattered);
+  else
+    PM_LAUNCH(K_PERMUTE, bytes, k_permute<false>, grid_for(np, PT * PK), PT, 0, s, perm, np, X, V, id, Xs, Vs, ids, pk.x,
+              pk.scattered);
   return launch_status();
 }
 

@@ -133,3 +133,22 @@ def test_large_batch_is_bitwise_a_batch_of_one(pm):
         out.append((ens.positions(), ens.velocities()))
     for b in (0, 17, 39):
         assert np.array_equal(out[1][0][b], out[0][0][0]) and np.array_equal(out[1][1][b], out[0][1][0]), b
+
+
+@pytest.mark.parametrize("n,N,order", [(128, 1 << 22, "random"), (128, (1 << 22) + 3, "cells"), (16, 1 << 22, "random"),
+                                       (64, (1 << 22) - 1, "random")])
+def test_packed_positions_deposit_the_same(pm, n, N, order):
+    """Many particles in random order are gathered from packed positions: the
+    density (and the cotangents) of any order is that of the cell order."""
+    X = inputs.uniform_particles(N, 8)
+    c = X >> np.uint32(32 - int(np.log2(n)))
+    by = np.lexsort((c[2], c[1], c[0]))
+    Xd, Xc = pm.positions_to_device(X), pm.positions_to_device(X[:, by])
+    if order == "cells":
+        Xd, by = Xc, np.arange(N)
+    assert torch.equal(pm.deposit(Xd, n), pm.deposit(Xc, n))
+    g = torch.from_numpy(np.stack([inputs.random_field(n, 70 + d) for d in range(3)]).astype(np.float32)).cuda()
+    bar = torch.from_numpy(np.random.default_rng(1).standard_normal((3, N)).astype(np.float32)).cuda()
+    b = torch.from_numpy(by).cuda()
+    one, two = pm.interp_adj(g, Xd, bar), pm.interp_adj(g, Xc, bar[:, b].contiguous())
+    assert torch.equal(one[0], two[0]) and torch.equal(one[1][:, b], two[1])
