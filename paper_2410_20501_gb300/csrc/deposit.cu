@@ -99,9 +99,9 @@ __global__ void __launch_bounds__(T * T * T) k_deposit(const uint32_t* __restric
 // destination planes a source plane reaches (9 (y, z) offsets each): the
 // particles of source plane x add their TSC weight products to destination
 // planes x - 1, x and x + 1, after which plane x - 1 has everything from this
-// column and its 9 sums go to shared memory.  Destination warps (two cells
-// per thread, rows ty and ty + DTY / 2) add, in a fixed order, the 9 column
-// sums that point at each of their cells and write the density.
+// column and its 9 sums go to shared memory.  A destination warp (eight
+// cells per thread, DTY / 8 rows apart) adds, in a fixed order, the 9 column
+// sums that point at each of its cells and writes the density.
 //
 // Its instructions bound it: a source warp weighs as many particles a plane as the
 // fullest of its 32 cells holds (3.6 on average at one a cell), and no plane's
@@ -109,11 +109,16 @@ __global__ void __launch_bounds__(T * T * T) k_deposit(const uint32_t* __restric
 // over the CTA: source and destination warps meet on two barriers per buffer of
 // column sums (full: every source warp has written; empty: the destinations have
 // read), where filling one and freeing one do not wait, and a source warp runs up
-// to kColBufs planes ahead of the slowest.  One barrier a plane -> four buffers:
-// 256^3 alone 269 -> 266 us, clustered 501 -> 469, 10^7 on 256^3 437 -> 413, with
-// values on 128^3 75 -> 68.  (Two columns a thread in
-// the paired float instructions halve the walks, but 128 registers leave 16 warps
-// an SM: 278 us against 277, clustered 668 against 570 with the moments' launch.)
+// to kColBufs planes ahead of the slowest.  Nor need the destinations be many: one
+// warp keeps up with eleven, and every warp fewer is registers for the others (80
+// a thread at two CTAs an SM; four destination warps leave 64 and spill).  Against
+// one barrier a plane and four destination warps: 256^3 280 -> 250 us (with the
+// moments' launch), clustered 501 -> 424, 10^7 on 256^3 437 -> 373, with values on
+// 128^3 75 -> 62, 512^3 1.87 -> 1.74 ms (the barriers alone, at 64 registers: 278,
+// 469, 413, 68 us, 1.94 ms).  (Two
+// columns a thread in the paired float instructions halve the walks, but 128
+// registers leave 16 warps an SM: clustered 668 us with the moments' launch
+// against 570.)
 //
 // Particle loads: a source thread copies the first KP particles of its cell
 // on the next plane into its own shared-memory slots with asynchronous copies
@@ -133,9 +138,9 @@ __global__ void __launch_bounds__(T * T * T) k_deposit(const uint32_t* __restric
 constexpr int DTY = 16, DTZ = 16, DEY = DTY + 2, DEZ = DTZ + 2, DNT = DTY * DTZ;
 constexpr int DPL = DEY * DEZ;                     // source cells of a plane (one per source thread)
 constexpr int DSRC_T = (DPL + 31) / 32 * 32;       // source warps
-constexpr int DDST_T = DNT / 2;                    // destination threads (two cells each)
+constexpr int DDST_T = DNT / 8;                    // destination threads (eight cells each)
 constexpr int DTHREADS = DSRC_T + DDST_T;
-static_assert(DDST_T % 32 == 0 && DTY % 2 == 0, "whole destination warps, two rows per thread");
+static_assert(DDST_T % 32 == 0 && DTY % 8 == 0, "whole destination warps, eight rows per thread");
 constexpr int kSumPlanes = 16;                    // planes of a partial sum of the density in a batch
 constexpr int kColBufs = 4;                        // column-sum buffers (a power of two)
 // Staged particles per cell and words per particle (x, y, z [, value]).
@@ -191,7 +196,7 @@ __global__ void __launch_bounds__(DTHREADS, 2) k_deposit_stream(const uint32_t* 
   const bool src = tid < PL, dst = tid >= DSRC_T;
   const int sly = tid / DEZ, slz = tid - sly * DEZ;            // source column of this thread (if src)
   const int dt = tid - DSRC_T;
-  const int ty = dt / DTZ, tz = dt - ty * DTZ;                 // destination cells (ty, tz), (ty + DTY / 2, tz) (if dst)
+  const int ty = dt / DTZ, tz = dt - ty * DTZ;                 // destination cells (ty + h DTY / 8, tz) (if dst)
   // copies the first KP particles [b, min(e, b + KP)) into slot buffer `buf`
   // (none for a cell whose moments are ready in `crowd`)
   auto stage = [&](int buf, uint32_t b, uint32_t e) {
@@ -327,8 +332,8 @@ __global__ void __launch_bounds__(DTHREADS, 2) k_deposit_stream(const uint32_t* 
         const float* ColR = Col + buf * 9 * PL;
         barrier_sync(FULL + buf);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int ry = ty + h * (DTY / 2);
+        for (int h = 0; h < 8; ++h) {
+          const int ry = ty + h * (DTY / 8);
           float a = 0.0f;
 #pragma unroll
           for (int oy = 0; oy < 3; ++oy)
@@ -630,7 +635,7 @@ pm_status deposit_sorted_values(const uint32_t* Xs, int64_t np, const uint32_t* 
     const float* crowd = cr.runs && np > 0 ? cr.moments : nullptr;
     int chunk, nitems;
     deposit_stream_plan(n, 0, &chunk, &nitems);
-    const unsigned grid = (unsigned)nitems;   // one item per CTA, two 512-thread CTAs per SM
+    const unsigned grid = (unsigned)nitems;   // one item per CTA, two CTAs per SM
     const double bytes = (vals ? 16.0 : 12.0) * np + 8.0 * n * n * (double)n + 4.0;
     if (vals) {
       PM_TRY(smem_attr(k_deposit_stream<true>, DepositStage<true>::smem));
