@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(256) k_resid_norm(const float* __restrict__ u,
   const float mean = load_mean(f);
   const int m = (1 << log2n) - 1;
   const uint32_t runs = 1u << (3 * log2n - 2);
-  PairSum D(both(0.0f)), F(both(0.0f));
+  float sd[2] = {0.0f, 0.0f}, cd[2] = {0.0f, 0.0f}, sf[2] = {0.0f, 0.0f}, cf[2] = {0.0f, 0.0f};
   for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < runs; t += gridDim.x * blockDim.x) {
     const int k = (int)(t << 2) & m, j = (int)(t >> (log2n - 2)) & m, i = (int)(t >> (2 * log2n - 2));
     auto row = [&](int x, int y) { return __ldg(reinterpret_cast<const float4*>(u + idx3(x & m, y & m, k, log2n))); };
@@ -273,12 +273,16 @@ __global__ void __launch_bounds__(256) k_resid_norm(const float* __restrict__ u,
       S.sub_times(6.0f, PairSum(two(c)));
       const float2 fv = mul2(both(f.s), add2(two(fr), both(-mean)));
       const float2 d = add2(fma2(both(-inv_h2), S.s, fv), mul2(both(-inv_h2), S.e));
-      D.add(mul2(d, d));
-      F.add(mul2(fv, fv));
+      kahan_add(sd[0], cd[0], d.x * d.x);
+      kahan_add(sd[1], cd[1], d.y * d.y);
+      kahan_add(sf[0], cf[0], fv.x * fv.x);
+      kahan_add(sf[1], cf[1], fv.y * fv.y);
     }
   }
-  block_sum_to(partial + blockIdx.x, D.s.x + D.s.y, -(D.e.x + D.e.y), scratch);
-  block_sum_to(partial + gridDim.x + blockIdx.x, F.s.x + F.s.y, -(F.e.x + F.e.y), scratch);
+  kahan_add(sd[0], cd[0], sd[1] - cd[1]);
+  kahan_add(sf[0], cf[0], sf[1] - cf[1]);
+  block_sum_to(partial + blockIdx.x, sd[0], cd[0], scratch);
+  block_sum_to(partial + gridDim.x + blockIdx.x, sf[0], cf[0], scratch);
 }
 
 // Block sum of per-thread float64 values, written by thread 0 to *out (a
