@@ -102,17 +102,4 @@ __device__ __forceinline__ float2 block_pair_sum(float sum, float comp, float2* 
   return scratch[32];
 }
 
-// Flat indices (32-bit: n <= 1024) of a cell's six periodic face neighbours in
-// the order x+, x-, y+, y-, z+, z-, for c = (i n + j) n + k.
-__device__ __forceinline__ void nb_index(uint32_t c, uint32_t i, uint32_t j, uint32_t k, int log2n,
-                                         uint32_t idx[6]) {
-  const uint32_t m = (1u << log2n) - 1, n = 1u << log2n, n2 = n << log2n;
-  idx[0] = i == m ? c - m * n2 : c + n2;
-  idx[1] = i == 0 ? c + m * n2 : c - n2;
-  idx[2] = j == m ? c - m * n : c + n;
-  idx[3] = j == 0 ? c + m * n : c - n;
-  idx[4] = k == m ? c - m : c + 1;
-  idx[5] = k == 0 ? c + m : c - 1;
-}
-
 }  // namespace pmgb
