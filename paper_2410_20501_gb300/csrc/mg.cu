@@ -766,13 +766,20 @@ pm_status march_attributes() {
   return PM_OK;
 }
 
-// `count` smoothing sweeps on level l with SOR factors w[0..count-1].
-// zero: the level's values start at 0; scale (sbox: per box): warm-start
-// factor applied to the values present before the first sweep.
-pm_status smooth(MG& g, int l, int count, const float* w, bool zero, float scale, const float* sbox = nullptr) {
+// SOR factor of sweep si of the `count` before (pre) or after the coarse
+// correction: 1 for the first before and the last after it, omega for the others.
+float sweep_factor(const mg_params& p, bool pre, int si, int count) {
+  return si == (pre ? 0 : count - 1) ? 1.0f : p.omega;
+}
+
+// `count` smoothing sweeps on level l, before (pre) or after the coarse
+// correction.  zero: the level's values start at 0; scale (sbox: per box):
+// warm-start factor applied to the values present before the first sweep.
+pm_status smooth(MG& g, int l, int count, bool pre, bool zero, float scale, const float* sbox = nullptr) {
   const int n = g.n0 >> l, log2n = ilog2(n);
   const float h2 = 1.0f / ((float)n * (float)n);
   const int64_t N = (int64_t)n * n * n;
+  auto factor = [&](int si) { return sweep_factor(*g.p, pre, si, count); };
   int done = 0;
   // fused sweeps (two per pass over memory) or colour passes (two per sweep),
   // bitwise the same result.  Two sweeps: 512^3 0.83 -> 0.40 ms, 256^3 130 -> 63
@@ -792,13 +799,13 @@ pm_status smooth(MG& g, int l, int count, const float* w, bool zero, float scale
     while (done < count) {
       const int S = count - done >= 2 ? 2 : 1;
       const int z = (done == 0 && zero) ? 1 : 0;
-      const bool one0 = w[done] == 1.0f, one1 = S == 2 && w[done + 1] == 1.0f;
+      const float w0 = factor(done), w1 = S == 2 ? factor(done + 1) : 1.0f;
+      const bool one0 = w0 == 1.0f, one1 = S == 2 && w1 == 1.0f;
       const int chunks = S == 2 ? march_chunks<2, kMarchTY, kMarchTZ>(n, g.B) : march_chunks<1, kMarchTY, kMarchTZ>(n, g.B);
       const dim3 grid = g.grid((unsigned)((n / kMarchTY) * (n / kMarchTZ) * chunks));
 #define PM_MARCH(SW, ONE0, ONE1)                                                                                   \
   do {                                                                                                             \
-    const LinearSweeps<ONE0, ONE1> sweeps{h2, done == 0 ? scale : 1.0f, w[done], SW == 2 ? w[done + 1] : 1.0f,      \
-                                          done == 0 ? sbox : nullptr};                                             \
+    const LinearSweeps<ONE0, ONE1> sweeps{h2, done == 0 ? scale : 1.0f, w0, w1, done == 0 ? sbox : nullptr};        \
     PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (z ? 8.0 : 12.0) * N * g.B,                                     \
               (k_rb_march<LinearSweeps<ONE0, ONE1>, SW, kMarchTY, kMarchTZ>), grid,                                \
               (MarchGeom<SW, kMarchTY, kMarchTZ>::THREADS), (MarchGeom<SW, kMarchTY, kMarchTZ>::smem), g.s, g.u[l], \
@@ -820,7 +827,7 @@ pm_status smooth(MG& g, int l, int count, const float* w, bool zero, float scale
   } else {
     const unsigned grid = grid_for(N / 4, kSweepThreads);
     for (; done < count; ++done) {
-      const PoissonUpdate upd{h2, w[done], done == 0 ? scale : 1.0f, done == 0 ? sbox : nullptr};
+      const PoissonUpdate upd{h2, factor(done), done == 0 ? scale : 1.0f, done == 0 ? sbox : nullptr};
       const int z = (done == 0 && zero) ? 1 : 0;
       const int first = done == 0 ? 1 : 0;
       PM_LAUNCH(l == 0 ? K_MG_SMOOTH0 : K_MG_SMOOTH, (z ? 4.0 : 6.0) * N * g.B, k_rb_sweep, g.grid(grid), kSweepThreads, 0,
@@ -835,11 +842,12 @@ pm_status smooth(MG& g, int l, int count, const float* w, bool zero, float scale
 
 // One side of the V-cycle on a small level (k_rb_tile); zero: from zeros.
 template <bool PRE>
-pm_status tile_side(MG& g, int l, int count, const float* w, bool zero, float scale, const float* sbox) {
+pm_status tile_side(MG& g, int l, int count, bool zero, float scale, const float* sbox) {
   const int n = g.n0 >> l, log2n = ilog2(n);
   const float h2 = 1.0f / ((float)n * (float)n);
   const double N = (double)n * n * n;
-  const PoissonUpdate u0{h2, w[0], scale, sbox}, u1{h2, count > 1 ? w[1] : 1.0f, 1.0f, nullptr};
+  const PoissonUpdate u0{h2, sweep_factor(*g.p, PRE, 0, count), scale, sbox};
+  const PoissonUpdate u1{h2, count > 1 ? sweep_factor(*g.p, PRE, 1, count) : 1.0f, 1.0f, nullptr};
   float* out = zero ? g.u[l] : g.alt[l];
   const float* in = zero ? nullptr : g.u[l];
   const float* uc = PRE ? nullptr : g.u[l + 1];
@@ -883,14 +891,11 @@ pm_status v_cycle(MG& g, int l, bool zero_guess) {
 #undef PM_COARSE
     return PM_OK;
   }
-  float w[64];
   if (p.smoother != 1 && n <= kTileN && p.npre >= 1 && p.npre <= 2 && p.npost >= 1 && p.npost <= 2 && g.alt[l] &&
       march_aligned(g.u[l], g.alt[l], g.f[l].p)) {
-    for (int si = 0; si < p.npre; ++si) w[si] = si == 0 ? 1.0f : p.omega;
-    PM_TRY(tile_side<true>(g, l, p.npre, w, zero_guess, scaled ? g.gscale : 1.0f, sbox));
+    PM_TRY(tile_side<true>(g, l, p.npre, zero_guess, scaled ? g.gscale : 1.0f, sbox));
     PM_TRY(v_cycle(g, l + 1, true));
-    for (int si = 0; si < p.npost; ++si) w[si] = si == p.npost - 1 ? 1.0f : p.omega;
-    return tile_side<false>(g, l, p.npost, w, false, 1.0f, nullptr);
+    return tile_side<false>(g, l, p.npost, false, 1.0f, nullptr);
   }
   if (p.npre == 0) {
     const int64_t N = (int64_t)n * n * n;
@@ -898,8 +903,7 @@ pm_status v_cycle(MG& g, int l, bool zero_guess) {
     else if (scaled)
       PM_LAUNCH(K_MG_GUESS, 8.0 * N * g.B, k_scale, g.grid(grid_for(N, 256)), 256, 0, g.s, g.u[l], N, g.gscale, sbox);
   } else {
-    for (int si = 0; si < p.npre; ++si) w[si] = si == 0 ? 1.0f : p.omega;
-    PM_TRY(smooth(g, l, p.npre, w, zero_guess, scaled ? g.gscale : 1.0f, sbox));
+    PM_TRY(smooth(g, l, p.npre, true, zero_guess, scaled ? g.gscale : 1.0f, sbox));
   }
   const int64_t nc = ((int64_t)n * n * n) / 8;
   const unsigned grid = grid_for(nc / 2, 128);
@@ -912,10 +916,7 @@ pm_status v_cycle(MG& g, int l, bool zero_guess) {
   PM_TRY(v_cycle(g, l + 1, true));
   PM_LAUNCH(K_MG_PROLONG, 68.0 * nc * g.B, k_prolong_correct<false>, g.grid(grid_for(nc / 2, 128)), 128, 0, g.s, g.u[l],
             g.u[l + 1], (const float*)nullptr, log2n);
-  if (p.npost > 0) {
-    for (int si = 0; si < p.npost; ++si) w[si] = si == p.npost - 1 ? 1.0f : p.omega;
-    PM_TRY(smooth(g, l, p.npost, w, false, 1.0f));
-  }
+  if (p.npost > 0) PM_TRY(smooth(g, l, p.npost, false, false, 1.0f));
   return PM_OK;
 }
 
