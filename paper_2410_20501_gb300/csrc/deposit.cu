@@ -170,10 +170,12 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 // Partial sums of the density: one per destination warp and chunk, or with
 // sum_planes < chunk one per warp and run of sum_planes planes (then they do not
 // depend on the chunk, which a batch's size may change).
+// A CTA takes one column and chunk (grid: every column times every chunk, by box): the
+// last kColBufs planes are never waited for, so a second one would overwrite them.
 template <bool VALS>
 __global__ void __launch_bounds__(DTHREADS, 2) k_deposit_stream(const uint32_t* __restrict__ Xs, int64_t np,
                                                                 const uint32_t* __restrict__ cellstart, int log2n,
-                                                                int chunk, int nitems, const float* __restrict__ vals,
+                                                                int chunk, const float* __restrict__ vals,
                                                                 float scale, float* __restrict__ rho,
                                                                 double* __restrict__ partial, int sum_planes,
                                                                 const float* __restrict__ crowd) {
@@ -185,7 +187,7 @@ __global__ void __launch_bounds__(DTHREADS, 2) k_deposit_stream(const uint32_t* 
     const int64_t off = (int64_t)blockIdx.z << (3 * log2n);
     cellstart += off;
     rho += off;
-    partial += (int64_t)blockIdx.z * nitems * (chunk / sum_planes) * DW;
+    partial += (int64_t)blockIdx.z * gridDim.x * (chunk / sum_planes) * DW;
   }
   float* Col = sm;                                                        // [kColBufs][9][PL] column sums
   uint32_t* Slot = reinterpret_cast<uint32_t*>(sm + kColBufs * 9 * PL);   // [2][KP][NC][PL]
@@ -211,144 +213,142 @@ __global__ void __launch_bounds__(DTHREADS, 2) k_deposit_stream(const uint32_t* 
       }
     }
   };
-  for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
-    const int tile = item % tiles, xc = item / tiles;
-    const int y0 = (tile / tiles_z) * DTY, z0 = (tile % tiles_z) * DTZ;
-    const int x0 = xc * chunk, x1 = x0 + chunk;
-    const uint32_t cy = (uint32_t)((y0 - 1 + sly) & mask), cz = (uint32_t)((z0 - 1 + slz) & mask);
-    auto cell_of = [&](int x) -> uint32_t { return ((((uint32_t)(x & mask)) << log2n | cy) << log2n) | cz; };
-    float wsum_s = 0.0f, wsum_c = 0.0f;
-    // pipeline registers: cell starts of planes xs and xs + 1
-    uint32_t b0 = 0, e0 = 0, b1 = 0, e1 = 0;
+  const int tile = blockIdx.x % tiles, xc = blockIdx.x / tiles;
+  const int y0 = (tile / tiles_z) * DTY, z0 = (tile % tiles_z) * DTZ;
+  const int x0 = xc * chunk, x1 = x0 + chunk;
+  const uint32_t cy = (uint32_t)((y0 - 1 + sly) & mask), cz = (uint32_t)((z0 - 1 + slz) & mask);
+  auto cell_of = [&](int x) -> uint32_t { return ((((uint32_t)(x & mask)) << log2n | cy) << log2n) | cz; };
+  float wsum_s = 0.0f, wsum_c = 0.0f;
+  // pipeline registers: cell starts of planes xs and xs + 1
+  uint32_t b0 = 0, e0 = 0, b1 = 0, e1 = 0;
+  if (src) {
+    const uint32_t c0 = cell_of(x0 - 1), c1 = cell_of(x0);
+    b0 = __ldg(cellstart + c0); e0 = __ldg(cellstart + c0 + 1);
+    b1 = __ldg(cellstart + c1); e1 = __ldg(cellstart + c1 + 1);
+    stage((x0 - 1) & 1, b0, e0);
+    cp_async_commit();
+  }
+  // one plane step of a source warp: source plane xs adds to the column sums of
+  // destination planes xs - 1 (A), xs (B) and xs + 1 (C, started here) and emits
+  // A.  The caller rotates the roles of the three register arrays.
+  auto step = [&](int xs, float (&A)[9], float (&B)[9], float (&C)[9]) {
+    uint32_t b2 = 0, e2 = 0;
     if (src) {
-      const uint32_t c0 = cell_of(x0 - 1), c1 = cell_of(x0);
-      b0 = __ldg(cellstart + c0); e0 = __ldg(cellstart + c0 + 1);
-      b1 = __ldg(cellstart + c1); e1 = __ldg(cellstart + c1 + 1);
-      stage((x0 - 1) & 1, b0, e0);
+      if (xs + 1 <= x1) stage((xs + 1) & 1, b1, e1);   // the next plane's particles, in flight
       cp_async_commit();
+      if (xs + 2 <= x1) {
+        const uint32_t c2 = cell_of(xs + 2);
+        b2 = __ldg(cellstart + c2); e2 = __ldg(cellstart + c2 + 1);
+      }
+      cp_async_wait1();                                  // this plane's particles have arrived
+#pragma unroll
+      for (int o = 0; o < 9; ++o) C[o] = 0.0f;
+      auto weigh = [&](uint32_t px, uint32_t py, uint32_t pz, float v) {
+        float wx[3], wy[3], wz[3];
+        tsc_weights(cell_offset(px, log2n), wx);
+        tsc_weights(cell_offset(py, log2n), wy);
+        tsc_weights(cell_offset(pz, log2n), wz);
+        if (VALS) {
+          wx[0] *= v; wx[1] *= v; wx[2] *= v;
+        }
+#pragma unroll
+        for (int oy = 0; oy < 3; ++oy) {
+          const float w0 = wx[0] * wy[oy], w1 = wx[1] * wy[oy], w2 = wx[2] * wy[oy];
+#pragma unroll
+          for (int oz = 0; oz < 3; ++oz) {
+            A[oy * 3 + oz] = fmaf(w0, wz[oz], A[oy * 3 + oz]);
+            B[oy * 3 + oz] = fmaf(w1, wz[oz], B[oy * 3 + oz]);
+            C[oy * 3 + oz] = fmaf(w2, wz[oz], C[oy * 3 + oz]);
+          }
+        }
+      };
+      const uint32_t* s0 = Slot + (xs & 1) * KP * NC * PL + tid;
+      const uint32_t cnt = e0 - b0;
+      if (crowd && cnt > kWalkRun) {   // its moments were summed already
+        const float* mo = crowd + kMomStride * (int64_t)b0;
+        float s[28];
+#pragma unroll
+        for (int o = 0; o < 26; o += 2) {
+          const float2 v = __ldg(reinterpret_cast<const float2*>(mo + o));
+          s[o] = v.x;
+          s[o + 1] = v.y;
+        }
+        s[26] = __ldg(mo + 26);
+#pragma unroll
+        for (int o = 0; o < 9; ++o) {
+          A[o] += s[o];
+          B[o] += s[9 + o];
+          C[o] += s[18 + o];
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < KP; ++k)
+          if ((uint32_t)k < cnt)
+            weigh(s0[(k * NC) * PL], s0[(k * NC + 1) * PL], s0[(k * NC + 2) * PL],
+                  VALS ? __uint_as_float(s0[(k * NC + 3) * PL]) : 1.0f);
+        if (cnt > (uint32_t)KP) {   // the rest from global memory
+          uint32_t p = b0 + KP;
+          uint32_t px = __ldg(Xs + p), py = __ldg(Xs + np + p), pz = __ldg(Xs + 2 * np + p);
+          for (; p < e0; ++p) {
+            // the next particle of the cell is loaded while this one is weighed
+            uint32_t qx = 0, qy = 0, qz = 0;
+            if (p + 1 < e0) { qx = __ldg(Xs + p + 1); qy = __ldg(Xs + np + p + 1); qz = __ldg(Xs + 2 * np + p + 1); }
+            weigh(px, py, pz, VALS ? __ldg(vals + p) : 1.0f);
+            px = qx;
+            py = qy;
+            pz = qz;
+          }
+        }
+      }
     }
-    // one plane step of a source warp: source plane xs adds to the column sums of
-    // destination planes xs - 1 (A), xs (B) and xs + 1 (C, started here) and emits
-    // A.  The caller rotates the roles of the three register arrays.
-    auto step = [&](int xs, float (&A)[9], float (&B)[9], float (&C)[9]) {
-      uint32_t b2 = 0, e2 = 0;
+    // destination plane xs - 1 has all of this column's contributions
+    const int done = xs - 1, buf = done & (kColBufs - 1);
+    if (done >= x0) {
+      if (done >= x0 + kColBufs) barrier_sync(EMPTY + buf);
       if (src) {
-        if (xs + 1 <= x1) stage((xs + 1) & 1, b1, e1);   // the next plane's particles, in flight
-        cp_async_commit();
-        if (xs + 2 <= x1) {
-          const uint32_t c2 = cell_of(xs + 2);
-          b2 = __ldg(cellstart + c2); e2 = __ldg(cellstart + c2 + 1);
-        }
-        cp_async_wait1();                                  // this plane's particles have arrived
 #pragma unroll
-        for (int o = 0; o < 9; ++o) C[o] = 0.0f;
-        auto weigh = [&](uint32_t px, uint32_t py, uint32_t pz, float v) {
-          float wx[3], wy[3], wz[3];
-          tsc_weights(cell_offset(px, log2n), wx);
-          tsc_weights(cell_offset(py, log2n), wy);
-          tsc_weights(cell_offset(pz, log2n), wz);
-          if (VALS) {
-            wx[0] *= v; wx[1] *= v; wx[2] *= v;
-          }
-#pragma unroll
-          for (int oy = 0; oy < 3; ++oy) {
-            const float w0 = wx[0] * wy[oy], w1 = wx[1] * wy[oy], w2 = wx[2] * wy[oy];
-#pragma unroll
-            for (int oz = 0; oz < 3; ++oz) {
-              A[oy * 3 + oz] = fmaf(w0, wz[oz], A[oy * 3 + oz]);
-              B[oy * 3 + oz] = fmaf(w1, wz[oz], B[oy * 3 + oz]);
-              C[oy * 3 + oz] = fmaf(w2, wz[oz], C[oy * 3 + oz]);
-            }
-          }
-        };
-        const uint32_t* s0 = Slot + (xs & 1) * KP * NC * PL + tid;
-        const uint32_t cnt = e0 - b0;
-        if (crowd && cnt > kWalkRun) {   // its moments were summed already
-          const float* mo = crowd + kMomStride * (int64_t)b0;
-          float s[28];
-#pragma unroll
-          for (int o = 0; o < 26; o += 2) {
-            const float2 v = __ldg(reinterpret_cast<const float2*>(mo + o));
-            s[o] = v.x;
-            s[o + 1] = v.y;
-          }
-          s[26] = __ldg(mo + 26);
-#pragma unroll
-          for (int o = 0; o < 9; ++o) {
-            A[o] += s[o];
-            B[o] += s[9 + o];
-            C[o] += s[18 + o];
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < KP; ++k)
-            if ((uint32_t)k < cnt)
-              weigh(s0[(k * NC) * PL], s0[(k * NC + 1) * PL], s0[(k * NC + 2) * PL],
-                    VALS ? __uint_as_float(s0[(k * NC + 3) * PL]) : 1.0f);
-          if (cnt > (uint32_t)KP) {   // the rest from global memory
-            uint32_t p = b0 + KP;
-            uint32_t px = __ldg(Xs + p), py = __ldg(Xs + np + p), pz = __ldg(Xs + 2 * np + p);
-            for (; p < e0; ++p) {
-              // the next particle of the cell is loaded while this one is weighed
-              uint32_t qx = 0, qy = 0, qz = 0;
-              if (p + 1 < e0) { qx = __ldg(Xs + p + 1); qy = __ldg(Xs + np + p + 1); qz = __ldg(Xs + 2 * np + p + 1); }
-              weigh(px, py, pz, VALS ? __ldg(vals + p) : 1.0f);
-              px = qx;
-              py = qy;
-              pz = qz;
-            }
-          }
-        }
+        for (int o = 0; o < 9; ++o) Col[(buf * 9 + o) * PL + tid] = A[o];
       }
-      // destination plane xs - 1 has all of this column's contributions
-      const int done = xs - 1, buf = done & (kColBufs - 1);
-      if (done >= x0) {
-        if (done >= x0 + kColBufs) barrier_sync(EMPTY + buf);
-        if (src) {
+      barrier_arrive(FULL + buf);
+    }
+    b0 = b1; e0 = e1; b1 = b2; e1 = e2;
+  };
+  if (!dst) {
+    // column sums of destination planes xs - 1 and xs (the first source plane
+    // reaches planes x0 - 2 .. x0; the first two are outside the chunk)
+    float R0[9], R1[9], R2[9];
 #pragma unroll
-          for (int o = 0; o < 9; ++o) Col[(buf * 9 + o) * PL + tid] = A[o];
-        }
-        barrier_arrive(FULL + buf);
+    for (int o = 0; o < 9; ++o) {
+      R0[o] = 0.0f;
+      R1[o] = 0.0f;
+    }
+    for (int xs = x0 - 1; xs <= x1; xs += 3) {
+      step(xs, R0, R1, R2);
+      if (xs + 1 <= x1) step(xs + 1, R1, R2, R0);
+      if (xs + 2 <= x1) step(xs + 2, R2, R0, R1);
+    }
+  } else {
+    for (int d = x0; d < x1; ++d) {
+      const int buf = d & (kColBufs - 1);
+      const float* ColR = Col + buf * 9 * PL;
+      barrier_sync(FULL + buf);
+#pragma unroll
+      for (int h = 0; h < 8; ++h) {
+        const int ry = ty + h * (DTY / 8);
+        float a = 0.0f;
+#pragma unroll
+        for (int oy = 0; oy < 3; ++oy)
+#pragma unroll
+          for (int oz = 0; oz < 3; ++oz) a += ColR[(oy * 3 + oz) * PL + (ry + 2 - oy) * DEZ + (tz + 2 - oz)];
+        const float r = a * scale;
+        rho[((((int64_t)d << log2n) | (y0 + ry)) << log2n) | (z0 + tz)] = r;
+        kahan_add(wsum_s, wsum_c, r);
       }
-      b0 = b1; e0 = e1; b1 = b2; e1 = e2;
-    };
-    if (!dst) {
-      // column sums of destination planes xs - 1 and xs (the first source plane
-      // reaches planes x0 - 2 .. x0; the first two are outside the chunk)
-      float R0[9], R1[9], R2[9];
-#pragma unroll
-      for (int o = 0; o < 9; ++o) {
-        R0[o] = 0.0f;
-        R1[o] = 0.0f;
-      }
-      for (int xs = x0 - 1; xs <= x1; xs += 3) {
-        step(xs, R0, R1, R2);
-        if (xs + 1 <= x1) step(xs + 1, R1, R2, R0);
-        if (xs + 2 <= x1) step(xs + 2, R2, R0, R1);
-      }
-    } else {
-      for (int d = x0; d < x1; ++d) {
-        const int buf = d & (kColBufs - 1);
-        const float* ColR = Col + buf * 9 * PL;
-        barrier_sync(FULL + buf);
-#pragma unroll
-        for (int h = 0; h < 8; ++h) {
-          const int ry = ty + h * (DTY / 8);
-          float a = 0.0f;
-#pragma unroll
-          for (int oy = 0; oy < 3; ++oy)
-#pragma unroll
-            for (int oz = 0; oz < 3; ++oz) a += ColR[(oy * 3 + oz) * PL + (ry + 2 - oy) * DEZ + (tz + 2 - oz)];
-          const float r = a * scale;
-          rho[((((int64_t)d << log2n) | (y0 + ry)) << log2n) | (z0 + tz)] = r;
-          kahan_add(wsum_s, wsum_c, r);
-        }
-        if (d + kColBufs < x1) barrier_arrive(EMPTY + buf);
-        if (((d + 1 - x0) & (sum_planes - 1)) == 0) {
-          const double ws = warp_sum_comp(wsum_s - wsum_c);
-          if ((dt & 31) == 0) partial[((int64_t)(d / sum_planes) * tiles + tile) * DW + (dt >> 5)] = ws;
-          wsum_s = wsum_c = 0.0f;
-        }
+      if (d + kColBufs < x1) barrier_arrive(EMPTY + buf);
+      if (((d + 1 - x0) & (sum_planes - 1)) == 0) {
+        const double ws = warp_sum_comp(wsum_s - wsum_c);
+        if ((dt & 31) == 0) partial[((int64_t)(d / sum_planes) * tiles + tile) * DW + (dt >> 5)] = ws;
+        wsum_s = wsum_c = 0.0f;
       }
     }
   }
@@ -635,16 +635,16 @@ pm_status deposit_sorted_values(const uint32_t* Xs, int64_t np, const uint32_t* 
     const float* crowd = cr.runs && np > 0 ? cr.moments : nullptr;
     int chunk, nitems;
     deposit_stream_plan(n, 0, &chunk, &nitems);
-    const unsigned grid = (unsigned)nitems;   // one item per CTA, two CTAs per SM
+    const unsigned grid = (unsigned)nitems;   // two CTAs per SM
     const double bytes = (vals ? 16.0 : 12.0) * np + 8.0 * n * n * (double)n + 4.0;
     if (vals) {
       PM_TRY(smem_attr(k_deposit_stream<true>, DepositStage<true>::smem));
       PM_LAUNCH(K_DEPOSIT, bytes, k_deposit_stream<true>, grid, DTHREADS, DepositStage<true>::smem, s, Xs, np,
-                cellstart, ilog2(n), chunk, nitems, vals, scale, rho, partials, chunk, crowd);
+                cellstart, ilog2(n), chunk, vals, scale, rho, partials, chunk, crowd);
     } else {
       PM_TRY(smem_attr(k_deposit_stream<false>, DepositStage<false>::smem));
       PM_LAUNCH(K_DEPOSIT, bytes, k_deposit_stream<false>, grid, DTHREADS, DepositStage<false>::smem, s, Xs, np,
-                cellstart, ilog2(n), chunk, nitems, vals, scale, rho, partials, chunk, crowd);
+                cellstart, ilog2(n), chunk, vals, scale, rho, partials, chunk, crowd);
     }
     const int64_t nsums = (int64_t)nitems * (DDST_T / 32);
     PM_LAUNCH(K_REDUCE, 8.0 * nsums, k_reduce_partials, 1, 1024, 0, s, partials, nsums, (int64_t)0, 1,
@@ -666,11 +666,11 @@ pm_status deposit_sorted_batch(const uint32_t* Xs, int64_t np_box, int B, const 
   // sums over a fixed number of planes, of which every chunk here is a multiple
   const int64_t nsums = (int64_t)nitems * (chunk / kSumPlanes) * (DDST_T / 32);
   const float scale = np_box > 0 ? (float)((double)n * n * n / (double)np_box) : 0.0f;
-  // one item per CTA: B x nitems CTAs balance over the SMs (two resident each)
+  // B x nitems CTAs balance over the SMs (two resident each)
   const int gx = nitems;
   const int64_t np = np_box * B;
   PM_LAUNCH(K_DEPOSIT, 12.0 * np + 8.0 * n * n * (double)n * B + 4.0, k_deposit_stream<false>, dim3(gx, 1, B),
-            DTHREADS, DepositStage<false>::smem, s, Xs, np, cellstart, ilog2(n), chunk, nitems, (const float*)nullptr, scale, rho,
+            DTHREADS, DepositStage<false>::smem, s, Xs, np, cellstart, ilog2(n), chunk, (const float*)nullptr, scale, rho,
             partials, kSumPlanes, cr.runs && np > 0 ? (const float*)cr.moments : nullptr);
   PM_LAUNCH(K_REDUCE, 8.0 * nsums * B, k_reduce_partials, B, 1024, 0, s, partials, nsums, nsums, B,
             1.0 / ((double)n * n * n), mean_out);
