@@ -574,9 +574,10 @@ int pm_timing_collect(const char** names, double* ms, int64_t* launches, double*
 
 /* ------------------------------------------------------------ autotuning --
  * Batched launches (pm_step_batch) tune how they tile their work, online: for
- * each launch site and shape (n, B) the candidate values of one parameter
- * (the x chunk of the force pass; colour passes or fused sweeps on 64^3
- * levels) take turns on successive real
+ * each launch site, shape (n, B) and kind of work the candidate values of one
+ * parameter (the x chunk of the force pass, for each stencil order; colour
+ * passes or fused sweeps on 64^3 levels, for each number of sweeps, before and
+ * after the coarse correction, from zeros or not) take turns on successive real
  * launches, timed with CUDA events on the launch stream and read back
  * without synchronising; after two timings each the fastest is kept for the
  * rest of the process.  Every candidate computes bitwise the same result, so
@@ -586,10 +587,10 @@ int pm_timing_collect(const char** names, double* ms, int64_t* launches, double*
 /* mode 0: fixed default tilings; 1 (the default): tune; 2: forget every
  * choice and timing, then tune.  PM_EINVAL for another mode. */
 pm_status pm_autotune(int mode);
-/* Reports the tuned sites, five ints each: site (0 force-pass chunk, 2
+/* Reports the tuned sites, one entry for each kind of work, five ints each: site (0 force-pass chunk, 2
  * multigrid smoother form: 0 colour passes, 1 fused; 1 is not in use),
  * n, B, the chosen value (-1 while undecided) and the timings read so far.
- * out (host, 5 * cap ints) may be NULL; returns the number of sites. */
+ * out (host, 5 * cap ints) may be NULL; returns the number of entries. */
 int pm_autotune_report(int* out, int cap);
 
 #ifdef __cplusplus

@@ -740,7 +740,7 @@ pm_status launch_force_interp(const float* phi, const float* eps, float alpha, i
   if (bt.B > 1) {   // batches: the x chunk is tuned (each particle's force is chunk-independent)
     int cand[3], nc = 0;
     for (int c = 16; c <= 64 && c <= n; c *= 2) cand[nc++] = c;
-    chunk = tune_begin(TUNE_FORCE_CHUNK, n, bt.B, cand, nc, chunk, s);
+    chunk = tune_begin(TUNE_FORCE_CHUNK, n, bt.B, ORDER, cand, nc, chunk, s);
   }
   const int nitems = tiles * (n / chunk);
   const dim3 grid((unsigned)nitems, 1, (unsigned)bt.B);

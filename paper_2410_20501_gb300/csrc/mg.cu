@@ -792,7 +792,7 @@ pm_status smooth(MG& g, int l, int count, bool pre, bool zero, float scale, cons
   const bool tune_form = fused_valid && g.B > 1 && n < 128;
   if (tune_form) {
     static const int forms[2] = {0, 1};
-    fused = tune_begin(TUNE_MG_SMOOTHER, n, g.B, forms, 2, 1, g.s) == 1;
+    fused = tune_begin(TUNE_MG_SMOOTHER, n, g.B, count << 2 | (zero ? 2 : 0) | (pre ? 1 : 0), forms, 2, 1, g.s) == 1;
   }
   const bool form_timed = tune_form && tune_active();
   if (fused) {

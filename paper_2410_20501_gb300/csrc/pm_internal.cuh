@@ -22,10 +22,11 @@ extern const char* const kKernelClassNames[K_NCLASS];
 
 // Online autotuner of batched launch tiling (tune.cu).  A site calls
 // tune_begin before its launch(es) with candidate values that compute bitwise
-// the same result, uses the value returned, and calls tune_end after them on
-// the same stream; tune_active() says whether this call is being timed.
+// the same result and a number for the kind of work (only launches of equal work
+// are compared), uses the value returned, and calls tune_end after them on the same
+// stream; tune_active() says whether this call is being timed.
 enum TuneSite { TUNE_FORCE_CHUNK = 0, TUNE_MG_SMOOTHER = 2 };
-int tune_begin(int site, int n, int B, const int* cand, int ncand, int dflt, cudaStream_t s);
+int tune_begin(int site, int n, int B, int work, const int* cand, int ncand, int dflt, cudaStream_t s);
 void tune_end(cudaStream_t s);
 bool tune_active();
 

@@ -2,12 +2,17 @@
 //
 // A tuned launch site has one launch parameter (an x chunk, a smoother form)
 // whose candidate values tile the same work differently and compute bitwise
-// the same result.  For each (site, n, B) the tuner hands out the candidates
+// the same result.  For each (site, n, B, work) the tuner hands out the candidates
 // in turn on successive real launches, times each launch with a pair of CUDA
 // events on the launching stream, reads the timings back once the events have
 // completed (no host synchronisation: a pending pair is simply read at a later
 // call), and after kSamples timings per candidate keeps the fastest (the
 // minimum of its samples, which discards the first launch's one-time costs).
+// `work` names what the launch does (the site says how), so that only launches of
+// equal work are compared: a level is smoothed strictly by turns before and after
+// its coarse correction, and two candidates handed out by turns would each be timed
+// on one of the two.  For the same reason every other round goes backwards: the
+// launches of a step differ in what the caches hold, with a period of a few.
 // While a stream is being captured into a CUDA graph nothing is timed or
 // queried: the site gets the choice made so far, else its default.
 #include <mutex>
@@ -21,7 +26,7 @@ namespace {
 constexpr int kMaxCand = 4, kSamples = 2, kSlots = 8, kEntries = 64;
 
 struct Entry {
-  int site = -1, n = 0, B = 0, dev = 0;   // key (events belong to device dev)
+  int site = -1, n = 0, B = 0, work = 0, dev = 0;   // key (events belong to device dev)
   int ncand = 0, cand[kMaxCand] = {};
   int chosen = -1;                    // index into cand once decided
   float best[kMaxCand] = {};          // minimum sample per candidate
@@ -83,14 +88,16 @@ void harvest(Entry& e) {
   }
 }
 
-Entry* find(int site, int n, int B, int dev, const int* cand, int ncand) {
+Entry* find(int site, int n, int B, int work, int dev, const int* cand, int ncand) {
   for (int i = 0; i < g_used; ++i)
-    if (g_tab[i].site == site && g_tab[i].n == n && g_tab[i].B == B && g_tab[i].dev == dev) return &g_tab[i];
+    if (g_tab[i].site == site && g_tab[i].n == n && g_tab[i].B == B && g_tab[i].work == work && g_tab[i].dev == dev)
+      return &g_tab[i];
   if (g_used == kEntries) return nullptr;
   Entry& e = g_tab[g_used++];
   e.site = site;
   e.n = n;
   e.B = B;
+  e.work = work;
   e.dev = dev;
   e.ncand = ncand;
   for (int c = 0; c < ncand; ++c) e.cand[c] = cand[c];
@@ -100,7 +107,7 @@ Entry* find(int site, int n, int B, int dev, const int* cand, int ncand) {
 
 }  // namespace
 
-int tune_begin(int site, int n, int B, const int* cand, int ncand, int dflt, cudaStream_t s) {
+int tune_begin(int site, int n, int B, int work, const int* cand, int ncand, int dflt, cudaStream_t s) {
   t_ticket = Ticket{};
   if (ncand <= 1 || ncand > kMaxCand) return ncand == 1 ? cand[0] : dflt;
   std::lock_guard<std::mutex> lock(g_mu);
@@ -110,7 +117,7 @@ int tune_begin(int site, int n, int B, const int* cand, int ncand, int dflt, cud
     cudaGetLastError();
     return dflt;
   }
-  Entry* e = find(site, n, B, dev, cand, ncand);
+  Entry* e = find(site, n, B, work, dev, cand, ncand);
   if (!e) return dflt;
   if (e->chosen >= 0) return e->cand[e->chosen];
   const bool cap = capturing(s);
@@ -122,16 +129,17 @@ int tune_begin(int site, int n, int B, const int* cand, int ncand, int dflt, cud
       if (e->count[c] > 0 && (b < 0 || e->best[c] < e->best[b])) b = c;
     return b >= 0 ? e->cand[b] : dflt;
   }
-  // the candidate with the fewest samples read or pending
+  // the candidate with the fewest samples read or pending, in odd rounds the last such
   int pend[kMaxCand] = {};
   int slot = -1;
   for (int k = 0; k < kSlots; ++k) {
     if (e->slot_cand[k] >= 0) ++pend[e->slot_cand[k]];
     else if (slot < 0) slot = k;
   }
+  auto taken = [&](int i) { return e->count[i] + pend[i]; };
   int c = 0;
   for (int i = 1; i < e->ncand; ++i)
-    if (e->count[i] + pend[i] < e->count[c] + pend[c]) c = i;
+    if (taken(i) < taken(c) || (taken(i) == taken(c) && (taken(i) & 1))) c = i;
   if (slot < 0 || e->count[c] + pend[c] >= kSamples) return e->cand[c];   // all samples in flight
   if (!e->ev0[slot]) {
     if (cudaEventCreate(&e->ev0[slot]) != cudaSuccess || cudaEventCreate(&e->ev1[slot]) != cudaSuccess) {

@@ -446,7 +446,8 @@ def autotune(mode):
 
 
 def autotune_report():
-    """The tuned launch sites: [{site, n, B, chosen (None while undecided), samples}]."""
+    """The tuned launch sites, an entry for each kind of work (stencil order; sweeps before or after the
+    coarse correction): [{site, n, B, chosen (None while undecided), samples}]."""
     cap = 64
     out = (ctypes.c_int * (5 * cap))()
     m = min(lib().pm_autotune_report(out, cap), cap)
