@@ -141,7 +141,7 @@ constexpr int DSRC_T = (DPL + 31) / 32 * 32;       // source warps
 constexpr int DDST_T = DNT / 8;                    // destination threads (eight cells each)
 constexpr int DTHREADS = DSRC_T + DDST_T;
 static_assert(DDST_T % 32 == 0 && DTY % 8 == 0, "whole destination warps, eight rows per thread");
-constexpr int kSumPlanes = 16;                    // planes of a partial sum of the density in a batch
+constexpr int kSumPlanes = 16;                    // planes of a partial sum of the density, at most
 constexpr int kColBufs = 4;                        // column-sum buffers (a power of two)
 // Staged particles per cell and words per particle (x, y, z [, value]).
 template <bool VALS> struct DepositStage {
@@ -167,9 +167,9 @@ __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
-// Partial sums of the density: one per destination warp and chunk, or with
-// sum_planes < chunk one per warp and run of sum_planes planes (then they do not
-// depend on the chunk, which a batch's size may change).
+// Partial sums of the density: one per destination warp and run of sum_planes planes,
+// which divides every chunk of a size n (deposit_stream_plan), so that the mean of a
+// box does not depend on the chunk, alone or in any batch.
 // A CTA takes one column and chunk (grid: every column times every chunk, by box): the
 // last kColBufs planes are never waited for, so a second one would overwrite them.
 template <bool VALS>
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(DTHREADS, 2) k_deposit_stream(const uint32_t* 
   const int x0 = xc * chunk, x1 = x0 + chunk;
   const uint32_t cy = (uint32_t)((y0 - 1 + sly) & mask), cz = (uint32_t)((z0 - 1 + slz) & mask);
   auto cell_of = [&](int x) -> uint32_t { return ((((uint32_t)(x & mask)) << log2n | cy) << log2n) | cz; };
-  float wsum_s = 0.0f, wsum_c = 0.0f;
+  float wsum_s = 0.0f, wsum_c = 0.0f;   // this thread's cells since the last partial sum, and its rounding
   // pipeline registers: cell starts of planes xs and xs + 1
   uint32_t b0 = 0, e0 = 0, b1 = 0, e1 = 0;
   if (src) {
@@ -342,11 +342,13 @@ __global__ void __launch_bounds__(DTHREADS, 2) k_deposit_stream(const uint32_t* 
           for (int oz = 0; oz < 3; ++oz) a += ColR[(oy * 3 + oz) * PL + (ry + 2 - oy) * DEZ + (tz + 2 - oz)];
         const float r = a * scale;
         rho[((((int64_t)d << log2n) | (y0 + ry)) << log2n) | (z0 + tz)] = r;
-        kahan_add(wsum_s, wsum_c, r);
+        float e;
+        two_sum(wsum_s, r, wsum_s, e);
+        wsum_c += e;
       }
       if (d + kColBufs < x1) barrier_arrive(EMPTY + buf);
       if (((d + 1 - x0) & (sum_planes - 1)) == 0) {
-        const double ws = warp_sum_comp(wsum_s - wsum_c);
+        const double ws = warp_sum_comp(wsum_s, wsum_c);
         if ((dt & 31) == 0) partial[((int64_t)(d / sum_planes) * tiles + tile) * DW + (dt >> 5)] = ws;
         wsum_s = wsum_c = 0.0f;
       }
@@ -523,13 +525,16 @@ __global__ void __launch_bounds__(CT, 4) k_list_moments(const uint32_t* __restri
 // 16 or more while the grid fills the SMs several times over (256^3 297 us at 32,
 // 316 at 16, 363 at 8), fewer only where SMs would have no CTA at all (32^3 with
 // its other launches 45 us at 16, 35 at 2; 64^3 47 at 16, 39 at 4; 128^3 77 at 16,
-// 79 at 8).
-inline void deposit_stream_plan(int n, int B, int* chunk, int* nitems) {   // B = 0: not a batch
+// 79 at 8).  The partial sums' planes go by n alone: the shortest chunk of that size.
+inline void deposit_stream_plan(int n, int B, int* chunk, int* nitems, int* sum_planes) {   // B = 0: not a batch
   const int tiles = (n / DTY) * (n / DTZ);
+  int shortest = kSumPlanes;
+  while (shortest > 2 && (int64_t)tiles * (n / shortest) < 152) shortest >>= 1;
   int c = n;
   while (c > kSumPlanes && (int64_t)tiles * (n / c) * (B ? B : 1) < 8 * 152) c >>= 1;
-  while (!B && c > 2 && (int64_t)tiles * (n / c) < 152) c >>= 1;
+  if (!B && shortest < c && (int64_t)tiles * (n / c) < 152) c = shortest;
   *chunk = c;
+  *sum_planes = shortest;
   *nitems = tiles * (n / c);
 }
 
@@ -633,20 +638,20 @@ pm_status deposit_sorted_values(const uint32_t* Xs, int64_t np, const uint32_t* 
   if (n >= 32) {
     PM_TRY(crowded_moments(Xs, np, cellstart, n, vals, cr, s));
     const float* crowd = cr.runs && np > 0 ? cr.moments : nullptr;
-    int chunk, nitems;
-    deposit_stream_plan(n, 0, &chunk, &nitems);
+    int chunk, nitems, sum_planes;
+    deposit_stream_plan(n, 0, &chunk, &nitems, &sum_planes);
     const unsigned grid = (unsigned)nitems;   // two CTAs per SM
     const double bytes = (vals ? 16.0 : 12.0) * np + 8.0 * n * n * (double)n + 4.0;
     if (vals) {
       PM_TRY(smem_attr(k_deposit_stream<true>, DepositStage<true>::smem));
       PM_LAUNCH(K_DEPOSIT, bytes, k_deposit_stream<true>, grid, DTHREADS, DepositStage<true>::smem, s, Xs, np,
-                cellstart, ilog2(n), chunk, vals, scale, rho, partials, chunk, crowd);
+                cellstart, ilog2(n), chunk, vals, scale, rho, partials, sum_planes, crowd);
     } else {
       PM_TRY(smem_attr(k_deposit_stream<false>, DepositStage<false>::smem));
       PM_LAUNCH(K_DEPOSIT, bytes, k_deposit_stream<false>, grid, DTHREADS, DepositStage<false>::smem, s, Xs, np,
-                cellstart, ilog2(n), chunk, vals, scale, rho, partials, chunk, crowd);
+                cellstart, ilog2(n), chunk, vals, scale, rho, partials, sum_planes, crowd);
     }
-    const int64_t nsums = (int64_t)nitems * (DDST_T / 32);
+    const int64_t nsums = (int64_t)nitems * (chunk / sum_planes) * (DDST_T / 32);
     PM_LAUNCH(K_REDUCE, 8.0 * nsums, k_reduce_partials, 1, 1024, 0, s, partials, nsums, (int64_t)0, 1,
               1.0 / ((double)n * n * n), mean_out);
     return launch_status();
@@ -660,18 +665,16 @@ pm_status deposit_sorted_batch(const uint32_t* Xs, int64_t np_box, int B, const 
   if (n < 32 || B < 1) return PM_EINVAL;
   PM_TRY(crowded_moments(Xs, np_box * B, cellstart, n, nullptr, cr, s));
   PM_TRY(smem_attr(k_deposit_stream<false>, DepositStage<false>::smem));
-  int chunk, nitems;
-  deposit_stream_plan(n, B, &chunk, &nitems);
-  // the mean of a box must not depend on the boxes it is batched with: partial
-  // sums over a fixed number of planes, of which every chunk here is a multiple
-  const int64_t nsums = (int64_t)nitems * (chunk / kSumPlanes) * (DDST_T / 32);
+  int chunk, nitems, sum_planes;
+  deposit_stream_plan(n, B, &chunk, &nitems, &sum_planes);
+  const int64_t nsums = (int64_t)nitems * (chunk / sum_planes) * (DDST_T / 32);
   const float scale = np_box > 0 ? (float)((double)n * n * n / (double)np_box) : 0.0f;
   // B x nitems CTAs balance over the SMs (two resident each)
   const int gx = nitems;
   const int64_t np = np_box * B;
   PM_LAUNCH(K_DEPOSIT, 12.0 * np + 8.0 * n * n * (double)n * B + 4.0, k_deposit_stream<false>, dim3(gx, 1, B),
             DTHREADS, DepositStage<false>::smem, s, Xs, np, cellstart, ilog2(n), chunk, (const float*)nullptr, scale, rho,
-            partials, kSumPlanes, cr.runs && np > 0 ? (const float*)cr.moments : nullptr);
+            partials, sum_planes, cr.runs && np > 0 ? (const float*)cr.moments : nullptr);
   PM_LAUNCH(K_REDUCE, 8.0 * nsums * B, k_reduce_partials, B, 1024, 0, s, partials, nsums, nsums, B,
             1.0 / ((double)n * n * n), mean_out);
   return launch_status();

@@ -30,9 +30,10 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   e = (a - (s - bp)) + (b - bp);
 }
 
-// Compensated warp sum; the result is valid in lane 0, as a double.
-__device__ __forceinline__ double warp_sum_comp(float v) {
-  float s = v, c = 0.0f;
+// Compensated warp sum of v + c (c: what rounding took from v); the result is
+// valid in lane 0, as a double.
+__device__ __forceinline__ double warp_sum_comp(float v, float c = 0.0f) {
+  float s = v;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     float os = __shfl_down_sync(0xffffffffu, s, o);
