@@ -291,10 +291,10 @@ pm_status pm_gradient(const float* phi, float* g, int n, int order, void* stream
  *   g [3][n^3] (read), X [3][np] (read), acc [3][np] (written). */
 pm_status pm_interp(const float* g, const uint32_t* X, int64_t np, int n,
                     float* acc, void* stream);
-/* The same, bitwise, for many particles in any order: where a sample of the
- * particles is scattered, the field is first packed into a workspace of
- * 16 n^3 + 256 bytes (256-byte aligned), so that a particle's rows come in wide
- * loads.  PM_ENOMEM: workspace too small. */
+/* The same, bitwise, with a workspace of 16 n^3 + 256 bytes (256-byte aligned):
+ * from 2^19 particles and a 24th of the cells on the field is packed into it
+ * first if a sample of the particles is scattered, so that a particle's rows
+ * come in wide loads; below, it is not touched.  PM_ENOMEM: workspace too small. */
 pm_status pm_interp_packed(const float* g, const uint32_t* X, int64_t np, int n, float* acc, void* ws,
                            size_t ws_bytes, void* stream);
 

@@ -422,8 +422,7 @@ pm_status pm_interp_packed(const float* g, const uint32_t* X, int64_t np, int n,
   if (!valid_n(n) || !valid_np(np) || !g || (np > 0 && (!X || !acc)) || !all_a16(g, X, acc)) return PM_EINVAL;
   if (!ws || !aligned(ws)) return PM_EINVAL;
   if (ws_bytes < (size_t)n * n * n * sizeof(float4) + 256) return PM_ENOMEM;
-  // from 2^17 particles and a fortieth of the cells on, random order pays for the extra launches and the packing
-  if (np < 1 << 17 || 40 * np < (int64_t)n * n * n) return pm_interp(g, X, np, n, acc, stream);
+  if (!interp_packs(np, n)) return pm_interp(g, X, np, n, acc, stream);
   return interp_packed_launch(g, X, np, n, acc, static_cast<int*>(ws),
                               reinterpret_cast<float4*>(static_cast<char*>(ws) + 256), as_stream(stream));
 }

@@ -191,41 +191,166 @@ __global__ void __launch_bounds__(256) k_interp_kdk(const float* __restrict__ g,
   }
 }
 
-// Whether packing what scattered particles look up is worth it, from a sample of
-// their order (one block): *flag = 1 if `gain` lookups saved per row of cells that
-// 32 neighbouring particles touch exceed `cost`.
+// How many blocks of 4 x 4 rows of cells (columns along z) the warp's particles with
+// cells (ix, iy, .) touch: few in cell order and on a displaced lattice, whose particles
+// change rows all the time but stay near each other, so that L1 holds what they look
+// up; nearly 32 in random order.
+__device__ __forceinline__ int row_blocks(uint32_t ix, uint32_t iy) {
+  const unsigned same = __match_any_sync(0xffffffffu, (ix >> 2) << 16 | iy >> 2);
+  return __popc(__ballot_sync(0xffffffffu, (same & ((1u << (threadIdx.x & 31)) - 1u)) == 0u));
+}
+// Up to this many, the particles of a warp look up their cells one by one: a lattice
+// displaced by one cell (rms, each particle on its own; 3.6 blocks) is 1.4 to 1.7 times as
+// fast so, one displaced by three (10.8) half as fast.
+constexpr int kNearBlocks = 7;
+
+// A particle's cell and weights.
+struct PointWeights {
+  float wx[3], wy[3], wz[3];
+  int ix, iy, iz;
+  __device__ __forceinline__ PointWeights(uint32_t x, uint32_t y, uint32_t z, int log2n) {
+    tsc_weights(cell_offset(x, log2n), wx);
+    tsc_weights(cell_offset(y, log2n), wy);
+    tsc_weights(cell_offset(z, log2n), wz);
+    const int sh = 32 - log2n;
+    ix = (int)(x >> sh);
+    iy = (int)(y >> sh);
+    iz = (int)(z >> sh);
+  }
+};
+__device__ __forceinline__ uint32_t box_cell(int i, int j, int k, int log2n) {   // offset inside one box (below 2^30)
+  return (uint32_t)i << (2 * log2n) | (uint32_t)j << log2n | (uint32_t)k;
+}
+// The sums of k_interp_kdk from the three planes, cell by cell.
+__device__ __forceinline__ void gather_cells(const float* __restrict__ g, const PointWeights& w, int log2n, float (&a)[3]) {
+  const int m = (1 << log2n) - 1;
+  const int64_t N = (int64_t)1 << (3 * log2n);
+#pragma unroll
+  for (int ox = 0; ox < 3; ++ox) {
+#pragma unroll
+    for (int oy = 0; oy < 3; ++oy) {
+      const float wxy = w.wx[ox] * w.wy[oy];
+#pragma unroll
+      for (int oz = 0; oz < 3; ++oz) {
+        const uint32_t c = box_cell((w.ix + ox - 1) & m, (w.iy + oy - 1) & m, (w.iz + oz - 1) & m, log2n);
+        const float wc = wxy * w.wz[oz];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) a[d] = fmaf(wc, __ldg(g + d * N + c), a[d]);
+      }
+    }
+  }
+}
+
+// Inverse TSC at particles in any order: the sums of k_interp_kdk in the same order
+// (bitwise the same).  A warp whose particles are near each other looks up cell by cell
+// (its lanes share lines); one whose particles are scattered is bound by the line
+// lookups of L1, one per load and lane, and takes the three z cells of a row and
+// component in the aligned 16 bytes that hold the first and, where they go on, the
+// next 8: 40 lookups a particle instead of 81.
+//
+// 48 registers (five CTAs an SM): at 64 dense cell-ordered particles are up to 6%
+// slower, at 40 sparse ones up to 25%.  Against all warps cell by cell: 262144 particles
+// in cell order on 128^3 13.4 -> 12.3 us, 10^7 on 256^3 232 -> 224; in random order 64 ->
+// 34 and 3410 -> 3254; 256^3 on a lattice displaced by 0.3, 1 and 3 cells 429 -> 413, 983 ->
+// 979, 3176 -> 1706 us.
+__global__ void __launch_bounds__(256, 5) k_interp_points(const float* __restrict__ g, const uint32_t* __restrict__ Xs,
+                                                          int64_t np, int log2n, float* __restrict__ acc) {
+  pdl_entry();
+  const int m = (1 << log2n) - 1;
+  const int64_t N = (int64_t)1 << (3 * log2n);
+  const int64_t p = blockIdx.x * (int64_t)256 + threadIdx.x;
+  const bool live = p < np;
+  const uint32_t x = live ? __ldg(Xs + p) : 0u, y = live ? __ldg(Xs + np + p) : 0u, z = live ? __ldg(Xs + 2 * np + p) : 0u;
+  const PointWeights w(x, y, z, log2n);
+  const bool near = row_blocks(w.ix, w.iy) <= kNearBlocks;   // the same for the whole warp
+  if (!live) return;
+  float a[3] = {0.0f, 0.0f, 0.0f};
+  if (near) {
+    gather_cells(g, w, log2n, a);
+  } else {
+    const int z0 = (w.iz - 1) & m, k0 = z0 & ~3, k1 = (k0 + 4) & m;
+    const bool two = (z0 & 3) >= 2, odd = z0 & 1;   // the row's cells are z0 & 3 and the two after it
+#pragma unroll
+    for (int ox = 0; ox < 3; ++ox) {
+#pragma unroll
+      for (int oy = 0; oy < 3; ++oy) {
+        const float wxy = w.wx[ox] * w.wy[oy];
+        const float w0 = wxy * w.wz[0], w1 = wxy * w.wz[1], w2 = wxy * w.wz[2];
+        const uint32_t row = box_cell((w.ix + ox - 1) & m, (w.iy + oy - 1) & m, 0, log2n);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          const float* r = g + d * N + row;
+          const float4 u = __ldg(reinterpret_cast<const float4*>(r + k0));
+          float2 v = make_float2(0.0f, 0.0f);
+          if (two) v = __ldg(reinterpret_cast<const float2*>(r + k1));
+          const float c0 = two ? u.z : u.x, c1 = two ? u.w : u.y, c2 = two ? v.x : u.z, c3 = two ? v.y : u.w;
+          a[d] = fmaf(w0, odd ? c1 : c0, a[d]);
+          a[d] = fmaf(w1, odd ? c2 : c1, a[d]);
+          a[d] = fmaf(w2, odd ? c3 : c2, a[d]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) acc[d * np + p] = a[d];
+}
+
+// Group k of K of 32 neighbouring particles, spread evenly over the particles (np >= 32):
+// this lane's x and y cells.
+__device__ __forceinline__ uint2 sample_cells(const uint32_t* __restrict__ Xs, int64_t np, int log2n, int k, int K) {
+  const int64_t p = (np - 32) * k / (K - 1) + (threadIdx.x & 31);
+  return make_uint2(__ldg(Xs + p) >> (32 - log2n), __ldg(Xs + np + p) >> (32 - log2n));
+}
+
+// *flag = 1 if 32 neighbouring particles change their row of cells more than `rows`
+// times (a sample's mean; one block).
 __global__ void __launch_bounds__(1024) k_order_sample(const uint32_t* __restrict__ Xs, int64_t np, int log2n,
-                                                       float gain, float cost, int* __restrict__ flag) {
+                                                       float rows, int* __restrict__ flag) {
   pdl_entry();
   __shared__ int total;
   constexpr int PER_WARP = 8, GROUPS = 32 * PER_WARP;
-  const int sh = 32 - log2n, lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) total = 0;
   __syncthreads();
-  uint32_t x[PER_WARP], y[PER_WARP];
+  uint2 c[PER_WARP];
 #pragma unroll
-  for (int k = 0; k < PER_WARP; ++k) {   // groups spread evenly over the particles (np >= 32)
-    const int64_t p = (np - 32) * ((threadIdx.x >> 5) * PER_WARP + k) / (GROUPS - 1) + lane;
-    x[k] = __ldg(Xs + p) >> sh;
-    y[k] = __ldg(Xs + np + p) >> sh;
-  }
-  int rows = 0;
+  for (int k = 0; k < PER_WARP; ++k) c[k] = sample_cells(Xs, np, log2n, (threadIdx.x >> 5) * PER_WARP + k, GROUPS);
+  int sum = 0;
 #pragma unroll
   for (int k = 0; k < PER_WARP; ++k) {
-    const uint32_t row = (x[k] << log2n) | y[k], prev = __shfl_up_sync(0xffffffffu, row, 1);
-    rows += __popc(__ballot_sync(0xffffffffu, lane == 0 || row != prev));
+    const uint32_t row = (c[k].x << log2n) | c[k].y, prev = __shfl_up_sync(0xffffffffu, row, 1);
+    sum += __popc(__ballot_sync(0xffffffffu, lane == 0 || row != prev));
   }
-  if (lane == 0) atomicAdd(&total, rows);   // integers: any order
+  if (lane == 0) atomicAdd(&total, sum);   // integers: any order
   __syncthreads();
-  if (threadIdx.x == 0) *flag = gain * ((float)total / GROUPS) > cost;
+  if (threadIdx.x == 0) *flag = (float)total / GROUPS > rows;
 }
 
-// Cells of the force field as float4 (g_x, g_y, g_z, 0), if *flag; a thread
-// packs four at a time.
-__global__ void __launch_bounds__(256) k_pack_force(const float* __restrict__ g, float4* __restrict__ out, int64_t N,
-                                                    const int* __restrict__ flag) {
+// Cells of the force field as float4 (g_x, g_y, g_z, 0), four at a time a thread, if 32
+// neighbouring particles touch more than `blocks` blocks of rows (row_blocks, a
+// sample's mean), which goes to *flag.  Every block takes the sample (8 loads a thread,
+// one wave of blocks, all deciding the same): as a kernel before this one it costs the
+// particles that need no packing a launch more.
+constexpr int kPackBlocks = 4 * 152;
+__global__ void __launch_bounds__(256, 4) k_pack_force(const float* __restrict__ g, float4* __restrict__ out, int64_t N,
+                                                       const uint32_t* __restrict__ Xs, int64_t np, int log2n,
+                                                       float blocks, int* __restrict__ flag) {
   pdl_entry();
-  if (!*flag) return;
+  __shared__ int total;
+  constexpr int PER_WARP = 4, GROUPS = 8 * PER_WARP;
+  if (threadIdx.x == 0) total = 0;
+  __syncthreads();
+  uint2 cell[PER_WARP];
+#pragma unroll
+  for (int k = 0; k < PER_WARP; ++k) cell[k] = sample_cells(Xs, np, log2n, (threadIdx.x >> 5) * PER_WARP + k, GROUPS);
+  int sum = 0;
+#pragma unroll
+  for (int k = 0; k < PER_WARP; ++k) sum += row_blocks(cell[k].x, cell[k].y);
+  if ((threadIdx.x & 31) == 0) atomicAdd(&total, sum);   // integers: any order
+  __syncthreads();
+  const bool scattered = (float)total / GROUPS > blocks;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *flag = scattered;
+  if (!scattered) return;
   for (int64_t c = 4 * (blockIdx.x * (int64_t)256 + threadIdx.x); c < N; c += 4 * (int64_t)gridDim.x * 256) {
     const float4 x = __ldg(reinterpret_cast<const float4*>(g + c));
     const float4 y = __ldg(reinterpret_cast<const float4*>(g + N + c));
@@ -249,70 +374,52 @@ __device__ __forceinline__ CellPair load_pair(const float4* p) {
   return v;
 }
 
-// Inverse TSC at particles in any order, from the packed field if *flag, else
-// from the three planes: the sums of k_interp_kdk in the same order (bitwise the
-// same).  What bounds the gather at scattered positions is the line lookups of
-// L1, one per load and lane, so the three z cells of a row come in two aligned
-// 32-byte loads instead of nine 4-byte ones.  10^7 random positions on 256^3:
-// 3.3 -> 1.6 ms with the packing.
-__global__ void __launch_bounds__(256) k_interp_packed(const float4* __restrict__ gp, const float* __restrict__ g,
-                                                       const uint32_t* __restrict__ Xs, int64_t np, int log2n,
-                                                       float* __restrict__ acc, const int* __restrict__ flag) {
+// Inverse TSC from the packed field if *flag, else from the three planes, cell by cell:
+// the sums of k_interp_kdk in the same order (bitwise the same).  At scattered
+// positions the line lookups of L1 and the sectors of L2 bound it, so the three z cells
+// of a row come in two aligned 32-byte loads: 18 lookups and sectors a particle against
+// 40 and 34 of k_interp_points.
+//
+// 40 registers (six CTAs an SM), which cell-ordered particles gain by; with the rows in
+// a loop that is not unrolled the packed form needs no more and is as fast as with 64
+// (10^7 random on 256^3 1.51 ms, in cell order 206 us against 224).
+__global__ void __launch_bounds__(256, 6) k_interp_packed(const float4* __restrict__ gp, const float* __restrict__ g,
+                                                          const uint32_t* __restrict__ Xs, int64_t np, int log2n,
+                                                          float* __restrict__ acc, const int* __restrict__ flag) {
   pdl_entry();
-  const int m = (1 << log2n) - 1, sh = 32 - log2n;
-  const int64_t N = (int64_t)1 << (3 * log2n);
+  const int m = (1 << log2n) - 1;
   const int64_t p = blockIdx.x * (int64_t)256 + threadIdx.x;
   if (p >= np) return;
   const bool packed = *flag != 0;
-  const uint32_t x = __ldg(Xs + p), y = __ldg(Xs + np + p), z = __ldg(Xs + 2 * np + p);
-  float wx[3], wy[3], wz[3];
-  tsc_weights(cell_offset(x, log2n), wx);
-  tsc_weights(cell_offset(y, log2n), wy);
-  tsc_weights(cell_offset(z, log2n), wz);
-  const int ix = (int)(x >> sh), iy = (int)(y >> sh), iz = (int)(z >> sh);
-  float ax = 0.0f, ay = 0.0f, az = 0.0f;
+  const PointWeights w(__ldg(Xs + p), __ldg(Xs + np + p), __ldg(Xs + 2 * np + p), log2n);
+  float a[3] = {0.0f, 0.0f, 0.0f};
   if (packed) {
-    const int z0 = (iz - 1) & m, k0 = z0 & ~1, k1 = (k0 + 2) & m;
+    const int z0 = (w.iz - 1) & m, k0 = z0 & ~1, k1 = (k0 + 2) & m;
     const bool odd = z0 & 1;                     // the row's cells are b, a, b of two pairs, else a, b, a
-#pragma unroll
-    for (int ox = 0; ox < 3; ++ox) {
-#pragma unroll
-      for (int oy = 0; oy < 3; ++oy) {
-        const float4* row = gp + idx3((ix + ox - 1) & m, (iy + oy - 1) & m, 0, log2n);
-        const CellPair u = load_pair(row + k0), v = load_pair(row + k1);
-        const float wxy = wx[ox] * wy[oy];
-        const float w0 = wxy * wz[0], w1 = wxy * wz[1], w2 = wxy * wz[2];
-        ax = fmaf(w0, odd ? u.b.x : u.a.x, ax);
-        ay = fmaf(w0, odd ? u.b.y : u.a.y, ay);
-        az = fmaf(w0, odd ? u.b.z : u.a.z, az);
-        ax = fmaf(w1, odd ? v.a.x : u.b.x, ax);
-        ay = fmaf(w1, odd ? v.a.y : u.b.y, ay);
-        az = fmaf(w1, odd ? v.a.z : u.b.z, az);
-        ax = fmaf(w2, odd ? v.b.x : v.a.x, ax);
-        ay = fmaf(w2, odd ? v.b.y : v.a.y, ay);
-        az = fmaf(w2, odd ? v.b.z : v.a.z, az);
-      }
+#pragma unroll 1
+    for (int o = 0; o < 9; ++o) {
+      const int ox = o / 3, oy = o - 3 * ox;
+      const float wx = ox == 0 ? w.wx[0] : ox == 1 ? w.wx[1] : w.wx[2];
+      const float wy = oy == 0 ? w.wy[0] : oy == 1 ? w.wy[1] : w.wy[2];
+      const float4* row = gp + box_cell((w.ix + ox - 1) & m, (w.iy + oy - 1) & m, 0, log2n);
+      const CellPair u = load_pair(row + k0), v = load_pair(row + k1);
+      const float wxy = wx * wy;
+      const float w0 = wxy * w.wz[0], w1 = wxy * w.wz[1], w2 = wxy * w.wz[2];
+      a[0] = fmaf(w0, odd ? u.b.x : u.a.x, a[0]);
+      a[1] = fmaf(w0, odd ? u.b.y : u.a.y, a[1]);
+      a[2] = fmaf(w0, odd ? u.b.z : u.a.z, a[2]);
+      a[0] = fmaf(w1, odd ? v.a.x : u.b.x, a[0]);
+      a[1] = fmaf(w1, odd ? v.a.y : u.b.y, a[1]);
+      a[2] = fmaf(w1, odd ? v.a.z : u.b.z, a[2]);
+      a[0] = fmaf(w2, odd ? v.b.x : v.a.x, a[0]);
+      a[1] = fmaf(w2, odd ? v.b.y : v.a.y, a[1]);
+      a[2] = fmaf(w2, odd ? v.b.z : v.a.z, a[2]);
     }
   } else {
-#pragma unroll
-    for (int ox = 0; ox < 3; ++ox) {
-#pragma unroll
-      for (int oy = 0; oy < 3; ++oy) {
-        const float wxy = wx[ox] * wy[oy];
-#pragma unroll
-        for (int oz = 0; oz < 3; ++oz) {
-          const int64_t c = idx3((ix + ox - 1) & m, (iy + oy - 1) & m, (iz + oz - 1) & m, log2n);
-          const float w = wxy * wz[oz];
-          ax = fmaf(w, __ldg(g + c), ax);
-          ay = fmaf(w, __ldg(g + N + c), ay);
-          az = fmaf(w, __ldg(g + 2 * N + c), az);
-        }
-      }
-    }
+    gather_cells(g, w, log2n, a);
   }
-  acc[p] = ax;
-  acc[np + p] = ay;
-  acc[2 * np + p] = az;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) acc[d * np + p] = a[d];
 }
 
 // Force and inverse TSC + kick-drift-kick in one pass for cell-sorted
@@ -691,27 +798,24 @@ pm_status gradient_launch(const float* phi, const float* eps, float alpha, float
   return PM_EINVAL;
 }
 
-pm_status order_sample(const uint32_t* X, int64_t np, int n, float gain, float cost, int* flag, cudaStream_t s) {
+pm_status order_sample(const uint32_t* X, int64_t np, int n, float rows, int* flag, cudaStream_t s) {
   if (np < 32) return PM_EINVAL;
-  PM_LAUNCH(K_INTERP, 0.0, k_order_sample, 1, 1024, 0, s, X, np, ilog2(n), gain, cost, flag);
+  PM_LAUNCH(K_INTERP, 0.0, k_order_sample, 1, 1024, 0, s, X, np, ilog2(n), rows, flag);
   return launch_status();
 }
 
-// The field is packed where that pays.  Per warp of particles the gather costs
-// 81 lookups for each row of cells the warp touches from the planes and 18 (and
-// some more for the wider cells) from the packed field; packing a cell costs
-// about as much as 43 lookups a warp at one particle per cell (all measured at
-// 256^3: cell-ordered particles planes 0.36, packed 0.40 ms at one particle per
-// cell and 0.13, 0.23 ms at a quarter; in random order 5.7 against 2.6 and 1.4
-// against 0.73 ms).
+// The field is packed where that pays: from 5 blocks of rows in 32 neighbouring
+// particles on, more where the particles are few for the cells to be packed.  256^3 on a
+// lattice displaced by d cells (rms), planes / packed: d = 0.3 (1.9 blocks) 415 / 590 us, 1
+// (3.6) 960 / 990, 2 (7) 1960 / 1048; 128^3 56 / 84, 108 / 126, 199 / 140.
 pm_status interp_packed_launch(const float* g, const uint32_t* X, int64_t np, int n, float* acc, int* flag,
                                float4* packed, cudaStream_t s) {
   if (np < 32) return PM_EINVAL;
   const int64_t N = (int64_t)n * n * n;
-  const float gain = 81.0f - 18.0f, cost = 108.0f + 43.0f * (float)N / (float)np;
-  PM_TRY(order_sample(X, np, n, gain, cost, flag, s));
-  // counted as small, so that its launch overlaps the sample (most of it exits at once where the flag is 0)
-  PM_LAUNCH(K_INTERP, 0.0, k_pack_force, grid_for(N / 4, 256, 152 * 8), 256, 0, s, g, packed, N, flag);
+  const float blocks = 5.0f + (float)N / (float)np;
+  // counted as small, so that its launch overlaps its predecessor (it ends after the sample where the flag is 0)
+  PM_LAUNCH(K_INTERP, 0.0, k_pack_force, grid_for(N / 4, 256, kPackBlocks), 256, 0, s, g, packed, N, X, np, ilog2(n), blocks,
+            flag);
   PM_LAUNCH(K_INTERP, 12.0 * N + 24.0 * np, k_interp_packed, grid_for(np, 256), 256, 0, s, packed, g, X, np, ilog2(n),
             acc, flag);
   return launch_status();
@@ -805,6 +909,10 @@ pm_status interp_launch(const float* g, const uint32_t* Xs, const float* Vs, con
   const int64_t np_box = bt.B > 1 ? bt.np_box : np;
   const dim3 grid(grid_for(np_box, 256), 1, (unsigned)bt.B);
   if (!max_out) blockmax = nullptr;
+  if (mode == 0 && bt.B == 1 && !blockmax) {
+    PM_LAUNCH(K_INTERP, bytes, k_interp_points, grid.x, 256, 0, s, g, Xs, np, ilog2(n), acc);
+    return launch_status();
+  }
 #define PM_INTERP(MX)                                                                                               \
   PM_LAUNCH(K_INTERP, bytes, k_interp_kdk<MX>, grid, 256, 0, s, g, Xs, Vs, ids_in, np, ilog2(n), acc, Xo, Vo, ids_out, \
             dt_kick, drift_scale, mode, np_box, bt.dt_kick, bt.dt_drift, blockmax)

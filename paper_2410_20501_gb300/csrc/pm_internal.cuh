@@ -162,9 +162,9 @@ struct Packed {
   uint4* x = nullptr;
   int* scattered = nullptr;
 };
-// *flag = 1 if `gain` times the rows of cells that 32 neighbouring particles touch
-// (a sample's mean) exceeds `cost`; np >= 32.
-pm_status order_sample(const uint32_t* X, int64_t np, int n, float gain, float cost, int* flag, cudaStream_t s);
+// *flag = 1 if 32 neighbouring particles change their row of cells more than `rows`
+// times (a sample's mean); np >= 32.
+pm_status order_sample(const uint32_t* X, int64_t np, int n, float rows, int* flag, cudaStream_t s);
 // Where to pack the positions of particles in an unknown order (*pk unchanged: not at all).
 pm_status pack_scattered(const uint32_t* X, int64_t np, int n, const Workspace& w, Packed* pk, cudaStream_t s);
 
@@ -245,6 +245,15 @@ pm_status interp_launch(const float* g, const uint32_t* Xs, const float* Vs, con
                         int64_t np, int n, float* acc, uint32_t* Xo, float* Vo, uint32_t* ids_out,
                         float dt_kick, float dt_drift, int mode, cudaStream_t s,
                         const Batch& bt = Batch{}, float2* blockmax = nullptr, double* max_out = nullptr);
+// Whether particles in scattered order would pay for the sample and the packing
+// (interp_packed_launch) against k_interp_points, and those in cell order hardly pay for
+// the launch more (3 us, and some 5 us of the host's).  With / without, in random order
+// (us): 390001 on 64^3 34 / 50, 262144 on 128^3 35 / 34, 524288 55 / 65, 2097152 149 / 243;
+// on 256^3 524288 184 / 163, 1048576 275 / 347.  In cell order: 64^3 12 / 9.4, 128^3 16 /
+// 12, 19.5 / 16.9, 39.6 / 39.6; on 256^3 1048576 74 / 64, 4194304 125 / 130.  With one
+// launch and cell by cell (every order): 128^3 17.5 and 43.5 in cell order, 129 and 497 in
+// random order.
+inline bool interp_packs(int64_t np, int n) { return np >= 1 << 19 && 24 * np >= (int64_t)n * n * n; }
 // acc = the force at X (np >= 32), by way of the field packed as float4 cells
 // (packed: n^3, 32-byte aligned) where the particles' order makes that the
 // faster one; bitwise interp_launch.

@@ -605,7 +605,7 @@ pm_status pack_scattered(const uint32_t* X, int64_t np, int n, const Workspace& 
   pk->x = reinterpret_cast<uint4*>(w.moments);   // free until the deposit sums the crowded cells
   pk->scattered = reinterpret_cast<int*>(w.scalars + 40);
   static_assert(kMomStride * sizeof(float) >= sizeof(uint4), "room for the packed positions");
-  return order_sample(X, np, n, 1.0f, 8.0f, pk->scattered, s);
+  return order_sample(X, np, n, 8.0f, pk->scattered, s);
 }
 
 pm_status sort_cells(const uint32_t* X, int64_t np, int n, Workspace& w, cudaStream_t s, uint32_t* cellstart,

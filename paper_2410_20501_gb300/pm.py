@@ -343,10 +343,14 @@ def gradient(phi, order=5):
 
 
 def interp(g, X):
+    """Inverse TSC of g [3, n, n, n] at particles X in any order, [3, np].  From 2^19
+    particles and a 24th of the cells on a call also takes 16 n^3 bytes of scratch for
+    the field packed by cells (used if a sample of the particles is scattered); where
+    the device has no room for it the planes serve alone, with the same bits."""
     n = g.shape[1]
     np_ = X.shape[1]
     acc = torch.empty((3, np_), dtype=torch.float32, device=X.device)
-    if np_ >= 2 ** 17 and 40 * np_ >= n ** 3:   # below, pm_interp_packed takes pm_interp's way
+    if np_ >= 2 ** 19 and 24 * np_ >= n ** 3:   # below, pm_interp_packed takes pm_interp's way (interp_packs)
         try:
             ws = torch.empty(16 * n ** 3 + 256, dtype=torch.uint8, device=X.device)
         except torch.cuda.OutOfMemoryError:
