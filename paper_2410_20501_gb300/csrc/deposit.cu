@@ -625,9 +625,9 @@ pm_status crowded_moments(const uint32_t* Xs, int64_t np, const uint32_t* cellst
                           const Crowded& cr, cudaStream_t s) {
   if (!cr.runs || np == 0) return PM_OK;
   if (vals)
-    PM_LAUNCH(K_DEPOSIT, 0.0, k_list_moments<true>, 8 * 152, CT, 0, s, Xs, np, cellstart, cr, ilog2(n), vals);
+    PM_LAUNCH_EARLY(K_DEPOSIT, 0.0, k_list_moments<true>, 8 * 152, CT, 0, s, Xs, np, cellstart, cr, ilog2(n), vals);
   else
-    PM_LAUNCH(K_DEPOSIT, 0.0, k_list_moments<false>, 8 * 152, CT, 0, s, Xs, np, cellstart, cr, ilog2(n), vals);
+    PM_LAUNCH_EARLY(K_DEPOSIT, 0.0, k_list_moments<false>, 8 * 152, CT, 0, s, Xs, np, cellstart, cr, ilog2(n), vals);
   return PM_OK;
 }
 }  // namespace

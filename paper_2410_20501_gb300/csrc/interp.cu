@@ -800,7 +800,7 @@ pm_status gradient_launch(const float* phi, const float* eps, float alpha, float
 
 pm_status order_sample(const uint32_t* X, int64_t np, int n, float rows, int* flag, cudaStream_t s) {
   if (np < 32) return PM_EINVAL;
-  PM_LAUNCH(K_INTERP, 0.0, k_order_sample, 1, 1024, 0, s, X, np, ilog2(n), rows, flag);
+  PM_LAUNCH_EARLY(K_INTERP, 0.0, k_order_sample, 1, 1024, 0, s, X, np, ilog2(n), rows, flag);
   return launch_status();
 }
 
@@ -813,9 +813,8 @@ pm_status interp_packed_launch(const float* g, const uint32_t* X, int64_t np, in
   if (np < 32) return PM_EINVAL;
   const int64_t N = (int64_t)n * n * n;
   const float blocks = 5.0f + (float)N / (float)np;
-  // counted as small, so that its launch overlaps its predecessor (it ends after the sample where the flag is 0)
-  PM_LAUNCH(K_INTERP, 0.0, k_pack_force, grid_for(N / 4, 256, kPackBlocks), 256, 0, s, g, packed, N, X, np, ilog2(n), blocks,
-            flag);
+  PM_LAUNCH_EARLY(K_INTERP, 0.0, k_pack_force, grid_for(N / 4, 256, kPackBlocks), 256, 0, s, g, packed, N, X, np,
+                  ilog2(n), blocks, flag);
   PM_LAUNCH(K_INTERP, 12.0 * N + 24.0 * np, k_interp_packed, grid_for(np, 256), 256, 0, s, packed, g, X, np, ilog2(n),
             acc, flag);
   return launch_status();

@@ -305,9 +305,11 @@ namespace pmgb {
 // First statement of every kernel: waits until the kernels before it in the
 // stream have finished and their writes are visible, then lets the next
 // kernel's blocks be placed as soon as this kernel's last ones are.  Loads
-// through __ldg count as invariant and may be moved across a memory clobber,
-// but not out of the block behind a branch on a value the compiler cannot see
-// (always 0): they stay behind the wait.
+// through __ldg count as invariant, and the compiler's front end may move them
+// across a memory clobber, but not out of the block behind a branch on a value
+// that it cannot see (an output of the assembly, always 0).  The assembler can see
+// that 0; there the order rests on the wait itself, which it keeps memory accesses
+// behind as behind a barrier.
 __device__ __forceinline__ void pdl_entry() {
   unsigned never;
   asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(never)::"memory");
@@ -315,10 +317,13 @@ __device__ __forceinline__ void pdl_entry() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Launches a kernel; one that moves less than kOverlapBytes is set up while
-// its predecessor in the stream drains (programmatic dependent launch;
-// pdl_entry() orders their memory), because its time is mostly the gap between
-// two launches.  Measured: a 32^3 step of 40 launches 350 -> 256 us, a 128^3
+// Launches a kernel; with early it is set up while its predecessor in the stream
+// drains (programmatic dependent launch; pdl_entry() orders their memory).  That is
+// done for kernels that move less than kOverlapBytes, because their time is mostly
+// the gap between two launches, and (PM_LAUNCH_EARLY) for those that a device-side
+// count or flag leaves with little to do in most calls of any size: the listed cells
+// of the sort and the deposit, the sample of an order and the packing behind one.
+// Measured: a 32^3 step of 40 launches 350 -> 256 us, a 128^3
 // refined Poisson solve of 350 launches 3.05 -> 2.47 ms.  The line lies at the
 // 64^3 levels: an overlapped kernel runs with the shared-memory / L1 split its
 // predecessor left behind, which costs the kernels that live on L1 (transfers
@@ -326,7 +331,7 @@ __device__ __forceinline__ void pdl_entry() {
 // gather at 10^7 random positions 3.2 -> 13 ms).
 constexpr double kOverlapBytes = 4e6;
 template <class... P, class... A>
-inline void launch_kernel(double bytes, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+inline void launch_kernel(bool early, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                           A&&... args) {
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -337,20 +342,25 @@ inline void launch_kernel(double bytes, void (*kern)(P...), dim3 grid, dim3 bloc
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = &at;
-  cfg.numAttrs = bytes < kOverlapBytes ? 1 : 0;
+  cfg.numAttrs = early ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 }  // namespace pmgb
 #endif
 
 // Launch with instrumentation: `bytes` is the kernel's algorithmic (compulsory)
-// DRAM traffic for this launch, accumulated per class while timing is on.
-#define PM_LAUNCH(cls, bytes, kern, grid, block, smem, st, ...)       \
-  do {                                                                 \
-    ::pmgb::launch_begin((cls), (double)(bytes), (st));                \
-    ::pmgb::launch_kernel((bytes), kern, dim3(grid), dim3(block), (smem), (st), __VA_ARGS__); \
-    ::pmgb::launch_end((cls), (st));                                   \
+// DRAM traffic for this launch, accumulated per class while timing is on (0 for a
+// pass that rereads or rewrites what another launch of the class has counted).
+#define PM_LAUNCH_IF(early, cls, bytes, kern, grid, block, smem, st, ...)                     \
+  do {                                                                                        \
+    ::pmgb::launch_begin((cls), (double)(bytes), (st));                                       \
+    ::pmgb::launch_kernel((early), kern, dim3(grid), dim3(block), (smem), (st), __VA_ARGS__); \
+    ::pmgb::launch_end((cls), (st));                                                          \
   } while (0)
+#define PM_LAUNCH(cls, bytes, kern, grid, block, smem, st, ...) \
+  PM_LAUNCH_IF((bytes) < ::pmgb::kOverlapBytes, cls, bytes, kern, grid, block, smem, st, __VA_ARGS__)
+#define PM_LAUNCH_EARLY(cls, bytes, kern, grid, block, smem, st, ...) \
+  PM_LAUNCH_IF(true, cls, bytes, kern, grid, block, smem, st, __VA_ARGS__)
 
 #define PM_TRY(expr)                       \
   do {                                     \

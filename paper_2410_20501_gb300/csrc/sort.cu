@@ -634,7 +634,7 @@ pm_status sort_cells(const uint32_t* X, int64_t np, int n, Workspace& w, cudaStr
             ListHeads{w.smalls, w.meds, w.runs, w.bigs});
   PM_LAUNCH(K_ORDER, 4.0 * ncells + 8.0 * np, k_cell_order, grid_for(ncells / OC, KT), KT, 0, s, cellstart, ncells,
             w.perm, w.smalls, w.meds, w.runs, w.bigs);
-  PM_LAUNCH(K_ORDER, 0.0, k_cell_order_lists, LIST_BLOCKS, LT, 0, s, cellstart, w.smalls, w.meds, w.runs, w.bigs,
+  PM_LAUNCH_EARLY(K_ORDER, 0.0, k_cell_order_lists, LIST_BLOCKS, LT, 0, s, cellstart, w.smalls, w.meds, w.runs, w.bigs,
             w.perm, reinterpret_cast<uint32_t*>(w.keyrank));
   return launch_status();
 }
