@@ -135,7 +135,6 @@ size_t layout_workspace(Workspace* w, void* base, int n, int64_t np, uint32_t fl
     const int nl = n >> l;
     if (nl < 4) break;
     const size_t bytes = (size_t)nl * nl * nl * 4 * batch;
-    const bool streamed = nl >= 64;   // f(R) levels smoothed out of place need a ping-pong partner
     if (mg) {
       if (l > 0) {
         w->mg_u[l] = (float*)take(bytes);
@@ -149,7 +148,7 @@ size_t layout_workspace(Workspace* w, void* base, int n, int64_t np, uint32_t fl
         w->fr_r[l] = (float*)take(bytes);
         w->fr_b[l] = (float*)take(bytes);
       }
-      if (streamed) w->fr_alt[l] = (float*)take(bytes);
+      if (nl >= 128) w->fr_alt[l] = (float*)take(bytes);   // the levels of the marched sweeps (fr_smooth_nh)
     }
   }
   w->base = b;
