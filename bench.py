@@ -916,7 +916,7 @@ def main():
                     help="time one stage alone on synthetic inputs (for profilers)")
     ap.add_argument("--n", type=int, default=256, help="grid size for --stage")
     ap.add_argument("--smoother", type=int, default=2,
-                    help="--stage mg/fr: 2 fused sweeps, 1 colour passes, 0 two-sweep streaming")
+                    help="--stage mg/fr: 2 (or 0) fused sweeps, 1 colour passes")
     args = ap.parse_args()
     if args.stage == "adjoint":
         print(json.dumps(run_adjoint(args.n, fd_dirs=args.steps)[0]))

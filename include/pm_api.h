@@ -259,9 +259,8 @@ typedef struct {
   int cycles;        /* cycles to run when tol <= 0                           */
   double tol;        /* > 0: cycle until ||b - N(u)|| <= tol ||b|| (synchronises) */
   int max_cycles;
-  int smoother;      /* 2: one fused sweep per pass on levels with n >= 128,
-                        colour passes below; 1: colour passes everywhere; 0: two
-                        sweeps per pass on levels with n >= 128                 */
+  int smoother;      /* 2 or 0: one fused sweep per pass on levels with
+                        n >= 128, colour passes below; 1: colour passes everywhere */
   int nhs;           /* Hu-Sawicki exponent n: 1 (cubic per cell) or 2 (quartic,
                         §3.10); 0 is taken as 1                                 */
 } fr_params;
@@ -507,8 +506,8 @@ pm_status pm_gradient_batch(const float* phi, float* g, int n, int B, int order,
  * per box).  The boxes share *prm: one scale factor, cosmology, f_R0 and box
  * size (ensembles over seeds).  Exactly prm->cycles cycles per box (tol and
  * max_cycles are not used: no box waits on a residual, nothing synchronises
- * with the host); smoother 0 is taken as 2.  Box b gives bitwise fr_solve on
- * rho + b n^3 with the same parameters, smoother 2 (or 1) and tol <= 0.
+ * with the host).  Box b gives bitwise fr_solve on rho + b n^3 with the same
+ * parameters and tol <= 0.
  *   rho  [B][n^3] float32 densities (read); each box's float64 mean is removed
  *   eps  [B][n^3] float32 in: guesses, out: solutions (16-byte aligned)
  *   ws   pm_fr_batch_workspace_size(n, B) bytes, 256-byte aligned
@@ -525,7 +524,7 @@ pm_status pm_interp_batch(const float* g, const uint32_t* X, int64_t np_box, int
  * have_prev), gradient, inverse TSC, kick by dt_kick[b], drift by
  * dt_drift[b]; then have_prev = 1.  Per-box arrays are read on the device
  * when the kernels run.  PM_EINVAL for bad sizes, pointers, parameters
- * (mg.fixed_cycles < 1, cold_cycles < 1, smoother 0 is taken as 2). */
+ * (mg.fixed_cycles < 1, cold_cycles < 1). */
 pm_status pm_step_batch(pm_batch_state* s, const pm_batch_params* prm, void* stream);
 
 /* ------------------------------------------------------ host utilities ---- */

@@ -806,7 +806,6 @@ pm_status pm_step_batch(pm_batch_state* st_, const pm_batch_params* prm, void* s
   PM_TRY(permute_particles(perm, np, S.X, S.V, nullptr, w.Xs, w.Vs, nullptr, s));
   PM_TRY(deposit_sorted_batch(w.Xs, np_box, B, w.cellstart, n, w.rho, w.partials, w.box_mean, s, crowded(w)));
   mg_params mp = prm->mg;
-  if (mp.smoother == 0) mp.smoother = 2;
   mp.first_guess = S.have_prev ? MG_GUESS_SCALED : MG_GUESS_JACOBI;
   if (!S.have_prev) mp.fixed_cycles = prm->cold_cycles;
   PM_TRY(mg_solve_batch_src(Src{w.rho, 0.0f, w.box_mean, prm->src_scale}, S.phi, n, B, mp, prm->phi_rescale, w, s));
@@ -847,9 +846,7 @@ pm_status mg_solve_batch(const float* f, float* phi, int n, int B, const mg_para
   cudaStream_t s = as_stream(stream);
   const int64_t N = (int64_t)n * n * n;
   for (int b = 0; b < B; ++b) PM_TRY(grid_mean(f + b * N, N, w.partials, w.box_mean + b, s));
-  mg_params mp = *prm;
-  if (mp.smoother == 0) mp.smoother = 2;
-  return mg_solve_batch_src(Src{f, 1.0f, w.box_mean, nullptr}, phi, n, B, mp, nullptr, w, s);
+  return mg_solve_batch_src(Src{f, 1.0f, w.box_mean, nullptr}, phi, n, B, *prm, nullptr, w, s);
 }
 
 pm_status pm_fr_batch_workspace_size(int n, int B, size_t* bytes) {
@@ -872,9 +869,7 @@ pm_status fr_solve_batch(const float* rho, float* eps, int n, int B, const fr_pa
   double fbar, kappa, c2;
   fr_background(*prm, &fbar, &kappa, &c2);
   const float sb = (float)(-prm->Om * prm->a / c2);
-  fr_params fp = *prm;
-  if (fp.smoother == 0) fp.smoother = 2;   // the two-sweep streaming kernel is single-box
-  return fr_solve_src(Src{rho, sb, w.box_mean, nullptr}, eps, n, fp, nullptr, w, s, B);
+  return fr_solve_src(Src{rho, sb, w.box_mean, nullptr}, eps, n, *prm, nullptr, w, s, B);
 }
 
 pm_status pm_gradient_batch(const float* phi, float* g, int n, int B, int order, void* stream) {

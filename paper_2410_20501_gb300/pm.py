@@ -441,7 +441,7 @@ def timing_enable(on=True):
     _check(lib().pm_timing_enable(1 if on else 0), "pm_timing_enable")
 
 
-TUNE_SITES = ("force_chunk", "mg_fused_chunk", "mg_smoother")
+TUNE_SITES = {0: "force_chunk", 2: "mg_smoother"}
 
 
 def autotune(mode):
