@@ -20,9 +20,6 @@ namespace {
 constexpr float kSixth = 1.0f / 6.0f;
 
 __device__ __forceinline__ float load_mean(const Src& f) { return f.mean ? (float)*f.mean : 0.0f; }
-__device__ __forceinline__ float src_at(const Src& f, int64_t i, float mean) {
-  return f.s * (__ldg(f.p + i) - mean);
-}
 
 // Offset of cell (i, j, k) inside one box (n <= 1024: below 2^30).
 __device__ __forceinline__ uint32_t idx3(int i, int j, int k, int log2n) {
