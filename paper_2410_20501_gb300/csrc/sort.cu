@@ -596,16 +596,19 @@ int64_t sort_smalls_capacity(int64_t np) { return np / (kWalkRun + 1) + 2; }
 
 // Packing pays where the gather in cell order is scattered: three lookups of four
 // bytes a particle become one of sixteen (10^7 in random order on 256^3: 294 ->
-// 158 us, the count that packs 144 -> 155).  A sample of the order decides: from
-// eight rows of cells in 32 neighbouring particles on the planes' lookups no longer
-// share their lines.  Below 2^22 particles the planes (48 MB) stay in L2 and
-// the sample costs what it could save.
+// 158 us, the count that packs 144 -> 155).  A sample of the order decides: a lattice
+// displaced by 0.3 cells (rms) has 10.7 row changes in 32 neighbouring particles, by 1
+// 29.8, random order nearly 32.  Whole deposits, planes / packed: displaced by 0.3,
+// 8 10^6 particles on 128^3 420 / 428 us, 256^3 645 / 667; by 1 511 / 498 and 872 / 868; by 4
+// 565 / 535 and 1013 / 958; random, 4 10^6 on 64^3 308 / 291, 10^7 on 128^3 833 / 745, on
+// 256^3 931 / 844, 10^8 on 512^3 18.4 / 14.8 ms.  Below 2^22 particles the planes (48 MB)
+// stay in L2 and the sample costs what it could save.
 pm_status pack_scattered(const uint32_t* X, int64_t np, int n, const Workspace& w, Packed* pk, cudaStream_t s) {
   if (np < 1 << 22) return PM_OK;
   pk->x = reinterpret_cast<uint4*>(w.moments);   // free until the deposit sums the crowded cells
   pk->scattered = reinterpret_cast<int*>(w.scalars + 40);
   static_assert(kMomStride * sizeof(float) >= sizeof(uint4), "room for the packed positions");
-  return order_sample(X, np, n, 8.0f, pk->scattered, s);
+  return order_sample(X, np, n, 16.0f, pk->scattered, s);
 }
 
 pm_status sort_cells(const uint32_t* X, int64_t np, int n, Workspace& w, cudaStream_t s, uint32_t* cellstart,
